@@ -507,9 +507,9 @@ int32_t problem_create_impl(firal_handle* H, const firal_pool* pool, const firal
                  pool->x_dtype, st));
   TRYC(copy_rows(P->dbl, P->Ha.p, h0 ? h0->ho : nullptr, P->m, pool->h, P->n, P->c,
                  pool->h_dtype, st));
-  // class-major copy of h for the CUDA-core kernels; the tensor-core path reads its own bf16
-  // operands, prepared below, and makes this copy only if Round asks for it
-  if (!is_mixed(precision)) TRYC(class_major_h(P));
+  // class-major copy of h for the FP64 kernels; the FP32 kernels read rows, and the tensor-core
+  // path reads its own bf16 operands, prepared below
+  if (P->dbl) TRYC(class_major_h(P));
   TRYC(P->w_sig.ensure((size_t)P->N * vs));
   TRYC(P->w_p.ensure((size_t)P->N * vs));
   TRYC(P->zsave.ensure((size_t)P->N * vs));
@@ -620,7 +620,7 @@ int32_t round_setup(firal_problem* P, const void* zr, RoundSetup& rs) {
   FIRAL_TRY(rs.L.ensure(blk * 8));
   // B(H_o): weights 1 on labelled rows, 0 on the pool; Sigma_diamond: z on the pool (C-15)
   FIRAL_TRY(fill_weights(P->dbl, P->zsave.p, P->m, 1.0, nullptr, 0.0, P->n, st));
-  FIRAL_TRY(syrk_blocks(P, P->zsave.p, 0.0, nullptr, P->lambda, P->HoBlk.as<double>()));
+  FIRAL_TRY(syrk_blocks(P, P->zsave.p, 0.0, nullptr, P->lambda, P->HoBlk.as<double>(), P->m));
   FIRAL_TRY(fill_weights(P->dbl, P->zsave.p, P->m, 1.0, zr, 0.0, P->n, st));
   FIRAL_TRY(syrk_blocks(P, P->zsave.p, 0.0, nullptr, P->lambda, rs.Sig.as<double>()));
   FIRAL_TRY(chol_inv(P->dbl, rs.Sig.as<double>(), P->c, P->d, nullptr, nullptr, rs.L.as<double>(),
@@ -1319,7 +1319,7 @@ int32_t firal_problem_destroy(firal_problem* P) {
   const bool synced = cudaStreamSynchronize(P->H->stream) == cudaSuccess;
   exact_release(P);
   for (DBuf* b : {&P->Xa, &P->Ha, &P->HaT, &P->w_sig, &P->w_p, &P->S_p, &P->S_sig, &P->Pblk,
-                  &P->Minv, &P->HoBlk, &P->walpha, &P->Dpart, &P->syrk_part, &P->cgX, &P->cgR,
+                  &P->Minv, &P->HoBlk, &P->walpha, &P->Dpart, &P->syrk_part, &P->form_part, &P->form_pk, &P->blk_w, &P->cgX, &P->cgR,
                   &P->cgP, &P->cgQ, &P->cgZ, &P->cgcols, &P->cgpart1, &P->cgpart2, &P->V, &P->U,
                   &P->W, &P->HU, &P->g, &P->red, &P->zsave, &P->Xb, &P->Hb, &P->HbT, &P->Pb, &P->vmean, &P->qmean, &P->Aw, &P->Zp, &P->Hlo, &P->gq_ab,
                   &P->gq_m, &P->gq_part, &P->rtab, &P->rM, &P->tdev, &P->cen, &P->cen_off,
@@ -1489,7 +1489,9 @@ int32_t firal_precond_blocks(firal_problem* P, const void* z, double* out) {
   if (!P || !out) return record(H, fail(FIRAL_ERR_ARG, "bad precond_blocks arguments"));
   cudaStream_t st = P->H->stream;
   int32_t rc = fill_weights(P->dbl, P->zsave.p, P->m, 1.0, z, 0.0, P->n, st);
-  if (rc == FIRAL_OK) rc = syrk_blocks(P, P->zsave.p, 0.0, nullptr, P->lambda, out);
+  // without z only the labelled rows carry weight
+  if (rc == FIRAL_OK)
+    rc = syrk_blocks(P, P->zsave.p, 0.0, nullptr, P->lambda, out, z ? -1 : P->m);
   return record(H, rc);
 }
 

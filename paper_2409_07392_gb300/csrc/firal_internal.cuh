@@ -185,6 +185,9 @@ struct firal_problem {
   bool S_p_ready = false;
   // scratch of the Hessian apply
   firal::DBuf walpha, Dpart, syrk_part;
+  firal::DBuf form_pk;           // CUDA-core row forms: packed coefficient tiles
+  firal::DBuf form_part;         // CUDA-core quadratic forms and scores: per-block row partials
+  firal::DBuf blk_w;             // f32 block sums of Round: w h (1 - h) (N x c)
   // PCG
   firal::DBuf cgX, cgR, cgP, cgQ, cgZ, cgcols, cgpart1, cgpart2;
   firal::DBuf bcg;               // block PCG: class partials, s x s matrices, breakdown flag
@@ -269,19 +272,13 @@ int32_t block_axpy(firal_problem* P, void* Y, const void* Z, const void* Pm, con
 int32_t precond_apply(firal_problem* P, const void* R, int s, void* Z);
 int32_t tick(int64_t* t_dev, cudaStream_t st);
 int32_t set_step(int64_t* t_dev, int64_t v, cudaStream_t st);
-int32_t syrk_blocks(firal_problem* P, const void* w, double lamS, void* outS, double lamP,
-                    double* outP);
 int32_t syrk_reduce_f32(firal_problem* P, const float* partS, const float* partP, int splits,
                         double lamS, float* outS, double lamP, double* outP,
                         const float* addS = nullptr);
-int32_t hessian_apply_simt(firal_problem* P, const void* w, const void* Sblk, const void* V,
-                           int s, void* out, double* pq);
 int32_t combine_f32(firal_problem* P, const float* Sblk, const float* V, int splits, int s,
                     float* out, double* pq, const float* vmean);
 int32_t cg_init(firal_problem* P, const void* B, int s, double tol, int fixed);
 int32_t cg_iterate_tail(firal_problem* P, int s, double tol, int fixed);
-int32_t quad_forms_simt(firal_problem* P, const void* A, const void* B, int s, double scale,
-                        void* g);
 int32_t dot_scaled(bool dbl, const void* a, const void* b, int64_t total, double scale,
                    double* part, double* out, cudaStream_t st);
 int32_t md_step_simt(bool dbl, void* z, const void* g, int64_t n, double budget, double beta0,
@@ -289,6 +286,15 @@ int32_t md_step_simt(bool dbl, void* z, const void* g, int64_t n, double budget,
 int32_t md_step_sharded(firal_problem* P, void* z, const void* g, double budget, double beta0,
                         double* red, cudaStream_t st);
 int32_t block_dots(firal_problem* P, const void* V, const void* out, int s, double* pq);
+// ---- k_rows.cu (contractions over the rows on the CUDA cores; rows < 0: all of them)
+int32_t syrk_blocks(firal_problem* P, const void* w, double lamS, void* outS, double lamP,
+                    double* outP, int64_t rows = -1);
+int32_t hessian_apply_simt(firal_problem* P, const void* w, const void* Sblk, const void* V,
+                           int s, void* out, double* pq);
+int32_t quad_forms_simt(firal_problem* P, const void* A, const void* B, int s, double scale,
+                        void* g);
+int32_t round_scores_f32(firal_problem* P, const float* M1, const float* M2, const uint8_t* mask,
+                         double eta, double* pv, int64_t* pi, int np);
 // ---- k_linalg.cu
 int32_t chol_inv(bool dbl, const double* A, int c, int d, void* inv_t, double* inv_d,
                  double* L_out, int32_t* not_spd, cudaStream_t st);

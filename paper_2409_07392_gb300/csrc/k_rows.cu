@@ -1,0 +1,1408 @@
+// Contractions over the rows (points) on the CUDA cores, for FIRAL_FP32 and FIRAL_FP64 and for
+// the block sums of Round in every precision:
+//
+//   k_row_form   per-row forms of x_i.V (f32): the alpha of Lemma 1, the gradient's quadratic
+//                forms (eq. 11) and the eq. 14 scores of Round
+//   k_row_form_d the first two in FP64
+//   k_row_outer  sums over the rows of A[i][m] B[i][n]: the low-rank part of the Hessian apply
+//                (m = (probe, class), n = feature) and the weighted block sums of eq. 13
+//                (m = class, n = pair of features)
+//
+// Both are dense products with one operand made on the fly.  f32: 8 x 8 outputs per thread from
+// shared memory, plain fmaf: the packed form (fma.rn.f32x2) has the same peak on this part and
+// needs one operand duplicated, which cost more in shared-memory reads than it saved in issue
+// slots (43 against 53 TFLOP/s with operands resident).  FP64: the part issues two FP64
+// multiply-adds per SM and cycle, so operand traffic is free and what counts is that no lane
+// multiplies padding and every SM has work; tiles are 2 x 2 outputs per thread with the tile's
+// width taken from the problem instead of a power of two.
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "firal_internal.cuh"
+
+namespace firal {
+namespace {
+
+// ------------------------------------------------------------------------------------------
+// helpers
+// ------------------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+// copies n bytes to shared memory, zeros when !ok (the source address must still be valid)
+template <int n>
+__device__ __forceinline__ void cp_async(void* dst, const void* src, bool ok) {
+  const int sz = ok ? n : 0;
+  if (n == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src),
+                 "r"(sz)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(smem_addr(dst)), "l"(src),
+                 "n"(n), "r"(sz)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void cp_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
+// pair p of the upper triangle, row by row: (0,0) (0,1) .. (0,d-1) (1,1) ..
+__host__ __device__ inline void pair_of(int p, int d, int& e, int& f) {
+  // row e starts at e d - e (e - 1) / 2
+  const float b = 2.0f * d + 1.0f;
+  int r = (int)((b - sqrtf(b * b - 8.0f * p)) * 0.5f);
+  if (r < 0) r = 0;
+  if (r > d - 1) r = d - 1;
+  while (r > 0 && r * d - r * (r - 1) / 2 > p) --r;
+  while (r + 1 < d && (r + 1) * d - (r + 1) * r / 2 <= p) ++r;
+  e = r;
+  f = r + p - (r * d - r * (r - 1) / 2);
+}
+
+// ------------------------------------------------------------------------------------------
+// k_row_outer: part[split][m][n] = sum over the split's rows of A[i][m] B[i][n]
+//   OP 0 (low-rank part): m = j c + k, A = h_ik walpha_ij; n = e, B = x_ie
+//   OP 1 (block sums):    m = which c + k, A = w_i h_ik (which 0) or w_i h_ik (1 - h_ik)
+//                         (which 1); n = pair (e, f), e <= f, B = x_ie x_if
+// The tile is GM TM x GN TN outputs, GM GN threads active; rows in steps of BK, the next
+// step's h, x and factors in flight (cp.async) while this one is multiplied.
+// ------------------------------------------------------------------------------------------
+constexpr int OUTER_BK = 16;
+
+template <class T>
+struct OuterArgs {
+  const T* Xa;
+  const T* Ha;
+  const T* w;        // OP 1: row weights; OP 0: walpha (N x s)
+  int64_t r0, r1;    // rows of the sum
+  int64_t rps;       // rows per split
+  int d, c, s;
+  int which0;        // OP 1: first output kind (0: w h, 1: w h (1 - h))
+  int M, Nn;         // outputs in all
+  int GM, GN;
+  T* part;
+};
+
+// FP64: 2 x 2 outputs per thread.
+template <int OP>
+__global__ __launch_bounds__(512, 1) void k_row_outer_d(const OuterArgs<double> a) {
+  constexpr int BK = OUTER_BK, TM = 2, TN = 2;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int BM = a.GM * TM, BN = a.GN * TN;
+  const int d = a.d, c = a.c;
+  const int dS = OP == 0 ? BN : (d + 1) & ~1;              // staged x row
+  const int bm0 = blockIdx.x * BM, bn0 = blockIdx.y * BN;
+  // probes (OP 0) the tile's rows m belong to; one factor per row otherwise
+  const int j0 = OP == 0 ? bm0 / c : 0;
+  const int nj = OP == 0 ? (min(bm0 + BM, a.M) - 1) / c - j0 + 1 : 1;
+  const int njS = OP == 0 ? (BM + c - 1) / c + 1 : 1;
+  double* As = (double*)smem_raw;              // [2][BK][BM]
+  double* Xs = As + 2 * BK * BM;               // [2][BK][dS]
+  double* Ws = Xs + 2 * BK * dS;               // [2][BK][njS]
+  double* Bs = Ws + 2 * BK * njS;              // OP 1: [BK][BN]
+  int* mcol = (int*)(OP == 0 ? Bs : Bs + BK * BN);   // [BM] class | (probe or kind) << 16
+  int* nmap = mcol + BM;                       // OP 1: [BN] e | f << 16
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+  const int mg = tid / a.GN, ng = tid - mg * a.GN;
+  const bool act = mg < a.GM;
+  for (int q = tid; q < BM; q += nt) {
+    const int m = bm0 + q;
+    mcol[q] = m < a.M ? (m % c) | ((OP == 0 ? m / c - j0 : m / c + a.which0) << 16) : -1;
+  }
+  if (OP == 1)
+    for (int q = tid; q < BN; q += nt) {
+      int e = 0, f = 0;
+      if (bn0 + q < a.Nn) pair_of(bn0 + q, d, e, f);
+      nmap[q] = bn0 + q < a.Nn ? e | (f << 16) : -1;
+    }
+  __syncthreads();
+  const int64_t i0 = a.r0 + (int64_t)blockIdx.z * a.rps;
+  const int64_t i1 = min(a.r1, i0 + a.rps);
+  const int steps = i0 < i1 ? (int)((i1 - i0 + BK - 1) / BK) : 0;
+
+  auto stage = [&](int t, int b) {
+    const int64_t ib = i0 + (int64_t)t * BK;
+    double* A = As + b * BK * BM;
+    double* X = Xs + b * BK * dS;
+    double* W = Ws + b * BK * njS;
+    for (int p = wid; p < BK; p += nw) {
+      const int64_t i = ib + p;
+      const bool rv = i < i1;
+      const double* hrow = a.Ha + (rv ? i : a.r0) * c;
+      for (int q = lane; q < BM; q += 32) {
+        const int mc = mcol[q];
+        cp_async<8>(A + p * BM + q, hrow + (mc < 0 ? 0 : mc & 0xffff), rv && mc >= 0);
+      }
+      const double* xrow = a.Xa + (rv ? i : a.r0) * d;
+      const int xo = OP == 0 ? bn0 : 0;
+      for (int q = lane; q < dS; q += 32)
+        cp_async<8>(X + p * dS + q, xrow + (xo + q < d ? xo + q : 0), rv && xo + q < d);
+      if (OP == 0) {
+        const double* wrow = a.w + (rv ? i : a.r0) * a.s + j0;
+        for (int q = lane; q < nj; q += 32) cp_async<8>(W + p * njS + q, wrow + q, rv);
+      } else if (lane == 0) {
+        cp_async<8>(W + p, a.w + (rv ? i : a.r0), rv);
+      }
+    }
+    cp_commit();
+  };
+
+  double acc[TM][TN] = {};
+  if (steps > 0) stage(0, 0);
+  for (int t = 0; t < steps; ++t) {
+    const int b = t & 1;
+    cp_wait0();
+    __syncthreads();   // step t has arrived for everyone; step t - 1 is multiplied
+    if (t + 1 < steps) stage(t + 1, b ^ 1);
+    double* A = As + b * BK * BM;
+    const double* X = Xs + b * BK * dS;
+    const double* W = Ws + b * BK * njS;
+    const int pn = (int)min((int64_t)BK, i1 - i0 - (int64_t)t * BK);
+    for (int p = wid; p < pn; p += nw) {
+      for (int q = lane; q < BM; q += 32) {
+        const int mc = mcol[q] >> 16;
+        const double h = A[p * BM + q];
+        if (OP == 0) {
+          A[p * BM + q] = mc < 0 ? 0.0 : h * W[p * njS + mc];
+        } else {
+          const double wh = W[p] * h;
+          A[p * BM + q] = mc == 1 ? wh * (1.0 - h) : wh;
+        }
+      }
+      if (OP == 1)
+        for (int q = lane; q < BN; q += 32) {
+          const int ef = nmap[q];
+          Bs[p * BN + q] = ef < 0 ? 0.0 : X[p * dS + (ef & 0xffff)] * X[p * dS + (ef >> 16)];
+        }
+    }
+    __syncthreads();
+    if (act) {
+      const double* B = OP == 0 ? X : Bs;
+#pragma unroll 4
+      for (int p = 0; p < pn; ++p) {
+        const double2 av = *reinterpret_cast<const double2*>(A + p * BM + mg * 2);
+        const double2 bv = *reinterpret_cast<const double2*>(B + p * BN + ng * 2);
+        acc[0][0] = fma(av.x, bv.x, acc[0][0]);
+        acc[0][1] = fma(av.x, bv.y, acc[0][1]);
+        acc[1][0] = fma(av.y, bv.x, acc[1][0]);
+        acc[1][1] = fma(av.y, bv.y, acc[1][1]);
+      }
+    }
+  }
+  if (!act) return;
+  double* out = a.part + (int64_t)blockIdx.z * a.M * a.Nn;
+#pragma unroll
+  for (int x = 0; x < TM; ++x) {
+    const int m = bm0 + mg * 2 + x;
+    if (m >= a.M) continue;
+#pragma unroll
+    for (int y = 0; y < TN; ++y) {
+      const int n = bn0 + ng * 2 + y;
+      if (n < a.Nn) out[(int64_t)m * a.Nn + n] = acc[x][y];
+    }
+  }
+}
+
+// f32: TM x 8 outputs per thread.  Row q of a thread's TM is tile row
+// (q / 4) 4 GM + 4 mg + q % 4, column y is (y / 4) 4 GN + 4 ng + y % 4; a warp covers 8 column
+// groups x 4 row groups where GN allows, which is the fewest shared-memory wavefronts.
+// One barrier per step.  A step's multiply-adds run in four quarters; each quarter first reads
+// its share of the next step's operands (h and its factors from global memory, OP 0's x too;
+// OP 1: two rows of pair factors from x in shared memory, and x of the step after from global
+// memory), multiplies, and then writes that share to the other buffer, so that the loads'
+// latency is covered and only one share is held in registers.
+// Bound by issue slots: the multiply-adds alone run at 53-57 TFLOP/s (78 is the part's peak, 65
+// an 8 x 8 outer product from registers), with the operands' loads and stores 43 (low-rank part,
+// n = 21,000, c = 1000, d = 64, s = 16: 1.01 ms, 2.88 before; Round's blocks at n = 1M, d = 128,
+// c = 100: 75 ms, 177 before) and, forming pairs, 29 (block sums, same n, c, d: 3.0 ms, 8.6
+// before).  Staging by cp.async with a separate pass over the tile ran at 31.
+// VH 4: rows of h and x 16-byte aligned, 16 rows per step; otherwise VH values of h per load
+// (8-byte aligned rows: 2), x by single values, 8 rows per step.
+template <int OP, int VH>
+struct OuterCfg {
+  static constexpr int BK = VH == 4 ? 16 : 8;
+  static constexpr int NI = VH == 4 ? 4 : VH == 2 ? 8 : 12;   // loads of h per thread and step
+  static constexpr int VX = VH == 4 ? 4 : 1;
+  static constexpr int NX = VH == 4 ? 4 : 8;                  // loads of x per thread and step
+};
+template <int OP, int TM, int VH>
+__global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a) {
+  using Cfg = OuterCfg<OP, VH>;
+  constexpr int BK = Cfg::BK, NI = Cfg::NI, NX = Cfg::NX, VX = Cfg::VX, TN = 8;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int BM = a.GM * TM, BN = a.GN * TN;
+  const int d = a.d, c = a.c;
+  const int dS = OP == 0 ? BN : (d + 3) & ~3;              // staged x row
+  const int bm0 = blockIdx.x * BM, bn0 = blockIdx.y * BN;
+  const int j0 = OP == 0 ? bm0 / c : 0;
+  float* As = (float*)smem_raw;                // [2][BK][BM]
+  float* Bs = As + 2 * BK * BM;                // [2][BK][BN]
+  float* Xs = Bs + 2 * BK * BN;                // OP 1: [2][BK][dS]
+  int* mcol = (int*)(OP == 0 ? Xs : Xs + 2 * BK * dS);   // [BM] class | (probe or kind) << 16
+  int* nmap = mcol + BM;                       // OP 1: [BN] e | f << 16
+  const int tid = threadIdx.x, nt = blockDim.x;
+  int mg, ng;
+  if ((a.GN & 7) == 0) {
+    mg = (tid >> 3) % a.GM;
+    ng = (tid >> 3) / a.GM * 8 + (tid & 7);
+  } else {
+    mg = tid / a.GN;
+    ng = tid - mg * a.GN;
+  }
+  const bool act = mg < a.GM && ng < a.GN;
+  for (int q = tid; q < BM; q += nt) {
+    const int m = bm0 + q;
+    mcol[q] = m < a.M ? (m % c) | ((OP == 0 ? m / c - j0 : m / c + a.which0) << 16) : -1;
+  }
+  if (OP == 1)
+    for (int q = tid; q < BN; q += nt) {
+      int e = 0, f = 0;
+      if (bn0 + q < a.Nn) pair_of(bn0 + q, d, e, f);
+      nmap[q] = bn0 + q < a.Nn ? e | (f << 16) : -1;
+    }
+  __syncthreads();
+  const int64_t i0 = a.r0 + (int64_t)blockIdx.z * a.rps;
+  const int64_t i1 = min(a.r1, i0 + a.rps);
+  const int rows = i0 < i1 ? (int)(i1 - i0) : 0;
+  const int steps = (rows + BK - 1) / BK;
+  const int hw = BM / VH, hn = BK * hw;        // loads of h per row and step
+  const int xw = dS / VX, xn = BK * xw;        // loads of x
+  const int xo = OP == 0 ? bn0 : 0;
+  // the loads' places, fixed over the steps: class | (probe or kind) << 12 | row of the step << 24
+  // (-1: none), and the offset of x
+  int hp[NI], xp[NX];
+#pragma unroll
+  for (int u = 0; u < NI; ++u) {
+    const int idx = tid + u * nt, pr = idx / hw, mc = idx < hn ? mcol[(idx - pr * hw) * VH] : -1;
+    hp[u] = mc < 0 ? -1 : (mc & 0xffff) | (mc >> 16) << 12 | pr << 24;
+  }
+#pragma unroll
+  for (int u = 0; u < NX; ++u) {
+    const int idx = tid + u * nt, pr = idx / xw, q = (idx - pr * xw) * VX;
+    xp[u] = idx < xn && xo + q < d ? pr * d + q : -1;
+  }
+  constexpr int QI = NI / 4, QX = NX / 4;   // loads per quarter
+  float hr[QI][VH], wr[QI], xr[QX][VX];
+  auto load_h = [&](int t, int qt) {
+    const int64_t ib = i0 + (int64_t)t * BK;
+    const int lim = min(BK, rows - t * BK);
+    const float* H = a.Ha + ib * c;
+    const float* W = OP == 0 ? a.w + ib * a.s + j0 : a.w + ib;
+#pragma unroll
+    for (int v = 0; v < QI; ++v) {
+      const int hu = hp[qt * QI + v], pr = hu >> 24;
+#pragma unroll
+      for (int z = 0; z < VH; ++z) hr[v][z] = 0.0f;
+      wr[v] = 0.0f;
+      if (hu >= 0 && pr < lim) {
+        const float* h = H + (pr * c + (hu & 0xfff));
+        if (VH == 4) {
+          const float4 r = *reinterpret_cast<const float4*>(h);
+          hr[v][0] = r.x;
+          hr[v][VH > 1 ? 1 : 0] = r.y;
+          hr[v][VH > 2 ? 2 : 0] = r.z;
+          hr[v][VH > 3 ? 3 : 0] = r.w;
+        } else if (VH == 2) {
+          const float2 r = *reinterpret_cast<const float2*>(h);
+          hr[v][0] = r.x;
+          hr[v][VH > 1 ? 1 : 0] = r.y;
+        } else {
+          hr[v][0] = *h;
+        }
+        wr[v] = OP == 0 ? W[pr * a.s + (hu >> 12 & 0xfff)] : W[pr];
+      }
+    }
+  };
+  auto store_a = [&](int t, int qt) {
+    float* A = As + (t & 1) * BK * BM;
+#pragma unroll
+    for (int v = 0; v < QI; ++v) {
+      const int idx = tid + (qt * QI + v) * nt;
+      if (idx >= hn) break;
+      float r[VH];
+#pragma unroll
+      for (int z = 0; z < VH; ++z) {
+        r[z] = wr[v] * hr[v][z];
+        if (OP == 1 && (hp[qt * QI + v] & 0x1000)) r[z] *= 1.0f - hr[v][z];
+      }
+      if (VH == 4)
+        *reinterpret_cast<float4*>(A + idx * VH) =
+            make_float4(r[0], r[VH > 1 ? 1 : 0], r[VH > 2 ? 2 : 0], r[VH > 3 ? 3 : 0]);
+      else if (VH == 2)
+        *reinterpret_cast<float2*>(A + idx * VH) = make_float2(r[0], r[VH > 1 ? 1 : 0]);
+      else
+        A[idx] = r[0];
+    }
+  };
+  auto load_x = [&](int t, int qt) {
+    const float* X = a.Xa + (i0 + (int64_t)t * BK) * d + xo;
+    const int lim = min(BK, rows - t * BK) * d;   // offsets of a step's rows lie below rows d
+#pragma unroll
+    for (int v = 0; v < QX; ++v) {
+      const int xu = xp[qt * QX + v];
+      const bool ok = xu >= 0 && xu < lim;
+      if (VX == 4) {
+        const float4 r = ok ? *reinterpret_cast<const float4*>(X + xu)
+                            : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        xr[v][0] = r.x;
+        xr[v][VX > 1 ? 1 : 0] = r.y;
+        xr[v][VX > 2 ? 2 : 0] = r.z;
+        xr[v][VX > 3 ? 3 : 0] = r.w;
+      } else {
+        xr[v][0] = ok ? X[xu] : 0.0f;
+      }
+    }
+  };
+  auto store_x = [&](int t, int qt) {
+    float* X = OP == 0 ? Bs + (t & 1) * BK * BN : Xs + (t & 1) * BK * dS;
+#pragma unroll
+    for (int v = 0; v < QX; ++v) {
+      const int idx = tid + (qt * QX + v) * nt;
+      if (idx >= xn) break;
+      if (VX == 4)
+        *reinterpret_cast<float4*>(X + idx * 4) = make_float4(
+            xr[v][0], xr[v][VX > 1 ? 1 : 0], xr[v][VX > 2 ? 2 : 0], xr[v][VX > 3 ? 3 : 0]);
+      else
+        X[idx] = xr[v][0];
+    }
+  };
+  // pairs of step t: warp w takes rows w, w + warps, ..; lane l columns l + 32 i, quarter by
+  // quarter of the multiply-adds (i = quarter, quarter + 4, ..)
+  const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
+  auto pair_rows = [&](int t, int q, int pr0) {
+    const float* X = Xs + (t & 1) * BK * dS;
+    float* B = Bs + (t & 1) * BK * BN + q;
+    const int ef = nmap[q];
+    const float* xe = X + (ef < 0 ? 0 : ef & 0xffff);
+    const float* xf = X + (ef < 0 ? 0 : ef >> 16);
+    for (int pr = pr0; pr < BK; pr += nw) B[pr * BN] = ef < 0 ? 0.0f : xe[pr * dS] * xf[pr * dS];
+  };
+
+  float acc[TM][TN];
+#pragma unroll
+  for (int x = 0; x < TM; ++x)
+#pragma unroll
+    for (int y = 0; y < TN; ++y) acc[x][y] = 0.0f;
+  if (steps > 0) {
+#pragma unroll
+    for (int qt = 0; qt < 4; ++qt) {
+      load_h(0, qt);
+      load_x(0, qt);
+      store_a(0, qt);
+      store_x(0, qt);
+      if (OP == 1 && steps > 1) {
+        load_x(1, qt);
+        store_x(1, qt);
+      }
+    }
+    if (OP == 1) {
+      __syncthreads();
+      for (int q = lane; q < BN; q += 32) pair_rows(0, q, wid);
+    }
+    __syncthreads();
+  }
+  for (int t = 0; t < steps; ++t) {
+    const bool more = t + 1 < steps, morex = OP == 0 ? more : t + 2 < steps;
+    const float* A = As + (t & 1) * BK * BM + mg * 4;
+    const float* B = Bs + (t & 1) * BK * BN + ng * 4;
+    const int va = a.GM * 4, vb = a.GN * 4;
+#pragma unroll
+    for (int qt = 0; qt < 4; ++qt) {
+      if (more) load_h(t + 1, qt);
+      if (morex) load_x(OP == 0 ? t + 1 : t + 2, qt);
+      float pe[2] = {0.0f, 0.0f}, pf[2] = {0.0f, 0.0f};
+      const int pq = lane + qt * 32;
+      const bool pair = OP == 1 && more && pq < BN;
+      if (pair) {
+        const int ef = nmap[pq];
+        const float* X = Xs + ((t + 1) & 1) * BK * dS + wid * dS;
+        if (ef >= 0) {
+          pe[0] = X[ef & 0xffff];
+          pf[0] = X[ef >> 16];
+          if (wid + nw < BK) {
+            pe[1] = X[nw * dS + (ef & 0xffff)];
+            pf[1] = X[nw * dS + (ef >> 16)];
+          }
+        }
+      }
+      if (act) {
+#pragma unroll
+        for (int q = 0; q < BK / 4; ++q) {   // rows past the end are zero in both tiles
+          float av[TM], bv[TN];
+#pragma unroll
+          for (int v = 0; v < TM / 4; ++v)
+            *reinterpret_cast<float4*>(av + 4 * v) =
+                *reinterpret_cast<const float4*>(A + q * BM + v * va);
+#pragma unroll
+          for (int v = 0; v < TN / 4; ++v)
+            *reinterpret_cast<float4*>(bv + 4 * v) =
+                *reinterpret_cast<const float4*>(B + q * BN + v * vb);
+#pragma unroll
+          for (int x = 0; x < TM; ++x)
+#pragma unroll
+            for (int y = 0; y < TN; ++y) acc[x][y] = fmaf(av[x], bv[y], acc[x][y]);
+        }
+        A += BK / 4 * BM;
+        B += BK / 4 * BN;
+      }
+      if (pair) {
+        float* P = Bs + ((t + 1) & 1) * BK * BN + wid * BN + pq;
+        P[0] = pe[0] * pf[0];
+        if (wid + nw < BK) P[nw * BN] = pe[1] * pf[1];
+        if (wid + 2 * nw < BK) pair_rows(t + 1, pq, wid + 2 * nw);
+        for (int q = pq + 128; q < BN; q += 128) pair_rows(t + 1, q, wid);
+      }
+      if (more) store_a(t + 1, qt);
+      if (morex) store_x(OP == 0 ? t + 1 : t + 2, qt);
+    }
+    __syncthreads();
+  }
+  if (!act) return;
+  float* out = a.part + (int64_t)blockIdx.z * a.M * a.Nn;
+#pragma unroll
+  for (int x = 0; x < TM; ++x) {
+    const int m = bm0 + (x / 4) * a.GM * 4 + mg * 4 + x % 4;
+    if (m >= a.M) continue;
+#pragma unroll
+    for (int y = 0; y < TN; ++y) {
+      const int n = bn0 + (y / 4) * a.GN * 4 + ng * 4 + y % 4;
+      if (n < a.Nn) out[(int64_t)m * a.Nn + n] = acc[x][y];
+    }
+  }
+}
+
+template <int OP>
+size_t outer_smem_d(int GM, int GN, int d, int c) {
+  constexpr int BK = OUTER_BK;
+  const int BM = GM * 2, BN = GN * 2;
+  const int dS = OP == 0 ? BN : (d + 1) & ~1;
+  const int njS = OP == 0 ? (BM + c - 1) / c + 1 : 1;
+  size_t el = (size_t)2 * BK * BM + 2 * BK * dS + 2 * BK * njS;
+  if (OP == 1) el += (size_t)BK * BN;
+  return el * sizeof(double) + ((size_t)BM + (OP == 1 ? BN : 0)) * sizeof(int);
+}
+
+bool aligned(const void* q, int bytes) { return reinterpret_cast<uintptr_t>(q) % bytes == 0; }
+// values of a row of `cols` f32 that one load may take
+int row_vec(const void* q, int cols) {
+  return cols % 4 == 0 && aligned(q, 16) ? 4 : cols % 2 == 0 && aligned(q, 8) ? 2 : 1;
+}
+// k_row_outer_f's VH: 4 needs both operands' rows aligned
+int outer_vh(const OuterArgs<float>& a) {
+  const int h = row_vec(a.Ha, a.c);
+  return h == 4 && row_vec(a.Xa, a.d) == 4 ? 4 : h >= 2 ? 2 : 1;
+}
+int outer_vh(const OuterArgs<double>&) { return 1; }
+
+// Tile and row splits for M x Nn outputs.
+struct OuterPlan {
+  int TM, GM, GN, threads, tm, tn, splits;
+  int64_t rps;
+};
+
+// The tile takes its width from the outputs (groups of TN columns up to 128 of them), then as
+// many row groups as the block has threads for, both cut to equal tiles, so that little of a
+// tile is padding at any class count or feature width (the fixed 64 x 64 tile multiplied 54
+// empty class columns at c = 10: 413 us a launch at n = 50,000, d = 50, s = 20; now 56).
+// Splits: enough blocks for two per SM (one at FP64: 512 threads), whole waves where the row
+// count allows it, at most 1024 rows in one f32 sum of the low-rank part, partials of at most
+// 512 MiB.  (The block sums take their ranges from block_ranges.)
+template <int OP, class T>
+OuterPlan outer_plan(const OuterArgs<T>& a, int sms) {
+  const bool dbl = sizeof(T) == 8;
+  const int M = a.M, Nn = a.Nn, vh = outer_vh(a);
+  const int64_t rows = a.r1 - a.r0;
+  const int TN = dbl ? 2 : 8;
+  OuterPlan p{};
+  p.TM = dbl ? 2 : (OP == 1 && M <= 32 ? 4 : 8);
+  const int nt = dbl ? 512 : 256;
+  const int max_gn = dbl ? 64 : 16;
+  const int ng = (Nn + TN - 1) / TN, mg = (M + p.TM - 1) / p.TM;
+  int gn = std::min(ng, max_gn);
+  if (mg < nt / gn) gn = std::min(ng, std::min(nt / mg, dbl ? 128 : 64));
+  p.tn = (ng + gn - 1) / gn;
+  p.GN = (ng + p.tn - 1) / p.tn;
+  int gm = std::min(mg, nt / p.GN);
+  // f32: the block's threads must also cover a step's loads
+  const int bk = vh == 4 ? 16 : 8, ni = vh == 4 ? 4 : vh == 2 ? 8 : 12, nx = vh == 4 ? 4 : 8;
+  for (;; --gm) {
+    p.tm = (mg + gm - 1) / gm;
+    p.GM = (mg + p.tm - 1) / p.tm;
+    int need = p.GM * p.GN;
+    if (!dbl) {
+      const int hn = bk * p.GM * p.TM / vh;
+      const int xn = bk * (OP == 0 ? p.GN * 8 : (a.d + 3) / 4 * 4) / (vh == 4 ? 4 : 1);
+      need = std::max({need, (hn + ni - 1) / ni, (xn + nx - 1) / nx});
+    }
+    p.threads = std::max(128, (need + 31) / 32 * 32);
+    if (p.threads <= nt || gm == 1) break;
+  }
+  const int64_t tiles = (int64_t)p.tm * p.tn;
+  const int64_t slots = (int64_t)sms * (dbl ? 1 : 2);
+  int64_t want = std::max<int64_t>(1, slots / tiles);
+  // several waves: round the block count to whole waves
+  const int64_t max_rows = dbl ? (int64_t)1 << 40 : 1024;
+  want = std::max<int64_t>(want, (rows + max_rows - 1) / max_rows);
+  if (want * tiles > slots) {
+    const int64_t waves = (want * tiles + slots - 1) / slots;
+    want = std::max<int64_t>(want, waves * slots / tiles);
+  }
+  const int64_t min_rows = dbl ? 4 : 2 * OUTER_BK;
+  want = std::min<int64_t>(want, (rows + min_rows - 1) / min_rows);
+  const int64_t cap = ((int64_t)1 << 29) / ((int64_t)M * Nn * sizeof(T));
+  want = std::max<int64_t>(1, std::min(want, std::max<int64_t>(1, cap)));
+  want = std::min<int64_t>(want, 65535);
+  p.rps = std::max<int64_t>(1, (rows + want - 1) / want);
+  if (!dbl && p.rps > 4 * OUTER_BK) p.rps = ((p.rps + OUTER_BK - 1) / OUTER_BK) * OUTER_BK;
+  p.splits = (int)std::max<int64_t>(1, (rows + p.rps - 1) / p.rps);
+  return p;
+}
+
+template <int OP, int TM, int VH>
+int32_t outer_launch_f(const OuterArgs<float>& a, const OuterPlan& p, cudaStream_t st) {
+  const int BK = OuterCfg<OP, VH>::BK, BM = p.GM * TM, BN = p.GN * 8, dS = (a.d + 3) & ~3;
+  const size_t smem =
+      ((size_t)2 * BK * (BM + BN + (OP == 1 ? dS : 0)) + BM + (OP == 1 ? BN : 0)) * 4;
+  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_outer_f<OP, TM, VH>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+  count_launch();
+  k_row_outer_f<OP, TM, VH><<<dim3(p.tm, p.tn, p.splits), p.threads, smem, st>>>(a);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+template <int OP>
+int32_t outer_run(OuterArgs<double> a, const OuterPlan& p, cudaStream_t st) {
+  a.GM = p.GM;
+  a.GN = p.GN;
+  a.rps = p.rps;
+  const size_t smem = outer_smem_d<OP>(p.GM, p.GN, a.d, a.c);
+  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_outer_d<OP>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+  count_launch();
+  k_row_outer_d<OP><<<dim3(p.tm, p.tn, p.splits), p.threads, smem, st>>>(a);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+template <int OP>
+int32_t outer_run(OuterArgs<float> a, const OuterPlan& p, cudaStream_t st) {
+  a.GM = p.GM;
+  a.GN = p.GN;
+  a.rps = p.rps;
+  const int vh = outer_vh(a);
+  if constexpr (OP == 1) if (p.TM == 4) {
+    if (vh == 4) return outer_launch_f<OP, 4, 4>(a, p, st);
+    if (vh == 2) return outer_launch_f<OP, 4, 2>(a, p, st);
+    return outer_launch_f<OP, 4, 1>(a, p, st);
+  }
+  if (vh == 4) return outer_launch_f<OP, 8, 4>(a, p, st);
+  if (vh == 2) return outer_launch_f<OP, 8, 2>(a, p, st);
+  return outer_launch_f<OP, 8, 1>(a, p, st);
+}
+
+// ------------------------------------------------------------------------------------------
+// reductions over the splits
+// ------------------------------------------------------------------------------------------
+// Block sums: the triangle's partials, added over the splits in double (8 threads per value,
+// fixed order), expanded to the full symmetric block with lam on the diagonal.
+template <class T>
+__global__ __launch_bounds__(256) void k_pair_expand(const T* __restrict__ part, int splits,
+                                                     int64_t count, int64_t stride, int np,
+                                                     int d, double lam,
+                                                     double* out_d, T* out_t) {
+  __shared__ double red[8][33];
+  const int64_t idx = blockIdx.x * (int64_t)32 + threadIdx.x;
+  double acc = 0.0;
+  if (idx < count) {
+#pragma unroll 8
+    for (int sp = threadIdx.y; sp < splits; sp += 8) acc += (double)part[sp * stride + idx];
+  }
+  red[threadIdx.y][threadIdx.x] = acc;
+  __syncthreads();
+  if (threadIdx.y != 0 || idx >= count) return;
+  for (int g = 1; g < 8; ++g) acc += red[g][threadIdx.x];
+  const int k = (int)(idx / np);
+  int e, f;
+  pair_of((int)(idx - (int64_t)k * np), d, e, f);
+  if (e == f) acc += lam;
+  const int64_t o1 = ((int64_t)k * d + e) * d + f, o2 = ((int64_t)k * d + f) * d + e;
+  if (out_d) out_d[o1] = out_d[o2] = acc;
+  if (out_t) out_t[o1] = out_t[o2] = (T)acc;
+}
+
+// out_j[k] = S_k V_j[k] - sum over the splits of part[split][j][k]; optional
+// pq[j c + k] = V_j[k] . out_j[k].  Block = class k, JB probes x SG groups x dpad features;
+// the groups share one output's splits and the terms of S_k V_j[k], added in a fixed order.
+template <class T>
+__global__ void k_row_combine(const T* __restrict__ S, const T* __restrict__ V,
+                              const T* __restrict__ part, int splits, int d, int c, int s,
+                              int64_t D, T* __restrict__ out, double* pq, int JB, int SG) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int dpad = (d + 31) & ~31;
+  T* vs = (T*)smem_raw;                  // JB * d
+  T* gs = vs + (size_t)JB * d;           // SG * JB * dpad (SG > 1)
+  __shared__ double red[32];
+  const int k = blockIdx.x;
+  const int e = threadIdx.x % dpad, q = threadIdx.x / dpad;
+  const int g = q / JB, jj = q - g * JB;
+  const int j = blockIdx.y * JB + jj;
+  for (int idx = threadIdx.x; idx < JB * d; idx += blockDim.x) {
+    const int qj = idx / d, f = idx - qj * d;
+    const int jx = blockIdx.y * JB + qj;
+    vs[idx] = jx < s ? V[(int64_t)jx * D + (int64_t)k * d + f] : T(0);
+  }
+  __syncthreads();
+  T acc = T(0);
+  if (j < s && e < d) {
+    const T* Sk = S + (int64_t)k * d * d + e;   // S symmetric: column e as row e
+#pragma unroll 4
+    for (int f = g; f < d; f += SG) acc = fma(Sk[(int64_t)f * d], vs[jj * d + f], acc);
+    T ds = T(0);
+    const T* dp = part + (int64_t)j * D + (int64_t)k * d + e;
+    const int64_t stride = (int64_t)s * D;
+#pragma unroll 8
+    for (int sp = g; sp < splits; sp += SG) ds += dp[sp * stride];
+    acc -= ds;
+  }
+  if (SG > 1) {
+    gs[(g * JB + jj) * dpad + e] = acc;
+    __syncthreads();
+    if (g == 0)
+      for (int x = 1; x < SG; ++x) acc += gs[(x * JB + jj) * dpad + e];
+  }
+  const bool own = g == 0 && j < s && e < d;
+  if (own) out[(int64_t)j * D + (int64_t)k * d + e] = acc;
+  if (pq) {
+    double v = own ? (double)vs[jj * d + e] * (double)acc : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (own && e == 0) {
+      double tot = 0.0;
+      for (int w = 0; w < dpad / 32; ++w) tot += red[(threadIdx.x >> 5) + w];
+      pq[(int64_t)j * c + k] = tot;
+    }
+  }
+}
+
+// ------------------------------------------------------------------------------------------
+// k_row_form (f32): 128 rows x 128 columns per tile, K = features.
+//   MODE 0  alpha:  columns (probe, class), walpha[i][j] = w_i sum_k h_ik (x_i.V_j[k])
+//   MODE 1  quad:   64 columns of A_j and the same 64 of B_j;
+//           sum_k h a b - (sum_k h a)(sum_k h b) per probe, summed over the block's probes
+//   MODE 2  scores: 64 columns of M1_k and the same 64 of M2_k; q = sum_e x_e (x.M_k[e]),
+//           sum over the block's classes of w q1 / (1 + eta w q2), w = h_ik (1 - h_ik)
+// The columns of one unit u (probe; class in MODE 2) are its inner index v (class; feature in
+// MODE 2) padded to kc, a multiple of 4 not above the tile, and PJ units share a tile when kc
+// is small; CC chunks cover inner ranges beyond the tile.  Each thread owns 8 rows and two
+// groups of 4 inner indices of one unit, so its share of a row's sum stays in registers; the
+// groups meet in shared memory once per tile.  Blocks: 128 rows x a range of units
+// (blockIdx.y).
+// Bound by issue slots and, per tile, the latency of the row coefficients: 40 TFLOP/s for alpha
+// at n = 21,000, c = 1000, d = 64, s = 16 (1.08 ms; one thread per row took 4.67), the quadratic
+// forms at n = 50,000, d = 50, c = 10, s = 20 100 us (175 before), the eq. 14 scores at
+// n = 5,000, d = c = 50 110 us (2,840 before: 40 blocks, one after another over the classes).
+// The coefficient tiles are packed first (k_form_pack), feature-major, so that a step of the
+// main loop is staged by whole 16-byte copies at any alignment.
+// ------------------------------------------------------------------------------------------
+constexpr int FORM_LD = 132;    // tile row in shared memory (16-byte rows, no 2-power stride)
+
+struct FormArgs {
+  const float* Xa;
+  const float* Ha;
+  const float* w;        // MODE 0: row weights
+  const float* A;        // coefficient blocks, unit u at A + u ustride + v d
+  const float* B;        // MODE 1, 2: the second block
+  float* pk;             // packed tiles [block y][chunk][tile][dK][128]
+  int64_t row0, N;       // first row, end row
+  int d, c;
+  int units, inner;      // units and inner extent (s, c; MODE 2: c, d)
+  int64_t ustride;       // elements between units
+  int kc, PJ, CC, UB;    // padded inner chunk, units per tile, chunks, units per block
+  int vec;               // float4 reads of the row coefficients are aligned
+  double eta;
+  float* walpha;         // MODE 0: N x units
+  double* part;          // MODE 1, 2: [blockIdx.y][row - row0]
+};
+
+// features padded to whole steps of 16
+__host__ __device__ inline int form_dk(int d) { return (d + 15) / 16 * 16; }
+
+// One thread: one tile column, 8 features.
+template <int MODE>
+__global__ __launch_bounds__(256) void k_form_pack(const FormArgs a, int64_t total) {
+  const int dK = form_dk(a.d), eb = dK / 8;
+  const int tpb = a.UB / a.PJ;
+  for (int64_t idx = blockIdx.x * (int64_t)256 + threadIdx.x; idx < total;
+       idx += (int64_t)gridDim.x * 256) {
+    const int col = (int)(idx & 127);
+    const int64_t q0 = idx >> 7;
+    const int T = (int)(q0 / eb), e0 = (int)(q0 - (int64_t)T * eb) * 8;
+    const int p = T % tpb, yc = T / tpb, cc = yc % a.CC, y = yc / a.CC;
+    const int q = MODE == 0 ? col : col & 63;
+    const int ul = q / a.kc, v = cc * a.kc + q - ul * a.kc;
+    const int u = y * a.UB + p * a.PJ + ul;
+    const bool ok = ul < a.PJ && u < a.units && v < a.inner;
+    const float* src =
+        (MODE != 0 && col >= 64 ? a.B : a.A) + (ok ? u * a.ustride + (int64_t)v * a.d : 0);
+    float* dst = a.pk + ((int64_t)T * dK + e0) * 128 + col;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) dst[e * 128] = ok && e0 + e < a.d ? src[e0 + e] : 0.0f;
+  }
+}
+
+// KC features per step: 16, or 8 where that lets two blocks share an SM
+template <int MODE, int KC>
+__global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
+  constexpr int NV = MODE == 0 ? 1 : MODE == 1 ? 3 : 2;   // values per (row, unit)
+  constexpr int GC = MODE == 0 ? 32 : 16;                 // column groups per tile
+  constexpr int LD = FORM_LD;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int d = a.d, dK = form_dk(d);
+  float* xs = (float*)smem_raw;              // [dK][LD]
+  float* vs = xs + (size_t)dK * LD;          // [2][KC][128]
+  float* red = vs + 2 * KC * 128;            // [NV][128][GC + 1]
+  float* sum = red + NV * 128 * (GC + 1);    // [NV][UB][128]
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  // a warp covers 8 column groups x 4 row groups
+  const int tx = (wid & 1) * 8 + (lane & 7), ty = (wid >> 1) * 4 + (lane >> 3);
+  const int64_t i0 = a.row0 + (int64_t)blockIdx.x * 128;
+  const int u0 = blockIdx.y * a.UB, u1 = min(a.units, u0 + a.UB);
+  const int tpb = a.UB / a.PJ;
+  const int tpc = (u1 - u0 + a.PJ - 1) / a.PJ;            // tiles per chunk
+  const int ntile = a.CC * tpc, nk = dK / KC;
+  const int gpu = a.kc / 4;                               // groups per unit
+  // x tile, feature-major: 8 features x 4 rows per warp instruction (32-byte reads, no bank
+  // conflicts at LD = 132)
+  {
+    const int el = lane & 7, rl = lane >> 3;
+    for (int q = wid; q < 32 * (dK / 8); q += 8) {
+      const int r = (q & 31) * 4 + rl, e = (q >> 5) * 8 + el;
+      const bool ok = i0 + r < a.N && e < d;
+      cp_async<4>(xs + e * LD + r, a.Xa + (ok ? (i0 + r) * d + e : 0), ok);
+    }
+  }
+  for (int q = tid; q < NV * a.UB * 128; q += 256) sum[q] = 0.0f;
+  // step kk of tile (cc, p): KC rows of 512 bytes
+  auto stage = [&](int cc, int p, int kk, int b) {
+    const float* src = a.pk + ((((int64_t)blockIdx.y * a.CC + cc) * tpb + p) * dK + kk * KC) * 128;
+    float* dst = vs + b * KC * 128;
+#pragma unroll
+    for (int x = 0; x < KC / 8; ++x)
+      cp_async<16>(dst + (x * 256 + tid) * 4, src + (x * 256 + tid) * 4, true);
+    cp_commit();
+  };
+  stage(0, 0, 0, 0);
+  float acc[8][8];
+  int step = 0, cc = 0, p = 0;
+  for (int t = 0; t < ntile; ++t) {
+    const int pn = p + 1 < tpc ? p + 1 : 0, cn = pn ? cc : cc + 1;   // the next tile
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) acc[x][y] = 0.0f;
+    for (int kk = 0; kk < nk; ++kk, ++step) {
+      const int b = step & 1;
+      cp_wait0();
+      __syncthreads();
+      if (kk + 1 < nk) stage(cc, p, kk + 1, b ^ 1);
+      else if (t + 1 < ntile) stage(cn, pn, 0, b ^ 1);
+      const float* X = xs + kk * KC * LD + ty * 4;
+      const float* Vt = vs + b * KC * 128 + tx * 4;
+#pragma unroll 4
+      for (int q = 0; q < KC; ++q) {
+        float av[8], bv[8];
+#pragma unroll
+        for (int v = 0; v < 2; ++v) {
+          *reinterpret_cast<float4*>(av + 4 * v) =
+              *reinterpret_cast<const float4*>(X + q * LD + v * 64);
+          *reinterpret_cast<float4*>(bv + 4 * v) =
+              *reinterpret_cast<const float4*>(Vt + q * 128 + v * 64);
+        }
+#pragma unroll
+        for (int x = 0; x < 8; ++x)
+#pragma unroll
+          for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(av[x], bv[y], acc[x][y]);
+      }
+    }
+    // per row: this thread's 4 (MODE 0: 2 x 4) inner indices
+#pragma unroll
+    for (int g = 0; g < (MODE == 0 ? 2 : 1); ++g) {
+      const int grp = g * 16 + tx;
+      const int ul = grp / gpu, v = cc * a.kc + (grp - ul * gpu) * 4;
+      const bool uv = ul < a.PJ && u0 + p * a.PJ + ul < u1;
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const int r = (x / 4) * 64 + ty * 4 + (x & 3);
+        const int64_t i = i0 + r;
+        float cf[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if (MODE == 2) {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+            if (uv && v + q < a.inner) cf[q] = xs[(v + q) * LD + r];
+        } else if (uv && i < a.N) {
+          const float* hp = a.Ha + i * a.c + v;
+          if (a.vec) {
+            if (v < a.inner) {
+              const float4 hv = *reinterpret_cast<const float4*>(hp);
+              cf[0] = hv.x;
+              cf[1] = hv.y;
+              cf[2] = hv.z;
+              cf[3] = hv.w;
+            }
+          } else {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              if (v + q < a.inner) cf[q] = hp[q];
+          }
+        }
+        float s0 = 0.0f, s1 = 0.0f, s2 = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float va = acc[x][g * 4 + q], vb = acc[x][4 + q];
+          if (MODE == 0) {
+            s0 = fmaf(cf[q], va, s0);
+          } else if (MODE == 1) {
+            const float ha = cf[q] * va;
+            s0 = fmaf(ha, vb, s0);
+            s1 += ha;
+            s2 = fmaf(cf[q], vb, s2);
+          } else {
+            s0 = fmaf(cf[q], va, s0);
+            s1 = fmaf(cf[q], vb, s1);
+          }
+        }
+        red[r * (GC + 1) + grp] = s0;
+        if (NV > 1) red[(128 + r) * (GC + 1) + grp] = s1;
+        if (NV > 2) red[(256 + r) * (GC + 1) + grp] = s2;
+      }
+    }
+    __syncthreads();
+    // groups of one unit, in order; the next write of red is behind at least one barrier
+    for (int q = tid; q < NV * a.PJ * 128; q += 256) {
+      const int r = q & 127, ul = (q >> 7) % a.PJ, nv = (q >> 7) / a.PJ;
+      const int slot = p * a.PJ + ul;
+      if (u0 + slot < u1) {
+        const float* rp = red + (nv * 128 + r) * (GC + 1) + ul * gpu;
+        float acc1 = 0.0f;
+        for (int x = 0; x < gpu; ++x) acc1 += rp[x];
+        sum[(nv * a.UB + slot) * 128 + r] += acc1;
+      }
+    }
+    cc = cn;
+    p = pn;
+  }
+  __syncthreads();
+  if (MODE == 0) {
+    for (int q = tid; q < (u1 - u0) * 128; q += 256) {
+      const int r = q & 127, ul = q >> 7;
+      if (i0 + r < a.N) a.walpha[(i0 + r) * a.units + u0 + ul] = a.w[i0 + r] * sum[ul * 128 + r];
+    }
+  } else if (tid < 128 && i0 + tid < a.N) {
+    const int64_t i = i0 + tid;
+    double q = 0.0;
+    for (int ul = 0; ul < u1 - u0; ++ul) {
+      const double v0 = sum[ul * 128 + tid], v1 = sum[(a.UB + ul) * 128 + tid];
+      if (MODE == 1) {
+        q += v0 - v1 * (double)sum[(2 * a.UB + ul) * 128 + tid];
+      } else {
+        const double hv = (double)a.Ha[i * a.c + u0 + ul];
+        const double wk = hv * (1.0 - hv);
+        q += wk * v0 / (1.0 + a.eta * wk * v1);
+      }
+    }
+    a.part[blockIdx.y * (a.N - a.row0) + (i - a.row0)] = q;
+  }
+}
+
+// Units per tile and block for `rows` rows: kc spreads the inner range over equal chunks of at
+// most the tile; units per block: as many as keep the grid's last wave full (two blocks per
+// SM), at most 16 (shared-memory sums).
+void form_plan(FormArgs& a, int tile, int64_t rows, int sms) {
+  a.CC = (a.inner + tile - 1) / tile;
+  a.kc = ((a.inner + a.CC - 1) / a.CC + 3) / 4 * 4;
+  a.PJ = std::min(std::max(1, tile / a.kc), std::min(a.units, 16));
+  const int64_t rt = (rows + 127) / 128;
+  double best = 1e300;
+  for (int nb = 1; nb <= 16 / a.PJ; ++nb) {
+    const int ub = nb * a.PJ;
+    const int64_t y = (a.units + ub - 1) / ub;
+    if (nb > 1 && (nb - 1) * a.PJ >= a.units) break;
+    const int64_t waves = (rt * y + 2 * sms - 1) / (2 * sms);
+    const double cost = (double)waves * (nb * a.CC + 0.35);   // 0.35: loading the x tile
+    if (cost < best) {
+      best = cost;
+      a.UB = ub;
+    }
+  }
+}
+
+template <int MODE, int KC>
+int32_t form_launch_k(const FormArgs& a, int64_t rows, int ny, cudaStream_t st) {
+  constexpr int NV = MODE == 0 ? 1 : MODE == 1 ? 3 : 2;
+  constexpr int GC = MODE == 0 ? 32 : 16;
+  const size_t smem = ((size_t)form_dk(a.d) * FORM_LD + 2 * KC * 128 +
+                       (size_t)NV * 128 * (GC + 1) + (size_t)NV * a.UB * 128) *
+                      4;
+  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_form<MODE, KC>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+  count_launch();
+  k_row_form<MODE, KC><<<dim3((unsigned)((rows + 127) / 128), ny), 256, smem, st>>>(a);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+template <int MODE>
+int32_t form_launch(firal_problem* P, FormArgs a, int64_t rows, int* ny, cudaStream_t st) {
+  *ny = (a.units + a.UB - 1) / a.UB;
+  const int dK = form_dk(a.d);
+  const int64_t tiles = (int64_t)*ny * a.CC * (a.UB / a.PJ);
+  FIRAL_TRY(P->form_pk.ensure((size_t)tiles * dK * 128 * sizeof(float)));
+  a.pk = P->form_pk.as<float>();
+  const int64_t total = tiles * (dK / 8) * 128;
+  count_launch();
+  k_form_pack<MODE><<<(unsigned)std::min<int64_t>((total + 255) / 256, 65536), 256, 0, st>>>(a, total);
+  if (a.d <= 96) return form_launch_k<MODE, 16>(a, rows, *ny, st);
+  return form_launch_k<MODE, 8>(a, rows, *ny, st);
+}
+
+// ------------------------------------------------------------------------------------------
+// k_row_form_d (FP64): 32 rows per block, one warp per probe, 4 classes at a time; h is read
+// class-major so that a warp's 32 rows are one run.  Bound by the FP64 rate (n = 3,000, d = 20,
+// c = s = 10: 23 us a launch, 137 with 128 rows per block; 10 us at 1.25 TFLOP/s).
+// ------------------------------------------------------------------------------------------
+template <int MODE>
+__global__ __launch_bounds__(256) void k_row_form_d(
+    const double* __restrict__ Xa, const double* __restrict__ HaT, const double* __restrict__ w,
+    const double* __restrict__ A, const double* __restrict__ B, int64_t row0, int64_t N, int d,
+    int c, int s, int64_t D, double* __restrict__ walpha, double* __restrict__ part) {
+  constexpr int KC = 4;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int ldx = d | 1;
+  double* xs = (double*)smem_raw;               // [32][ldx]
+  double* va = xs + 32 * ldx;                   // [nw][KC][d]
+  double* vb = va + (size_t)nw * KC * d;        // MODE 1
+  __shared__ double red[8][33];
+  const int64_t i0 = row0 + (int64_t)blockIdx.x * 32;
+  const int64_t i = i0 + lane;
+  const bool rv = i < N;
+  const int j = blockIdx.y * nw + wid;
+  for (int q = threadIdx.x; q < 32 * d; q += blockDim.x) {
+    const int r = q / d, e = q - r * d;
+    xs[r * ldx + e] = i0 + r < N ? Xa[(i0 + r) * d + e] : 0.0;
+  }
+  double s0 = 0.0, s1 = 0.0, s2 = 0.0;
+  const double* x = xs + lane * ldx;
+  for (int k0 = 0; k0 < c; k0 += KC) {
+    __syncthreads();
+    if (j < s) {
+      const int kn = min(KC, c - k0) * d;
+      const int64_t o = (int64_t)j * D + (int64_t)k0 * d;
+      for (int q = lane; q < KC * d; q += 32) {
+        va[wid * KC * d + q] = q < kn ? A[o + q] : 0.0;
+        if (MODE == 1) vb[wid * KC * d + q] = q < kn ? B[o + q] : 0.0;
+      }
+    }
+    __syncthreads();
+    if (j >= s) continue;
+    double ga[KC], gb[KC];
+#pragma unroll
+    for (int q = 0; q < KC; ++q) ga[q] = gb[q] = 0.0;
+    const double* pa = va + wid * KC * d;
+    const double* pb = vb + wid * KC * d;
+    double hv[KC];
+#pragma unroll
+    for (int q = 0; q < KC; ++q)
+      hv[q] = rv && k0 + q < c ? HaT[(int64_t)(k0 + q) * N + i] : 0.0;
+    if (k0 + KC <= c) {
+#pragma unroll 2
+      for (int e = 0; e < d; ++e) {
+        const double xe = x[e];
+#pragma unroll
+        for (int q = 0; q < KC; ++q) {
+          ga[q] = fma(xe, pa[q * d + e], ga[q]);
+          if (MODE == 1) gb[q] = fma(xe, pb[q * d + e], gb[q]);
+        }
+      }
+    } else {                       // the last classes: no multiply-adds on padding
+      const int kn = c - k0;
+      for (int e = 0; e < d; ++e) {
+        const double xe = x[e];
+#pragma unroll
+        for (int q = 0; q < KC - 1; ++q)
+          if (q < kn) {
+            ga[q] = fma(xe, pa[q * d + e], ga[q]);
+            if (MODE == 1) gb[q] = fma(xe, pb[q * d + e], gb[q]);
+          }
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < KC; ++q) {
+      if (MODE == 0) {
+        s0 = fma(hv[q], ga[q], s0);
+      } else {
+        const double ha = hv[q] * ga[q];
+        s0 = fma(ha, gb[q], s0);
+        s1 += ha;
+        s2 = fma(hv[q], gb[q], s2);
+      }
+    }
+  }
+  if (MODE == 0) {
+    if (j < s && rv) walpha[i * s + j] = w[i] * s0;
+    return;
+  }
+  red[wid][lane] = j < s ? s0 - s1 * s2 : 0.0;
+  __syncthreads();
+  if (wid == 0 && rv) {
+    double q = 0.0;
+    for (int x2 = 0; x2 < nw; ++x2) q += red[x2][lane];
+    part[blockIdx.y * (N - row0) + (i - row0)] = q;
+  }
+}
+
+int form_d_warps(int s) { return (s + (s + 7) / 8 - 1) / ((s + 7) / 8); }
+
+template <int MODE>
+int32_t form_d_launch(const double* Xa, const double* HaT, const double* w, const double* A,
+                      const double* B, int64_t row0, int64_t N, int d, int c, int s, int64_t D,
+                      double* walpha, double* part, cudaStream_t st) {
+  const int nw = form_d_warps(s);
+  const size_t smem = ((size_t)32 * (d | 1) + (size_t)(MODE == 1 ? 2 : 1) * nw * 4 * d) * 8;
+  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_form_d<MODE>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
+  count_launch();
+  k_row_form_d<MODE><<<dim3((unsigned)((N - row0 + 31) / 32), (s + nw - 1) / nw), nw * 32, smem,
+                       st>>>(Xa, HaT, w, A, B, row0, N, d, c, s, D, walpha, part);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+// g_i = -(scale / s) sum over the blocks' partials
+template <class T>
+__global__ void k_form_sum(const double* __restrict__ part, int ny, int64_t n, double f,
+                           T* __restrict__ g) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    double q = 0.0;
+    for (int y = 0; y < ny; ++y) q += part[y * n + i];
+    g[i] = (T)(f * q);
+  }
+}
+
+// eq. 14: the blocks' partial scores added per row, then the masked argmax of each 128 rows
+// (lowest index on ties)
+__global__ __launch_bounds__(128) void k_score_argmax(const double* __restrict__ part, int ny,
+                                                      int64_t n, const uint8_t* __restrict__ mask,
+                                                      double* part_val, int64_t* part_idx) {
+  __shared__ double bv[4];
+  __shared__ int64_t bi[4];
+  const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
+  double val = -INFINITY;
+  int64_t idx = INT64_MAX;
+  if (i < n && !mask[i]) {
+    double q = 0.0;
+    for (int y = 0; y < ny; ++y) q += part[y * n + i];
+    if (q == q) {
+      val = q;
+      idx = i;
+    }
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ov = __shfl_xor_sync(0xffffffffu, val, o);
+    const int64_t oi = __shfl_xor_sync(0xffffffffu, idx, o);
+    if (ov > val || (ov == val && oi < idx)) {
+      val = ov;
+      idx = oi;
+    }
+  }
+  if ((threadIdx.x & 31) == 0) {
+    bv[threadIdx.x >> 5] = val;
+    bi[threadIdx.x >> 5] = idx;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 4; ++w)
+      if (bv[w] > val || (bv[w] == val && bi[w] < idx)) {
+        val = bv[w];
+        idx = bi[w];
+      }
+    part_val[blockIdx.x] = val;
+    part_idx[blockIdx.x] = idx;
+  }
+}
+
+// Row ranges of the f32 block sums.  The rows' weights span the labelled rows' 1 and the pool's
+// b / n, so a long f32 chain drops part of the small terms: at n = 1M, d = 128, c = 100 Round's
+// blocks come out 2e-4 low and its nu 6e-4, and an apply over 400,000 rows and 360 classes
+// carries 3e-5.  That error is part of the results, so the ranges depend on the shape alone and
+// stay as they are (finer ones move those results by more than f32 calls may differ between
+// versions); rows run in order within each.
+void block_ranges(OuterPlan& p, int64_t N, int64_t rows, int d, int c, int sms) {
+  const int64_t groups = d > 64 ? c : (c + 3) / 4;
+  int64_t n = std::max<int64_t>((4 * (int64_t)sms + groups - 1) / groups, (N + 65535) / 65536);
+  n = std::max<int64_t>(1, std::min({n, (N + 255) / 256, (int64_t)4096}));
+  p.rps = (N + n - 1) / n;
+  p.splits = (int)std::max<int64_t>(1, (rows + p.rps - 1) / p.rps);   // ranges that hold rows
+}
+
+template <class T>
+int32_t syrk_t(firal_problem* P, const T* w, int64_t rows, double lamS, T* outS, double lamP,
+               double* outP) {
+  cudaStream_t st = P->H->stream;
+  const int d = P->d, c = P->c;
+  const int nw = (outS ? 1 : 0) + (outP ? 1 : 0);
+  if (nw == 0) return FIRAL_OK;
+  const int np = d * (d + 1) / 2;
+  OuterArgs<T> a{};
+  a.Xa = P->Xa.as<T>();
+  a.Ha = P->Ha.as<T>();
+  a.w = w;
+  a.r0 = 0;
+  a.r1 = rows;
+  a.d = d;
+  a.c = c;
+  a.s = 1;
+  a.which0 = outS ? 0 : 1;
+  a.M = nw * c;
+  a.Nn = np;
+  OuterPlan p = outer_plan<1>(a, P->sms);
+  if (sizeof(T) == 4) block_ranges(p, P->N, rows, d, c, P->sms);
+  FIRAL_TRY(P->syrk_part.ensure((size_t)a.M * a.Nn * p.splits * sizeof(T)));
+  a.part = P->syrk_part.as<T>();
+  ProfScope ps(st, PF_SYRK);
+  FIRAL_TRY(outer_run<1>(a, p, st));
+  const int64_t per = (int64_t)a.M * np, half = (int64_t)c * np;
+  const dim3 blk(32, 8);
+  const unsigned grid = (unsigned)((half + 31) / 32);
+  if (outS) {
+    count_launch();
+    k_pair_expand<T><<<grid, blk, 0, st>>>(a.part, p.splits, half, per, np, d, lamS, nullptr, outS);
+  }
+  if (outP) {
+    count_launch();
+    k_pair_expand<T><<<grid, blk, 0, st>>>(a.part + (outS ? half : 0), p.splits, half, per, np, d,
+                                           lamP, outP, nullptr);
+  }
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+// pw[i][k] = w_i h_ik (1 - h_ik)
+__global__ void k_block_weights(const float* __restrict__ Ha, const float* __restrict__ w,
+                                int64_t rows, int c, float* __restrict__ pw) {
+  for (int64_t i = blockIdx.x; i < rows; i += gridDim.x) {
+    const float wi = w[i];
+    for (int k = threadIdx.x; k < c; k += blockDim.x) {
+      const float h = Ha[i * c + k];
+      pw[i * c + k] = wi * h * (1.0f - h);
+    }
+  }
+}
+
+// B_k alone in f32 (Round's Sigma blocks and B(H_o), firal_precond_blocks).  nu and the scores
+// amplify the chains' rounding, so here every addition is kept: each term is (p x_e) x_f with
+// p = w h (1 - h), over the full square, as both (e, f) and (f, e) are used.  It is OP 0's
+// product with m = (class k, feature e): A = x_e p_k, B = x_f.
+int32_t blocks_only_f32(firal_problem* P, const float* w, int64_t rows, double lamP,
+                        double* outP) {
+  cudaStream_t st = P->H->stream;
+  const int d = P->d, c = P->c;
+  const int64_t per = (int64_t)c * d * d;
+  OuterArgs<float> a{};
+  a.Xa = a.Ha = P->Xa.as<float>();
+  a.r0 = 0;
+  a.r1 = rows;
+  a.d = a.c = d;
+  a.s = c;
+  a.M = c * d;
+  a.Nn = d;
+  OuterPlan p = outer_plan<0>(a, P->sms);
+  block_ranges(p, P->N, rows, d, c, P->sms);
+  FIRAL_TRY(P->syrk_part.ensure((size_t)per * p.splits * sizeof(float)));
+  FIRAL_TRY(P->blk_w.ensure((size_t)std::max<int64_t>(rows, 1) * c * sizeof(float)));
+  a.part = P->syrk_part.as<float>();
+  a.w = P->blk_w.as<float>();
+  {
+    ProfScope ps(st, PF_SYRK);
+    if (rows > 0) {
+      count_launch();
+      k_block_weights<<<(unsigned)std::min<int64_t>(rows, 65536), std::min(256, (c + 31) / 32 * 32),
+                        0, st>>>(P->Ha.as<float>(), w, rows, c, P->blk_w.as<float>());
+      FIRAL_CUDA_TRY(cudaGetLastError());
+    }
+    FIRAL_TRY(outer_run<0>(a, p, st));
+  }
+  return syrk_reduce_f32(P, nullptr, a.part, p.splits, 0.0, nullptr, lamP, outP);
+}
+
+template <class T>
+int32_t apply_t(firal_problem* P, const T* w, const T* Sblk, const T* V, int s, T* out,
+                double* pq) {
+  cudaStream_t st = P->H->stream;
+  const int d = P->d, c = P->c;
+  const int64_t N = P->N, D = P->D;
+  FIRAL_TRY(P->walpha.ensure((size_t)N * s * sizeof(T)));
+  {
+    ProfScope ps(st, PF_ALPHA);
+    if constexpr (sizeof(T) == 8) {
+      FIRAL_TRY(form_d_launch<0>(P->Xa.as<double>(), P->HaT.as<double>(), w, V, nullptr, 0, N, d,
+                                 c, s, D, P->walpha.as<double>(), nullptr, st));
+    } else {
+      FormArgs a{};
+      a.Xa = P->Xa.as<float>();
+      a.Ha = P->Ha.as<float>();
+      a.w = w;
+      a.A = V;
+      a.N = N;
+      a.d = d;
+      a.c = c;
+      a.units = s;
+      a.inner = c;
+      a.ustride = D;
+      a.vec = row_vec(a.Ha, c) == 4;
+      a.walpha = P->walpha.as<float>();
+      form_plan(a, 128, N, P->sms);
+      int ny = 0;
+      FIRAL_TRY(form_launch<0>(P, a, N, &ny, st));
+    }
+  }
+  OuterArgs<T> o{};
+  o.Xa = P->Xa.as<T>();
+  o.Ha = P->Ha.as<T>();
+  o.w = P->walpha.as<T>();
+  o.r0 = 0;
+  o.r1 = N;
+  o.d = d;
+  o.c = c;
+  o.s = s;
+  o.M = s * c;
+  o.Nn = d;
+  OuterPlan p = outer_plan<0>(o, P->sms);
+  if (forced_splits() > 0) {
+    p.splits = (int)std::min<int64_t>(forced_splits(), (N + 31) / 32);
+    p.rps = (N + p.splits - 1) / p.splits;
+    p.splits = (int)((N + p.rps - 1) / p.rps);
+  }
+  FIRAL_TRY(P->Dpart.ensure((size_t)p.splits * s * D * sizeof(T)));
+  o.part = P->Dpart.as<T>();
+  {
+    ProfScope ps(st, PF_DTERM);
+    FIRAL_TRY(outer_run<0>(o, p, st));
+  }
+  // one probe per block and the splits over up to 8 thread groups while that leaves the blocks
+  // few; 4 probes per block once the classes alone fill the chip
+  const int dpad = (d + 31) / 32 * 32;
+  const bool few = (int64_t)c * ((s + 3) / 4) < 4 * P->sms;
+  const int JB = few ? 1 : 4;
+  const int SG = few ? std::max(1, std::min({8, 1024 / dpad, p.splits})) : 1;
+  const size_t smem = ((size_t)JB * d + (size_t)SG * JB * dpad) * sizeof(T);
+  ProfScope ps(st, PF_COMBINE);
+  count_launch();
+  k_row_combine<T><<<dim3(c, (s + JB - 1) / JB), dpad * JB * SG, smem, st>>>(
+      Sblk, V, o.part, p.splits, d, c, s, D, out, pq, JB, SG);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+}  // namespace
+
+int32_t syrk_blocks(firal_problem* P, const void* w, double lamS, void* outS, double lamP,
+                    double* outP, int64_t rows) {
+  if (rows < 0) rows = P->N;
+  if (!P->dbl && !outS) return blocks_only_f32(P, (const float*)w, rows, lamP, outP);
+  if (P->dbl) return syrk_t<double>(P, (const double*)w, rows, lamS, (double*)outS, lamP, outP);
+  return syrk_t<float>(P, (const float*)w, rows, lamS, (float*)outS, lamP, outP);
+}
+
+int32_t hessian_apply_simt(firal_problem* P, const void* w, const void* Sblk, const void* V,
+                           int s, void* out, double* pq) {
+  if (P->dbl) {
+    FIRAL_TRY(class_major_h(P));
+    return apply_t<double>(P, (const double*)w, (const double*)Sblk, (const double*)V, s,
+                           (double*)out, pq);
+  }
+  return apply_t<float>(P, (const float*)w, (const float*)Sblk, (const float*)V, s, (float*)out,
+                        pq);
+}
+
+// Per-point quadratic forms (eq. 11): g_i = -(scale/s) sum_j a_j^T H_i b_j for pool rows,
+//   a_j^T H_i b_j = sum_k h_ik (x_i.A_j[k]) (x_i.B_j[k]) - (sum_k h_ik x_i.A_j[k])(sum_k h_ik x_i.B_j[k]).
+int32_t quad_forms_simt(firal_problem* P, const void* A, const void* B, int s, double scale,
+                        void* g) {
+  cudaStream_t st = P->H->stream;
+  const int d = P->d, c = P->c;
+  ProfScope ps(st, PF_QUAD);
+  int ny = 0;
+  if (P->dbl) {
+    FIRAL_TRY(class_major_h(P));
+    ny = (s + form_d_warps(s) - 1) / form_d_warps(s);
+    FIRAL_TRY(P->form_part.ensure((size_t)ny * P->n * sizeof(double)));
+    FIRAL_TRY(form_d_launch<1>(P->Xa.as<double>(), P->HaT.as<double>(), nullptr,
+                               (const double*)A, (const double*)B, P->m, P->N, d, c, s, P->D,
+                               nullptr, P->form_part.as<double>(), st));
+  } else {
+    FormArgs a{};
+    a.Xa = P->Xa.as<float>();
+    a.Ha = P->Ha.as<float>();
+    a.A = (const float*)A;
+    a.B = (const float*)B;
+    a.row0 = P->m;
+    a.N = P->N;
+    a.d = d;
+    a.c = c;
+    a.units = s;
+    a.inner = c;
+    a.ustride = P->D;
+    a.vec = row_vec(a.Ha, c) == 4;
+    form_plan(a, 64, P->n, P->sms);
+    FIRAL_TRY(P->form_part.ensure((size_t)((s + a.UB - 1) / a.UB) * P->n * sizeof(double)));
+    a.part = P->form_part.as<double>();
+    FIRAL_TRY(form_launch<1>(P, a, P->n, &ny, st));
+  }
+  count_launch();
+  const unsigned grid = (unsigned)std::min<int64_t>((P->n + 255) / 256, 4096);
+  if (P->dbl)
+    k_form_sum<double><<<grid, 256, 0, st>>>(P->form_part.as<double>(), ny, P->n, -scale / s,
+                                             (double*)g);
+  else
+    k_form_sum<float><<<grid, 256, 0, st>>>(P->form_part.as<double>(), ny, P->n, -scale / s,
+                                            (float*)g);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+// eq. 14 scores of the pool rows in f32 and the masked argmax of each 128 rows
+int32_t round_scores_f32(firal_problem* P, const float* M1, const float* M2, const uint8_t* mask,
+                         double eta, double* pv, int64_t* pi, int np) {
+  cudaStream_t st = P->H->stream;
+  FormArgs a{};
+  a.Xa = P->Xa.as<float>();
+  a.Ha = P->Ha.as<float>();
+  a.A = M1;
+  a.B = M2;
+  a.row0 = P->m;
+  a.N = P->N;
+  a.d = P->d;
+  a.c = P->c;
+  a.units = P->c;
+  a.inner = P->d;
+  a.ustride = (int64_t)P->d * P->d;
+  a.eta = eta;
+  form_plan(a, 64, P->n, P->sms);
+  FIRAL_TRY(P->form_part.ensure((size_t)((a.units + a.UB - 1) / a.UB) * P->n * sizeof(double)));
+  a.part = P->form_part.as<double>();
+  ProfScope ps(st, PF_ROUND);
+  int ny = 0;
+  FIRAL_TRY(form_launch<2>(P, a, P->n, &ny, st));
+  count_launch();
+  k_score_argmax<<<np, 128, 0, st>>>(a.part, ny, P->n, mask, pv, pi);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+}  // namespace firal

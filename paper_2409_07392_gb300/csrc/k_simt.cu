@@ -247,93 +247,8 @@ int32_t set_step(int64_t* t_dev, int64_t v, cudaStream_t st) {
 }
 
 // ------------------------------------------------------------------------------------------
-// Weighted block sums (eq. 13 and the diagonal part of the apply), partial over row splits:
-//   partS[split][k][e][f] = sum_{i in split} w_i h_ik x_ie x_if
-//   partP[split][k][e][f] = sum_{i in split} w_i h_ik (1 - h_ik) x_ie x_if
-// 256 threads as 16 x 16, each owning a TE x TE tile of the (16 TE)^2 output; G classes per CTA.
+// Reductions of the tensor-core path's split sums (the CUDA-core paths' are in k_rows.cu)
 // ------------------------------------------------------------------------------------------
-template <class T, int TE, int G>
-__global__ __launch_bounds__(256) void k_syrk(const T* __restrict__ Xa, const T* __restrict__ HaT,
-                                              const T* __restrict__ w, int64_t N, int d, int c,
-                                              int64_t rows_per_split, T* partS, T* partP) {
-  constexpr int DP = 16 * TE;
-  constexpr int PC = 32;
-  __shared__ __align__(16) T xs[PC][DP];
-  __shared__ T wsS[G][PC];
-  __shared__ T wsP[G][PC];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int k0 = blockIdx.x * G;
-  const int split = blockIdx.y;
-  const int64_t i0 = (int64_t)split * rows_per_split;
-  const int64_t i1 = min(N, i0 + rows_per_split);
-  T accS[G][TE][TE], accP[G][TE][TE];
-#pragma unroll
-  for (int g = 0; g < G; ++g)
-#pragma unroll
-    for (int r = 0; r < TE; ++r)
-#pragma unroll
-      for (int q = 0; q < TE; ++q) accS[g][r][q] = accP[g][r][q] = T(0);
-
-  for (int64_t ib = i0; ib < i1; ib += PC) {
-    for (int idx = threadIdx.x; idx < PC * DP; idx += 256) {
-      const int p = idx / DP, e = idx - p * DP;
-      const int64_t i = ib + p;
-      xs[p][e] = (i < i1 && e < d) ? Xa[i * d + e] : T(0);
-    }
-    for (int idx = threadIdx.x; idx < G * PC; idx += 256) {
-      const int g = idx / PC, p = idx - g * PC;
-      const int64_t i = ib + p;
-      const int k = k0 + g;
-      const T hv = (i < i1 && k < c) ? HaT[(int64_t)k * N + i] : T(0);
-      const T wv = (i < i1) ? w[i] : T(0);
-      wsS[g][p] = wv * hv;
-      wsP[g][p] = wv * hv * (T(1) - hv);
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int p = 0; p < PC; ++p) {
-      T a[TE], b[TE];
-#pragma unroll
-      for (int r = 0; r < TE; ++r) {
-        a[r] = xs[p][ty * TE + r];
-        b[r] = xs[p][tx * TE + r];
-      }
-#pragma unroll
-      for (int g = 0; g < G; ++g) {
-        const T sS = wsS[g][p], sP = wsP[g][p];
-#pragma unroll
-        for (int r = 0; r < TE; ++r) {
-          const T as = sS * a[r], ap = sP * a[r];
-#pragma unroll
-          for (int q = 0; q < TE; ++q) {
-            accS[g][r][q] = fma(as, b[q], accS[g][r][q]);
-            accP[g][r][q] = fma(ap, b[q], accP[g][r][q]);
-          }
-        }
-      }
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int g = 0; g < G; ++g) {
-    const int k = k0 + g;
-    if (k >= c) continue;
-#pragma unroll
-    for (int r = 0; r < TE; ++r) {
-      const int e = ty * TE + r;
-      if (e >= d) continue;
-#pragma unroll
-      for (int q = 0; q < TE; ++q) {
-        const int f = tx * TE + q;
-        if (f >= d) continue;
-        const int64_t o = (((int64_t)split * c + k) * d + e) * d + f;
-        if (partS) partS[o] = accS[g][r][q];
-        if (partP) partP[o] = accP[g][r][q];
-      }
-    }
-  }
-}
-
 // out[k][e][f] = sum_split part[split][k][e][f] (+ lam on the diagonal), as double and/or T
 template <class T>
 __global__ void k_syrk_reduce(const T* part, int splits, int64_t per, int d, double lam,
@@ -351,50 +266,6 @@ __global__ void k_syrk_reduce(const T* part, int splits, int64_t per, int d, dou
   }
 }
 
-static int syrk_splits(int64_t N, int cgroups, int sms) {
-  int64_t want = (4LL * sms + cgroups - 1) / cgroups;
-  int64_t by_rows = (N + 65535) / 65536;
-  int64_t s = want > by_rows ? want : by_rows;
-  int64_t max_by_size = (N + 255) / 256;
-  if (s > max_by_size) s = max_by_size;
-  if (s < 1) s = 1;
-  if (s > 4096) s = 4096;
-  return (int)s;
-}
-
-template <class T>
-static int32_t syrk_t(firal_problem* P, const T* w, double lamS, T* outS, double lamP,
-                      double* outP) {
-  cudaStream_t st = P->H->stream;
-  const int d = P->d, c = P->c;
-  const int TE = d <= 32 ? 2 : (d <= 64 ? 4 : 8);
-  const int G = (sizeof(T) == 8 || TE == 8) ? 1 : 4;
-  const int cgroups = (c + G - 1) / G;
-  const int splits = syrk_splits(P->N, cgroups, P->sms);
-  const int64_t rps = (P->N + splits - 1) / splits;
-  const int64_t per = (int64_t)c * d * d;
-  FIRAL_TRY(P->syrk_part.ensure((size_t)per * splits * 2 * sizeof(T)));
-  T* partS = outS ? P->syrk_part.as<T>() : nullptr;
-  T* partP = outP ? P->syrk_part.as<T>() + per * splits : nullptr;
-  dim3 grid(cgroups, splits);
-  ProfScope ps(st, PF_SYRK);
-  count_launch(1 + (outS ? 1 : 0) + (outP ? 1 : 0));
-  const T* Xa = P->Xa.as<T>();
-  const T* HaT = P->HaT.as<T>();
-#define FIRAL_SYRK(TE_, G_) \
-  k_syrk<T, TE_, G_><<<grid, 256, 0, st>>>(Xa, HaT, w, P->N, d, c, rps, partS, partP)
-  if (TE == 2) { if (G == 4) FIRAL_SYRK(2, 4); else FIRAL_SYRK(2, 1); }
-  else if (TE == 4) { if (G == 4) FIRAL_SYRK(4, 4); else FIRAL_SYRK(4, 1); }
-  else FIRAL_SYRK(8, 1);
-#undef FIRAL_SYRK
-  FIRAL_CUDA_TRY(cudaGetLastError());
-  const int g = grid_for(per, 256, 4096);
-  if (outS) k_syrk_reduce<T><<<g, 256, 0, st>>>(partS, splits, per, d, lamS, nullptr, outS);
-  if (outP) k_syrk_reduce<T><<<g, 256, 0, st>>>(partP, splits, per, d, lamP, outP, nullptr);
-  FIRAL_CUDA_TRY(cudaGetLastError());
-  return FIRAL_OK;
-}
-
 int32_t syrk_reduce_f32(firal_problem* P, const float* partS, const float* partP, int splits,
                         double lamS, float* outS, double lamP, double* outP, const float* addS) {
   cudaStream_t st = P->H->stream;
@@ -407,129 +278,6 @@ int32_t syrk_reduce_f32(firal_problem* P, const float* partS, const float* partP
   if (outP) k_syrk_reduce<float><<<g, 256, 0, st>>>(partP, splits, per, P->d, lamP, outP, nullptr);
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
-}
-
-int32_t syrk_blocks(firal_problem* P, const void* w, double lamS, void* outS, double lamP,
-                    double* outP) {
-  FIRAL_TRY(class_major_h(P));
-  if (P->dbl) return syrk_t<double>(P, (const double*)w, lamS, (double*)outS, lamP, outP);
-  return syrk_t<float>(P, (const float*)w, lamS, (float*)outS, lamP, outP);
-}
-
-// ------------------------------------------------------------------------------------------
-// Low-rank part of the apply, step 1:  walpha[i][j] = w_i sum_k h_ik (x_i . V_j[:,k]).
-// One thread per row; x_i staged (transposed) in shared memory; probe block in chunks.
-// ------------------------------------------------------------------------------------------
-template <class T, int KC>
-__global__ __launch_bounds__(128) void k_alpha(const T* __restrict__ Xa, const T* __restrict__ HaT,
-                                               const T* __restrict__ w, const T* __restrict__ V,
-                                               int64_t N, int d, int c, int s, int64_t D,
-                                               T* __restrict__ walpha) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* xs = (T*)smem_raw;              // [d][128]
-  T* Vs = xs + (size_t)d * 128;      // [d][KC]
-  T* hs = Vs + (size_t)d * KC;       // [KC][128]
-  const int tid = threadIdx.x;
-  const int64_t i0 = (int64_t)blockIdx.x * 128;
-  const int64_t i = i0 + tid;
-  for (int idx = tid; idx < d * 128; idx += 128) {
-    const int r = idx / d, e = idx - r * d;     // coalesced read of row-major X
-    const int64_t ii = i0 + r;
-    xs[e * 128 + r] = ii < N ? Xa[ii * d + e] : T(0);
-  }
-  const T wi = i < N ? w[i] : T(0);
-  for (int j = 0; j < s; ++j) {
-    T acc = T(0);
-    for (int k0 = 0; k0 < c; k0 += KC) {
-      __syncthreads();
-      for (int idx = tid; idx < KC * d; idx += 128) {
-        const int kk = idx / d, e = idx - kk * d;
-        const int k = k0 + kk;
-        Vs[e * KC + kk] = k < c ? V[(int64_t)j * D + (int64_t)k * d + e] : T(0);
-      }
-      for (int idx = tid; idx < KC * 128; idx += 128) {
-        const int kk = idx / 128, r = idx - kk * 128;
-        const int k = k0 + kk;
-        const int64_t ii = i0 + r;
-        hs[kk * 128 + r] = (k < c && ii < N) ? HaT[(int64_t)k * N + ii] : T(0);
-      }
-      __syncthreads();
-      T gam[KC];
-#pragma unroll
-      for (int kk = 0; kk < KC; ++kk) gam[kk] = T(0);
-      for (int e = 0; e < d; ++e) {
-        const T xe = xs[e * 128 + tid];
-#pragma unroll
-        for (int kk = 0; kk < KC; ++kk) gam[kk] = fma(xe, Vs[e * KC + kk], gam[kk]);
-      }
-#pragma unroll
-      for (int kk = 0; kk < KC; ++kk) acc = fma(hs[kk * 128 + tid], gam[kk], acc);
-    }
-    if (i < N) walpha[i * s + j] = wi * acc;
-  }
-}
-
-// Low-rank part, step 2:  Dpart[split][k][j d + e] = sum_{i in split} h_ik walpha[i][j] x_ie.
-// 64 (j,e) x 64 k tile per CTA; 256 threads, 4 x 4 register tiles; rows in chunks of 32.
-template <class T>
-__global__ __launch_bounds__(256) void k_dterm(const T* __restrict__ Xa, const T* __restrict__ Ha,
-                                               const T* __restrict__ walpha, int64_t N, int d,
-                                               int c, int s, int64_t rows_per_split,
-                                               T* __restrict__ Dpart) {
-  constexpr int PC = 32;
-  __shared__ __align__(16) T Ys[PC][64];
-  __shared__ __align__(16) T Hs[PC][64];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int r0 = blockIdx.x * 64, k0 = blockIdx.y * 64;
-  const int split = blockIdx.z;
-  const int sd = s * d;
-  const int64_t i0 = (int64_t)split * rows_per_split;
-  const int64_t i1 = min(N, i0 + rows_per_split);
-  T acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
-  for (int64_t ib = i0; ib < i1; ib += PC) {
-    for (int idx = threadIdx.x; idx < PC * 64; idx += 256) {
-      const int p = idx >> 6, col = idx & 63;
-      const int64_t i = ib + p;
-      const int r = r0 + col;
-      T y = T(0);
-      if (i < i1 && r < sd) {
-        const int j = r / d, e = r - j * d;
-        y = walpha[i * s + j] * Xa[i * d + e];
-      }
-      Ys[p][col] = y;
-      const int k = k0 + col;
-      Hs[p][col] = (i < i1 && k < c) ? Ha[i * c + k] : T(0);
-    }
-    __syncthreads();
-#pragma unroll 8
-    for (int p = 0; p < PC; ++p) {
-      T a[4], b[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        a[q] = Ys[p][ty * 4 + q];
-        b[q] = Hs[p][tx * 4 + q];
-      }
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) acc[x][y] = fma(a[x], b[y], acc[x][y]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int y = 0; y < 4; ++y) {
-    const int k = k0 + tx * 4 + y;
-    if (k >= c) continue;
-#pragma unroll
-    for (int x = 0; x < 4; ++x) {
-      const int r = r0 + ty * 4 + x;
-      if (r < sd) Dpart[((int64_t)split * c + k) * sd + r] = acc[x][y];
-    }
-  }
 }
 
 // out_j[k] = S_k V_j[k] - sum_split Dpart[split][k][j d + .]; optional pq[j c + k] = V_j[k].out_j[k]
@@ -633,64 +381,6 @@ __global__ void k_combine4(const float* __restrict__ S, const float* __restrict_
       make_float4(acc.x - dsum.x, acc.y - dsum.y, acc.z - dsum.z, acc.w - dsum.w);
 }
 
-static int dterm_splits(int tiles, int64_t N, int sms) {
-  int64_t want = (3LL * sms + tiles - 1) / tiles;
-  int64_t max_by_rows = (N + 1023) / 1024;
-  if (want > max_by_rows) want = max_by_rows;
-  if (want < 1) want = 1;
-  if (want > 256) want = 256;
-  return (int)want;
-}
-
-template <class T>
-static int32_t apply_t(firal_problem* P, const T* w, const T* Sblk, const T* V, int s, T* out,
-                       double* pq) {
-  cudaStream_t st = P->H->stream;
-  const int d = P->d, c = P->c;
-  const int64_t N = P->N, D = P->D;
-  FIRAL_TRY(P->walpha.ensure((size_t)N * s * sizeof(T)));
-  constexpr int KC = 16;
-  const size_t smem_a = ((size_t)d * 128 + (size_t)d * KC + (size_t)KC * 128) * sizeof(T);
-  static bool attr_set[2] = {false, false};
-  if (!attr_set[sizeof(T) == 8]) {
-    FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_alpha<T, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        200 * 1024));
-    FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_combine<T, 4>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    attr_set[sizeof(T) == 8] = true;
-  }
-  {
-  ProfScope ps(st, PF_ALPHA);
-  count_launch();
-  k_alpha<T, KC><<<(unsigned)((N + 127) / 128), 128, smem_a, st>>>(
-      P->Xa.as<T>(), P->HaT.as<T>(), w, V, N, d, c, s, D, P->walpha.as<T>());
-  }
-  FIRAL_CUDA_TRY(cudaGetLastError());
-  const int sd = s * d;
-  const int tr = (sd + 63) / 64, tk = (c + 63) / 64;
-  const int splits = forced_splits() > 0 ? (int)std::min<int64_t>(forced_splits(), (N + 31) / 32)
-                                         : dterm_splits(tr * tk, N, P->sms);
-  const int64_t rps = (N + splits - 1) / splits;
-  FIRAL_TRY(P->Dpart.ensure((size_t)splits * c * sd * sizeof(T)));
-  {
-  ProfScope ps(st, PF_DTERM);
-  count_launch();
-  k_dterm<T><<<dim3(tr, tk, splits), 256, 0, st>>>(P->Xa.as<T>(), P->Ha.as<T>(),
-                                                   P->walpha.as<T>(), N, d, c, s, rps,
-                                                   P->Dpart.as<T>());
-  }
-  FIRAL_CUDA_TRY(cudaGetLastError());
-  const int threads = ((d + 31) / 32) * 32 * 4;   // 4 probes in parallel
-  const size_t smem_c = ((size_t)d * d + 4 * (size_t)d) * sizeof(T);
-  ProfScope ps(st, PF_COMBINE);
-  count_launch();
-  k_combine<T, 4><<<dim3(c, (s + 3) / 4), threads, smem_c, st>>>(Sblk, V, P->Dpart.as<T>(),
-                                                                  splits, d, c, s, D, out, pq,
-                                                                  nullptr, P->pt);
-  FIRAL_CUDA_TRY(cudaGetLastError());
-  return FIRAL_OK;
-}
-
 int32_t combine_f32(firal_problem* P, const float* Sblk, const float* V, int splits, int s,
                     float* out, double* pq, const float* vmean) {
   const int d = P->d, c = P->c;
@@ -723,16 +413,6 @@ int32_t combine_f32(firal_problem* P, const float* Sblk, const float* V, int spl
       Sblk, V, P->Dpart.as<float>(), splits, d, c, s, P->D, out, pq, vmean, P->pt);
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
-}
-
-int32_t hessian_apply_simt(firal_problem* P, const void* w, const void* Sblk, const void* V,
-                           int s, void* out, double* pq) {
-  FIRAL_TRY(class_major_h(P));
-  if (P->dbl)
-    return apply_t<double>(P, (const double*)w, (const double*)Sblk, (const double*)V, s,
-                           (double*)out, pq);
-  return apply_t<float>(P, (const float*)w, (const float*)Sblk, (const float*)V, s, (float*)out,
-                        pq);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -982,100 +662,6 @@ int32_t cg_iterate_tail(firal_problem* P, int s, double tol, int fixed) {
     k_cg_beta<<<(slots + 3) / 4, 128, 0, st>>>(p1, p2, c, s, tol, fixed, cols, P->pt);
     k_cg_pupdate<float><<<grid_for(total, 256), 256, 0, st>>>(cols, s, P->D, P->cgZ.as<float>(),
                                                              P->cgP.as<float>(), P->pt, d);
-  }
-  FIRAL_CUDA_TRY(cudaGetLastError());
-  return FIRAL_OK;
-}
-
-// ------------------------------------------------------------------------------------------
-// Per-point quadratic forms (eq. 11):  g_i = -(scale/s) sum_j a_j^T H_i b_j for pool rows,
-//   a_j^T H_i b_j = sum_k h_ik (x_i.A_j[k]) (x_i.B_j[k]) - (sum_k h_ik x_i.A_j[k])(sum_k h_ik x_i.B_j[k]).
-// ------------------------------------------------------------------------------------------
-template <class T, int KC>
-__global__ __launch_bounds__(128) void k_quad(const T* __restrict__ Xa, const T* __restrict__ HaT,
-                                              const T* __restrict__ A, const T* __restrict__ B,
-                                              int64_t m, int64_t N, int d, int c, int s, int64_t D,
-                                              double scale, T* __restrict__ g) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  T* xs = (T*)smem_raw;               // [d][128]
-  T* As = xs + (size_t)d * 128;       // [d][KC]
-  T* Bs = As + (size_t)d * KC;        // [d][KC]
-  T* hs = Bs + (size_t)d * KC;        // [KC][128]
-  const int tid = threadIdx.x;
-  const int64_t i0 = m + (int64_t)blockIdx.x * 128;
-  const int64_t i = i0 + tid;
-  for (int idx = tid; idx < d * 128; idx += 128) {
-    const int r = idx / d, e = idx - r * d;
-    const int64_t ii = i0 + r;
-    xs[e * 128 + r] = ii < N ? Xa[ii * d + e] : T(0);
-  }
-  double q = 0.0;
-  for (int j = 0; j < s; ++j) {
-    T s1 = T(0), sa = T(0), sb = T(0);
-    for (int k0 = 0; k0 < c; k0 += KC) {
-      __syncthreads();
-      for (int idx = tid; idx < KC * d; idx += 128) {
-        const int kk = idx / d, e = idx - kk * d;
-        const int k = k0 + kk;
-        const int64_t src = (int64_t)j * D + (int64_t)k * d + e;
-        As[e * KC + kk] = k < c ? A[src] : T(0);
-        Bs[e * KC + kk] = k < c ? B[src] : T(0);
-      }
-      for (int idx = tid; idx < KC * 128; idx += 128) {
-        const int kk = idx / 128, r = idx - kk * 128;
-        const int k = k0 + kk;
-        const int64_t ii = i0 + r;
-        hs[kk * 128 + r] = (k < c && ii < N) ? HaT[(int64_t)k * N + ii] : T(0);
-      }
-      __syncthreads();
-      T ga[KC], gb[KC];
-#pragma unroll
-      for (int kk = 0; kk < KC; ++kk) ga[kk] = gb[kk] = T(0);
-      for (int e = 0; e < d; ++e) {
-        const T xe = xs[e * 128 + tid];
-#pragma unroll
-        for (int kk = 0; kk < KC; ++kk) {
-          ga[kk] = fma(xe, As[e * KC + kk], ga[kk]);
-          gb[kk] = fma(xe, Bs[e * KC + kk], gb[kk]);
-        }
-      }
-#pragma unroll
-      for (int kk = 0; kk < KC; ++kk) {
-        const T hv = hs[kk * 128 + tid];
-        const T ha = hv * ga[kk];
-        s1 = fma(ha, gb[kk], s1);
-        sa += ha;
-        sb = fma(hv, gb[kk], sb);
-      }
-    }
-    q += (double)s1 - (double)sa * (double)sb;
-  }
-  if (i < N) g[i - m] = (T)(-scale / s * q);
-}
-
-int32_t quad_forms_simt(firal_problem* P, const void* A, const void* B, int s, double scale,
-                        void* g) {
-  FIRAL_TRY(class_major_h(P));
-  cudaStream_t st = P->H->stream;
-  const int d = P->d, c = P->c;
-  constexpr int KC = 16;
-  const unsigned grid = (unsigned)((P->n + 127) / 128);
-  ProfScope ps(st, PF_QUAD);
-  count_launch();
-  if (P->dbl) {
-    const size_t sm = ((size_t)d * 128 + 2 * (size_t)d * KC + KC * 128) * sizeof(double);
-    FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_quad<double, KC>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    k_quad<double, KC><<<grid, 128, sm, st>>>(P->Xa.as<double>(), P->HaT.as<double>(),
-                                              (const double*)A, (const double*)B, P->m, P->N, d,
-                                              c, s, P->D, scale, (double*)g);
-  } else {
-    const size_t sm = ((size_t)d * 128 + 2 * (size_t)d * KC + KC * 128) * sizeof(float);
-    FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_quad<float, KC>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    k_quad<float, KC><<<grid, 128, sm, st>>>(P->Xa.as<float>(), P->HaT.as<float>(),
-                                             (const float*)A, (const float*)B, P->m, P->N, d, c,
-                                             s, P->D, scale, (float*)g);
   }
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
