@@ -648,9 +648,8 @@ int32_t round_chains(firal_problem* P, const RoundSetup& rs, int32_t b, const do
       bf->release();
   };
   const int np = (int)std::max<int64_t>((P->n + 127) / 128, P->sms);
-  // per chain: tridiagonal forms (2 c d), Gershgorin bounds (2 c), nu step state and
-  // per-SM partials (4 + 3 * 1024)
-  const size_t tri_sz = (size_t)2 * c * d, gb_sz = (size_t)2 * c, work_sz = 4 + 3 * 1024;
+  // per chain: tridiagonal forms (2 c d), Gershgorin bounds (2 c), nu's per-SM partials
+  const size_t tri_sz = (size_t)2 * c * d, gb_sz = (size_t)2 * c, work_sz = 6 * 1024;
   int32_t rc = FIRAL_OK;
 #define TRYR(x)                    \
   do {                             \
@@ -719,8 +718,9 @@ int32_t round_chains(firal_problem* P, const RoundSetup& rs, int32_t b, const do
     // of H~_k (the eigenvalues enter only through that trace)
     TRYR(sym_tri(Ht.as<double>(), c * ne, d, tri, gb, st));
     for (int e = 0; e < ne; ++e)
-      TRYR(nu_of_tri(tri + e * tri_sz, gb + e * gb_sz, c, d, etas[e], work + e * work_sz,
-                     nu.as<double>() + e, st));
+      TRYR(nu_of_tri(tri + e * tri_sz, gb + e * gb_sz, c, d, etas[e],
+                     t > 0 ? nu.as<double>() + e : nullptr, work + e * work_sz,
+                     nu.as<double>() + e, st));   // from the last pick's nu
     // line 11: B = nu Sigma + eta H + (eta/b) H_o, inverted
     for (int e = 0; e < ne; ++e)
       TRYR(lincomb_nu(Bm_e(e), nu.as<double>() + e, Sig, etas[e], Hk_e(e), etas[e] / b,

@@ -300,13 +300,9 @@ int32_t chol_inv(bool dbl, const double* A, int c, int d, void* inv_t, double* i
                  double* L_out, int32_t* not_spd, cudaStream_t st);
 int32_t tilde_eigvals(const double* L, const double* H, int c, int d, double* eig,
                       cudaStream_t st);
-int32_t tilde_nu(const double* L, const double* H, int c, int d, double eta, double* tri,
-                 double* gb, double* nu_out, cudaStream_t st);
-int32_t sym_tri_nu(const double* Ht, int c, int d, double eta, double* tri, double* gb,
-                   double* nu_out, cudaStream_t st);
 int32_t sym_tri(const double* Ht, int nblocks, int d, double* tri, double* gb, cudaStream_t st);
-int32_t nu_of_tri(const double* tri, const double* gb, int c, int d, double eta, double* work,
-                  double* nu_out, cudaStream_t st);
+int32_t nu_of_tri(const double* tri, const double* gb, int c, int d, double eta,
+                  const double* nu0, double* part, double* nu_out, cudaStream_t st);
 int32_t similarity_blocks(const double* L, const double* H, int c, int d, double* out,
                           cudaStream_t st);
 int32_t nu_bisect_dev(const double* lam, int64_t count, double scale, double* nu_out,

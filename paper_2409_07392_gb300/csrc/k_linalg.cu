@@ -1,8 +1,10 @@
 // FP64 block linear algebra and the Round-step kernels (Algorithm 3).
 //
-//  * k_chol_inv   -- Cholesky of c SPD d x d blocks (one CTA per block, shared memory),
+//  * k_chol_inv   -- Cholesky of c SPD d x d blocks (one CTA per block, in registers),
 //                    explicit inverse A^{-1} = L^{-T} L^{-1}; a non-positive pivot raises a
 //                    device flag (FIRAL_ERR_NOT_SPD) instead of trapping.
+//  * k_sym_tri    -- Householder tridiagonal forms, and k_nu_coop, the root nu of eq. 10 from
+//                    them (Round's per-pick path).
 //  * k_tilde_eig  -- eigenvalues of L^{-1} H L^{-T} (similar to Sigma^{-1/2} H Sigma^{-1/2}):
 //                    two in-place triangular solves, Householder tridiagonalisation and
 //                    Sturm-sequence bisection (Golub & Van Loan, Sections 8.3 and 8.4).
@@ -10,6 +12,8 @@
 //  * Round kernels -- eq. 14 scores with a masked argmax, the block update of H, and the
 //                    assembly of B_t (Algorithm 3 lines 7-11).
 #include <cooperative_groups.h>
+
+#include <algorithm>
 
 #include "firal_internal.cuh"
 
@@ -38,83 +42,159 @@ __device__ double block_sum_d(double v, double* red) {
 // ------------------------------------------------------------------------------------------
 // Cholesky + inverse of c blocks
 // ------------------------------------------------------------------------------------------
-// Shared-memory layout: the block in rows of ld = d + 1 doubles (an odd stride: the threads of
-// a half-warp reading one column each hit distinct banks).  The factor L fills the lower
-// triangle; Y = L^{-1} goes to the strict upper triangle transposed (Y[i][c], i > c, at row c,
-// column i) with its diagonal in yd.  TPR = blockDim / d threads (at least 1) share each row or
-// column, so no index is divided by a run-time size.
-template <class T>
-__global__ void k_chol_inv(const double* __restrict__ A, int d, T* __restrict__ inv_t,
-                           double* __restrict__ inv_d, double* __restrict__ L_out,
-                           int32_t* not_spd) {
+// One block per matrix, 16 x 16 threads; thread (ti, tk) holds the lower elements
+// (ti + 16 x, tk + 16 y), x >= y, in registers.  Factor and inverse are one elimination: after
+// step j the columns up to j hold Y = L^{-1} (rows past j: its partial sums) and the columns
+// past j the trailing matrix, so a step is one update a_ik -= l_i v_k of every row past j with
+//   v_k = Y_jk (k < j), 1 / L_jj (k = j), l_k (k > j),
+// published through shared memory by the owners of row and column j.  The owner of the next
+// pivot takes its square root and reciprocal while the other threads still update.  The inverse
+// is then Y^T Y from shared memory, each 16-row slab only into the columns it reaches.
+// d^3 / 2 FP64 multiply-adds per block at two per SM and cycle bound it (d = 64, c = 1000: 0.22
+// of 0.57 ms; the rest is the pivots' latency); the form before it kept the matrix in shared memory, three barriers and a
+// serial pivot per column, and dot-product chains of up to d dependent multiply-adds (64 cycles
+// each) in the inverse: 883 us there, 590 us at d = 100, c = 101 (now 307), 188 us at
+// d = 50, c = 10 (now 80).
+template <class T, int R>
+__global__ __launch_bounds__(256) void k_chol_inv(const double* __restrict__ A, int d,
+                                                  T* __restrict__ inv_t,
+                                                  double* __restrict__ inv_d,
+                                                  double* __restrict__ L_out, int32_t* not_spd) {
   extern __shared__ double sh[];
-  const int ld = d + 1;
-  double* Ls = sh;              // d x ld
-  double* yd = sh + d * ld;     // d
-  const int k = blockIdx.x, tid = threadIdx.x, bd = blockDim.x;
-  const int tpr = bd >= d ? bd / d : 1;
-  const int row = tid % d, ph = tid / d;        // this thread's row (or column) and phase
-  const bool act = ph < tpr;
-  const double* Ak = A + (int64_t)k * d * d;
-  for (int i = 0; i < d; ++i)
-    for (int e = tid; e < d; e += bd) Ls[i * ld + e] = Ak[(int64_t)i * d + e];
-  __syncthreads();
-  // right-looking Cholesky: pivot, column below it, trailing lower triangle
-  for (int j = 0; j < d; ++j) {
-    if (tid == 0) {
-      double v = Ls[j * ld + j];
-      if (!(v > 0.0)) {
-        atomicExch(not_spd, 1);
-        v = fabs(v) > 1e-300 ? fabs(v) : 1e-300;
+  __shared__ double vec[16 * R];
+  __shared__ double piv[2];          // L_jj and its reciprocal
+  const int k0 = blockIdx.x, tid = threadIdx.x, ti = tid >> 4, tk = tid & 15;
+  const double* Ak = A + (int64_t)k0 * d * d;
+  double* Lk = L_out ? L_out + (int64_t)k0 * d * d : nullptr;
+  double a[R * (R + 1) / 2];         // (x, y) at x (x + 1) / 2 + y
+#pragma unroll
+  for (int x = 0; x < R; ++x)
+#pragma unroll
+    for (int y = 0; y <= x; ++y) {
+      const int i = ti + 16 * x, k = tk + 16 * y;
+      a[x * (x + 1) / 2 + y] = i < d && k < d ? Ak[(int64_t)i * d + k] : (i == k ? 1.0 : 0.0);
+    }
+  if (Lk)
+    for (int i = ti; i < d; i += 16)
+      for (int k = tk; k < d; k += 16)
+        if (k > i) Lk[(int64_t)i * d + k] = 0.0;
+  auto pivot = [&](double v) {
+    if (!(v > 0.0)) {
+      atomicExch(not_spd, 1);
+      v = fabs(v) > 1e-300 ? fabs(v) : 1e-300;
+    }
+    const double r = rsqrt(v);       // a third of the latency of a square root and a division
+    piv[0] = v * r;
+    piv[1] = r;
+  };
+  if (tid == 0) pivot(a[0]);
+  // steps 16 bj .. 16 bj + 15: bj is a constant, so every register index is one
+#pragma unroll
+  for (int bj = 0; bj < R; ++bj) {
+    const int jn = min(16, d - 16 * bj);
+    for (int tj = 0; tj < jn; ++tj) {
+      const int j = 16 * bj + tj;
+      __syncthreads();               // pivot j is there; the last step's reads of vec are done
+      const double r = piv[1];
+      if (tk == tj) {                // column j: l_i = a_ij / L_jj, then its column of Y
+#pragma unroll
+        for (int x = bj; x < R; ++x) {
+          const int i = ti + 16 * x;
+          double& v = a[x * (x + 1) / 2 + bj];
+          if (i > j) {
+            const double l = v * r;
+            vec[i] = l;
+            if (Lk && i < d) Lk[(int64_t)i * d + j] = l;
+            v = 0.0;
+          } else if (i == j) {
+            vec[j] = r;
+            if (Lk) Lk[(int64_t)j * d + j] = piv[0];
+            v = r;
+          }
+        }
       }
-      Ls[j * ld + j] = sqrt(v);
-      yd[j] = 1.0 / Ls[j * ld + j];
+      if (ti == tj) {                // row j: Y_jk, k < j
+#pragma unroll
+        for (int y = 0; y <= bj; ++y) {
+          const int k = tk + 16 * y;
+          double& v = a[bj * (bj + 1) / 2 + y];
+          if (k < j) {
+            v *= r;
+            vec[k] = v;
+          }
+        }
+      }
+      __syncthreads();
+      // the next pivot first: its square root and reciprocal overlap the update
+      if (tj < 15) {
+        if (j + 1 < d && ti == tj + 1 && tk == tj + 1) {
+          const double l = vec[j + 1];
+          pivot(fma(-l, l, a[bj * (bj + 1) / 2 + bj]));
+        }
+      } else if (bj + 1 < R && j + 1 < d && tid == 0) {
+        const double l = vec[j + 1];
+        pivot(fma(-l, l, a[bj + 1 < R ? (bj + 1) * (bj + 2) / 2 + bj + 1 : 0]));
+      }
+      double vk[R];
+#pragma unroll
+      for (int y = 0; y < R; ++y) vk[y] = vec[tk + 16 * y];
+#pragma unroll
+      for (int x = bj; x < R; ++x) {
+        const int i = ti + 16 * x;
+        if (i > j && i < d) {          // (whole warps of padding rows skip)
+          const double li = -vec[i];
+#pragma unroll
+          for (int y = 0; y <= x; ++y)
+            a[x * (x + 1) / 2 + y] = fma(li, vk[y], a[x * (x + 1) / 2 + y]);
+        }
+      }
     }
-    __syncthreads();
-    const double rjj = yd[j];   // FP64 division is several FMAs: one per pivot
-    for (int i = j + 1 + tid; i < d; i += bd) Ls[i * ld + j] *= rjj;
-    __syncthreads();
-    if (act && row > j) {
-      const double lij = Ls[row * ld + j];
-      for (int kk = j + 1 + ph; kk <= row; kk += tpr) Ls[row * ld + kk] -= lij * Ls[kk * ld + j];
-    }
-    __syncthreads();
-  }
-  if (L_out) {
-    for (int i = 0; i < d; ++i)
-      for (int e = tid; e < d; e += bd)
-        L_out[(int64_t)k * d * d + (int64_t)i * d + e] = e <= i ? Ls[i * ld + e] : 0.0;
   }
   if (!inv_t && !inv_d) return;
-  // Y = L^{-1} by rows: Y[i][c] = -(L[i][c] Y[c][c] + sum_{c < p < i} L[i][p] Y[p][c]) Y[i][i],
-  // Y[i][i] = 1 / L[i][i] (yd, from the factorisation)
-  for (int i = 1; i < d; ++i) {
-    for (int c = tid; c < i; c += bd) {
-      double acc = Ls[i * ld + c] * yd[c];
-      for (int p = c + 1; p < i; ++p) acc += Ls[i * ld + p] * Ls[c * ld + p];
-      Ls[c * ld + i] = -acc * yd[i];
+  // Y to shared memory (zeros above the diagonal)
+  const int ld = d | 1;
+#pragma unroll
+  for (int x = 0; x < R; ++x)
+#pragma unroll
+    for (int y = 0; y < R; ++y) {
+      const int i = ti + 16 * x, k = tk + 16 * y;
+      if (i < d && k < d) sh[i * ld + k] = y <= x && k <= i ? a[x * (x + 1) / 2 + (y <= x ? y : 0)] : 0.0;
     }
-    __syncthreads();
-  }
-  // A^{-1}[a][b] = sum_{i >= max(a,b)} Y[i][a] Y[i][b]: thread (column b, phase) takes
-  // a = ph, ph + TPR, ... <= b and writes both (a, b) and (b, a)
-  if (act) {
-    const int b = row;
-    for (int a = ph; a <= b; a += tpr) {
-      double acc = (a == b ? yd[a] : Ls[a * ld + b]) * yd[b];
-      for (int i = b + 1; i < d; ++i) acc += Ls[a * ld + i] * Ls[b * ld + i];
-      const int64_t o1 = (int64_t)k * d * d + (int64_t)a * d + b;
-      const int64_t o2 = (int64_t)k * d * d + (int64_t)b * d + a;
-      if (inv_t) {
-        inv_t[o1] = (T)acc;
-        inv_t[o2] = (T)acc;
+  __syncthreads();
+  // element (p, q) = sum_{i >= p} Y_ip Y_iq, p = ti + 16 x >= 16 x
+#pragma unroll
+  for (int x = 0; x < R * (R + 1) / 2; ++x) a[x] = 0.0;
+#pragma unroll
+  for (int s = 0; s < R; ++s) {      // rows 16 s .. 16 s + 15 reach the tiles x <= s
+    const int i1 = min(d, 16 * s + 16);
+    for (int i = 16 * s; i < i1; ++i) {
+      double yk[R], yi[R];
+#pragma unroll
+      for (int y = 0; y <= s; ++y) {
+        yk[y] = tk + 16 * y < d ? sh[i * ld + tk + 16 * y] : 0.0;
+        yi[y] = ti + 16 * y < d ? sh[i * ld + ti + 16 * y] : 0.0;
       }
-      if (inv_d) {
-        inv_d[o1] = acc;
-        inv_d[o2] = acc;
-      }
+#pragma unroll
+      for (int x = 0; x <= s; ++x)
+        if (ti + 16 * x < d)
+#pragma unroll
+          for (int y = 0; y <= x; ++y)
+            a[x * (x + 1) / 2 + y] = fma(yi[x], yk[y], a[x * (x + 1) / 2 + y]);
     }
   }
+#pragma unroll
+  for (int x = 0; x < R; ++x)
+#pragma unroll
+    for (int y = 0; y <= x; ++y) {
+      const int p = ti + 16 * x, q = tk + 16 * y;
+      if (p < d && q <= p) {
+        const double v = a[x * (x + 1) / 2 + y];
+        const int64_t o1 = (int64_t)k0 * d * d + (int64_t)p * d + q;
+        const int64_t o2 = (int64_t)k0 * d * d + (int64_t)q * d + p;
+        if (inv_t) inv_t[o1] = inv_t[o2] = (T)v;
+        if (inv_d) inv_d[o1] = inv_d[o2] = v;
+      }
+    }
 }
 
 static int threads_for(int d) {
@@ -124,25 +204,35 @@ static int threads_for(int d) {
   return t;
 }
 
-int32_t chol_inv(bool dbl, const double* A, int c, int d, void* inv_t, double* inv_d,
-                 double* L_out, int32_t* not_spd, cudaStream_t st) {
-  const size_t smem = ((size_t)d * (d + 1) + d) * sizeof(double);
-  const int thr = threads_for(d);
-  if (smem > 200 * 1024 || thr < d)
-    return fail(FIRAL_ERR_UNSUPPORTED, "block factorisation needs d <= 158");
-  ProfScope ps(st, PF_CHOL);
-  count_launch();
-  if (dbl) {
-    FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_chol_inv<double>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    k_chol_inv<double><<<c, thr, smem, st>>>(A, d, (double*)inv_t, inv_d, L_out, not_spd);
-  } else {
-    FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_chol_inv<float>,
-                                        cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-    k_chol_inv<float><<<c, thr, smem, st>>>(A, d, (float*)inv_t, inv_d, L_out, not_spd);
-  }
+template <class T, int R>
+static int32_t chol_inv_r(const double* A, int c, int d, T* inv_t, double* inv_d, double* L_out,
+                          int32_t* not_spd, cudaStream_t st) {
+  const size_t smem = (size_t)d * (d | 1) * sizeof(double);
+  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_chol_inv<T, R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      200 * 1024));
+  k_chol_inv<T, R><<<c, 256, inv_t || inv_d ? smem : 0, st>>>(A, d, inv_t, inv_d, L_out, not_spd);
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
+}
+
+template <class T>
+static int32_t chol_inv_t(const double* A, int c, int d, T* inv_t, double* inv_d, double* L_out,
+                          int32_t* not_spd, cudaStream_t st) {
+  if (d <= 16) return chol_inv_r<T, 1>(A, c, d, inv_t, inv_d, L_out, not_spd, st);
+  if (d <= 32) return chol_inv_r<T, 2>(A, c, d, inv_t, inv_d, L_out, not_spd, st);
+  if (d <= 48) return chol_inv_r<T, 3>(A, c, d, inv_t, inv_d, L_out, not_spd, st);
+  if (d <= 64) return chol_inv_r<T, 4>(A, c, d, inv_t, inv_d, L_out, not_spd, st);
+  if (d <= 96) return chol_inv_r<T, 6>(A, c, d, inv_t, inv_d, L_out, not_spd, st);
+  return chol_inv_r<T, 8>(A, c, d, inv_t, inv_d, L_out, not_spd, st);
+}
+
+int32_t chol_inv(bool dbl, const double* A, int c, int d, void* inv_t, double* inv_d,
+                 double* L_out, int32_t* not_spd, cudaStream_t st) {
+  if (d > 128) return fail(FIRAL_ERR_UNSUPPORTED, "block factorisation needs d <= 128");
+  ProfScope ps(st, PF_CHOL);
+  count_launch();
+  if (dbl) return chol_inv_t<double>(A, c, d, (double*)inv_t, inv_d, L_out, not_spd, st);
+  return chol_inv_t<float>(A, c, d, (float*)inv_t, inv_d, L_out, not_spd, st);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -290,65 +380,164 @@ __global__ void k_tilde_eig(const double* __restrict__ L, const double* __restri
   }
 }
 
-// The tridiagonal forms alone (Round's nu needs no individual eigenvalue): tri[k] = dg (d) then
-// e2 (d) of block k; gb[k] = its Gershgorin interval (lo, hi).
-__global__ void k_tilde_tri(const double* __restrict__ L, const double* __restrict__ H, int d,
-                            double* __restrict__ tri, double* __restrict__ gb) {
-  extern __shared__ double sh[];
-  double* M = sh;
-  double* v = M + d * d;
-  double* p = v + d;
-  double* dg = p + d;
-  double* e2 = dg + d;
-  double* rl = e2 + d;
-  __shared__ double red[32];
-  const int k = blockIdx.x, tid = threadIdx.x, bd = blockDim.x;
-  tilde_tridiag(L + (int64_t)k * d * d, H + (int64_t)k * d * d, d, M, v, p, dg, e2, rl, red);
-  for (int i = tid; i < d; i += bd) {
-    tri[(int64_t)k * 2 * d + i] = dg[i];
-    tri[(int64_t)k * 2 * d + d + i] = i + 1 < d ? e2[i] : 0.0;
-  }
-  if (tid == 0) {
-    double lo = 1e300, hi = -1e300;
-    for (int i = 0; i < d; ++i) {
-      const double r = (i > 0 ? sqrt(e2[i - 1]) : 0.0) + (i + 1 < d ? sqrt(e2[i]) : 0.0);
-      lo = fmin(lo, dg[i] - r);
-      hi = fmax(hi, dg[i] + r);
+// Tridiagonal forms of blocks that are already L^{-1} H L^{-T} (Ht, kept up to date by
+// k_round_hupdate): tri[k] = diagonal (d) then squared off-diagonal (d) of block k, gb[k] = its
+// Gershgorin interval (lo, hi).  Householder reduction with the matrix in registers: thread
+// (ti, tk) of 16 x 16 holds the elements (ti + 16 x, tk + 16 y).  A step publishes its column,
+// one warp forms the reflector's scalars, p = tau M v is summed over the 16 threads of a row by
+// a butterfly that halves the rows each lane keeps, and M -= v w^T + w v^T runs on registers.
+// d^3 FP64 multiply-adds at two per SM and cycle bound it (d = 128: 0.5 ms of 1.05; d = 50:
+// 0.03 of 0.22, where the steps' serial part, four barriers, a square root and a division,
+// is most).  With the matrix in shared memory and one thread per row of M v, 64 cycles per
+// dependent multiply-add, it took 1.77 ms at d = 128, c = 100 and 0.28 ms at d = c = 50.
+template <int R>
+__global__ __launch_bounds__(256) void k_sym_tri(const double* __restrict__ Ht, int d,
+                                                 double* __restrict__ tri,
+                                                 double* __restrict__ gb) {
+  __shared__ double col[16 * R], w[16 * R], dg[16 * R], e2[16 * R];
+  __shared__ double sc[2];           // tau, v_{j+1}
+  const int k0 = blockIdx.x, tid = threadIdx.x, ti = tid >> 4, tk = tid & 15, lane = tid & 31;
+  const double* Hk = Ht + (int64_t)k0 * d * d;
+  double m[R][R];
+#pragma unroll
+  for (int x = 0; x < R; ++x)
+#pragma unroll
+    for (int y = 0; y < R; ++y) {
+      const int i = ti + 16 * x, k = tk + 16 * y;
+      m[x][y] = i < d && k < d ? Hk[(int64_t)i * d + k] : 0.0;
     }
-    gb[2 * k] = lo;
-    gb[2 * k + 1] = hi;
+#pragma unroll
+  for (int b = 0; b < R; ++b) {
+    for (int tj = 0; tj < 16; ++tj) {
+      const int j = 16 * b + tj;
+      if (j + 2 >= d) break;
+      // column j below the diagonal; the diagonal entry is final
+      if (tk == tj) {
+#pragma unroll
+        for (int x = b; x < R; ++x) {
+          const int i = ti + 16 * x;
+          if (i > j) col[i] = i < d ? m[x][b] : 0.0;
+          else if (i == j) dg[j] = m[x][b];
+        }
+      }
+      __syncthreads();
+      if (tid < 32) {
+        double sg = 0.0;
+        for (int i = j + 2 + lane; i < d; i += 32) sg = fma(col[i], col[i], sg);
+        sg = warp_sum_d(sg);
+        const double x0 = col[j + 1];
+        if (lane == 0) {
+          if (sg == 0.0) {
+            sc[0] = 0.0;
+            e2[j] = x0 * x0;
+          } else {
+            // u = x0 - alpha, |alpha| = mu; u^2 + sg = 2 mu (mu + |x0|), so tau = 1 / (mu |u|)
+            const double a2 = fma(x0, x0, sg), r = rsqrt(a2), mu = a2 * r;
+            const double u = x0 > 0 ? x0 + mu : x0 - mu;
+            sc[0] = r / fabs(u);
+            sc[1] = u;
+            e2[j] = a2;
+          }
+        }
+      }
+      __syncthreads();
+      const double tau = sc[0];
+      if (tau == 0.0) {
+        __syncthreads();             // col and sc are rewritten by the next step
+        continue;
+      }
+      const double u = sc[1];
+      double vk[R], vi[R];
+#pragma unroll
+      for (int y = b; y < R; ++y) {
+        const int k = tk + 16 * y, i = ti + 16 * y;
+        vk[y] = k <= j ? 0.0 : (k == j + 1 ? u : col[k]);
+        vi[y] = i <= j ? 0.0 : (i == j + 1 ? u : col[i]);
+      }
+      // p = tau M v: row i's 16 partial sums lie in one half-warp
+      double ps[8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) ps[x] = 0.0;
+#pragma unroll
+      for (int x = b; x < R; ++x) {
+        const int i = ti + 16 * x;
+        if (i > j && i < d)            // (whole warps of finished or padding rows skip)
+#pragma unroll
+          for (int y = b; y < R; ++y) ps[x] = fma(m[x][y], vk[y], ps[x]);
+      }
+      // lane bits 0, 1, 2 pick which of the 8 rows a lane goes on with; bit 3 adds the halves
+#pragma unroll
+      for (int h = 4, bit = 1; h >= 1; h >>= 1, bit <<= 1) {
+        const bool up = tk & bit;
+#pragma unroll
+        for (int x = 0; x < h; ++x) {
+          const double send = up ? ps[x] : ps[x + h], keep = up ? ps[x + h] : ps[x];
+          ps[x] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+        }
+      }
+      ps[0] += __shfl_xor_sync(0xffffffffu, ps[0], 8);
+      if (tk < 8) {
+        const int xr = ((tk & 1) << 2) | (tk & 2) | ((tk >> 2) & 1);   // the row this lane kept
+        const int i = ti + 16 * xr;
+        if (xr < R && i > j) w[i] = tau * ps[0];
+      }
+      __syncthreads();
+      if (tid < 32) {
+        double pv = 0.0;
+        for (int i = j + 1 + lane; i < d; i += 32)
+          pv = fma(w[i], i == j + 1 ? u : col[i], pv);
+        pv = warp_sum_d(pv);
+        const double K = 0.5 * tau * pv;
+        for (int i = j + 1 + lane; i < d; i += 32)      // p becomes w
+          w[i] = fma(-K, i == j + 1 ? u : col[i], w[i]);
+      }
+      __syncthreads();
+      double wk[R];
+#pragma unroll
+      for (int y = b; y < R; ++y) {
+        const int k = tk + 16 * y;
+        wk[y] = k <= j || k >= d ? 0.0 : w[k];
+      }
+#pragma unroll
+      for (int x = b; x < R; ++x) {
+        const int i = ti + 16 * x;
+        if (i > j && i < d) {
+          const double nv = -vi[x], nw = -w[i];
+#pragma unroll
+          for (int y = b; y < R; ++y) m[x][y] = fma(nv, wk[y], fma(nw, vk[y], m[x][y]));
+        }
+      }
+    }
   }
-}
-
-// Tridiagonal forms (as k_tilde_tri) of blocks that are already L^{-1} H L^{-T} (Ht, kept up
-// to date by k_round_hupdate): copy to shared memory, Householder reduction.
-__global__ void k_sym_tri(const double* __restrict__ Ht, int d, double* __restrict__ tri,
-                          double* __restrict__ gb) {
-  extern __shared__ double sh[];
-  double* M = sh;
-  double* v = M + d * d;
-  double* p = v + d;
-  double* dg = p + d;
-  double* e2 = dg + d;
-  __shared__ double red[32];
-  const int k = blockIdx.x, tid = threadIdx.x, bd = blockDim.x;
-  const double* Hk = Ht + (int64_t)k * d * d;
-  for (int t = tid; t < d * d; t += bd) M[t] = Hk[t];
+  // the last 2 x 2 block (1 x 1 at d = 1)
+#pragma unroll
+  for (int x = 0; x < R; ++x)
+#pragma unroll
+    for (int y = 0; y < R; ++y) {
+      const int i = ti + 16 * x, k = tk + 16 * y;
+      if (i < d && i == k && i + 2 >= d) dg[i] = m[x][y];
+      if (i == d - 1 && k == d - 2) e2[d - 2] = m[x][y] * m[x][y];
+    }
   __syncthreads();
-  householder_tridiag(d, M, v, p, dg, e2, red);
-  for (int i = tid; i < d; i += bd) {
-    tri[(int64_t)k * 2 * d + i] = dg[i];
-    tri[(int64_t)k * 2 * d + d + i] = i + 1 < d ? e2[i] : 0.0;
+  for (int i = tid; i < d; i += 256) {
+    tri[(int64_t)k0 * 2 * d + i] = dg[i];
+    tri[(int64_t)k0 * 2 * d + d + i] = i + 1 < d ? e2[i] : 0.0;
   }
-  if (tid == 0) {
+  if (tid < 32) {
     double lo = 1e300, hi = -1e300;
-    for (int i = 0; i < d; ++i) {
+    for (int i = lane; i < d; i += 32) {
       const double r = (i > 0 ? sqrt(e2[i - 1]) : 0.0) + (i + 1 < d ? sqrt(e2[i]) : 0.0);
       lo = fmin(lo, dg[i] - r);
       hi = fmax(hi, dg[i] + r);
     }
-    gb[2 * k] = lo;
-    gb[2 * k + 1] = hi;
+    for (int o = 16; o > 0; o >>= 1) {
+      lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+      hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+    if (lane == 0) {
+      gb[2 * k0] = lo;
+      gb[2 * k0 + 1] = hi;
+    }
   }
 }
 
@@ -385,187 +574,173 @@ __global__ void k_similarity(const double* __restrict__ L, const double* __restr
   }
 }
 
-// For A = nu I + eta T (T tridiagonal: diagonal dg, squared off-diagonal e2), the leading
-// principal minors theta_i of A (the continuants theta_i = a_i theta_{i-1} - b_i theta_{i-2},
-// a_i = nu + eta dg_i, b_i = eta^2 e2_{i-1}) and their first three nu-derivatives follow the
-// same three-term recurrence, with no division (rescaled by 2^-400 or 2^400 as they grow or
-// shrink; only ratios are used).  With p = theta'/theta, q = theta''/theta, u = theta'''/theta
-// of the last minor (theta_d = det A, so p = Tr A^-1):
-//   Tr A^-2 = p^2 - q,   d/dnu Tr A^-2 = -2 Tr A^-3 = 3 p q - 2 p^3 - u.
-// Returns false when a minor is not positive (nu at or left of -eta lambda_min).
-__device__ bool tri_trace2(const double* dg, const double* e2, int d, double nu, double eta,
-                           double* f, double* fp) {
-  double u0 = 1.0, u1 = 0.0, u2 = 0.0, u3 = 0.0;                  // theta_{i-2} and derivatives
-  double v0 = nu + eta * dg[0], v1 = 1.0, v2 = 0.0, v3 = 0.0;     // theta_{i-1}
-  if (!(v0 > 0.0)) return false;
-  const double eta2 = eta * eta;
-  for (int i = 1; i < d; ++i) {
-    const double a = nu + eta * dg[i], b = eta2 * e2[i - 1];
-    const double w0 = a * v0 - b * u0;
-    const double w1 = fma(a, v1, v0) - b * u1;
-    const double w2 = fma(a, v2, 2.0 * v1) - b * u2;
-    const double w3 = fma(a, v3, 3.0 * v2) - b * u3;
-    if (!(w0 > 0.0)) return false;
-    u0 = v0; u1 = v1; u2 = v2; u3 = v3;
-    v0 = w0; v1 = w1; v2 = w2; v3 = w3;
-    const double sc = v0 > 0x1p400 ? 0x1p-400 : (v0 < 0x1p-400 ? 0x1p400 : 1.0);
-    if (sc != 1.0) {
-      u0 *= sc; u1 *= sc; u2 *= sc; u3 *= sc;
-      v0 *= sc; v1 *= sc; v2 *= sc; v3 *= sc;
-    }
-  }
-  const double r = 1.0 / v0;
-  const double p = v1 * r, q = v2 * r, uu = v3 * r;
-  *f = p * p - q;
-  *fp = 3.0 * p * q - 2.0 * p * p * p - uu;
-  return true;
-}
-
 // nu of eq. 10 from the c tridiagonal forms: the root of F(nu) = sum_k Tr((nu I + eta T_k)^-2)
 // = 1, which is what sum_j (nu + eta lambda_j)^-2 = 1 states, the trace taken without the
-// eigenvalues.  Newton runs on psi(nu) = F^(-1/2) - 1: a power mean of the nu + eta lambda_j
-// (exponent -2) minus 1, increasing, concave and close to linear right of -eta lambda_min, so
-// the iterates reach the root in a few steps; they stay inside the bracket
-// [-eta max Gershgorin, sqrt(c d) - eta min Gershgorin], and a step that leaves it, or a trial
-// outside the SPD domain, bisects instead.  One block; thread k evaluates block k (and
-// k + blockDim, ...).
-__global__ void k_nu_tri(const double* __restrict__ tri, const double* __restrict__ gb, int c,
-                         int d, double eta, double* nu_out) {
-  __shared__ double red[32];
-  __shared__ double wmn[32], wmx[32];
-  __shared__ double s_lo, s_hi, s_nu;
-  __shared__ int s_bad, s_done;
-  double mn = 1e300, mx = -1e300;
-  for (int k = threadIdx.x; k < c; k += blockDim.x) {
-    mn = fmin(mn, gb[2 * k]);
-    mx = fmax(mx, gb[2 * k + 1]);
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-    mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-  }
-  if ((threadIdx.x & 31) == 0) {
-    wmn[threadIdx.x >> 5] = mn;
-    wmx[threadIdx.x >> 5] = mx;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double a = 1e300, b = -1e300;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      a = fmin(a, wmn[w]);
-      b = fmax(b, wmx[w]);
-    }
-    s_lo = -eta * b;
-    s_hi = sqrt((double)c * d) - eta * a;
-    s_nu = s_hi;
-    s_done = 0;
-  }
-  __syncthreads();
-  for (int it = 0; it < 300; ++it) {
-    const double nu = s_nu;
-    double f = 0.0, fp = 0.0;
-    int bad = 0;
-    for (int k = threadIdx.x; k < c; k += blockDim.x) {
-      double fk, fpk;
-      if (tri_trace2(tri + (int64_t)k * 2 * d, tri + (int64_t)k * 2 * d + d, d, nu, eta, &fk,
-                     &fpk)) {
-        f += fk;
-        fp += fpk;
-      } else {
-        bad = 1;
-      }
-    }
-    if (threadIdx.x == 0) s_bad = 0;
-    __syncthreads();
-    if (bad) atomicOr(&s_bad, 1);
-    const double F = block_sum_d(f, red);   // (synchronises: s_bad is complete after it)
-    const double FP = block_sum_d(fp, red);
-    if (threadIdx.x == 0) {
-      double lo = s_lo, hi = s_hi;
-      const bool left = s_bad || F - 1.0 > 0.0;   // left of the root, or of the domain
-      if (left) lo = nu;
-      else hi = nu;
-      if (!s_bad && F - 1.0 == 0.0) {
-        s_done = 1;
-      } else {
-        // psi = F^-1/2 - 1, psi' = -F^-3/2 F' / 2: nu - psi / psi' = nu + 2 (F - F^3/2) / F'
-        const bool newton = !s_bad && FP < 0.0 && F > 0.0;
-        const double step = newton ? 2.0 * (F - F * sqrt(F)) / FP : 0.0;
-        if (newton && fabs(step) <= 1e-12 * fabs(nu)) {
-          s_nu = nu + step;   // converged (as in k_nu_coop)
-          s_done = 1;
-        } else {
-          double nx = newton ? nu + step : 0.5 * (lo + hi);
-          if (!(nx > lo && nx < hi)) nx = 0.5 * (lo + hi);
-          if (nx == nu || hi - lo <= 4e-16 * fmax(fabs(lo), fabs(hi))) s_done = 1;
-          s_nu = nx;
-        }
-      }
-      s_lo = lo;
-      s_hi = hi;
-    }
-    __syncthreads();
-    if (s_done) break;
-  }
-  if (threadIdx.x == 0) *nu_out = s_nu;
-}
+// eigenvalues.
+//
+// For A = nu I + eta T (diagonal dg, squared off-diagonal e2), the leading principal minors
+// theta_i of A (the continuants theta_i = a_i theta_{i-1} - b_i theta_{i-2}, a_i = nu + eta dg_i,
+// b_i = eta^2 e2_{i-1}) and their nu-derivatives follow the same three-term recurrence, with no
+// division (rescaled by 2^-400 or 2^400 as they grow or shrink; only ratios are used).  With
+// t_q = theta^(q) / q!, t_q,i = a_i t_q,i-1 + t_{q-1},i-1 - b_i t_q,i-2, and with p, q2, u the
+// ratios of the first, second and third derivative of theta to theta at the last minor (theta_d = det A):
+//   Tr A^-2 = p^2 - q2,   d/dnu Tr A^-2 = -2 Tr A^-3 = 3 p q2 - 2 p^3 - u.
+//
+// Newton runs on psi(nu) = F^(-1/2) - 1: a power mean of the nu + eta lambda_j (exponent -2)
+// minus 1, increasing, concave and close to linear right of -eta lambda_min, so the iterates
+// reach the root in a few steps; they stay inside the bracket [-eta max Gershgorin,
+// sqrt(c d) - eta min Gershgorin], and a step that leaves it, or a trial outside the SPD domain
+// (a minor that is not positive), bisects instead.
+//
+// An SM sub-partition takes a warp's FP64 instruction in 64 cycles however few lanes it has, so
+// the four recurrences t_0..t_3 of a class lie in four lanes (two multiply-adds a step, the
+// neighbour's term by shuffle) and a warp runs eight classes; a_i is formed by all threads
+// before each evaluation.  Blocks of four warps, one grid barrier per step (partials double-
+// buffered by step parity; every block takes the same step from them).  c = 100, d = 128:
+// 0.29 ms a call, 1.6 ms with one lane per class and 14 FP64 instructions a step; c = d = 50:
+// 0.11, 0.58 ms before.
+// part: 2 x 3 doubles per block; nu0: a first iterate (taken when inside the bracket) or NULL.
+constexpr int NU_CLASSES = 32;   // classes per block
 
-// The same root on many SMs at once.  GB300 runs FP64 at a small fraction of its FP32 rate per
-// SM, and each block's recursion is sequential, so one block evaluating all c blocks spends
-// most of its time waiting on one SM's FP64 pipe: here block b evaluates classes b, b + grid,
-// ... (its lane 0 runs each recursion), and block 0 combines the partials in a fixed order and
-// takes the step.  Cooperative launch (every block resident), two grid barriers per step.
-// st: [lo, hi, nu, done]; part: 3 doubles per block (F, F', out-of-domain).
-__global__ void k_nu_coop(const double* __restrict__ tri, const double* __restrict__ gb, int c,
-                          int d, double eta, double* st, double* part, double* nu_out) {
+__global__ __launch_bounds__(128) void k_nu_coop(const double* __restrict__ tri,
+                                                 const double* __restrict__ gb, int c, int d,
+                                                 double eta, const double* nu0, double* part,
+                                                 double* nu_out) {
   cg::grid_group grid = cg::this_grid();
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  extern __shared__ double sh[];
+  __shared__ double red[3][4], st[4];   // lo, hi, nu, done
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int ld = d | 1;
+  double* as = sh;                      // [32][ld] a_i
+  double* es = as + NU_CLASSES * ld;    // [32][ld] eta dg_i
+  double* bs = es + NU_CLASSES * ld;    // [32][ld] -b_i
+  const bool once = c <= (int)gridDim.x * NU_CLASSES;   // this block's classes: loaded once
+  const int ci = tid >> 2, q = tid & 3; // class of the block, derivative
+  const double eta2 = eta * eta;
+  {
     double a = 1e300, b = -1e300;
-    for (int k = 0; k < c; ++k) {
+    for (int k = tid; k < c; k += 128) {
       a = fmin(a, gb[2 * k]);
       b = fmax(b, gb[2 * k + 1]);
     }
-    st[0] = -eta * b;
-    st[1] = sqrt((double)c * d) - eta * a;
-    st[2] = st[1];
-    st[3] = 0.0;
+    for (int o = 16; o > 0; o >>= 1) {
+      a = fmin(a, __shfl_xor_sync(0xffffffffu, a, o));
+      b = fmax(b, __shfl_xor_sync(0xffffffffu, b, o));
+    }
+    if (lane == 0) {
+      red[0][wid] = a;
+      red[1][wid] = b;
+    }
+    __syncthreads();
+    if (tid == 0) {
+      for (int x = 1; x < 4; ++x) {
+        a = fmin(a, red[0][x]);
+        b = fmax(b, red[1][x]);
+      }
+      st[0] = -eta * b;
+      st[1] = sqrt((double)c * d) - eta * a;
+      const double n0 = nu0 ? *nu0 : st[1];
+      st[2] = n0 > st[0] && n0 < st[1] ? n0 : st[1];
+      st[3] = 0.0;
+    }
   }
-  grid.sync();
   for (int it = 0; it < 300; ++it) {
+    __syncthreads();
     const double nu = st[2];
-    if (threadIdx.x == 0) {
-      double f = 0.0, fp = 0.0, bad = 0.0;
-      for (int k = blockIdx.x; k < c; k += gridDim.x) {
-        double fk, fpk;
-        if (tri_trace2(tri + (int64_t)k * 2 * d, tri + (int64_t)k * 2 * d + d, d, nu, eta, &fk,
-                       &fpk)) {
-          f += fk;
-          fp += fpk;
+    double f = 0.0, fp = 0.0, bad = 0.0;
+    for (int base = blockIdx.x * NU_CLASSES; base < c; base += gridDim.x * NU_CLASSES) {
+      const int nc = min(NU_CLASSES, c - base);
+      if (it == 0 || !once) {
+        __syncthreads();
+        for (int x = wid; x < nc; x += 4) {
+          const double* t = tri + (int64_t)(base + x) * 2 * d;
+#pragma unroll 4
+          for (int i = lane; i < d; i += 32) {
+            es[x * ld + i] = eta * t[i];
+            bs[x * ld + i] = i > 0 ? -eta2 * t[d + i - 1] : 0.0;
+          }
+        }
+        __syncthreads();
+      }
+      for (int x = wid; x < nc; x += 4)
+        for (int i = lane; i < d; i += 32) as[x * ld + i] = nu + es[x * ld + i];
+      __syncthreads();
+      const int x = min(ci, nc - 1);    // idle lanes repeat the last class
+      double u = q == 0 ? 1.0 : 0.0, v = q == 0 ? as[x * ld] : (q == 1 ? 1.0 : 0.0);
+      // sign and exponent of theta by integer tests (no FP64 issue): the sign of every minor in
+      // the group's first lane, the exponent every fourth step (a step scales by at most
+      // |a_i| + |b_i|, far below 2^150)
+      bool ok = __double2hiint(v) > 0;
+      auto step = [&](int i) {
+        double lower = __shfl_up_sync(0xffffffffu, v, 1, 4);
+        if (q == 0) lower = 0.0;
+        const double nv = fma(as[x * ld + i], v, fma(bs[x * ld + i], u, lower));
+        u = v;
+        v = nv;
+        const int hi = __double2hiint(v);
+        ok = ok && hi > 0 && hi < 0x7ff00000;
+      };
+      int i = 1;
+      for (; i + 3 < d; i += 4) {
+        step(i);
+        step(i + 1);
+        step(i + 2);
+        step(i + 3);
+        const int ex = __shfl_sync(0xffffffffu, __double2hiint(v), lane & ~3) >> 20 & 0x7ff;
+        if (ex > 1023 + 400 || (ex < 1023 - 400 && ex > 0)) {
+          const double sc = ex > 1023 ? 0x1p-400 : 0x1p400;
+          u *= sc;
+          v *= sc;
+        }
+      }
+      for (; i < d; ++i) step(i);
+      const double t0 = __shfl_sync(0xffffffffu, v, lane & ~3);
+      const double t1 = __shfl_sync(0xffffffffu, v, (lane & ~3) + 1);
+      const double t2 = __shfl_sync(0xffffffffu, v, (lane & ~3) + 2);
+      const double t3 = __shfl_sync(0xffffffffu, v, (lane & ~3) + 3);
+      if (q == 0 && ci < nc) {
+        if (ok) {
+          const double r = 1.0 / t0;
+          const double p = t1 * r, qq = 2.0 * t2 * r, uu = 6.0 * t3 * r;
+          f += p * p - qq;
+          fp += 3.0 * p * qq - 2.0 * p * p * p - uu;
         } else {
           bad = 1.0;
         }
       }
-      part[3 * blockIdx.x] = f;
-      part[3 * blockIdx.x + 1] = fp;
-      part[3 * blockIdx.x + 2] = bad;
+    }
+    f = warp_sum_d(f);
+    fp = warp_sum_d(fp);
+    bad = warp_sum_d(bad);
+    if (lane == 0) {
+      red[0][wid] = f;
+      red[1][wid] = fp;
+      red[2][wid] = bad;
+    }
+    __syncthreads();
+    double* pt = part + (size_t)(it & 1) * 3 * gridDim.x;
+    if (tid < 3) {
+      double a = 0.0;
+      for (int x = 0; x < 4; ++x) a += red[tid][x];
+      pt[3 * blockIdx.x + tid] = a;
     }
     grid.sync();
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      double F = 0.0, FP = 0.0;
-      bool bad = false;
+    if (tid == 0) {
+      double F = 0.0, FP = 0.0, nbad = 0.0;
       for (int b = 0; b < (int)gridDim.x; ++b) {
-        F += part[3 * b];
-        FP += part[3 * b + 1];
-        bad = bad || part[3 * b + 2] != 0.0;
+        F += __ldcg(pt + 3 * b);
+        FP += __ldcg(pt + 3 * b + 1);
+        nbad += __ldcg(pt + 3 * b + 2);
       }
+      const bool off = nbad > 0.0;
       double lo = st[0], hi = st[1];
-      if (bad || F - 1.0 > 0.0) lo = nu;   // left of the root, or of the domain
+      if (off || F - 1.0 > 0.0) lo = nu;   // left of the root, or of the domain
       else hi = nu;
-      if (!bad && F - 1.0 == 0.0) {
+      if (!off && F - 1.0 == 0.0) {
         st[3] = 1.0;
       } else {
         // psi = F^-1/2 - 1, psi' = -F^-3/2 F' / 2: nu - psi / psi' = nu + 2 (F - F^3/2) / F'
-        const bool newton = !bad && FP < 0.0 && F > 0.0;
+        const bool newton = !off && FP < 0.0 && F > 0.0;
         const double step = newton ? 2.0 * (F - F * sqrt(F)) / FP : 0.0;
         // Newton converges quadratically: a step below 1e-12 nu leaves the next one far below
         // the accuracy of F itself (~1e-13, the continuant ratios), so take it and stop
@@ -582,47 +757,43 @@ __global__ void k_nu_coop(const double* __restrict__ tri, const double* __restri
       st[0] = lo;
       st[1] = hi;
     }
-    grid.sync();
+    __syncthreads();
     if (st[3] != 0.0) break;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) *nu_out = st[2];
+  if (blockIdx.x == 0 && tid == 0) *nu_out = st[2];
 }
 
 int32_t sym_tri(const double* Ht, int nblocks, int d, double* tri, double* gb, cudaStream_t st) {
-  const size_t smem = ((size_t)d * d + 4 * (size_t)d) * sizeof(double);
-  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_sym_tri, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      200 * 1024));
+  if (d > 128) return fail(FIRAL_ERR_UNSUPPORTED, "tridiagonal forms need d <= 128");
   ProfScope ps(st, PF_ROUND);
   count_launch();
-  k_sym_tri<<<nblocks, threads_for(d), smem, st>>>(Ht, d, tri, gb);
+  if (d <= 16) k_sym_tri<1><<<nblocks, 256, 0, st>>>(Ht, d, tri, gb);
+  else if (d <= 32) k_sym_tri<2><<<nblocks, 256, 0, st>>>(Ht, d, tri, gb);
+  else if (d <= 64) k_sym_tri<4><<<nblocks, 256, 0, st>>>(Ht, d, tri, gb);
+  else if (d <= 96) k_sym_tri<6><<<nblocks, 256, 0, st>>>(Ht, d, tri, gb);
+  else k_sym_tri<8><<<nblocks, 256, 0, st>>>(Ht, d, tri, gb);
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
 }
 
 // nu from c tridiagonal forms (tri: 2 c d doubles, gb: 2 c) on up to one block per SM;
-// work: 4 + 3 * SMs doubles of step state and per-block partials.
-int32_t nu_of_tri(const double* tri, const double* gb, int c, int d, double eta, double* work,
-                  double* nu_out, cudaStream_t st) {
+// part: 6 doubles per SM; nu0 (device) may be NULL.
+int32_t nu_of_tri(const double* tri, const double* gb, int c, int d, double eta,
+                  const double* nu0, double* part, double* nu_out, cudaStream_t st) {
   ProfScope ps(st, PF_ROUND);
   count_launch();
   int dev = 0, sms = 0;
   FIRAL_CUDA_TRY(cudaGetDevice(&dev));
   FIRAL_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-  int nb = c < sms ? c : sms;
-  double* state = work;
-  double* part = state + 4;
-  void* args[] = {(void*)&tri, (void*)&gb, (void*)&c, (void*)&d, (void*)&eta, (void*)&state,
-                  (void*)&part, (void*)&nu_out};
-  FIRAL_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_nu_coop, dim3(nb), dim3(32), args, 0,
-                                             st));
+  const int nb = std::min((c + NU_CLASSES - 1) / NU_CLASSES, sms);
+  const size_t smem = (size_t)3 * NU_CLASSES * (d | 1) * sizeof(double);
+  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_nu_coop, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      128 * 1024));
+  void* args[] = {(void*)&tri, (void*)&gb,  (void*)&c,    (void*)&d,
+                  (void*)&eta, (void*)&nu0, (void*)&part, (void*)&nu_out};
+  FIRAL_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)k_nu_coop, dim3(nb), dim3(128), args,
+                                             smem, st));
   return FIRAL_OK;
-}
-
-int32_t sym_tri_nu(const double* Ht, int c, int d, double eta, double* tri, double* gb,
-                   double* nu_out, cudaStream_t st) {
-  FIRAL_TRY(sym_tri(Ht, c, d, tri, gb, st));
-  // the step state and the per-block partials live after the bounds in the caller's buffer
-  return nu_of_tri(tri, gb, c, d, eta, gb + 2 * (size_t)c, nu_out, st);
 }
 
 int32_t similarity_blocks(const double* L, const double* H, int c, int d, double* out,
@@ -633,19 +804,6 @@ int32_t similarity_blocks(const double* L, const double* H, int c, int d, double
   ProfScope ps(st, PF_ROUND);
   count_launch();
   k_similarity<<<c, threads_for(d), smem, st>>>(L, H, d, out);
-  FIRAL_CUDA_TRY(cudaGetLastError());
-  return FIRAL_OK;
-}
-
-int32_t tilde_nu(const double* L, const double* H, int c, int d, double eta, double* tri,
-                 double* gb, double* nu_out, cudaStream_t st) {
-  const size_t smem = ((size_t)d * d + 5 * (size_t)d) * sizeof(double);
-  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_tilde_tri, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      200 * 1024));
-  ProfScope ps(st, PF_ROUND);
-  count_launch(2);
-  k_tilde_tri<<<c, threads_for(d), smem, st>>>(L, H, d, tri, gb);
-  k_nu_tri<<<1, 256, 0, st>>>(tri, gb, c, d, eta, nu_out);
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
 }
