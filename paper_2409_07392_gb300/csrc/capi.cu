@@ -185,6 +185,30 @@ int32_t DBuf::ensure(size_t nbytes) {
   return FIRAL_OK;
 }
 
+int32_t CGStateRead::ensure(int n) {
+  for (auto& e : ev)
+    if (!e) FIRAL_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+  if (n <= cap && host) return FIRAL_OK;
+  if (host) cudaFreeHost(host);
+  host = nullptr;
+  cap = 0;
+  void* p = nullptr;
+  FIRAL_CUDA_TRY(cudaMallocHost(&p, (size_t)2 * n * sizeof(int)));
+  host = static_cast<int*>(p);
+  cap = n;
+  return FIRAL_OK;
+}
+
+void CGStateRead::release() {
+  if (host) cudaFreeHost(host);
+  host = nullptr;
+  cap = 0;
+  for (auto& e : ev) {
+    if (e) cudaEventDestroy(e);
+    e = nullptr;
+  }
+}
+
 void DBuf::release() {
   if (p) cudaFree(p);
   p = nullptr;
@@ -303,9 +327,9 @@ int32_t ensure_cg(firal_problem* P, int s) {
   FIRAL_TRY(P->cgP.ensure(vb));
   FIRAL_TRY(P->cgQ.ensure(vb));
   FIRAL_TRY(P->cgZ.ensure(vb));
-  FIRAL_TRY(P->cgcols.ensure((size_t)s * pool_count(P->pt) * sizeof(CGCol)));
+  FIRAL_TRY(P->cgcols.ensure((size_t)2 * s * pool_count(P->pt) * sizeof(CGCol)));
   FIRAL_TRY(P->cgpart1.ensure((size_t)s * P->c * sizeof(double)));
-  FIRAL_TRY(P->cgpart2.ensure((size_t)s * P->c * sizeof(double)));
+  FIRAL_TRY(P->cgpart2.ensure((size_t)2 * s * P->c * sizeof(double)));
   // block PCG: c * s * s partials, six s x s matrices, flag
   FIRAL_TRY(P->bcg.ensure(((size_t)P->c * s * s + 6 * (size_t)s * s + 1) * sizeof(double)));
   return FIRAL_OK;
@@ -414,8 +438,28 @@ int32_t pcg_run(firal_problem* P, const void* B, int s, const firal_cg_opts& cg,
   FIRAL_TRY(cg_init(P, B, s, tol, fixed));
   const int ns = s * pool_count(P->pt);   // one CG scalar set per (column, pool)
   std::vector<CGCol> cols(ns);
+  // Tolerance mode reads the columns' states back to know when to stop.  Waiting for each
+  // iteration's state leaves the GPU idle for the read and the next launches (about 30 us); when
+  // an apply costs no more than that, the next iteration is enqueued first and the state of the
+  // one before it is waited for: stopped columns do not change, so the one extra iteration at
+  // the end leaves every result as it is.
+  const double apply_us =
+      4.0 * P->N * P->D * s / (P->dbl ? 1e6 : is_mixed(P->prec) ? 5e8 : 3e7);
+  const bool lag = !fixed && !sharded(P) && apply_us <= 60.0;
+  // (the last kernel of an iteration writes the flags to page-locked host memory: a copy on the
+  // stream between the kernels cost another 10 us an iteration)
+  CGStateRead& rd = P->H->cg_state;
+  if (lag) FIRAL_TRY(rd.ensure(ns));
   for (int it = 0; it < iters; ++it) {
-    if (!fixed) {
+    if (lag && it > 1) {
+      const int slot = (it - 1) & 1;     // the flags after it - 1 iterations
+      FIRAL_CUDA_TRY(cudaEventSynchronize(rd.ev[slot]));
+      const volatile int* active = rd.at(slot, ns);
+      bool any = false;
+      for (int j = 0; j < ns; ++j) any |= active[j] != 0;
+      if (!any) break;
+    }
+    if (!fixed && !lag) {
       FIRAL_CUDA_TRY(cudaMemcpyAsync(cols.data(), P->cgcols.p, ns * sizeof(CGCol),
                                      cudaMemcpyDeviceToHost, st));
       FIRAL_CUDA_TRY(cudaStreamSynchronize(st));
@@ -424,7 +468,9 @@ int32_t pcg_run(firal_problem* P, const void* B, int s, const firal_cg_opts& cg,
       if (!any) break;
     }
     FIRAL_TRY(apply(P, P->w_sig.p, P->S_sig.p, P->cgP.p, s, P->cgQ.p, P->cgpart1.as<double>()));
-    FIRAL_TRY(cg_iterate_tail(P, s, tol, fixed));
+    const int slot = (it + 1) & 1;
+    FIRAL_TRY(cg_iterate_tail(P, s, tol, fixed, lag ? rd.at(slot, ns) : nullptr));
+    if (lag) FIRAL_CUDA_TRY(cudaEventRecord(rd.ev[slot], st));
   }
   FIRAL_CUDA_TRY(cudaMemcpyAsync(X_out, P->cgX.p, (size_t)s * P->D * vsize(P),
                                  cudaMemcpyDeviceToDevice, st));
@@ -580,7 +626,7 @@ int32_t relax_step_impl(firal_problem* P, const firal_relax_opts* o, int32_t t, 
   void* zdev = (char*)P->w_sig.p + P->m * vsize(P);
   if (P->pt.Q) FIRAL_TRY(md_step_pooled(P, zdev, P->g.p, o->beta0, st));   // per-pool simplex
   else if (sharded(P)) FIRAL_TRY(md_step_sharded(P, zdev, P->g.p, budget, o->beta0, red, st));
-  else FIRAL_TRY(md_step_simt(P->dbl, zdev, P->g.p, P->n, budget, o->beta0, red, st));
+  else FIRAL_TRY(md_step_simt(P->dbl, zdev, P->g.p, P->n, budget, o->beta0, red, want, st));
   FIRAL_CUDA_TRY(cudaMemcpyAsync(z, zdev, P->n * vsize(P), cudaMemcpyDeviceToDevice, st));
   if (device_t) FIRAL_TRY(tick(P->tdev.as<int64_t>(), st));
   if (stats) {
@@ -1289,6 +1335,7 @@ int32_t firal_destroy(firal_handle* H) {
   cudaStreamSynchronize(H->stream);
   H->flags.release();
   H->scratch.release();
+  H->cg_state.release();
   delete H;
   return FIRAL_OK;
 }
@@ -1528,7 +1575,7 @@ int32_t firal_md_step(firal_problem* P, void* z, const void* g, double budget, d
   firal_handle* H = P ? P->H : nullptr;
   if (!P || !z || !g || !(budget > 0)) return record(H, fail(FIRAL_ERR_ARG, "bad md_step arguments"));
   return record(H, md_step_simt(P->dbl, z, g, P->n, budget, beta0, P->red.as<double>(),
-                                P->H->stream));
+                                false, P->H->stream));
 }
 
 int32_t firal_objective_fwd(firal_problem* P, const void* z, uint64_t seed, int32_t t, int32_t s,

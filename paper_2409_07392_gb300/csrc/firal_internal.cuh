@@ -66,6 +66,17 @@ struct CGCol {
   int32_t iters;    // iterations taken
 };
 
+// Two page-locked sets of the columns' active flags, written by the CG kernels, and their events
+// (one handle's solves run one after another).
+struct CGStateRead {
+  int* host = nullptr;
+  int cap = 0;
+  cudaEvent_t ev[2] = {nullptr, nullptr};
+  int32_t ensure(int n);
+  void release();
+  int* at(int slot, int n) const { return host + (size_t)slot * n; }
+};
+
 // Device-side status words written by kernels and read by the host on synchronising calls.
 struct DevFlags {
   int32_t not_spd;     // set by a Cholesky that met a non-positive pivot
@@ -113,6 +124,7 @@ struct firal_handle {
   cudaStream_t stream = nullptr;
   firal::DBuf flags;       // firal::DevFlags
   firal::DBuf scratch;     // small reductions
+  firal::CGStateRead cg_state;   // tolerance-mode solves: the columns' states read back
   std::string err;
 };
 
@@ -278,11 +290,12 @@ int32_t syrk_reduce_f32(firal_problem* P, const float* partS, const float* partP
 int32_t combine_f32(firal_problem* P, const float* Sblk, const float* V, int splits, int s,
                     float* out, double* pq, const float* vmean);
 int32_t cg_init(firal_problem* P, const void* B, int s, double tol, int fixed);
-int32_t cg_iterate_tail(firal_problem* P, int s, double tol, int fixed);
+int32_t cg_iterate_tail(firal_problem* P, int s, double tol, int fixed,
+                        int* host_active = nullptr);
 int32_t dot_scaled(bool dbl, const void* a, const void* b, int64_t total, double scale,
                    double* part, double* out, cudaStream_t st);
 int32_t md_step_simt(bool dbl, void* z, const void* g, int64_t n, double budget, double beta0,
-                     double* red, cudaStream_t st);
+                     double* red, bool want_zmax, cudaStream_t st);
 int32_t md_step_sharded(firal_problem* P, void* z, const void* g, double budget, double beta0,
                         double* red, cudaStream_t st);
 int32_t block_dots(firal_problem* P, const void* V, const void* out, int s, double* pq);

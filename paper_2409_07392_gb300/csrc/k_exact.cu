@@ -1189,7 +1189,8 @@ int32_t exact_relax(firal_problem* P, double budget, int T, double beta0, const 
     double f = 0.0;
     FIRAL_TRY(exact_objective(P, z, &f, P->g.p));          // Algorithm 1 lines 5-6
     if (hist) hist[t] = f;
-    FIRAL_TRY(md_step_simt(P->dbl, z, P->g.p, P->n, budget, beta0, P->red.as<double>(), st));
+    FIRAL_TRY(md_step_simt(P->dbl, z, P->g.p, P->n, budget, beta0, P->red.as<double>(), false,
+                           st));
   }
   return FIRAL_OK;
 }

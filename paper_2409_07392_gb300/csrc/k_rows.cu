@@ -666,25 +666,26 @@ __global__ void k_row_combine(const T* __restrict__ S, const T* __restrict__ V,
     for (int sp = g; sp < splits; sp += SG) ds += dp[sp * stride];
     acc -= ds;
   }
-  if (SG > 1) {
-    gs[(g * JB + jj) * dpad + e] = acc;
+  for (int h = SG >> 1; h > 0; h >>= 1) {   // SG is a power of two
+    T* slot = gs + (size_t)(jj * dpad + e);
     __syncthreads();
-    if (g == 0)
-      for (int x = 1; x < SG; ++x) acc += gs[(x * JB + jj) * dpad + e];
+    if (g >= h && g < 2 * h) slot[(size_t)g * JB * dpad] = acc;
+    __syncthreads();
+    if (g < h) acc += slot[(size_t)(g + h) * JB * dpad];
   }
   const bool own = g == 0 && j < s && e < d;
   if (own) out[(int64_t)j * D + (int64_t)k * d + e] = acc;
-  if (pq) {
+  if (pq && g == 0) {   // (whole warps; the others have no share)
     double v = own ? (double)vs[jj * d + e] * (double)acc : 0.0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (own && e == 0) {
-      double tot = 0.0;
-      for (int w = 0; w < dpad / 32; ++w) tot += red[(threadIdx.x >> 5) + w];
-      pq[(int64_t)j * c + k] = tot;
-    }
+  }
+  __syncthreads();
+  if (pq && own && e == 0) {
+    double tot = 0.0;
+    for (int w = 0; w < dpad / 32; ++w) tot += red[(threadIdx.x >> 5) + w];
+    pq[(int64_t)j * c + k] = tot;
   }
 }
 
@@ -972,8 +973,10 @@ int32_t form_launch(firal_problem* P, FormArgs a, int64_t rows, int* ny, cudaStr
 // ------------------------------------------------------------------------------------------
 // k_row_form_d (FP64): 32 rows per block, one warp per probe, 4 classes at a time; h is read
 // class-major so that a warp's 32 rows are one run.  Bound by the FP64 rate (n = 3,000, d = 20,
-// c = s = 10: 23 us a launch, 137 with 128 rows per block; 10 us at 1.25 TFLOP/s).
+// c = s = 10: 20 us a launch, 137 with 128 rows per block; 10 us at 1.25 TFLOP/s).
 // ------------------------------------------------------------------------------------------
+constexpr int FORM_D_STAGE = 512;   // doubles of a probe's coefficients staged at a time, per warp
+
 template <int MODE>
 __global__ __launch_bounds__(256) void k_row_form_d(
     const double* __restrict__ Xa, const double* __restrict__ HaT, const double* __restrict__ w,
@@ -984,71 +987,74 @@ __global__ __launch_bounds__(256) void k_row_form_d(
   const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int ldx = d | 1;
   double* xs = (double*)smem_raw;               // [32][ldx]
-  double* va = xs + 32 * ldx;                   // [nw][KC][d]
-  double* vb = va + (size_t)nw * KC * d;        // MODE 1
+  double* va = xs + 32 * ldx + (size_t)wid * FORM_D_STAGE;                 // this warp's
+  double* vb = va + (size_t)nw * FORM_D_STAGE;                             // MODE 1
   __shared__ double red[8][33];
   const int64_t i0 = row0 + (int64_t)blockIdx.x * 32;
   const int64_t i = i0 + lane;
   const bool rv = i < N;
   const int j = blockIdx.y * nw + wid;
-  for (int q = threadIdx.x; q < 32 * d; q += blockDim.x) {
-    const int r = q / d, e = q - r * d;
-    xs[r * ldx + e] = i0 + r < N ? Xa[(i0 + r) * d + e] : 0.0;
-  }
+#pragma unroll 8
+  for (int r = wid; r < 32; r += nw)
+    for (int e = lane; e < d; e += 32) xs[r * ldx + e] = i0 + r < N ? Xa[(i0 + r) * d + e] : 0.0;
+  __syncthreads();
   double s0 = 0.0, s1 = 0.0, s2 = 0.0;
   const double* x = xs + lane * ldx;
-  for (int k0 = 0; k0 < c; k0 += KC) {
-    __syncthreads();
-    if (j < s) {
-      const int kn = min(KC, c - k0) * d;
-      const int64_t o = (int64_t)j * D + (int64_t)k0 * d;
-      for (int q = lane; q < KC * d; q += 32) {
-        va[wid * KC * d + q] = q < kn ? A[o + q] : 0.0;
-        if (MODE == 1) vb[wid * KC * d + q] = q < kn ? B[o + q] : 0.0;
+  const int ks = max(KC, min((c + KC - 1) / KC * KC, FORM_D_STAGE / d / KC * KC));
+  if (j < s) {
+    for (int kb = 0; kb < c; kb += ks) {
+      const int kn = min(ks, c - kb) * d;
+      const int64_t o = (int64_t)j * D + (int64_t)kb * d;
+      __syncwarp();
+#pragma unroll 4
+      for (int q = lane; q < FORM_D_STAGE; q += 32) {
+        if (q >= ks * d) break;
+        va[q] = q < kn ? A[o + q] : 0.0;
+        if (MODE == 1) vb[q] = q < kn ? B[o + q] : 0.0;
       }
-    }
-    __syncthreads();
-    if (j >= s) continue;
-    double ga[KC], gb[KC];
-#pragma unroll
-    for (int q = 0; q < KC; ++q) ga[q] = gb[q] = 0.0;
-    const double* pa = va + wid * KC * d;
-    const double* pb = vb + wid * KC * d;
-    double hv[KC];
-#pragma unroll
-    for (int q = 0; q < KC; ++q)
-      hv[q] = rv && k0 + q < c ? HaT[(int64_t)(k0 + q) * N + i] : 0.0;
-    if (k0 + KC <= c) {
-#pragma unroll 2
-      for (int e = 0; e < d; ++e) {
-        const double xe = x[e];
+      __syncwarp();
+      for (int k0 = kb; k0 < min(c, kb + ks); k0 += KC) {
+        double ga[KC], gb[KC], hv[KC];
+        const double* pa = va + (k0 - kb) * d;
+        const double* pb = vb + (k0 - kb) * d;
 #pragma unroll
         for (int q = 0; q < KC; ++q) {
-          ga[q] = fma(xe, pa[q * d + e], ga[q]);
-          if (MODE == 1) gb[q] = fma(xe, pb[q * d + e], gb[q]);
+          ga[q] = gb[q] = 0.0;
+          hv[q] = rv && k0 + q < c ? HaT[(int64_t)(k0 + q) * N + i] : 0.0;
         }
-      }
-    } else {                       // the last classes: no multiply-adds on padding
-      const int kn = c - k0;
-      for (int e = 0; e < d; ++e) {
-        const double xe = x[e];
+        if (k0 + KC <= c) {
+#pragma unroll 2
+          for (int e = 0; e < d; ++e) {
+            const double xe = x[e];
 #pragma unroll
-        for (int q = 0; q < KC - 1; ++q)
-          if (q < kn) {
-            ga[q] = fma(xe, pa[q * d + e], ga[q]);
-            if (MODE == 1) gb[q] = fma(xe, pb[q * d + e], gb[q]);
+            for (int q = 0; q < KC; ++q) {
+              ga[q] = fma(xe, pa[q * d + e], ga[q]);
+              if (MODE == 1) gb[q] = fma(xe, pb[q * d + e], gb[q]);
+            }
           }
-      }
-    }
+        } else {                   // the last classes: no multiply-adds on padding
+          const int kr = c - k0;
+          for (int e = 0; e < d; ++e) {
+            const double xe = x[e];
 #pragma unroll
-    for (int q = 0; q < KC; ++q) {
-      if (MODE == 0) {
-        s0 = fma(hv[q], ga[q], s0);
-      } else {
-        const double ha = hv[q] * ga[q];
-        s0 = fma(ha, gb[q], s0);
-        s1 += ha;
-        s2 = fma(hv[q], gb[q], s2);
+            for (int q = 0; q < KC - 1; ++q)
+              if (q < kr) {
+                ga[q] = fma(xe, pa[q * d + e], ga[q]);
+                if (MODE == 1) gb[q] = fma(xe, pb[q * d + e], gb[q]);
+              }
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < KC; ++q) {
+          if (MODE == 0) {
+            s0 = fma(hv[q], ga[q], s0);
+          } else {
+            const double ha = hv[q] * ga[q];
+            s0 = fma(ha, gb[q], s0);
+            s1 += ha;
+            s2 = fma(hv[q], gb[q], s2);
+          }
+        }
       }
     }
   }
@@ -1065,14 +1071,20 @@ __global__ __launch_bounds__(256) void k_row_form_d(
   }
 }
 
-int form_d_warps(int s) { return (s + (s + 7) / 8 - 1) / ((s + 7) / 8); }
+// Warps (probes) per block: 4 while the grid is small, so that every block loads all four
+// sub-partitions and the blocks spread evenly over the SMs (n = 3,000, s = 10: 285 blocks, at
+// most two per SM; 190 blocks of 5 warps took 23 us, 475 of 2 warps, on two sub-partitions, 22),
+// up to 8 to share the x tile.
+int form_d_warps(int64_t rows, int s, int sms) {
+  if ((rows + 31) / 32 * ((s + 7) / 8) < 8LL * sms) return std::min(4, s);
+  return (s + (s + 7) / 8 - 1) / ((s + 7) / 8);
+}
 
 template <int MODE>
 int32_t form_d_launch(const double* Xa, const double* HaT, const double* w, const double* A,
                       const double* B, int64_t row0, int64_t N, int d, int c, int s, int64_t D,
-                      double* walpha, double* part, cudaStream_t st) {
-  const int nw = form_d_warps(s);
-  const size_t smem = ((size_t)32 * (d | 1) + (size_t)(MODE == 1 ? 2 : 1) * nw * 4 * d) * 8;
+                      double* walpha, double* part, int nw, cudaStream_t st) {
+  const size_t smem = ((size_t)32 * (d | 1) + (size_t)(MODE == 1 ? 2 : 1) * nw * FORM_D_STAGE) * 8;
   FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_form_d<MODE>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   count_launch();
@@ -1251,7 +1263,8 @@ int32_t apply_t(firal_problem* P, const T* w, const T* Sblk, const T* V, int s, 
     ProfScope ps(st, PF_ALPHA);
     if constexpr (sizeof(T) == 8) {
       FIRAL_TRY(form_d_launch<0>(P->Xa.as<double>(), P->HaT.as<double>(), w, V, nullptr, 0, N, d,
-                                 c, s, D, P->walpha.as<double>(), nullptr, st));
+                                 c, s, D, P->walpha.as<double>(), nullptr, form_d_warps(N, s, P->sms),
+                                 st));
     } else {
       FormArgs a{};
       a.Xa = P->Xa.as<float>();
@@ -1294,12 +1307,13 @@ int32_t apply_t(firal_problem* P, const T* w, const T* Sblk, const T* V, int s, 
     ProfScope ps(st, PF_DTERM);
     FIRAL_TRY(outer_run<0>(o, p, st));
   }
-  // one probe per block and the splits over up to 8 thread groups while that leaves the blocks
-  // few; 4 probes per block once the classes alone fill the chip
+  // one probe per block and the splits over thread groups (a power of two, at most 1024 threads)
+  // while that leaves the blocks few; 4 probes per block once the classes alone fill the chip
   const int dpad = (d + 31) / 32 * 32;
   const bool few = (int64_t)c * ((s + 3) / 4) < 4 * P->sms;
   const int JB = few ? 1 : 4;
-  const int SG = few ? std::max(1, std::min({8, 1024 / dpad, p.splits})) : 1;
+  int SG = 1;
+  while (few && 2 * SG * dpad <= 1024 && 2 * SG <= p.splits) SG *= 2;
   const size_t smem = ((size_t)JB * d + (size_t)SG * JB * dpad) * sizeof(T);
   ProfScope ps(st, PF_COMBINE);
   count_launch();
@@ -1340,11 +1354,12 @@ int32_t quad_forms_simt(firal_problem* P, const void* A, const void* B, int s, d
   int ny = 0;
   if (P->dbl) {
     FIRAL_TRY(class_major_h(P));
-    ny = (s + form_d_warps(s) - 1) / form_d_warps(s);
+    const int nw = form_d_warps(P->n, s, P->sms);
+    ny = (s + nw - 1) / nw;
     FIRAL_TRY(P->form_part.ensure((size_t)ny * P->n * sizeof(double)));
     FIRAL_TRY(form_d_launch<1>(P->Xa.as<double>(), P->HaT.as<double>(), nullptr,
                                (const double*)A, (const double*)B, P->m, P->N, d, c, s, P->D,
-                               nullptr, P->form_part.as<double>(), st));
+                               nullptr, P->form_part.as<double>(), nw, st));
   } else {
     FormArgs a{};
     a.Xa = P->Xa.as<float>();
