@@ -308,6 +308,27 @@ int32_t quad_forms_simt(firal_problem* P, const void* A, const void* B, int s, d
                         void* g);
 int32_t round_scores_f32(firal_problem* P, const float* M1, const float* M2, const uint8_t* mask,
                          double eta, double* pv, int64_t* pi, int np);
+// class pairs (k, l), k <= l, of Exact-FIRAL: partial sums of w (delta_kl h_k - h_k h_l) x x^T
+// (part: splits x npairs x upper feature triangle), and g_i = -sum (2 - delta_kl)
+// (delta_kl h_k - h_k h_l) x_i^T M_kl x_i over the pool (*done = false: left to the caller)
+int32_t pair_sums_f32(firal_problem* P, int64_t r0, int64_t rows, const float* w, double wsc,
+                      const int2* pairs, int npairs, DBuf& part, int* splits);
+int32_t pair_forms_f32(firal_problem* P, const int2* pairs, int npairs, const float* M, float* g,
+                       bool* done);
+#ifdef __CUDACC__
+// pair p of the upper triangle of d features, row by row: (0,0) (0,1) .. (0,d-1) (1,1) ..
+__host__ __device__ inline void feature_pair(int p, int d, int& e, int& f) {
+  // row e starts at e d - e (e - 1) / 2
+  const float b = 2.0f * d + 1.0f;
+  int r = (int)((b - sqrtf(b * b - 8.0f * p)) * 0.5f);
+  if (r < 0) r = 0;
+  if (r > d - 1) r = d - 1;
+  while (r > 0 && r * d - r * (r - 1) / 2 > p) --r;
+  while (r + 1 < d && (r + 1) * d - (r + 1) * r / 2 <= p) ++r;
+  e = r;
+  f = r + p - (r * d - r * (r - 1) / 2);
+}
+#endif
 // ---- k_linalg.cu
 int32_t chol_inv(bool dbl, const double* A, int c, int d, void* inv_t, double* inv_d,
                  double* L_out, int32_t* not_spd, cudaStream_t st);

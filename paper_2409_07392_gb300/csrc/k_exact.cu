@@ -31,7 +31,9 @@
 namespace firal {
 namespace {
 
-constexpr int NB = 64;    // panel width of the blocked Cholesky and triangular inverse
+// panel width of the blocked Cholesky and triangular inverse: the widest tile one block factors
+// in registers, not above the GEMM tile
+template <class T> constexpr int NB_OF = sizeof(T) == 4 ? 128 : 64;
 constexpr int GBK = 8;    // K depth of one GEMM stage
 
 // ------------------------------------------------------------------------------ vector loads
@@ -73,7 +75,7 @@ __device__ __forceinline__ void ld_vec<double, 8>(const double* p, double* out) 
 
 // ------------------------------------------------------------------------------ dense GEMM
 template <class T> struct GemmCfg;
-template <> struct GemmCfg<float> { static constexpr int BM = 128, PAD = 4; };
+template <> struct GemmCfg<float> { static constexpr int BM = 128; };   // (k_gemm_f)
 template <> struct GemmCfg<double> { static constexpr int BM = 64, PAD = 2; };
 
 // K-range flags for triangular operands (tile-level bounds; every skipped term is zero):
@@ -192,6 +194,120 @@ __global__ __launch_bounds__(256) void k_gemm(int M, int N, int K, T alpha, cons
   }
 }
 
+// The same product in f32: every element adds its k terms in the same order, so the results are
+// those of k_gemm<float>.  128 x 128 x 16 tiles, 8 x 8 outputs per thread, a warp 8 x 4 thread
+// groups; 16-byte loads where the operands allow (VEC), each quarter of a step reading one item
+// of the next tile before its multiply-adds and storing it after them, one barrier per step.
+// D = 2500: about 38 TFLOP/s on full products (400 tiles, 1.3 waves of two blocks per SM); scalar
+// loads of 8-deep stages with the whole next tile held in registers ran at 33.
+template <bool TA, bool TB, bool VEC>
+__global__ __launch_bounds__(256, 2) void k_gemm_f(int M, int N, int K, float alpha, const float* A,
+                                                   int64_t lda, const float* B, int64_t ldb,
+                                                   float beta, float* C, int64_t ldc, int lower,
+                                                   int kflags, int64_t sA, int64_t sB,
+                                                   int64_t sC) {
+  A += blockIdx.z * sA;
+  B += blockIdx.z * sB;
+  C += blockIdx.z * sC;
+  constexpr int BM = 128, BK = 16, LD = BM + 4;
+  __shared__ __align__(16) float As[2][BK][LD];
+  __shared__ __align__(16) float Bs[2][BK][LD];
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int tx = (wid & 1) * 8 + (lane & 7), ty = (wid >> 1) * 4 + (lane >> 3);
+  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BM;
+  if (lower && n0 >= m0 + BM) return;
+  int kb = 0, ke = K;
+  if (kflags & K_FROM_N0) kb = max(kb, n0);
+  if (kflags & K_FROM_M0) kb = max(kb, m0);
+  if (kflags & K_TO_M1) ke = min(ke, m0 + BM);
+  // item u of a tile: 4 consecutive k of one row (KM: k is the fast index) or 4 consecutive
+  // rows of one k
+  auto load = [&](float (&r)[4], const float* P, int64_t ld, bool kfast, int lim, int o0, int k0,
+                  int u) {
+    const int idx = tid + u * 256;
+    const int o = o0 + (kfast ? idx >> 2 : (idx & 31) * 4);
+    const int k = k0 + (kfast ? (idx & 3) * 4 : idx >> 5);
+    const float* p = P + (kfast ? (int64_t)o * ld + k : (int64_t)k * ld + o);
+    const bool in = kfast ? o < lim : k < ke;
+    const int left = kfast ? ke - k : lim - o;       // values of the 4 that exist
+    if (VEC && in && left >= 4) {
+      const float4 v = *reinterpret_cast<const float4*>(p);
+      r[0] = v.x;
+      r[1] = v.y;
+      r[2] = v.z;
+      r[3] = v.w;
+    } else {
+#pragma unroll
+      for (int z = 0; z < 4; ++z) r[z] = in && z < left ? p[z] : 0.0f;
+    }
+  };
+  auto store = [&](float (*S)[LD], const float (&r)[4], bool kfast, int u) {
+    const int idx = tid + u * 256;
+    if (kfast) {
+#pragma unroll
+      for (int z = 0; z < 4; ++z) S[(idx & 3) * 4 + z][idx >> 2] = r[z];
+    } else {
+      *reinterpret_cast<float4*>(&S[idx >> 5][(idx & 31) * 4]) =
+          make_float4(r[0], r[1], r[2], r[3]);
+    }
+  };
+  float acc[8][8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 8; ++j) acc[i][j] = 0.0f;
+  const int nk = ke > kb ? (ke - kb + BK - 1) / BK : 0;
+  if (nk > 0) {
+#pragma unroll
+    for (int qt = 0; qt < 4; ++qt) {
+      float r[4];
+      load(r, qt < 2 ? A : B, qt < 2 ? lda : ldb, qt < 2 ? !TA : TB, qt < 2 ? M : N,
+           qt < 2 ? m0 : n0, kb, qt & 1);
+      store(qt < 2 ? As[0] : Bs[0], r, qt < 2 ? !TA : TB, qt & 1);
+    }
+    __syncthreads();
+  }
+  for (int kt = 0; kt < nk; ++kt) {
+    const int buf = kt & 1;
+    const bool more = kt + 1 < nk;
+#pragma unroll
+    for (int qt = 0; qt < 4; ++qt) {
+      float r[4];
+      if (more)
+        load(r, qt < 2 ? A : B, qt < 2 ? lda : ldb, qt < 2 ? !TA : TB, qt < 2 ? M : N,
+             qt < 2 ? m0 : n0, kb + (kt + 1) * BK, qt & 1);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int kk = qt * 4 + q;
+        float a[8], b[8];
+        ld_vec<float, 4>(&As[buf][kk][ty * 4], a);
+        ld_vec<float, 4>(&As[buf][kk][64 + ty * 4], a + 4);
+        ld_vec<float, 4>(&Bs[buf][kk][tx * 4], b);
+        ld_vec<float, 4>(&Bs[buf][kk][64 + tx * 4], b + 4);
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+#pragma unroll
+          for (int j = 0; j < 8; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+      }
+      if (more) store(qt < 2 ? As[buf ^ 1] : Bs[buf ^ 1], r, qt < 2 ? !TA : TB, qt & 1);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    const int gm = m0 + (i / 4) * 64 + ty * 4 + (i % 4);
+    if (gm >= M) continue;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const int gn = n0 + (j / 4) * 64 + tx * 4 + (j % 4);
+      if (gn >= N) continue;
+      float v = alpha * acc[i][j];
+      if (beta != 0.0f) v = fmaf(beta, C[(int64_t)gm * ldc + gn], v);
+      C[(int64_t)gm * ldc + gn] = v;
+    }
+  }
+}
+
 template <class T>
 int32_t gemm(cudaStream_t st, bool ta, bool tb, int M, int N, int K, double alpha, const T* A,
              int64_t lda, const T* B, int64_t ldb, double beta, T* C, int64_t ldc,
@@ -205,7 +321,22 @@ int32_t gemm(cudaStream_t st, bool ta, bool tb, int M, int N, int K, double alph
   const T a = (T)alpha, b = (T)beta;
   const int lw = lower ? 1 : 0;
 #define FIRAL_GEMM_ARGS M, N, K, a, A, lda, B, ldb, b, C, ldc, lw, kflags, sA, sB, sC
-  if (!ta && !tb) k_gemm<T, false, false><<<grid, 256, 0, st>>>(FIRAL_GEMM_ARGS);
+  if constexpr (sizeof(T) == 4) {
+    const auto al = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+    const bool vec = al(A) && al(B) && lda % 4 == 0 && ldb % 4 == 0 && sA % 4 == 0 && sB % 4 == 0;
+#define FIRAL_GEMM_F(TA_, TB_)                                                             \
+  if (ta == TA_ && tb == TB_) {                                                            \
+    if (vec) k_gemm_f<TA_, TB_, true><<<grid, 256, 0, st>>>(FIRAL_GEMM_ARGS);              \
+    else k_gemm_f<TA_, TB_, false><<<grid, 256, 0, st>>>(FIRAL_GEMM_ARGS);                 \
+  }
+    FIRAL_GEMM_F(false, false)
+    FIRAL_GEMM_F(false, true)
+    FIRAL_GEMM_F(true, false)
+    FIRAL_GEMM_F(true, true)
+#undef FIRAL_GEMM_F
+    FIRAL_CUDA_TRY(cudaGetLastError());
+    return FIRAL_OK;
+  } else if (!ta && !tb) k_gemm<T, false, false><<<grid, 256, 0, st>>>(FIRAL_GEMM_ARGS);
   else if (!ta && tb) k_gemm<T, false, true><<<grid, 256, 0, st>>>(FIRAL_GEMM_ARGS);
   else if (ta && !tb) k_gemm<T, true, false><<<grid, 256, 0, st>>>(FIRAL_GEMM_ARGS);
   else k_gemm<T, true, true><<<grid, 256, 0, st>>>(FIRAL_GEMM_ARGS);
@@ -215,73 +346,116 @@ int32_t gemm(cudaStream_t st, bool ta, bool tb, int M, int N, int K, double alph
 }
 
 // ------------------------------------------------------------------ Cholesky / inverse tiles
-// Cholesky of the diagonal tile A[j0 .. j0+jb)^2 (lower) in shared memory, in the vec type
-// (like the GEMM updates around it), written back in place (zeros above its diagonal), and the
-// tile's inverse written to Winv at the same place (lower, zeros above).  One CTA runs the jb
-// sequential steps, so the kernel is latency-bound (about 60 us for a 64 x 64 tile on GB300).
-// A pivot that is not positive and finite sets *flag and leaves both tiles unwritten.
-template <class T>
+// Cholesky of the diagonal tile A[j0 .. j0+jb)^2 (lower), written back in place (zeros above its
+// diagonal), and the tile's inverse written to Winv at the same place (lower, zeros above).  One
+// block of 16 x 16 threads with the tile in registers, factor and inverse in one elimination:
+// after step j the columns up to j hold Y = L^{-1} (its partial sums below row j), the columns
+// past j the trailing matrix, and a step is one update a_ik -= l_i v_k with v_k = Y_jk, 1 / L_jj
+// or l_k left, at and right of column j, published through shared memory.  Latency-bound (two
+// barriers, a square root and a reciprocal per step, the next pivot's overlapped with the
+// update): 68 us for a 128 x 128 f32 tile; in shared memory, with the inverse as a second
+// pass of row-by-row substitutions, a 64 x 64 tile took 59.
+// A pivot that is not positive and finite sets *flag; the tiles are then not to be used.
+template <class T, int R>
 __global__ __launch_bounds__(256) void k_potrf_diag(T* A, T* Winv, int64_t ld, int j0, int jb,
                                                     int* flag) {
-  extern __shared__ __align__(16) unsigned char potrf_raw[];   // L | Li (NB x NB+1 each) | red
-  T(*L)[NB + 1] = reinterpret_cast<T(*)[NB + 1]>(potrf_raw);
-  T(*Li)[NB + 1] = L + NB;
-  T(*red)[NB] = reinterpret_cast<T(*)[NB]>(&Li[NB][0]);
+  __shared__ T vec[16 * R];
+  __shared__ T piv[2];               // L_jj and its reciprocal
   __shared__ int bad;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, ti = tid >> 4, tk = tid & 15;
+  T* At = A + (int64_t)j0 * ld + j0;
+  T* Wt = Winv + (int64_t)j0 * ld + j0;
+  T a[R * (R + 1) / 2];              // element (ti + 16 x, tk + 16 y), x >= y
+#pragma unroll
+  for (int x = 0; x < R; ++x)
+#pragma unroll
+    for (int y = 0; y <= x; ++y) {
+      const int i = ti + 16 * x, k = tk + 16 * y;
+      a[x * (x + 1) / 2 + y] = i < jb && k <= i ? At[(int64_t)i * ld + k] : T(0);
+    }
   if (tid == 0) bad = 0;
-  for (int idx = tid; idx < jb * jb; idx += blockDim.x) {
-    const int i = idx / jb, j = idx - i * jb;
-    L[i][j] = j <= i ? A[(int64_t)(j0 + i) * ld + j0 + j] : T(0);
-  }
   __syncthreads();
-  // column k: every thread takes the pivot from L[k][k] (final after step k-1), scales the
-  // column below it, and after one barrier updates its share of the trailing triangle; the
-  // pivot itself is stored after that barrier, when no thread reads L[k][k] any more.
-  const int tx = tid & 15, ty = tid >> 4;
-  for (int k = 0; k < jb; ++k) {
-    const T p = L[k][k];
-    if (!(p > T(0)) || !(p < T(INFINITY))) {
-      if (tid == 0) bad = 1;
-      break;
+  for (int i = ti; i < jb; i += 16)
+    for (int k = tk; k < jb; k += 16)
+      if (k > i) At[(int64_t)i * ld + k] = Wt[(int64_t)i * ld + k] = T(0);
+  auto pivot = [&](T v) {
+    if (!(v > T(0)) || !(v < T(INFINITY))) bad = 1;
+    const T r = rsqrt(v);
+    piv[0] = v * r;
+    piv[1] = r;
+  };
+  if (tid == 0) pivot(a[0]);
+#pragma unroll
+  for (int bj = 0; bj < R; ++bj) {
+    const int jn = min(16, jb - 16 * bj);
+    for (int tj = 0; tj < jn; ++tj) {
+      const int j = 16 * bj + tj;
+      __syncthreads();               // pivot j is there; the last step's reads of vec are done
+      if (bad) {
+        if (tid == 0) atomicExch(flag, 1);
+        return;
+      }
+      const T r = piv[1];
+      if (tk == tj) {                // column j
+#pragma unroll
+        for (int x = bj; x < R; ++x) {
+          const int i = ti + 16 * x;
+          T& v = a[x * (x + 1) / 2 + bj];
+          if (i > j) {
+            const T l = v * r;
+            vec[i] = l;
+            if (i < jb) At[(int64_t)i * ld + j] = l;
+            v = T(0);
+          } else if (i == j) {
+            vec[j] = r;
+            At[(int64_t)j * ld + j] = piv[0];
+            v = r;
+          }
+        }
+      }
+      if (ti == tj) {                // row j of Y
+#pragma unroll
+        for (int y = 0; y <= bj; ++y) {
+          const int k = tk + 16 * y;
+          T& v = a[bj * (bj + 1) / 2 + y];
+          if (k < j) {
+            v *= r;
+            vec[k] = v;
+          }
+        }
+      }
+      __syncthreads();
+      if (tj < 15) {
+        if (j + 1 < jb && ti == tj + 1 && tk == tj + 1) {
+          const T l = vec[j + 1];
+          pivot(fma(-l, l, a[bj * (bj + 1) / 2 + bj]));
+        }
+      } else if (bj + 1 < R && j + 1 < jb && tid == 0) {
+        const T l = vec[j + 1];
+        pivot(fma(-l, l, a[bj + 1 < R ? (bj + 1) * (bj + 2) / 2 + bj + 1 : 0]));
+      }
+      T vk[R];
+#pragma unroll
+      for (int y = 0; y < R; ++y) vk[y] = vec[tk + 16 * y];
+#pragma unroll
+      for (int x = bj; x < R; ++x) {
+        const int i = ti + 16 * x;
+        if (i > j && i < jb) {
+          const T li = -vec[i];
+#pragma unroll
+          for (int y = 0; y <= x; ++y)
+            a[x * (x + 1) / 2 + y] = fma(li, vk[y], a[x * (x + 1) / 2 + y]);
+        }
+      }
     }
-    const T piv = sqrt(p);
-    if (tid > k && tid < jb) L[tid][k] /= piv;
-    __syncthreads();
-    if (tid == 0) L[k][k] = piv;
-    for (int i = k + 1 + ty; i < jb; i += 16) {
-      const T lik = L[i][k];
-      for (int j = k + 1 + tx; j <= i; j += 16) L[i][j] = fma(-lik, L[j][k], L[i][j]);
+  }
+#pragma unroll
+  for (int x = 0; x < R; ++x)
+#pragma unroll
+    for (int y = 0; y <= x; ++y) {
+      const int i = ti + 16 * x, k = tk + 16 * y;
+      if (i < jb && k <= i) Wt[(int64_t)i * ld + k] = a[x * (x + 1) / 2 + y];
     }
-    __syncthreads();
-  }
-  __syncthreads();
-  if (bad) {
-    if (tid == 0) atomicExch(flag, 1);
-    return;
-  }
-  // inverse of the lower-triangular tile: forward substitution on the identity, row by row,
-  // all NB right-hand sides at once; row i = (e_i - L[i][0:i] Li[0:i][:]) / L[i][i], each dot
-  // product split over four threads (entries above the diagonal come out as exact zeros)
-  const int col = tid & (NB - 1), part = tid >> 6;
-  for (int i = 0; i < jb; ++i) {
-    T acc = T(0);
-    for (int k = part; k < i; k += 4) acc = fma(L[i][k], Li[k][col], acc);
-    red[part][col] = acc;
-    __syncthreads();
-    if (part == 0 && col < jb) {
-      const T v = (col == i ? T(1) : T(0)) -
-                  ((red[0][col] + red[1][col]) + (red[2][col] + red[3][col]));
-      Li[i][col] = v / L[i][i];
-    }
-    __syncthreads();
-  }
-  for (int idx = tid; idx < jb * jb; idx += blockDim.x) {
-    const int i = idx / jb, j = idx - i * jb;
-    const int64_t o = (int64_t)(j0 + i) * ld + j0 + j;
-    A[o] = L[i][j];
-    Winv[o] = Li[i][j];
-  }
 }
 
 // Blocked right-looking Cholesky A = L L^T in place (lower triangle; the strict upper triangle
@@ -289,9 +463,7 @@ __global__ __launch_bounds__(256) void k_potrf_diag(T* A, T* Winv, int64_t ld, i
 // scratch of D * D / 4 elements.  A non-SPD matrix sets *flag.
 template <class T>
 int32_t potrf_trtri(cudaStream_t st, T* A, T* W, T* Tmp, int64_t D, int* flag) {
-  const size_t psm = (2 * NB * (NB + 1) + 4 * NB) * sizeof(T);
-  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_potrf_diag<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)psm));
+  constexpr int NB = NB_OF<T>;
   {
     ProfScope ps(st, PF_EXACT_FACTOR);
     FIRAL_CUDA_TRY(cudaMemsetAsync(W, 0, (size_t)D * D * sizeof(T), st));
@@ -301,7 +473,7 @@ int32_t potrf_trtri(cudaStream_t st, T* A, T* W, T* Tmp, int64_t D, int* flag) {
     {
       ProfScope ps(st, PF_EXACT_FACTOR);
       count_launch();
-      k_potrf_diag<T><<<1, 256, psm, st>>>(A, W, D, (int)j0, jb, flag);
+      k_potrf_diag<T, NB / 16><<<1, 256, 0, st>>>(A, W, D, (int)j0, jb, flag);
       FIRAL_CUDA_TRY(cudaGetLastError());
     }
     const int rest = (int)(D - j0 - jb);
@@ -482,6 +654,33 @@ __global__ void k_pair_reduce(const T* __restrict__ part, int nsplit, int npairs
     if (kl.x == kl.y && e == f) v += diag;
     out[pos] = (T)v;
     if (kl.x != kl.y) out[((int64_t)kl.y * d + f) * D + (int64_t)kl.x * d + e] = (T)v;
+  }
+}
+
+// The same from pair_sums_f32's partials: per class pair the upper triangle of features, row by
+// row, which is the whole block (it is symmetric).
+__global__ void k_pair_reduce_tri(const float* __restrict__ part, int nsplit, int npairs, int fp,
+                                  int d, const int2* __restrict__ pairs, const float* base,
+                                  double s2, const float* base2, double diag, float* out,
+                                  int64_t D) {
+  const int64_t tot = (int64_t)npairs * fp;
+  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < tot;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int p = (int)(idx / fp);
+    int e, f;
+    feature_pair((int)(idx - (int64_t)p * fp), d, e, f);
+    const int2 kl = pairs[p];
+    double acc = 0.0;
+    for (int s = 0; s < nsplit; ++s) acc += (double)part[(int64_t)s * tot + idx];
+    for (int side = 0; side < (e == f ? 1 : 2); ++side) {
+      const int64_t r = (int64_t)kl.x * d + (side ? f : e), q = (int64_t)kl.y * d + (side ? e : f);
+      double v = acc;
+      if (base) v += (double)base[r * D + q];
+      if (base2) v += s2 * (double)base2[r * D + q];
+      if (kl.x == kl.y && e == f) v += diag;
+      out[r * D + q] = (float)v;
+      if (kl.x != kl.y) out[q * D + r] = (float)v;
+    }
   }
 }
 
@@ -797,6 +996,21 @@ int32_t pair_build(firal_problem* P, int64_t r0, int64_t rows, const T* w, doubl
   cudaStream_t st = P->H->stream;
   const int d = P->d, c = P->c, dpb = dpb_of(d), DP = 16 * dpb;
   const int np = ex.npairs;
+  if constexpr (sizeof(T) == 4)
+    if (rows > 0) {
+      // x x^T is symmetric: one product over class pairs x feature pairs
+      const int fp = d * (d + 1) / 2;
+      int splits = 0;
+      FIRAL_TRY(pair_sums_f32(P, r0, rows, w, wsc, ex.pairs.as<int2>(), np, ex.part, &splits));
+      ProfScope ps(st, PF_EXACT_BUILD);
+      count_launch();
+      const int64_t tot = (int64_t)np * fp;
+      k_pair_reduce_tri<<<(unsigned)std::min<int64_t>((tot + 255) / 256, 8192), 256, 0, st>>>(
+          ex.part.as<float>(), splits, np, fp, d, ex.pairs.as<int2>(), base, s2, base2, diag, out,
+          P->D);
+      FIRAL_CUDA_TRY(cudaGetLastError());
+      return FIRAL_OK;
+    }
   int ns = (int)std::max<int64_t>(1, std::min<int64_t>((2LL * P->sms + np - 1) / np, rows / 256));
   ns = std::max(1, std::min(ns, 64));
   FIRAL_TRY(ex.part.ensure((size_t)ns * np * DP * DP * sizeof(T)));
@@ -941,7 +1155,13 @@ int32_t objective_t(firal_problem* P, const T* z, double* f_host, T* g) {
     // M = Sigma^{-1} H_p Sigma^{-1}, then g_i = -Tr(H_i M) (eq. 6)
     FIRAL_TRY(gemm<T>(st, false, false, (int)D, (int)D, (int)D, 1.0, S, D, mat<T>(ex, EX_HP), D,
                       0.0, T1, D));
-    FIRAL_TRY(gemm<T>(st, false, false, (int)D, (int)D, (int)D, 1.0, T1, D, S, D, 0.0, M, D));
+    FIRAL_TRY(gemm<T>(st, false, false, (int)D, (int)D, (int)D, 1.0, T1, D, S, D, 0.0, M, D,
+                      true));      // symmetric: the lower tiles, then mirrored
+    FIRAL_TRY(sym_from_lower<T>(st, M, D));
+    bool done = false;
+    if constexpr (sizeof(T) == 4)
+      FIRAL_TRY(pair_forms_f32(P, ex.pairs.as<int2>(), ex.npairs, M, g, &done));
+    if (!done) {
     int ng = 1;
     const int PTS = 16 * (dpb_of(P->d) == 8 ? 4 : 8);
     const int64_t tiles = (P->n + PTS - 1) / PTS;
@@ -954,6 +1174,7 @@ int32_t objective_t(firal_problem* P, const T* z, double* f_host, T* g) {
     const int blocks = (int)std::min<int64_t>((P->n + 255) / 256, 4096);
     k_sum_groups<T><<<blocks, 256, 0, st>>>(ex.gpart.as<double>(), ng, P->n, g);
     FIRAL_CUDA_TRY(cudaGetLastError());
+    }
   }
   double hv[1];
   FIRAL_CUDA_TRY(cudaMemcpyAsync(hv, f_dev, sizeof(double), cudaMemcpyDeviceToHost, st));

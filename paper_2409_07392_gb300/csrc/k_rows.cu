@@ -46,22 +46,11 @@ __device__ __forceinline__ void cp_async(void* dst, const void* src, bool ok) {
 __device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void cp_wait0() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
 
-// pair p of the upper triangle, row by row: (0,0) (0,1) .. (0,d-1) (1,1) ..
-__host__ __device__ inline void pair_of(int p, int d, int& e, int& f) {
-  // row e starts at e d - e (e - 1) / 2
-  const float b = 2.0f * d + 1.0f;
-  int r = (int)((b - sqrtf(b * b - 8.0f * p)) * 0.5f);
-  if (r < 0) r = 0;
-  if (r > d - 1) r = d - 1;
-  while (r > 0 && r * d - r * (r - 1) / 2 > p) --r;
-  while (r + 1 < d && (r + 1) * d - (r + 1) * r / 2 <= p) ++r;
-  e = r;
-  f = r + p - (r * d - r * (r - 1) / 2);
-}
-
 // ------------------------------------------------------------------------------------------
 // k_row_outer: part[split][m][n] = sum over the split's rows of A[i][m] B[i][n]
 //   OP 0 (low-rank part): m = j c + k, A = h_ik walpha_ij; n = e, B = x_ie
+//   OP 2 (Exact-FIRAL):   m = class pair (k, l), A = wsc w_i (delta_kl h_ik - h_ik h_il); n and B
+//                         as OP 1 (f32 only)
 //   OP 1 (block sums):    m = which c + k, A = w_i h_ik (which 0) or w_i h_ik (1 - h_ik)
 //                         (which 1); n = pair (e, f), e <= f, B = x_ie x_if
 // The tile is GM TM x GN TN outputs, GM GN threads active; rows in steps of BK, the next
@@ -78,6 +67,8 @@ struct OuterArgs {
   int64_t rps;       // rows per split
   int d, c, s;
   int which0;        // OP 1: first output kind (0: w h, 1: w h (1 - h))
+  const int2* pairs; // OP 2: class pairs; w may be null (weights 1), all scaled by wsc
+  float wsc;
   int M, Nn;         // outputs in all
   int GM, GN;
   T* part;
@@ -113,7 +104,7 @@ __global__ __launch_bounds__(512, 1) void k_row_outer_d(const OuterArgs<double> 
   if (OP == 1)
     for (int q = tid; q < BN; q += nt) {
       int e = 0, f = 0;
-      if (bn0 + q < a.Nn) pair_of(bn0 + q, d, e, f);
+      if (bn0 + q < a.Nn) feature_pair(bn0 + q, d, e, f);
       nmap[q] = bn0 + q < a.Nn ? e | (f << 16) : -1;
     }
   __syncthreads();
@@ -253,12 +244,15 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
   const bool act = mg < a.GM && ng < a.GN;
   for (int q = tid; q < BM; q += nt) {
     const int m = bm0 + q;
-    mcol[q] = m < a.M ? (m % c) | ((OP == 0 ? m / c - j0 : m / c + a.which0) << 16) : -1;
+    if (OP == 2)
+      mcol[q] = m < a.M ? a.pairs[m].x | a.pairs[m].y << 16 : -1;
+    else
+      mcol[q] = m < a.M ? (m % c) | ((OP == 0 ? m / c - j0 : m / c + a.which0) << 16) : -1;
   }
-  if (OP == 1)
+  if (OP != 0)
     for (int q = tid; q < BN; q += nt) {
       int e = 0, f = 0;
-      if (bn0 + q < a.Nn) pair_of(bn0 + q, d, e, f);
+      if (bn0 + q < a.Nn) feature_pair(bn0 + q, d, e, f);
       nmap[q] = bn0 + q < a.Nn ? e | (f << 16) : -1;
     }
   __syncthreads();
@@ -309,8 +303,14 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
           hr[v][VH > 1 ? 1 : 0] = r.y;
         } else {
           hr[v][0] = *h;
+          if (OP == 2) {
+            const int l = hu >> 12 & 0xfff;
+            const float hk = *h;
+            hr[v][0] = (l == (hu & 0xfff) ? hk : 0.0f) - hk * H[pr * c + l];
+          }
         }
-        wr[v] = OP == 0 ? W[pr * a.s + (hu >> 12 & 0xfff)] : W[pr];
+        wr[v] = OP == 0 ? W[pr * a.s + (hu >> 12 & 0xfff)]
+                        : OP == 1 ? W[pr] : a.wsc * (a.w ? W[pr] : 1.0f);
       }
     }
   };
@@ -391,12 +391,12 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
       load_x(0, qt);
       store_a(0, qt);
       store_x(0, qt);
-      if (OP == 1 && steps > 1) {
+      if (OP != 0 && steps > 1) {
         load_x(1, qt);
         store_x(1, qt);
       }
     }
-    if (OP == 1) {
+    if (OP != 0) {
       __syncthreads();
       for (int q = lane; q < BN; q += 32) pair_rows(0, q, wid);
     }
@@ -413,7 +413,7 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
       if (morex) load_x(OP == 0 ? t + 1 : t + 2, qt);
       float pe[2] = {0.0f, 0.0f}, pf[2] = {0.0f, 0.0f};
       const int pq = lane + qt * 32;
-      const bool pair = OP == 1 && more && pq < BN;
+      const bool pair = OP != 0 && more && pq < BN;
       if (pair) {
         const int ef = nmap[pq];
         const float* X = Xs + ((t + 1) & 1) * BK * dS + wid * dS;
@@ -490,6 +490,7 @@ int row_vec(const void* q, int cols) {
 }
 // k_row_outer_f's VH: 4 needs both operands' rows aligned
 int outer_vh(const OuterArgs<float>& a) {
+  if (a.pairs) return 1;   // two values of h per element
   const int h = row_vec(a.Ha, a.c);
   return h == 4 && row_vec(a.Xa, a.d) == 4 ? 4 : h >= 2 ? 2 : 1;
 }
@@ -563,7 +564,7 @@ template <int OP, int TM, int VH>
 int32_t outer_launch_f(const OuterArgs<float>& a, const OuterPlan& p, cudaStream_t st) {
   const int BK = OuterCfg<OP, VH>::BK, BM = p.GM * TM, BN = p.GN * 8, dS = (a.d + 3) & ~3;
   const size_t smem =
-      ((size_t)2 * BK * (BM + BN + (OP == 1 ? dS : 0)) + BM + (OP == 1 ? BN : 0)) * 4;
+      ((size_t)2 * BK * (BM + BN + (OP != 0 ? dS : 0)) + BM + (OP != 0 ? BN : 0)) * 4;
   FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_outer_f<OP, TM, VH>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
   count_launch();
@@ -592,6 +593,7 @@ int32_t outer_run(OuterArgs<float> a, const OuterPlan& p, cudaStream_t st) {
   a.GN = p.GN;
   a.rps = p.rps;
   const int vh = outer_vh(a);
+  if constexpr (OP == 2) return outer_launch_f<2, 8, 1>(a, p, st);
   if constexpr (OP == 1) if (p.TM == 4) {
     if (vh == 4) return outer_launch_f<OP, 4, 4>(a, p, st);
     if (vh == 2) return outer_launch_f<OP, 4, 2>(a, p, st);
@@ -625,7 +627,7 @@ __global__ __launch_bounds__(256) void k_pair_expand(const T* __restrict__ part,
   for (int g = 1; g < 8; ++g) acc += red[g][threadIdx.x];
   const int k = (int)(idx / np);
   int e, f;
-  pair_of((int)(idx - (int64_t)k * np), d, e, f);
+  feature_pair((int)(idx - (int64_t)k * np), d, e, f);
   if (e == f) acc += lam;
   const int64_t o1 = ((int64_t)k * d + e) * d + f, o2 = ((int64_t)k * d + f) * d + e;
   if (out_d) out_d[o1] = out_d[o2] = acc;
@@ -694,6 +696,8 @@ __global__ void k_row_combine(const T* __restrict__ S, const T* __restrict__ V,
 //   MODE 0  alpha:  columns (probe, class), walpha[i][j] = w_i sum_k h_ik (x_i.V_j[k])
 //   MODE 1  quad:   64 columns of A_j and the same 64 of B_j;
 //           sum_k h a b - (sum_k h a)(sum_k h b) per probe, summed over the block's probes
+//   MODE 3  class pairs (Exact-FIRAL): unit (k, l), columns M_kl[e]; sum_e x_e (x.M_kl[e]) times
+//           -(2 - delta_kl)(delta_kl h_k - h_k h_l), summed over the block's pairs
 //   MODE 2  scores: 64 columns of M1_k and the same 64 of M2_k; q = sum_e x_e (x.M_k[e]),
 //           sum over the block's classes of w q1 / (1 + eta w q2), w = h_ik (1 - h_ik)
 // The columns of one unit u (probe; class in MODE 2) are its inner index v (class; feature in
@@ -725,6 +729,8 @@ struct FormArgs {
   int kc, PJ, CC, UB;    // padded inner chunk, units per tile, chunks, units per block
   int vec;               // float4 reads of the row coefficients are aligned
   double eta;
+  const int2* pairs;     // MODE 3
+  int64_t ldm;           // MODE 3: row length of M
   float* walpha;         // MODE 0: N x units
   double* part;          // MODE 1, 2: [blockIdx.y][row - row0]
 };
@@ -743,12 +749,18 @@ __global__ __launch_bounds__(256) void k_form_pack(const FormArgs a, int64_t tot
     const int64_t q0 = idx >> 7;
     const int T = (int)(q0 / eb), e0 = (int)(q0 - (int64_t)T * eb) * 8;
     const int p = T % tpb, yc = T / tpb, cc = yc % a.CC, y = yc / a.CC;
-    const int q = MODE == 0 ? col : col & 63;
+    const int q = MODE == 0 || MODE == 3 ? col : col & 63;
     const int ul = q / a.kc, v = cc * a.kc + q - ul * a.kc;
     const int u = y * a.UB + p * a.PJ + ul;
     const bool ok = ul < a.PJ && u < a.units && v < a.inner;
-    const float* src =
-        (MODE != 0 && col >= 64 ? a.B : a.A) + (ok ? u * a.ustride + (int64_t)v * a.d : 0);
+    const float* src = a.A;
+    if (MODE == 3) {
+      const int2 kl = a.pairs[ok ? u : 0];
+      src += ok ? (int64_t)(kl.x * a.d + v) * a.ldm + (int64_t)kl.y * a.d : 0;
+    } else {
+      if (MODE != 0 && col >= 64) src = a.B;
+      src += ok ? u * a.ustride + (int64_t)v * a.d : 0;
+    }
     float* dst = a.pk + ((int64_t)T * dK + e0) * 128 + col;
 #pragma unroll
     for (int e = 0; e < 8; ++e) dst[e * 128] = ok && e0 + e < a.d ? src[e0 + e] : 0.0f;
@@ -758,8 +770,9 @@ __global__ __launch_bounds__(256) void k_form_pack(const FormArgs a, int64_t tot
 // KC features per step: 16, or 8 where that lets two blocks share an SM
 template <int MODE, int KC>
 __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
-  constexpr int NV = MODE == 0 ? 1 : MODE == 1 ? 3 : 2;   // values per (row, unit)
-  constexpr int GC = MODE == 0 ? 32 : 16;                 // column groups per tile
+  constexpr bool ONE = MODE == 0 || MODE == 3;            // one coefficient block
+  constexpr int NV = ONE ? 1 : MODE == 1 ? 3 : 2;         // values per (row, unit)
+  constexpr int GC = ONE ? 32 : 16;                       // column groups per tile
   constexpr int LD = FORM_LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int d = a.d, dK = form_dk(d);
@@ -813,8 +826,9 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
       else if (t + 1 < ntile) stage(cn, pn, 0, b ^ 1);
       const float* X = xs + kk * KC * LD + ty * 4;
       const float* Vt = vs + b * KC * 128 + tx * 4;
-#pragma unroll 4
-      for (int q = 0; q < KC; ++q) {
+      // the last step stops at the last feature (the padding is zero)
+      const int qn = min(KC, d - kk * KC);
+      auto multiply = [&](int q) {
         float av[8], bv[8];
 #pragma unroll
         for (int v = 0; v < 2; ++v) {
@@ -827,11 +841,17 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
         for (int x = 0; x < 8; ++x)
 #pragma unroll
           for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(av[x], bv[y], acc[x][y]);
+      };
+      if (qn == KC) {
+#pragma unroll 4
+        for (int q = 0; q < KC; ++q) multiply(q);
+      } else {
+        for (int q = 0; q < qn; ++q) multiply(q);
       }
     }
     // per row: this thread's 4 (MODE 0: 2 x 4) inner indices
 #pragma unroll
-    for (int g = 0; g < (MODE == 0 ? 2 : 1); ++g) {
+    for (int g = 0; g < (ONE ? 2 : 1); ++g) {
       const int grp = g * 16 + tx;
       const int ul = grp / gpu, v = cc * a.kc + (grp - ul * gpu) * 4;
       const bool uv = ul < a.PJ && u0 + p * a.PJ + ul < u1;
@@ -840,7 +860,7 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
         const int r = (x / 4) * 64 + ty * 4 + (x & 3);
         const int64_t i = i0 + r;
         float cf[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        if (MODE == 2) {
+        if (MODE >= 2) {
 #pragma unroll
           for (int q = 0; q < 4; ++q)
             if (uv && v + q < a.inner) cf[q] = xs[(v + q) * LD + r];
@@ -864,7 +884,7 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
           const float va = acc[x][g * 4 + q], vb = acc[x][4 + q];
-          if (MODE == 0) {
+          if (ONE) {
             s0 = fmaf(cf[q], va, s0);
           } else if (MODE == 1) {
             const float ha = cf[q] * va;
@@ -906,8 +926,13 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
     const int64_t i = i0 + tid;
     double q = 0.0;
     for (int ul = 0; ul < u1 - u0; ++ul) {
-      const double v0 = sum[ul * 128 + tid], v1 = sum[(a.UB + ul) * 128 + tid];
-      if (MODE == 1) {
+      const double v0 = sum[ul * 128 + tid], v1 = ONE ? 0.0 : sum[(a.UB + ul) * 128 + tid];
+      if (MODE == 3) {
+        const int2 kl = a.pairs[u0 + ul];
+        const double hk = (double)a.Ha[i * a.c + kl.x], hl = (double)a.Ha[i * a.c + kl.y];
+        const double w = (kl.x == kl.y ? hk : 0.0) - hk * hl;
+        q -= (kl.x == kl.y ? 1.0 : 2.0) * w * v0;
+      } else if (MODE == 1) {
         q += v0 - v1 * (double)sum[(2 * a.UB + ul) * 128 + tid];
       } else {
         const double hv = (double)a.Ha[i * a.c + u0 + ul];
@@ -943,8 +968,8 @@ void form_plan(FormArgs& a, int tile, int64_t rows, int sms) {
 
 template <int MODE, int KC>
 int32_t form_launch_k(const FormArgs& a, int64_t rows, int ny, cudaStream_t st) {
-  constexpr int NV = MODE == 0 ? 1 : MODE == 1 ? 3 : 2;
-  constexpr int GC = MODE == 0 ? 32 : 16;
+  constexpr int NV = MODE == 0 || MODE == 3 ? 1 : MODE == 1 ? 3 : 2;
+  constexpr int GC = MODE == 0 || MODE == 3 ? 32 : 16;
   const size_t smem = ((size_t)form_dk(a.d) * FORM_LD + 2 * KC * 128 +
                        (size_t)NV * 128 * (GC + 1) + (size_t)NV * a.UB * 128) *
                       4;
@@ -1204,39 +1229,45 @@ int32_t syrk_t(firal_problem* P, const T* w, int64_t rows, double lamS, T* outS,
   return FIRAL_OK;
 }
 
-// pw[i][k] = w_i h_ik (1 - h_ik)
+// pw[i][k] = w_i h_ik, then (both) w_i h_ik (1 - h_ik); only the second when !both
 __global__ void k_block_weights(const float* __restrict__ Ha, const float* __restrict__ w,
-                                int64_t rows, int c, float* __restrict__ pw) {
+                                int64_t rows, int c, bool both, float* __restrict__ pw) {
+  const int cc = both ? 2 * c : c;
   for (int64_t i = blockIdx.x; i < rows; i += gridDim.x) {
     const float wi = w[i];
     for (int k = threadIdx.x; k < c; k += blockDim.x) {
-      const float h = Ha[i * c + k];
-      pw[i * c + k] = wi * h * (1.0f - h);
+      const float h = Ha[i * c + k], wh = wi * h;
+      if (both) pw[i * cc + k] = wh;
+      pw[i * cc + cc - c + k] = wh * (1.0f - h);
     }
   }
 }
 
-// B_k alone in f32 (Round's Sigma blocks and B(H_o), firal_precond_blocks).  nu and the scores
-// amplify the chains' rounding, so here every addition is kept: each term is (p x_e) x_f with
-// p = w h (1 - h), over the full square, as both (e, f) and (f, e) are used.  It is OP 0's
-// product with m = (class k, feature e): A = x_e p_k, B = x_f.
-int32_t blocks_only_f32(firal_problem* P, const float* w, int64_t rows, double lamP,
-                        double* outP) {
+// Block sums with every addition in a fixed order: each term is (p x_e) x_f with p = w h (1 - h)
+// (and w h for S), rows in order within their range, over the full square, as both (e, f) and
+// (f, e) are used.  For results that amplify the sums' rounding: Round's nu and scores (B_k
+// alone: its Sigma blocks and B(H_o), firal_precond_blocks), and the classifier refit, whose line
+// search compares losses at their f32 noise (S and B_k over few rows).  It is OP 0's product with
+// m = (kind and class k, feature e): A = x_e p_k, B = x_f.
+constexpr int64_t FEW_ROWS = 256;   // one range at any class count
+
+int32_t blocks_ordered_f32(firal_problem* P, const float* w, int64_t rows, double lamS,
+                           float* outS, double lamP, double* outP) {
   cudaStream_t st = P->H->stream;
-  const int d = P->d, c = P->c;
+  const int d = P->d, c = P->c, cc = (outS ? 1 : 0) * c + c;
   const int64_t per = (int64_t)c * d * d;
   OuterArgs<float> a{};
   a.Xa = a.Ha = P->Xa.as<float>();
   a.r0 = 0;
   a.r1 = rows;
   a.d = a.c = d;
-  a.s = c;
-  a.M = c * d;
+  a.s = cc;
+  a.M = cc * d;
   a.Nn = d;
   OuterPlan p = outer_plan<0>(a, P->sms);
   block_ranges(p, P->N, rows, d, c, P->sms);
-  FIRAL_TRY(P->syrk_part.ensure((size_t)per * p.splits * sizeof(float)));
-  FIRAL_TRY(P->blk_w.ensure((size_t)std::max<int64_t>(rows, 1) * c * sizeof(float)));
+  FIRAL_TRY(P->syrk_part.ensure((size_t)cc * d * d * p.splits * sizeof(float)));
+  FIRAL_TRY(P->blk_w.ensure((size_t)std::max<int64_t>(rows, 1) * cc * sizeof(float)));
   a.part = P->syrk_part.as<float>();
   a.w = P->blk_w.as<float>();
   {
@@ -1244,12 +1275,103 @@ int32_t blocks_only_f32(firal_problem* P, const float* w, int64_t rows, double l
     if (rows > 0) {
       count_launch();
       k_block_weights<<<(unsigned)std::min<int64_t>(rows, 65536), std::min(256, (c + 31) / 32 * 32),
-                        0, st>>>(P->Ha.as<float>(), w, rows, c, P->blk_w.as<float>());
+                        0, st>>>(P->Ha.as<float>(), w, rows, c, outS != nullptr,
+                                 P->blk_w.as<float>());
       FIRAL_CUDA_TRY(cudaGetLastError());
     }
     FIRAL_TRY(outer_run<0>(a, p, st));
   }
-  return syrk_reduce_f32(P, nullptr, a.part, p.splits, 0.0, nullptr, lamP, outP);
+  // S and B_k together: one range (few rows), S's blocks before B_k's
+  return syrk_reduce_f32(P, a.part, a.part + (outS ? per : 0), p.splits, lamS, outS, lamP, outP);
+}
+
+// The apply of one vector over few rows (the classifier refit's solves), f32, in two launches and
+// in a fixed order of additions: alpha row by row (x.V_j[k] by one thread per class, features in
+// order; the classes in order by one thread), then per class the rows in order and S_k V_j[k].
+__global__ __launch_bounds__(256) void k_few_alpha(const float* __restrict__ Xa,
+                                                   const float* __restrict__ Ha,
+                                                   const float* __restrict__ w,
+                                                   const float* __restrict__ V, int d, int c,
+                                                   float* __restrict__ walpha) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* xs = (float*)smem_raw;   // d
+  float* gs = xs + d;             // c
+  float* hs = gs + c;             // c
+  const int64_t i = blockIdx.x;
+  for (int e = threadIdx.x; e < d; e += blockDim.x) xs[e] = Xa[i * d + e];
+  for (int k = threadIdx.x; k < c; k += blockDim.x) hs[k] = Ha[i * c + k];
+  __syncthreads();
+  for (int k = threadIdx.x; k < c; k += blockDim.x) {
+    const float* v = V + (int64_t)k * d;
+    float g = 0.0f;
+#pragma unroll 8
+    for (int e = 0; e < d; ++e) g = fmaf(xs[e], v[e], g);
+    gs[k] = g;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float acc = 0.0f;
+#pragma unroll 8
+    for (int k = 0; k < c; ++k) acc = fmaf(hs[k], gs[k], acc);
+    walpha[i] = w[i] * acc;
+  }
+}
+
+__global__ __launch_bounds__(128) void k_few_apply(const float* __restrict__ Xa,
+                                                   const float* __restrict__ Ha,
+                                                   const float* __restrict__ walpha, int rows,
+                                                   const float* __restrict__ S,
+                                                   const float* __restrict__ V, int d, int c,
+                                                   float* __restrict__ out, double* pq) {
+  __shared__ float vs[128];
+  __shared__ double red[4];
+  const int k = blockIdx.x, e = threadIdx.x;
+  if (e < d) vs[e] = V[(int64_t)k * d + e];
+  __syncthreads();
+  float q = 0.0f;
+  if (e < d) {
+    float ds = 0.0f;
+#pragma unroll 8
+    for (int i = 0; i < rows; ++i)
+      ds = fmaf(walpha[i] * Xa[(int64_t)i * d + e], Ha[(int64_t)i * c + k], ds);
+    const float* Sk = S + (int64_t)k * d * d + e;   // S symmetric: column e as row e
+    float acc = 0.0f;
+#pragma unroll 8
+    for (int f = 0; f < d; ++f) acc = fmaf(Sk[(int64_t)f * d], vs[f], acc);
+    q = acc - ds;
+    out[(int64_t)k * d + e] = q;
+  }
+  if (!pq) return;
+  double v = e < d ? (double)vs[e] * (double)q : 0.0;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((e & 31) == 0) red[e >> 5] = v;
+  __syncthreads();
+  if (e == 0) {
+    for (int x = 1; x < (int)(blockDim.x >> 5); ++x) v += red[x];
+    pq[k] = v;
+  }
+}
+
+int32_t few_apply(firal_problem* P, const float* w, const float* S, const float* V, float* out,
+                  double* pq) {
+  cudaStream_t st = P->H->stream;
+  const int d = P->d, c = P->c;
+  FIRAL_TRY(P->walpha.ensure((size_t)P->N * sizeof(float)));
+  {
+    ProfScope ps(st, PF_ALPHA);
+    count_launch();
+    k_few_alpha<<<(unsigned)P->N, std::min(256, (c + 31) / 32 * 32), (d + 2 * c) * sizeof(float),
+                  st>>>(P->Xa.as<float>(), P->Ha.as<float>(), w, V, d, c, P->walpha.as<float>());
+    FIRAL_CUDA_TRY(cudaGetLastError());
+  }
+  ProfScope ps(st, PF_DTERM);
+  count_launch();
+  k_few_apply<<<c, (d + 31) / 32 * 32, 0, st>>>(P->Xa.as<float>(), P->Ha.as<float>(),
+                                               P->walpha.as<float>(), (int)P->N, S, V, d, c, out,
+                                               pq);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
 }
 
 template <class T>
@@ -1328,7 +1450,8 @@ int32_t apply_t(firal_problem* P, const T* w, const T* Sblk, const T* V, int s, 
 int32_t syrk_blocks(firal_problem* P, const void* w, double lamS, void* outS, double lamP,
                     double* outP, int64_t rows) {
   if (rows < 0) rows = P->N;
-  if (!P->dbl && !outS) return blocks_only_f32(P, (const float*)w, rows, lamP, outP);
+  if (!P->dbl && (!outS || (outP && rows == P->N && rows <= FEW_ROWS)))
+    return blocks_ordered_f32(P, (const float*)w, rows, lamS, (float*)outS, lamP, outP);
   if (P->dbl) return syrk_t<double>(P, (const double*)w, rows, lamS, (double*)outS, lamP, outP);
   return syrk_t<float>(P, (const float*)w, rows, lamS, (float*)outS, lamP, outP);
 }
@@ -1340,6 +1463,8 @@ int32_t hessian_apply_simt(firal_problem* P, const void* w, const void* Sblk, co
     return apply_t<double>(P, (const double*)w, (const double*)Sblk, (const double*)V, s,
                            (double*)out, pq);
   }
+  if (s == 1 && P->N <= FEW_ROWS)
+    return few_apply(P, (const float*)w, (const float*)Sblk, (const float*)V, (float*)out, pq);
   return apply_t<float>(P, (const float*)w, (const float*)Sblk, (const float*)V, s, (float*)out,
                         pq);
 }
@@ -1417,6 +1542,65 @@ int32_t round_scores_f32(firal_problem* P, const float* M1, const float* M2, con
   count_launch();
   k_score_argmax<<<np, 128, 0, st>>>(a.part, ny, P->n, mask, pv, pi);
   FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+// Exact-FIRAL in f32 (class pairs k <= l).  The partial sums are one product of npairs x d (d +
+// 1) / 2 outputs, x x^T being symmetric, and the gradient's forms run on k_row_form: at n = 5,000,
+// d = c = 50 1,010 and 1,060 us, where a CTA per class pair over full blocks, and per group of
+// pairs with M_kl staged pair by pair, took 1,830 and 2,760.
+int32_t pair_sums_f32(firal_problem* P, int64_t r0, int64_t rows, const float* w, double wsc,
+                      const int2* pairs, int npairs, DBuf& part, int* splits) {
+  OuterArgs<float> a{};
+  a.Xa = P->Xa.as<float>();
+  a.Ha = P->Ha.as<float>();
+  a.w = w ? w - r0 : nullptr;
+  a.r0 = r0;
+  a.r1 = r0 + rows;
+  a.d = P->d;
+  a.c = P->c;
+  a.s = 1;
+  a.pairs = pairs;
+  a.wsc = (float)wsc;
+  a.M = npairs;
+  a.Nn = P->d * (P->d + 1) / 2;
+  const OuterPlan p = outer_plan<2>(a, P->sms);
+  FIRAL_TRY(part.ensure((size_t)a.M * a.Nn * p.splits * sizeof(float)));
+  a.part = part.as<float>();
+  *splits = p.splits;
+  ProfScope ps(P->H->stream, PF_EXACT_BUILD);
+  return outer_run<2>(a, p, P->H->stream);
+}
+
+int32_t pair_forms_f32(firal_problem* P, const int2* pairs, int npairs, const float* M, float* g,
+                       bool* done) {
+  cudaStream_t st = P->H->stream;
+  FormArgs a{};
+  a.Xa = P->Xa.as<float>();
+  a.Ha = P->Ha.as<float>();
+  a.A = M;
+  a.row0 = P->m;
+  a.N = P->N;
+  a.d = P->d;
+  a.c = P->c;
+  a.units = npairs;
+  a.inner = P->d;
+  a.pairs = pairs;
+  a.ldm = P->D;
+  form_plan(a, 128, P->n, P->sms);
+  const int64_t ny = (npairs + a.UB - 1) / a.UB;
+  *done = false;
+  if (ny > 4096) return FIRAL_OK;   // very many classes of few features: partials too large
+  FIRAL_TRY(P->form_part.ensure((size_t)ny * P->n * sizeof(double)));
+  a.part = P->form_part.as<double>();
+  ProfScope ps(st, PF_EXACT_QUAD);
+  int y = 0;
+  FIRAL_TRY(form_launch<3>(P, a, P->n, &y, st));
+  count_launch();
+  k_form_sum<float><<<(unsigned)std::min<int64_t>((P->n + 255) / 256, 4096), 256, 0, st>>>(
+      P->form_part.as<double>(), y, P->n, 1.0, g);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  *done = true;
   return FIRAL_OK;
 }
 
