@@ -223,6 +223,7 @@ void DBuf::park() {
 
 // tensor-core entry points (k_tc.cu); return FIRAL_ERR_UNSUPPORTED when not built
 int32_t tc_prepare(firal_problem* P);
+int32_t tc_prepare_operands(firal_problem* P);
 int32_t tc_hessian_apply(firal_problem* P, const void* w, const void* Sblk, const void* V, int s,
                          void* out, double* pq, double lam_null);
 int32_t tc_quad_forms(firal_problem* P, const void* A, const void* B, int s, double scale,
@@ -508,8 +509,10 @@ int32_t validate_pool(const firal_pool* pool, const firal_hess0* h0) {
   return FIRAL_OK;
 }
 
+// stacked: the rows of several pools; their tables and the operands that depend on them follow in
+// pooled_create
 int32_t problem_create_impl(firal_handle* H, const firal_pool* pool, const firal_hess0* h0,
-                            int32_t precision, firal_problem** out) {
+                            int32_t precision, firal_problem** out, bool stacked = false) {
   if (!H || !out) return fail(FIRAL_ERR_ARG, "handle and out must be non-null");
   FIRAL_TRY(validate_pool(pool, h0));
   if (precision < FIRAL_FP64 || precision > FIRAL_MIXED_BF16_FAST)
@@ -570,11 +573,12 @@ int32_t problem_create_impl(firal_handle* H, const firal_pool* pool, const firal
   TRYC(P->red.ensure(2048 * sizeof(double)));
   TRYC(P->g.ensure((size_t)P->n * vs));
   if (is_mixed(precision)) TRYC(tc_prepare(P));
-  // at most 32 classes: the fused per-point apply (one pool; a pooled problem replaces these
-  // tables with its pools')
-  if (is_mixed(precision))
+  // at most 32 classes: the fused per-point apply
+  if (is_mixed(precision) && !stacked) {
     TRYC(tc_setup_pw(P, std::vector<int>{0, (int)P->c}, std::vector<int64_t>{0, P->m},
                      std::vector<int64_t>{0, P->n}));
+    TRYC(tc_prepare_operands(P));
+  }
 #undef TRYC
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cleanup(fail(FIRAL_ERR_CUDA, cudaGetErrorString(e)));
@@ -990,7 +994,7 @@ int32_t pooled_create(firal_handle* H, const std::vector<int>& idx, const firal_
   firal_pool sp{Xs.p, Hs.p, n, dg, (int32_t)C, p0.x_dtype, p0.h_dtype};
   firal_hess0 sh{Xos.p, Hos.p, M, h0s ? h0s[idx[0]].lambda : 0.0};
   firal_problem* P = nullptr;
-  TRYP(problem_create_impl(H, &sp, &sh, prec, &P));
+  TRYP(problem_create_impl(H, &sp, &sh, prec, &P, true));
   rel();
 #undef TRYP
 #undef CUDP
@@ -1083,7 +1087,9 @@ int32_t pooled_create(firal_handle* H, const std::vector<int>& idx, const firal_
       e = cudaMemcpyAsync(P->kr_bsum.p, kbs.data(), kbs.size() * sizeof(int4),
                           cudaMemcpyHostToDevice, st);
     // pools of at most 32 classes (and dp <= 64): the fused per-point apply
-    if (e == cudaSuccess && (rc = tc_setup_pw(P, coff, loff, poff)) != FIRAL_OK) return bail(rc);
+    if (e == cudaSuccess && ((rc = tc_setup_pw(P, coff, loff, poff)) != FIRAL_OK ||
+                             (rc = tc_prepare_operands(P)) != FIRAL_OK))
+      return bail(rc);
   }
   // the host vectors above are read by the copies: wait for them before they go out of scope
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -1732,7 +1732,7 @@ __global__ void __launch_bounds__(256, 1)
 // [i / 64][p][i % 64] (npp rows per block): every 128 x 64 TMA tile is one contiguous 16 KB
 // run.  Block = 64 points (staged point-major in shared memory) x every pair; a thread takes
 // pairs p, p + 256, ... (consecutive threads read consecutive e' of the staged rows) and
-// writes each pair's 64 points as four 32-byte pieces.
+// writes each pair's 64 points as four 32-byte pieces.  Zlo may be NULL: the lo part is left out.
 __global__ void __launch_bounds__(256) k_build_z(bf16* Zhi, bf16* Zlo, const bf16* Xb, int d,
                                                  int dp, int npairs, int64_t npp) {
   __shared__ __align__(16) bf16 xs[64 * 128];
@@ -1756,7 +1756,7 @@ __global__ void __launch_bounds__(256) k_build_z(bf16* Zhi, bf16* Zlo, const bf1
       e2 = e + (p - (e * d - e * (e - 1) / 2));
     }
     bf16* zh = Zhi + ((int64_t)blockIdx.x * npp + p) * 64;
-    bf16* zl = Zlo + ((int64_t)blockIdx.x * npp + p) * 64;
+    bf16* zl = Zlo ? Zlo + ((int64_t)blockIdx.x * npp + p) * 64 : nullptr;
 #pragma unroll 1
     for (int c16 = 0; c16 < 4; ++c16) {
       uint4 hv[2], lv[2];
@@ -1777,11 +1777,13 @@ __global__ void __launch_bounds__(256) k_build_z(bf16* Zhi, bf16* Zlo, const bf1
         }
       }
       uint4* oh = reinterpret_cast<uint4*>(zh + c16 * 16);
-      uint4* ol = reinterpret_cast<uint4*>(zl + c16 * 16);
       oh[0] = hv[0];
       oh[1] = hv[1];
-      ol[0] = lv[0];
-      ol[1] = lv[1];
+      if (Zlo) {
+        uint4* ol = reinterpret_cast<uint4*>(zl + c16 * 16);
+        ol[0] = lv[0];
+        ol[1] = lv[1];
+      }
     }
   }
 }
@@ -2285,6 +2287,21 @@ static int32_t tc_prepare_centred(firal_problem* P, int cpb2) {
   return FIRAL_OK;
 }
 
+// bf16 h, row-major (Np x cp)
+static int32_t make_hb(firal_problem* P) {
+  FIRAL_TRY(P->Hb.ensure((size_t)P->Np * P->cp * 2));
+  dim3 g, b;
+  bf16_pad_grid(P->Np, P->cp, g, b);
+  count_launch();
+  k_bf16_pad<0><<<g, b, 0, P->H->stream>>>(P->Hb.as<bf16>(), P->Ha.as<float>(), nullptr, P->N,
+                                           P->c, P->Np, P->cp);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+// The bf16 features every mixed problem reads: x row-major and x^T K-block-major.  The operands
+// that depend on which Hessian apply the problem takes follow in tc_prepare_operands, once
+// tc_setup_pw has decided that.
 int32_t tc_prepare(firal_problem* P) {
   cudaStream_t st = P->H->stream;
   if (P->d > 128) return fail(FIRAL_ERR_UNSUPPORTED, "mixed path supports d <= 128");
@@ -2292,36 +2309,49 @@ int32_t tc_prepare(firal_problem* P) {
   P->cp = (int32_t)((P->c + 63) / 64 * 64);
   P->Np = (P->N + 127) / 128 * 128;
   const int64_t Np = P->Np;
-  FIRAL_TRY(P->Hb.ensure((size_t)Np * P->cp * 2));
-  const int cpb2 = (P->cp + d_cfg::MT * d_cfg::BM - 1) / (d_cfg::MT * d_cfg::BM) * (d_cfg::MT * d_cfg::BM);
-  FIRAL_TRY(P->HbT.ensure((size_t)Np * cpb2 * 2));
   FIRAL_TRY(P->Xb.ensure((size_t)Np * P->dp * 2 * 2));   // X (Np x dp) then X^T (dp x Np)
   const int64_t tot_x = Np * P->dp;
   ProfScope ps(st, PF_PREP);
-  count_launch(3);
-  {
-    dim3 g, b;
-    bf16_pad_grid(Np, P->cp, g, b);
-    k_bf16_pad<0><<<g, b, 0, st>>>(P->Hb.as<bf16>(), P->Ha.as<float>(), nullptr, P->N, P->c, Np,
-                                   P->cp);
-    bf16_pad_grid(Np, P->dp, g, b);
-    k_bf16_pad<0><<<g, b, 0, st>>>(P->Xb.as<bf16>(), P->Xa.as<float>(), nullptr, P->N, P->d, Np,
-                                   P->dp);
-  }
+  count_launch(2);
+  dim3 g, b;
+  bf16_pad_grid(Np, P->dp, g, b);
+  k_bf16_pad<0><<<g, b, 0, st>>>(P->Xb.as<bf16>(), P->Xa.as<float>(), nullptr, P->N, P->d, Np,
+                                 P->dp);
   FIRAL_CUDA_TRY(cudaGetLastError());
-  // h^T and x^T of the D-GEMM, K-block-major
-  k_block_transpose_bf16<<<dim3((unsigned)(Np / 32), (unsigned)(cpb2 / 32)), dim3(32, 8), 0, st>>>(
-      P->HbT.as<bf16>(), P->Hb.as<bf16>(), Np, P->cp, cpb2);
   k_block_transpose_bf16<<<dim3((unsigned)(Np / 32), (unsigned)((P->dp + 31) / 32)), dim3(32, 8),
                            0, st>>>(P->Xb.as<bf16>() + tot_x, P->Xb.as<bf16>(), Np, P->dp, P->dp);
   FIRAL_CUDA_TRY(cudaGetLastError());
-  FIRAL_TRY(tc_prepare_centred(P, cpb2));
+  return FIRAL_OK;
+}
+
+// The constant operands of the problem's Hessian apply and block sums.  The fused per-point
+// apply (P->pw) reads h itself and sums the preconditioner blocks only, against the bf16 part of
+// the pair operand: it takes no bf16 h, no h^T, no centred copies and no lo part of Z (row
+// shards, whose gradient forms take the general path, make the bf16 h on first use).  64 pools
+// of 0.5 M rows and 1,000 classes together: 1 GB of h copies and 2 GB of Z_lo not written.
+int32_t tc_prepare_operands(firal_problem* P) {
+  cudaStream_t st = P->H->stream;
+  const int64_t Np = P->Np;
+  ProfScope ps(st, PF_PREP);
+  if (!P->pw) {
+    const int cpb2 =
+        (P->cp + d_cfg::MT * d_cfg::BM - 1) / (d_cfg::MT * d_cfg::BM) * (d_cfg::MT * d_cfg::BM);
+    FIRAL_TRY(make_hb(P));
+    FIRAL_TRY(P->HbT.ensure((size_t)Np * cpb2 * 2));
+    // h^T of the D-GEMM, K-block-major
+    count_launch();
+    k_block_transpose_bf16<<<dim3((unsigned)(Np / 32), (unsigned)(cpb2 / 32)), dim3(32, 8), 0,
+                             st>>>(P->HbT.as<bf16>(), P->Hb.as<bf16>(), Np, P->cp, cpb2);
+    FIRAL_CUDA_TRY(cudaGetLastError());
+    FIRAL_TRY(tc_prepare_centred(P, cpb2));
+  }
   // pair operand of the block sums (problem constant): Z = x (x) x on the pair triangle
   const int npairs = P->d * (P->d + 1) / 2;
   const int64_t npp = (npairs + b_cfg::NPP_ALIGN - 1) / b_cfg::NPP_ALIGN * b_cfg::NPP_ALIGN;
-  FIRAL_TRY(P->Zp.ensure((size_t)2 * npp * Np * 2));
+  FIRAL_TRY(P->Zp.ensure((size_t)(P->pw ? 1 : 2) * npp * Np * 2));
   k_build_z<<<(unsigned)(Np / 64), 256, 0, st>>>(
-      P->Zp.as<bf16>(), P->Zp.as<bf16>() + npp * Np, P->Xb.as<bf16>(), P->d, P->dp, npairs, npp);
+      P->Zp.as<bf16>(), P->pw ? nullptr : P->Zp.as<bf16>() + npp * Np, P->Xb.as<bf16>(), P->d,
+      P->dp, npairs, npp);
   count_launch();
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
@@ -2651,7 +2681,7 @@ int32_t tc_syrk_blocks(firal_problem* P, const void* wv, double lamS, void* outS
     FIRAL_TRY(make_map(&mA1, Alo, arows, BK, BM, BK, true));
     FIRAL_TRY(make_map(&mA2, AP, arows, BK, BM, BK, true));
     FIRAL_TRY(make_map(&mZ0, P->Zp.p, zrows, BK, BN, BK, true));
-    FIRAL_TRY(make_map(&mZ1, P->Zp.as<bf16>() + npp * Np, zrows, BK, BN, BK, true));
+    if (outS) FIRAL_TRY(make_map(&mZ1, P->Zp.as<bf16>() + npp * Np, zrows, BK, BN, BK, true));
     const int grid = std::min(units, sms);
     if (outS && s1) {
       // one product: A_hi against the pair operand's bf16 part
@@ -2757,6 +2787,7 @@ __global__ void k_quad_combine(const float* part1, int n_nt1, const float* a32, 
 static int32_t ensure_hlo(firal_problem* P) {
   const size_t bytes = (size_t)P->Np * P->cp * 2;
   if (P->Hlo.p && P->Hlo.bytes >= bytes && P->hlo_ready) return FIRAL_OK;
+  if (P->pw) FIRAL_TRY(make_hb(P));
   FIRAL_TRY(P->Hlo.ensure(bytes));
   ProfScope ps(P->H->stream, PF_PREP);
   count_launch();
