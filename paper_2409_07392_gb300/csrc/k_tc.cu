@@ -3496,18 +3496,19 @@ int32_t tc_round_scores(firal_problem* P, const void* M1, const void* M2, const 
 // staged x^T tile, K-major, 128 rows of which the first dp are features) and psi as an
 // MN-major operand, so each epilogue thread writes its row's psi values as 16-byte runs.
 // Work list: segments of at most SEG_TILES 128-row tiles of one pool's rows (its labelled
-// rows and its pool rows are separate segments); the host deals the segments to the CTAs
-// longest first (sched: per-CTA offsets, then segment indices), and a CTA takes every probe
-// group of each of its segments (an item).  A tile that also holds rows of another pool runs once per pool with
-// the other rows masked.  An item accumulates out in TMEM and writes one partial; a
+// rows and its pool rows are separate segments); an item is one probe group of a segment, and
+// the host deals the items to the CTAs longest first (sched: per-CTA offsets, then items as
+// segment GRP_MAX + group), so a single pool of 50,000 rows (49 segments) still fills the chip.
+// A tile that also holds rows of another pool runs once per pool with the other rows masked.  An item accumulates out in TMEM and writes one partial; a
 // per-class combine adds a pool's partials in segment order.
 // Pipeline: the x and x^T tiles, the S accumulator (TMEM), the psi operand (shared memory) and
 // the D accumulator are double-buffered: the TMA loads of tile t+1, MMA1 of tile t+1, the
 // epilogue of tile t and MMA2 of tile t-1 overlap.  Each epilogue thread loads its row's h for
 // the next tile while it works on the current one, from the class-major copy of h (one
 // coalesced run of 128 rows per class).
-// Roles (384 threads): warp 0 TMA producer, warp 1 MMA issuer, warp 2 TMEM owner, warps 4-11
-// epilogue (warp & 3 = TMEM lane quarter, (warp - 4) >> 2 = which 32-column chunks).
+// Roles (384 threads): warp 0 TMA producer (P~ and x), warp 1 MMA issuer, warp 2 TMEM owner,
+// warp 3 TMA producer (x^T), warps 4-11 epilogue (warp & 3 = TMEM lane quarter, (warp - 4) >> 2
+// = which 32-column chunks).
 // ------------------------------------------------------------------------------------------
 namespace pw_cfg {
 constexpr int NU = 128;                           // columns per unit (probe group)
@@ -3521,6 +3522,7 @@ constexpr int OFF_PT = 0, OFF_XA = 2 * PT_HALF, OFF_XT = OFF_XA + 2 * XA_BYTES;
 constexpr int OFF_PSI = OFF_XT + 2 * XT_BYTES, OFF_CTL = OFF_PSI + 2 * PSI_BUF;
 constexpr int SMEM = OFF_CTL + 256 + 1024;
 constexpr uint32_t TS = 0, TD = 256;              // TMEM columns: S (2 x 128) | D (2 x 128)
+constexpr int GRP_MAX = 64;   // probe groups of a segment: 32 classes x 256 probes / NU
 }  // namespace pw_cfg
 
 struct PwCtl {   // < 256 bytes
@@ -3764,56 +3766,69 @@ __global__ void __launch_bounds__(384, 1)
   };
 
   if (warp == 0 && lane == 0) {
-    // ---------------- TMA producer: P~ of each item, x and x^T of each of its tiles
+    // ---------------- TMA producer: P~ of each item, x of each of its tiles
     tma_prefetch(&mapX);
-    tma_prefetch(&mapXT);
     tma_prefetch(&mapPT);
     uint32_t nt = 0, ni = 0;   // tiles and items loaded
     bool ok = true;
     for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
-      const int4 sg = seg_tab[sched[gridDim.x + 1 + it]];
+      const int code = sched[gridDim.x + 1 + it], grp = code & (GRP_MAX - 1);
+      const int4 sg = seg_tab[code / GRP_MAX];
       const int4 pq = pool_tab[sg.x];
       const int n1 = pq.z * sp, pbase = 2 * sp * pq.w;
-      const int ng = pw_ngrp(pq.z, sp);
-      for (int grp = 0; grp < ng && ok; ++grp) {
-        const int nc = pw_ncols(pq.z, sp, grp);
-        if (!mbar_wait(&ctl->pt_empty, (ni & 1) ^ 1, abort_w)) { give_up(41); ok = false; break; }
-        mbar_expect_tx(&ctl->pt_full, 2 * nc * 128);
-        for (int part = 0; part < 2; ++part)
-          for (int r = 0; r < nc; r += 64)
-            tma_load_2d(sm + OFF_PT + part * PT_HALF + r * 128, &mapPT, &ctl->pt_full, 0,
-                        pbase + part * n1 + grp * NU + r);
-        ++ni;
-        for (int t = sg.y >> 7; t <= (sg.z - 1) >> 7; ++t) {
-          const int b = nt & 1;
-          const uint32_t ph = (nt >> 1) & 1;
-          // both buffers free before either load is issued: a wait that gives up leaves no
-          // load of this tile in flight
-          if (!mbar_wait(&ctl->x_empty[b], ph ^ 1, abort_w) ||
-              !mbar_wait(&ctl->xt_empty[b], ph ^ 1, abort_w)) {
-            give_up(42);
-            ok = false;
-            break;
-          }
-          mbar_expect_tx(&ctl->x_full[b], XA_BYTES);
-          tma_load_2d(sm + OFF_XA + b * XA_BYTES, &mapX, &ctl->x_full[b], 0, t * 128);
-          mbar_expect_tx(&ctl->xt_full[b], 2 * DP * 128);
-          unsigned char* xt = sm + OFF_XT + b * XT_BYTES;
-          tma_load_2d(xt, &mapXT, &ctl->xt_full[b], 0, (2 * t) * DP);
-          tma_load_2d(xt + DP * 128, &mapXT, &ctl->xt_full[b], 0, (2 * t + 1) * DP);
-          ++nt;
+      const int nc = pw_ncols(pq.z, sp, grp);
+      if (!mbar_wait(&ctl->pt_empty, (ni & 1) ^ 1, abort_w)) { give_up(41); break; }
+      mbar_expect_tx(&ctl->pt_full, 2 * nc * 128);
+      for (int part = 0; part < 2; ++part)
+        for (int r = 0; r < nc; r += 64)
+          tma_load_2d(sm + OFF_PT + part * PT_HALF + r * 128, &mapPT, &ctl->pt_full, 0,
+                      pbase + part * n1 + grp * NU + r);
+      ++ni;
+      for (int t = sg.y >> 7; t <= (sg.z - 1) >> 7; ++t) {
+        const int b = nt & 1;
+        if (!mbar_wait(&ctl->x_empty[b], ((nt >> 1) & 1) ^ 1, abort_w)) {
+          give_up(42);
+          ok = false;
+          break;
         }
+        mbar_expect_tx(&ctl->x_full[b], XA_BYTES);
+        tma_load_2d(sm + OFF_XA + b * XA_BYTES, &mapX, &ctl->x_full[b], 0, t * 128);
+        ++nt;
       }
     }
     // every issued load lands before the CTA can exit (buffer b took loads nt = b, b + 2, ...)
     for (int b = 0; b < 2; ++b) {
       const uint32_t cnt = (nt + 1 - b) / 2;
-      if (cnt) {
-        mbar_wait_drain(&ctl->x_full[b], (cnt - 1) & 1);
-        mbar_wait_drain(&ctl->xt_full[b], (cnt - 1) & 1);
-      }
+      if (cnt) mbar_wait_drain(&ctl->x_full[b], (cnt - 1) & 1);
     }
     if (ni) mbar_wait_drain(&ctl->pt_full, (ni - 1) & 1);
+  } else if (warp == 3 && lane == 0) {
+    // ---------------- TMA producer of the x^T tiles.  Its own thread: an x^T buffer is free
+    // after MMA2, an x buffer already after MMA1, and a single producer that waits for both
+    // puts the loads' latency between one tile's MMA2 and the next tile's MMA1.
+    tma_prefetch(&mapXT);
+    uint32_t nt = 0;
+    bool ok = true;
+    for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
+      const int4 sg = seg_tab[sched[gridDim.x + 1 + it] / GRP_MAX];
+      for (int t = sg.y >> 7; t <= (sg.z - 1) >> 7; ++t) {
+        const int b = nt & 1;
+        if (!mbar_wait(&ctl->xt_empty[b], ((nt >> 1) & 1) ^ 1, abort_w)) {
+          give_up(43);
+          ok = false;
+          break;
+        }
+        mbar_expect_tx(&ctl->xt_full[b], 2 * DP * 128);
+        unsigned char* xt = sm + OFF_XT + b * XT_BYTES;
+        tma_load_2d(xt, &mapXT, &ctl->xt_full[b], 0, (2 * t) * DP);
+        tma_load_2d(xt + DP * 128, &mapXT, &ctl->xt_full[b], 0, (2 * t + 1) * DP);
+        ++nt;
+      }
+    }
+    for (int b = 0; b < 2; ++b) {
+      const uint32_t cnt = (nt + 1 - b) / 2;
+      if (cnt) mbar_wait_drain(&ctl->xt_full[b], (cnt - 1) & 1);
+    }
   } else if (warp == 1 && lane == 0) {
     // ---------------- MMA issuer: MMA1 of unit u, then MMA2 of unit u - 1
     struct Pend {
@@ -3855,36 +3870,35 @@ __global__ void __launch_bounds__(384, 1)
       return true;
     };
     for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
-      const int4 sg = seg_tab[sched[gridDim.x + 1 + it]];
+      const int code = sched[gridDim.x + 1 + it], grp = code & (GRP_MAX - 1);
+      const int4 sg = seg_tab[code / GRP_MAX];
       const int4 pq = pool_tab[sg.x];
-      const int ng = pw_ngrp(pq.z, sp);
       const int t0 = sg.y >> 7, t1 = (sg.z - 1) >> 7;
-      for (int grp = 0; grp < ng && ok; ++grp) {
-        const uint32_t idesc1 = idesc_bf16_f32(128, pw_ncols(pq.z, sp, grp));
-        if (!mbar_wait(&ctl->pt_full, ni & 1, abort_w)) { give_up(44); ok = false; break; }
-        const uint32_t item = ni++;
-        for (int t = t0; t <= t1; ++t) {
-          const uint32_t u = nt;
-          const int b = u & 1;
-          const uint32_t ph = (u >> 1) & 1;
-          if (!mbar_wait(&ctl->x_full[b], ph, abort_w) ||
-              !mbar_wait(&ctl->s_empty[b], ph ^ 1, abort_w)) { give_up(45); ok = false; break; }
-          tc_fence_after();
-          const uint32_t xa = smem_u32(sm + OFF_XA + b * XA_BYTES), pt = smem_u32(sm + OFF_PT);
+      const int nc = pw_ncols(pq.z, sp, grp);
+      const uint32_t idesc1 = idesc_bf16_f32(128, nc);
+      if (!mbar_wait(&ctl->pt_full, ni & 1, abort_w)) { give_up(44); ok = false; break; }
+      const uint32_t item = ni++;
+      for (int t = t0; t <= t1; ++t) {
+        const uint32_t u = nt;
+        const int b = u & 1;
+        const uint32_t ph = (u >> 1) & 1;
+        if (!mbar_wait(&ctl->x_full[b], ph, abort_w) ||
+            !mbar_wait(&ctl->s_empty[b], ph ^ 1, abort_w)) { give_up(45); ok = false; break; }
+        tc_fence_after();
+        const uint32_t xa = smem_u32(sm + OFF_XA + b * XA_BYTES), pt = smem_u32(sm + OFF_PT);
 #pragma unroll
-          for (int k = 0; k < DP / 16; ++k) {
-            const uint64_t ad = sdesc_sw128(xa + k * 32);
-            umma_bf16(tmem + TS + b * NU, ad, sdesc_sw128(pt + k * 32), idesc1, k > 0 ? 1u : 0u);
-            umma_bf16(tmem + TS + b * NU, ad, sdesc_sw128(pt + PT_HALF + k * 32), idesc1, 1u);
-          }
-          umma_commit(&ctl->s_full[b]);
-          umma_commit(&ctl->x_empty[b]);
-          if (t == t1) umma_commit(&ctl->pt_empty);
-          ++nt;
-          if (have && !mma2(pend)) { give_up(46); ok = false; break; }
-          pend = Pend{u, item, t == t0, t == t1, pw_ncols(pq.z, sp, grp)};
-          have = true;
+        for (int k = 0; k < DP / 16; ++k) {
+          const uint64_t ad = sdesc_sw128(xa + k * 32);
+          umma_bf16(tmem + TS + b * NU, ad, sdesc_sw128(pt + k * 32), idesc1, k > 0 ? 1u : 0u);
+          umma_bf16(tmem + TS + b * NU, ad, sdesc_sw128(pt + PT_HALF + k * 32), idesc1, 1u);
         }
+        umma_commit(&ctl->s_full[b]);
+        umma_commit(&ctl->x_empty[b]);
+        if (t == t1) umma_commit(&ctl->pt_empty);
+        ++nt;
+        if (have && !mma2(pend)) { give_up(46); ok = false; break; }
+        pend = Pend{u, item, t == t0, t == t1, nc};
+        have = true;
       }
     }
     if (ok && have && !*abort_w && !mma2(pend)) give_up(46);
@@ -3898,16 +3912,14 @@ __global__ void __launch_bounds__(384, 1)
     uint32_t u = 0, ni = 0;
     bool ok = true;
     for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
-      const int4 sg = seg_tab[sched[gridDim.x + 1 + it]];
+      const int code = sched[gridDim.x + 1 + it], grp = code & (GRP_MAX - 1);
+      const int4 sg = seg_tab[code / GRP_MAX];
       const int4 pq = pool_tab[sg.x];
-      const int ng = pw_ngrp(pq.z, sp);
-      for (int grp = 0; grp < ng && ok; ++grp) {
-        const int nc = pw_ncols(pq.z, sp, grp);
-        const uint32_t item = ni++;
-        if (pq.z == 8) ok = pw_epi_item<8, DP>(E, u, item, sg, pq, grp, nc);
-        else if (pq.z == 16) ok = pw_epi_item<16, DP>(E, u, item, sg, pq, grp, nc);
-        else ok = pw_epi_item<32, DP>(E, u, item, sg, pq, grp, nc);
-      }
+      const int nc = pw_ncols(pq.z, sp, grp);
+      const uint32_t item = ni++;
+      if (pq.z == 8) ok = pw_epi_item<8, DP>(E, u, item, sg, pq, grp, nc);
+      else if (pq.z == 16) ok = pw_epi_item<16, DP>(E, u, item, sg, pq, grp, nc);
+      else ok = pw_epi_item<32, DP>(E, u, item, sg, pq, grp, nc);
     }
   }
   __syncthreads();
@@ -3978,13 +3990,25 @@ __global__ void __launch_bounds__(PWF_THREADS) k_pw_finish(float* out, const flo
   const int q = blockIdx.x, j = blockIdx.y;
   const int4 pt = pool_tab[q];
   const int2 sr = pseg[q];
-  const int cq = pt.y;
+  const int cq = pt.y, ns = sr.y - sr.x;
   const float* vm = vmean + (j * Qe + q) * d;
   for (int idx = threadIdx.x; idx < cq * d; idx += blockDim.x) {
     const int kl = idx / d, e = idx - kl * d;
     const int64_t o = (int64_t)j * D + (int64_t)(pt.x + kl) * d + e;
     float acc = lam * (V[o] - vm[e]);
-    for (int g = sr.x; g < sr.y; ++g) acc += part[((int64_t)(seg_tab[g].w + kl) * sp + j) * d + e];
+    // a pool's segments are consecutive: its partial of segment g lies g cq rows after the first;
+    // eight loads in flight, added in segment order
+    const float* ps = part + ((int64_t)((ns ? seg_tab[sr.x].w : 0) + kl) * sp + j) * d + e;
+    const int64_t step = (int64_t)cq * sp * d;
+    int g = 0;
+    for (; g + 8 <= ns; g += 8) {
+      float v[8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) v[x] = ps[(g + x) * step];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) acc += v[x];
+    }
+    for (; g < ns; ++g) acc += ps[g * step];
     t[kl * 64 + e] = acc;
   }
   __syncthreads();
@@ -4138,9 +4162,14 @@ static int32_t pw_schedule(firal_problem* P, int sp, bool quad, int* grid_out,
     const int4 sg = P->pw_seg_h[g];
     if (quad && (int64_t)sg.z <= P->m) continue;
     const int4 pq = P->pw_pool_h[sg.x];
-    const int64_t ng = ((int64_t)pq.z * sp + pw_cfg::NU - 1) / pw_cfg::NU;
+    const int ng = (pq.z * sp + pw_cfg::NU - 1) / pw_cfg::NU;
     const int64_t tiles = (sg.z - 1) / 128 - sg.y / 128 + 1;
-    items.push_back({(tiles + 1) * ng, g});
+    // apply: an item is one probe group of a segment (each group writes its own partial);
+    // gradient: a segment (its groups add to the same entries of g in group order)
+    if (quad)
+      items.push_back({(tiles + 1) * ng, g});
+    else
+      for (int grp = 0; grp < ng; ++grp) items.push_back({tiles + 1, g * pw_cfg::GRP_MAX + grp});
   }
   const int grid = std::max(1, std::min<int>(P->sms, (int)items.size()));
   std::stable_sort(items.begin(), items.end(),
