@@ -509,12 +509,13 @@ int32_t validate_pool(const firal_pool* pool, const firal_hess0* h0) {
   return FIRAL_OK;
 }
 
-// stacked: the rows of several pools; their tables and the operands that depend on them follow in
-// pooled_create
+// stacked: the rows of several pools (checked by the caller; pool and h0 then give the total sizes
+// and no pointers); their tables and the operands that depend on them follow in pooled_create
 int32_t problem_create_impl(firal_handle* H, const firal_pool* pool, const firal_hess0* h0,
-                            int32_t precision, firal_problem** out, bool stacked = false) {
+                            int32_t precision, firal_problem** out,
+                            const std::vector<StackRows>* stacked = nullptr) {
   if (!H || !out) return fail(FIRAL_ERR_ARG, "handle and out must be non-null");
-  FIRAL_TRY(validate_pool(pool, h0));
+  if (!stacked) FIRAL_TRY(validate_pool(pool, h0));
   if (precision < FIRAL_FP64 || precision > FIRAL_MIXED_BF16_FAST)
     return fail(FIRAL_ERR_ARG, "unknown precision");
   if (is_mixed(precision) && !tc_available())
@@ -552,10 +553,20 @@ int32_t problem_create_impl(firal_handle* H, const firal_pool* pool, const firal
   } while (0)
   TRYC(P->Xa.ensure((size_t)P->N * P->d * vs));
   TRYC(P->Ha.ensure((size_t)P->N * P->c * vs));
-  TRYC(copy_rows(P->dbl, P->Xa.p, h0 ? h0->Xo : nullptr, P->m, pool->X, P->n, P->d,
-                 pool->x_dtype, st));
-  TRYC(copy_rows(P->dbl, P->Ha.p, h0 ? h0->ho : nullptr, P->m, pool->h, P->n, P->c,
-                 pool->h_dtype, st));
+  if (stacked) {
+    const size_t tb = stacked->size() * sizeof(StackRows);
+    TRYC(P->stack_tab.ensure(tb));
+    if (cudaMemcpyAsync(P->stack_tab.p, stacked->data(), tb, cudaMemcpyHostToDevice, st) !=
+        cudaSuccess)
+      return cleanup(fail(FIRAL_ERR_CUDA, "copy of the pools' row table"));
+    TRYC(stack_rows(P->dbl, P->Xa.p, P->Ha.p, P->stack_tab.as<StackRows>(), (int)stacked->size(),
+                    P->N, P->d, P->c, pool->x_dtype, pool->h_dtype, st));
+  } else {
+    TRYC(copy_rows(P->dbl, P->Xa.p, h0 ? h0->Xo : nullptr, P->m, pool->X, P->n, P->d,
+                   pool->x_dtype, st));
+    TRYC(copy_rows(P->dbl, P->Ha.p, h0 ? h0->ho : nullptr, P->m, pool->h, P->n, P->c,
+                   pool->h_dtype, st));
+  }
   // class-major copy of h for the FP64 kernels; the FP32 kernels read rows, and the tensor-core
   // path reads its own bf16 operands, prepared below
   if (P->dbl) TRYC(class_major_h(P));
@@ -910,17 +921,12 @@ firal_relax_opts default_relax_opts() {
 // h row holds its pool's probabilities in that pool's class columns and zeros elsewhere, so
 // every Hessian, Sigma_z and the preconditioner are block diagonal over pools.
 // ------------------------------------------------------------------------------------------
-static size_t dtype_size(int32_t dt) {
-  return dt == FIRAL_DT_BF16 ? 2 : dt == FIRAL_DT_F32 ? 4 : 8;
-}
-
 int32_t pooled_create(firal_handle* H, const std::vector<int>& idx, const firal_pool* pools,
                       const firal_hess0* h0s, const double* budgets, int32_t prec,
                       firal_problem** out) {
   const int Q = (int)idx.size();
   cudaStream_t st = H->stream;
   const firal_pool& p0 = pools[idx[0]];
-  const size_t xs = dtype_size(p0.x_dtype), hs = dtype_size(p0.h_dtype);
   int dg = 0;
   int64_t C = 0, M = 0, n = 0;
   std::vector<int> coff(Q + 1), pdim(Q);
@@ -941,63 +947,23 @@ int32_t pooled_create(firal_handle* H, const std::vector<int>& idx, const firal_
   loff[Q] = M;
   poff[Q] = n;
   if (C > 4096) return fail(FIRAL_ERR_UNSUPPORTED, "pooled classes exceed 4096");
-  // stacked inputs (temporaries)
-  DBuf Xs, Hs, Xos, Hos;
-  auto rel = [&]() {
-    Xs.release();
-    Hs.release();
-    Xos.release();
-    Hos.release();
-  };
-  int32_t rc = FIRAL_OK;
-#define TRYP(x)                    \
-  do {                             \
-    rc = (x);                      \
-    if (rc != FIRAL_OK) {          \
-      rel();                       \
-      return rc;                   \
-    }                              \
-  } while (0)
-#define CUDP(x)                                                           \
-  do {                                                                    \
-    cudaError_t e_ = (x);                                                 \
-    if (e_ != cudaSuccess) {                                              \
-      rel();                                                              \
-      return fail(FIRAL_ERR_CUDA, std::string(#x) + ": " + cudaGetErrorString(e_)); \
-    }                                                                     \
-  } while (0)
-  TRYP(Xs.ensure((size_t)n * dg * xs));
-  TRYP(Hs.ensure((size_t)n * C * hs));
-  CUDP(cudaMemsetAsync(Xs.p, 0, (size_t)n * dg * xs, st));
-  CUDP(cudaMemsetAsync(Hs.p, 0, (size_t)n * C * hs, st));
-  if (M > 0) {
-    TRYP(Xos.ensure((size_t)M * dg * xs));
-    TRYP(Hos.ensure((size_t)M * C * hs));
-    CUDP(cudaMemsetAsync(Xos.p, 0, (size_t)M * dg * xs, st));
-    CUDP(cudaMemsetAsync(Hos.p, 0, (size_t)M * C * hs, st));
-  }
+  // the stacked rows: every pool's labelled rows, then every pool's own
+  std::vector<StackRows> rows;
+  for (int q = 0; q < Q; ++q)
+    if (loff[q + 1] > loff[q]) {
+      const firal_hess0& h0 = h0s[idx[q]];
+      rows.push_back({h0.Xo, h0.ho, loff[q], h0.m, coff[q], pools[idx[q]].c, pools[idx[q]].d});
+    }
   for (int q = 0; q < Q; ++q) {
     const firal_pool& pl = pools[idx[q]];
-    CUDP(cudaMemcpy2DAsync((char*)Xs.p + (size_t)poff[q] * dg * xs, dg * xs, pl.X, pl.d * xs,
-                           pl.d * xs, pl.n, cudaMemcpyDeviceToDevice, st));
-    CUDP(cudaMemcpy2DAsync((char*)Hs.p + ((size_t)poff[q] * C + coff[q]) * hs, C * hs, pl.h,
-                           pl.c * hs, pl.c * hs, pl.n, cudaMemcpyDeviceToDevice, st));
-    const int64_t mq = loff[q + 1] - loff[q];
-    if (mq > 0) {
-      const firal_hess0& h0 = h0s[idx[q]];
-      CUDP(cudaMemcpy2DAsync((char*)Xos.p + (size_t)loff[q] * dg * xs, dg * xs, h0.Xo,
-                             pl.d * xs, pl.d * xs, mq, cudaMemcpyDeviceToDevice, st));
-      CUDP(cudaMemcpy2DAsync((char*)Hos.p + ((size_t)loff[q] * C + coff[q]) * hs, C * hs, h0.ho,
-                             pl.c * hs, pl.c * hs, mq, cudaMemcpyDeviceToDevice, st));
-    }
+    rows.push_back({pl.X, pl.h, M + poff[q], pl.n, coff[q], pl.c, pl.d});
   }
-  firal_pool sp{Xs.p, Hs.p, n, dg, (int32_t)C, p0.x_dtype, p0.h_dtype};
-  firal_hess0 sh{Xos.p, Hos.p, M, h0s ? h0s[idx[0]].lambda : 0.0};
+  firal_pool sp{nullptr, nullptr, n, dg, (int32_t)C, p0.x_dtype, p0.h_dtype};
+  firal_hess0 sh{nullptr, nullptr, M, h0s ? h0s[idx[0]].lambda : 0.0};
   firal_problem* P = nullptr;
-  TRYP(problem_create_impl(H, &sp, &sh, prec, &P, true));
-  rel();
-#undef TRYP
-#undef CUDP
+  // (the row table lives until the synchronisation below, or the one in firal_problem_destroy)
+  FIRAL_TRY(problem_create_impl(H, &sp, &sh, prec, &P, &rows));
+  int32_t rc = FIRAL_OK;
   auto bail = [&](int32_t code) {
     firal_problem_destroy(P);
     return code;
@@ -1377,7 +1343,7 @@ int32_t firal_problem_destroy(firal_problem* P) {
                   &P->W, &P->HU, &P->g, &P->red, &P->zsave, &P->Xb, &P->Hb, &P->HbT, &P->Pb, &P->vmean, &P->qmean, &P->Aw, &P->Zp, &P->Hlo, &P->gq_ab,
                   &P->gq_m, &P->gq_part, &P->rtab, &P->rM, &P->tdev, &P->cen, &P->cen_off,
                   &P->cen_idx, &P->Ub, &P->UbT, &P->cen_am, &P->cen_rho, &P->cen_lab, &P->cen_items, &P->cen_part,
-                  &P->pool_tabs, &P->pool_z, &P->md_part, &P->kr_alpha, &P->kr_dterm,
+                  &P->pool_tabs, &P->stack_tab, &P->pool_z, &P->md_part, &P->kr_alpha, &P->kr_dterm,
                   &P->kr_bsum, &P->bcg, &P->pw_pool, &P->pw_seg, &P->pw_pseg, &P->pw_pk,
                   &P->pw_part, &P->X64, &P->S_lab, &P->w_lab, &P->cm_scr}) {
     if (synced) b->park();

@@ -212,6 +212,7 @@ struct firal_problem {
   bool hlo_ready = false;        // made on first use)
   firal::DBuf vmean, qmean;      // class means of the probe block / of the raw apply (s x d)
   firal::DBuf Aw;                // block sums: (w h)^T hi, lo and (w h (1 - h))^T (3 x cp x Np)
+  firal::DBuf stack_tab;         // pooled problems: the StackRows the rows came from
   firal::DBuf Zp;                // block sums: x (x) x on the pair triangle, bf16 hi and lo
   firal::DBuf gq_ab, gq_m, gq_part;  // tensor-core quadratic forms: [A;B], M~ pairs, partials
   firal::DBuf rtab, rM;          // Round on tensor cores: 8-pair chunk table, M~ hi/lo rows
@@ -266,6 +267,16 @@ int32_t shard_allreduce(firal_problem* P, void* buf, int64_t count, int32_t dtyp
 // ---- k_simt.cu
 int32_t copy_rows(bool dbl, void* dst, const void* a, int64_t ma, const void* b, int64_t nb,
                   int cols, int32_t src_dtype, cudaStream_t st);
+// rows [row0, row0 + rows) of a pooled problem: one pool's labelled or pool rows (c classes from
+// column c0, d features), in the problem's storage types
+struct StackRows {
+  const void* X;
+  const void* h;
+  int64_t row0, rows;
+  int c0, c, d;
+};
+int32_t stack_rows(bool dbl, void* X, void* H, const StackRows* tab, int nent, int64_t N, int dg,
+                   int C, int32_t x_dtype, int32_t h_dtype, cudaStream_t st);
 int32_t transpose(bool dbl, void* dst, const void* src, int64_t rows, int cols, cudaStream_t st);
 int32_t class_major_h(firal_problem* P);
 int32_t fill_weights(bool dbl, void* w, int64_t m, double lab_val, const void* z, double zconst,

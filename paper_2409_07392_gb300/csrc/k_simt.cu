@@ -136,6 +136,70 @@ int32_t copy_rows(bool dbl, void* dst, const void* a, int64_t ma, const void* b,
   return copy_rows_t<float, __nv_bfloat16>(dst, a, ma, b, nb, cols, st);
 }
 
+// The rows of several pools stacked (pooled problems): row r of entry t takes the pool's features
+// (zero up to the common width dg) and its probabilities in the pool's class columns (zero
+// elsewhere).  One pass that writes every element of X and h once: no zero fill, no stacked copy
+// of the inputs in their own type.  Bound by the writes of h (N x C, of which a pool's columns
+// are a few percent).  A warp takes 8 consecutive rows; its entry is found by bisection.
+// Stacking and copying 64 pools of 1.3 M rows, 3 groups of up to 400 classes (3.2 GB of h): 6.3 ms
+// as fills, 2-D copies and a copy; 0.43 ms here (7.6 TB/s).
+constexpr int STACK_RW = 8;
+template <class T, class Tx, class Th>
+__global__ void __launch_bounds__(256) k_stack_rows(T* __restrict__ X, T* __restrict__ H,
+                                                    const StackRows* __restrict__ tab, int nent,
+                                                    int64_t N, int dg, int C) {
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  int64_t r = ((int64_t)blockIdx.x * 8 + warp) * STACK_RW;
+  const int64_t rend = r + STACK_RW < N ? r + STACK_RW : N;
+  if (r >= rend) return;
+  int lo = 0, hi = nent - 1;
+  while (lo < hi) {   // the last entry that starts at or before r
+    const int mid = (lo + hi + 1) >> 1;
+    if (tab[mid].row0 <= r) lo = mid;
+    else hi = mid - 1;
+  }
+  StackRows e = tab[lo];
+  for (; r < rend; ++r) {
+    while (r >= e.row0 + e.rows) e = tab[++lo];
+    const int64_t i = r - e.row0;
+    const Tx* x = static_cast<const Tx*>(e.X) + i * e.d;
+    for (int k = lane; k < dg; k += 32) X[r * dg + k] = k < e.d ? (T)to_double(x[k]) : T(0);
+    const Th* h = static_cast<const Th*>(e.h) + i * e.c;
+    for (int k = lane; k < C; k += 32) {
+      const int kl = k - e.c0;
+      H[r * C + k] = (kl >= 0 && kl < e.c) ? (T)to_double(h[kl]) : T(0);
+    }
+  }
+}
+
+template <class T>
+static int32_t stack_rows_t(T* X, T* H, const StackRows* tab, int nent, int64_t N, int dg, int C,
+                            int32_t xdt, int32_t hdt, cudaStream_t st) {
+  const unsigned g = (unsigned)((N + 8 * STACK_RW - 1) / (8 * STACK_RW));
+  const bool h64 = hdt == FIRAL_DT_F64;
+  if (xdt == FIRAL_DT_F64) {
+    if (h64) k_stack_rows<T, double, double><<<g, 256, 0, st>>>(X, H, tab, nent, N, dg, C);
+    else k_stack_rows<T, double, float><<<g, 256, 0, st>>>(X, H, tab, nent, N, dg, C);
+  } else if (xdt == FIRAL_DT_F32) {
+    if (h64) k_stack_rows<T, float, double><<<g, 256, 0, st>>>(X, H, tab, nent, N, dg, C);
+    else k_stack_rows<T, float, float><<<g, 256, 0, st>>>(X, H, tab, nent, N, dg, C);
+  } else {
+    if (h64) k_stack_rows<T, __nv_bfloat16, double><<<g, 256, 0, st>>>(X, H, tab, nent, N, dg, C);
+    else k_stack_rows<T, __nv_bfloat16, float><<<g, 256, 0, st>>>(X, H, tab, nent, N, dg, C);
+  }
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+int32_t stack_rows(bool dbl, void* X, void* H, const StackRows* tab, int nent, int64_t N, int dg,
+                   int C, int32_t x_dtype, int32_t h_dtype, cudaStream_t st) {
+  ProfScope ps(st, PF_PREP);
+  count_launch();
+  if (dbl)
+    return stack_rows_t<double>((double*)X, (double*)H, tab, nent, N, dg, C, x_dtype, h_dtype, st);
+  return stack_rows_t<float>((float*)X, (float*)H, tab, nent, N, dg, C, x_dtype, h_dtype, st);
+}
+
 int32_t transpose(bool dbl, void* dst, const void* src, int64_t rows, int cols, cudaStream_t st) {
   dim3 grid((unsigned)((rows + 31) / 32), (unsigned)((cols + 31) / 32));
   dim3 blk(32, 8);
