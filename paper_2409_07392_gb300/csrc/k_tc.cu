@@ -1854,18 +1854,42 @@ __global__ void k_weighted_hT(bf16* Ahi, bf16* Alo, bf16* AP, const float* Ha, c
 //   q_ik = sum_pairs Z_i(e,e') M~_k(e,e'),  Z_i(e,e') = x_ie x_ie',
 // pairs ordered by e with e' running over [8 floor(e/8), d8) so every 8-pair chunk is one
 // aligned 16-byte run of x (pairs with e' < e carry weight 0 in M~).  M~ = symmetric weights
-// (M_ee on the diagonal, M_ee' + M_e'e above it), fed as bf16 hi + lo.  One unit = one
-// 128-point tile; it loops over chunks of 128 classes (N = 256: M1 rows then M2 rows) and keeps
-// a running masked argmax per thread (ties to the lowest index).
+// (M_ee on the diagonal, M_ee' + M_e'e above it), fed as bf16 hi + lo.
+//
+// An item is NT 128-point tiles against a chunk of 128 classes (N = 256: M1 rows then M2 rows).
+// What bounds it: M~ (8.9 MB at d = 128 and 128 classes) streams from L2 once per item, and with
+// one tile per item that stream asks 64 B per clock of every SM.  So two tiles share each M~
+// piece (NT = 2, half the stream), whose accumulators fill TMEM; an item of one tile (few tiles,
+// or several class chunks) double-buffers its accumulator instead.  M~ moves in 32 KB pieces of
+// 32 pairs, hi and lo side by side in one 128-byte row, three to five of them in flight: the
+// L2 latency of a piece passes under the products of the others.
+//
+// The eq. 14 sum takes FP64 divisions (a class of a 32-row group is about 20 FP64 instructions of
+// 64 cycles: 63 us per 128 x 100 tile, against 73 us of products).  With one class chunk the
+// epilogue first forms the score in f32 with a bound on its error, and does the FP64 sum only
+// where that bound reaches the block's best score so far; the result is the FP64 argmax, as if
+// every score had been formed.  With several chunks the FP64 sums run on their own warps beside
+// the next chunk's products.
+//
+// 1 M points, d = 128, 100 classes: 10.4 ms a pick with one tile per item, 64 KB stages, and the
+// FP64 epilogue on the builders' warps; 5.2 ms here (4.6 ms of products at the measured bf16
+// rate).
+//
+// Roles: warp 0 TMA producer, warp 1 MMA issuer, warps 2-7 build Z, warps 8 .. 8 + 4 NT epilogue
+// (warp & 3 = TMEM lane quarter, (warp - 8) >> 2 = tile of the item).
 // ------------------------------------------------------------------------------------------
 namespace r_cfg {
-constexpr int BM = 128, BN = 256, BK = 64, STAGES = 2, NBUILD = 6;
+constexpr int BM = 128, BN = 256, BK = 64, NBUILD = 6;
 constexpr int Z_BYTES = BM * BK * 2;
-constexpr int M_BYTES = BN * BK * 2;
-constexpr int STAGE_BYTES = Z_BYTES + 2 * M_BYTES;       // 80 KB
-template <int DP> struct L {
-  static constexpr int X_BYTES = BM * DP * 2;
-  static constexpr int SMEM = STAGES * STAGE_BYTES + X_BYTES + 1024 + 1024;
+constexpr int UNIT = BN * 128;                           // 32 pairs, hi | lo: 32 KB
+template <int DP, int NT> struct L {
+  static constexpr int X_BYTES = BM * DP * 2;            // one tile's x
+  static constexpr int MST = NT == 1 ? 5 : DP == 128 ? 3 : 4;   // M~ pieces in flight
+  static constexpr int OFF_M = 2 * NT * Z_BYTES, OFF_X = OFF_M + MST * UNIT;
+  static constexpr int OFF_CTL = OFF_X + NT * X_BYTES;
+  static constexpr int SMEM = OFF_CTL + 1400 + 1024;
+  static constexpr int NACC = 2 / NT;                    // accumulator buffers of 256 NT columns
+  static constexpr int THREADS = 256 + 128 * NT;
 };
 }  // namespace r_cfg
 
@@ -1880,43 +1904,67 @@ struct RoundChains {
 };
 
 struct RoundCtl {
-  uint64_t full[2], empty[2], zfull[2], xfull, xempty, tfull, tempty, drain;
+  uint64_t full[5], empty[5], zfull[2], zempty[2], xfull, xempty, tfull[2], tempty[2], drain;
   uint32_t tmem_base;
   int abort_w;
-  double bval[4 * RC_MAX];
-  long long bidx[4 * RC_MAX];
+  int thr[RC_MAX];   // per chain: the block's best score so far, rounded down (float_key)
+  double bval[8 * RC_MAX];
+  long long bidx[8 * RC_MAX];
 };
+static_assert(sizeof(RoundCtl) <= 1400, "control block must fit");
 
-template <int DP>
-__global__ void __launch_bounds__(256, 1)
-    k_tc_round(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapMh,
-               const __grid_constant__ CUtensorMap mapMl, const short2* __restrict__ tab,
-               const float* __restrict__ Ha, const uint8_t* __restrict__ mask, int64_t m,
-               int64_t n, int c, int n_kc, int kblocks, const RoundChains rc,
-               double* part_val, int64_t* part_idx, int32_t* err) {
+// order-preserving integer of a float
+__device__ __forceinline__ int float_key(float f) {
+  const int i = __float_as_int(f);
+  return i ^ ((i >> 31) & 0x7fffffff);
+}
+__device__ __forceinline__ float key_float(int k) {
+  return __int_as_float(k ^ ((k >> 31) & 0x7fffffff));
+}
+
+// FP64 part of eq. 14's sum for one class
+__device__ __forceinline__ void round_term(double& score, float h, float q1, float q2, double eta) {
+  const double hv = (double)h;
+  const double wk = hv * (1.0 - hv);
+  score += wk * (double)q1 / (1.0 + eta * wk * (double)q2);
+}
+
+template <int DP, int NT>
+__global__ void __launch_bounds__(r_cfg::L<DP, NT>::THREADS, 1)
+    k_tc_round(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapM,
+               const short2* __restrict__ tab, const float* __restrict__ Ha,
+               const uint8_t* __restrict__ mask, int64_t m, int64_t n, int c, int n_kc,
+               int kblocks, const RoundChains rc, double* part_val, int64_t* part_idx,
+               int32_t* err) {
   using namespace r_cfg;
-  using LL = L<DP>;
+  using LL = L<DP, NT>;
+  constexpr int MST = LL::MST, NACC = LL::NACC;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  unsigned char* xs = sm + STAGES * STAGE_BYTES;                 // x tile, row i = 2*DP bytes
-  RoundCtl* ctl = (RoundCtl*)(xs + LL::X_BYTES);
+  unsigned char* ms = sm + LL::OFF_M;
+  unsigned char* xs = sm + LL::OFF_X;                 // x tiles, row i = 2*DP bytes
+  RoundCtl* ctl = (RoundCtl*)(sm + LL::OFF_CTL);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int i = 0; i < STAGES; ++i) {
+    for (int i = 0; i < MST; ++i) {
       mbar_init(&ctl->full[i], 1);
       mbar_init(&ctl->empty[i], 1);
+    }
+    for (int i = 0; i < 2; ++i) {
       mbar_init(&ctl->zfull[i], NBUILD);
+      mbar_init(&ctl->zempty[i], 1);
+      mbar_init(&ctl->tfull[i], 1);
+      mbar_init(&ctl->tempty[i], 4 * NT);
     }
     mbar_init(&ctl->xfull, 1);
     mbar_init(&ctl->xempty, NBUILD);
-    mbar_init(&ctl->tfull, 1);
-    mbar_init(&ctl->tempty, 4);
     mbar_init(&ctl->drain, 1);
     ctl->abort_w = 0;
+    for (int e = 0; e < RC_MAX; ++e) ctl->thr[e] = float_key(-INFINITY);
     mbar_fence_init();
   }
   if (warp == 1) {
-    tmem_alloc(&ctl->tmem_base, 256);
+    tmem_alloc(&ctl->tmem_base, 512);
     tmem_relinquish();
   }
   tc_fence_before();
@@ -1924,133 +1972,121 @@ __global__ void __launch_bounds__(256, 1)
   tc_fence_after();
   const uint32_t tmem = ctl->tmem_base;
   volatile int* abort_w = &ctl->abort_w;
-  const int n_mt = (int)((n + BM - 1) / BM);
+  const int64_t n_it = (n + BM * NT - 1) / (BM * NT);
   const int n_ch = rc.n * n_kc;   // (chain, class chunk) pairs, chain-major
-  constexpr uint32_t TX = 2 * M_BYTES;
+  auto give_up = [&](int code) {
+    atomicExch(err, code);
+    ctl->abort_w = 1;
+  };
 
   if (warp == 0 && lane == 0) {
     tma_prefetch(&mapX);
-    tma_prefetch(&mapMh);
-    tma_prefetch(&mapMl);
-    int stage = 0;
-    uint32_t phase = 0, xphase = 0;
+    tma_prefetch(&mapM);
+    uint32_t nx = 0, nm = 0;   // x and M~ loads issued
     bool ok = true;
-    for (int mt = blockIdx.x; mt < n_mt && ok && !*abort_w; mt += gridDim.x) {
-      if (!mbar_wait(&ctl->xempty, xphase ^ 1, abort_w)) {
-        atomicExch(err, 31);
-        ctl->abort_w = 1;
-        break;
-      }
-      mbar_expect_tx(&ctl->xfull, LL::X_BYTES);
-      tma_load_2d(xs, &mapX, &ctl->xfull, 0, (int)(m + (int64_t)mt * BM));
-      xphase ^= 1;
-      for (int kc = 0; kc < n_ch && ok; ++kc) {
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&ctl->empty[stage], phase ^ 1, abort_w)) {
-            atomicExch(err, 32);
-            ctl->abort_w = 1;
+    for (int64_t mt = blockIdx.x; mt < n_it && ok && !*abort_w; mt += gridDim.x) {
+      if (!mbar_wait(&ctl->xempty, (nx & 1) ^ 1, abort_w)) { give_up(31); break; }
+      mbar_expect_tx(&ctl->xfull, NT * LL::X_BYTES);
+#pragma unroll
+      for (int t = 0; t < NT; ++t)
+        tma_load_2d(xs + t * LL::X_BYTES, &mapX, &ctl->xfull, 0, (int)(m + (mt * NT + t) * BM));
+      ++nx;
+      for (int kc = 0; kc < n_ch && ok; ++kc)
+        for (int u = 0; u < 2 * kblocks; ++u) {
+          const int b = nm % MST;
+          if (!mbar_wait(&ctl->empty[b], ((nm / MST) & 1) ^ 1, abort_w)) {
+            give_up(32);
             ok = false;
             break;
           }
-          unsigned char* st = sm + stage * STAGE_BYTES;
-          mbar_expect_tx(&ctl->full[stage], TX);
-          tma_load_2d(st + Z_BYTES, &mapMh, &ctl->full[stage], kb * BK, kc * BN);
-          tma_load_2d(st + Z_BYTES + M_BYTES, &mapMl, &ctl->full[stage], kb * BK, kc * BN);
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
+          mbar_expect_tx(&ctl->full[b], UNIT);
+          tma_load_2d(ms + b * UNIT, &mapM, &ctl->full[b], u * 64, kc * BN);
+          ++nm;
         }
-      }
     }
-    for (int i = 0; i < STAGES; ++i) {
-      if (!mbar_wait(&ctl->empty[stage], phase ^ 1, abort_w)) break;
-      if (++stage == STAGES) {
-        stage = 0;
-        phase ^= 1;
-      }
+    // every issued load lands before the CTA can exit (buffer b took loads b, b + MST, ...)
+    for (uint32_t b = 0; b < MST; ++b) {
+      const uint32_t cnt = (nm + MST - 1 - b) / MST;
+      if (cnt) mbar_wait_drain(&ctl->full[b], (cnt - 1) & 1);
     }
+    if (nx) mbar_wait_drain(&ctl->xfull, (nx - 1) & 1);
   } else if (warp == 1 && lane == 0) {
     constexpr uint32_t idesc = idesc_bf16_f32(BM, BN);
-    int stage = 0;
-    uint32_t phase = 0, acc_phase = 0;
+    uint32_t nm = 0, nz = 0, na = 0;   // M~ pieces, Z blocks and accumulators taken
     bool ok = true;
-    for (int mt = blockIdx.x; mt < n_mt && ok && !*abort_w; mt += gridDim.x) {
+    for (int64_t mt = blockIdx.x; mt < n_it && ok && !*abort_w; mt += gridDim.x) {
       for (int kc = 0; kc < n_ch && ok; ++kc) {
-        if (!mbar_wait(&ctl->tempty, acc_phase ^ 1, abort_w)) {
-          atomicExch(err, 33);
-          ctl->abort_w = 1;
+        const int ab = na % NACC;
+        if (!mbar_wait(&ctl->tempty[ab], ((na / NACC) & 1) ^ 1, abort_w)) {
+          give_up(33);
           ok = false;
           break;
         }
         tc_fence_after();
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!mbar_wait(&ctl->zfull[stage], phase, abort_w) ||
-              !mbar_wait(&ctl->full[stage], phase, abort_w)) {
-            atomicExch(err, 34);
-            ctl->abort_w = 1;
+        for (int kb = 0; kb < kblocks && ok; ++kb) {
+          const int zb = nz & 1;
+          if (!mbar_wait(&ctl->zfull[zb], (nz >> 1) & 1, abort_w)) {
+            give_up(34);
             ok = false;
             break;
           }
-          tc_fence_after();
-          const uint32_t z0 = smem_u32(sm + stage * STAGE_BYTES);
-          const uint32_t mh = z0 + Z_BYTES, ml = mh + M_BYTES;
+          const uint32_t z0 = smem_u32(sm + zb * NT * Z_BYTES);
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t dz = sdesc_sw128(z0 + k * 32);
-            umma_bf16(tmem, dz, sdesc_sw128(mh + k * 32), idesc, (kb | k) != 0);
-            umma_bf16(tmem, dz, sdesc_sw128(ml + k * 32), idesc, 1u);
+          for (int u = 0; u < 2; ++u) {
+            const int b = nm % MST;
+            if (!mbar_wait(&ctl->full[b], (nm / MST) & 1, abort_w)) {
+              give_up(38);
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+            const uint32_t mm = smem_u32(ms + b * UNIT);
+#pragma unroll
+            for (int t = 0; t < NT; ++t)
+#pragma unroll
+              for (int k = 0; k < 2; ++k) {
+                const uint64_t dz = sdesc_sw128(z0 + t * Z_BYTES + (2 * u + k) * 32);
+                const uint32_t acc = tmem + ab * BN + t * BN;
+                umma_bf16(acc, dz, sdesc_sw128(mm + k * 32), idesc, (kb | u | k) != 0);
+                umma_bf16(acc, dz, sdesc_sw128(mm + 64 + k * 32), idesc, 1u);
+              }
+            umma_commit(&ctl->empty[b]);
+            ++nm;
           }
-          umma_commit(&ctl->empty[stage]);
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
+          if (!ok) break;
+          umma_commit(&ctl->zempty[zb]);
+          ++nz;
         }
         if (!ok) break;
-        umma_commit(&ctl->tfull);
-        acc_phase ^= 1;
+        umma_commit(&ctl->tfull[ab]);
+        ++na;
       }
     }
     umma_commit(&ctl->drain);
     mbar_wait_drain(&ctl->drain, 0);
-  } else if (warp >= 2) {
-    const int bw = warp - 2;
-    const int tid_b = bw * 32 + lane;
-    int stage = 0;
-    uint32_t phase = 0, xphase = 0, acc_phase = 0;
+  } else if (warp >= 2 && warp < 2 + NBUILD) {
+    // ---------------- Z blocks: (row i, 8-pair chunk c8); 8 consecutive threads share row i
+    const int tid_b = (warp - 2) * 32 + lane;
+    const int c8 = tid_b & 7;
+    uint32_t nz = 0, nx = 0;
     bool ok = true;
-    double best[RC_MAX];
-    long long besti[RC_MAX];
-#pragma unroll
-    for (int e = 0; e < RC_MAX; ++e) {
-      best[e] = -INFINITY;
-      besti[e] = LLONG_MAX;
-    }
-    for (int mt = blockIdx.x; mt < n_mt && ok && !*abort_w; mt += gridDim.x) {
-      if (!mbar_wait(&ctl->xfull, xphase, abort_w)) {
-        atomicExch(err, 35);
-        ctl->abort_w = 1;
-        break;
-      }
-      xphase ^= 1;
-      double score = 0.0;   // epilogue threads: this point's eq. 14 sum over class chunks
-      for (int ch = 0; ch < n_ch && ok; ++ch) {
-        const int ce = ch / n_kc, kc = ch - ce * n_kc;   // chain, class chunk
-        const double eta = rc.eta[ce];
-        if (kc == 0) score = 0.0;
+    for (int64_t mt = blockIdx.x; mt < n_it && ok && !*abort_w; mt += gridDim.x) {
+      if (!mbar_wait(&ctl->xfull, nx & 1, abort_w)) { give_up(35); break; }
+      ++nx;
+      for (int ch = 0; ch < n_ch && ok; ++ch)
         for (int kb = 0; kb < kblocks; ++kb) {
-          // the MMA warp must have released this stage (previous round) before Z is rewritten
-          if (!mbar_wait(&ctl->empty[stage], phase ^ 1, abort_w)) {
-            atomicExch(err, 36);
-            ctl->abort_w = 1;
+          const int zb = nz & 1;
+          const short2 ee = tab[kb * 8 + c8];
+          // the MMA warp must have released this block before Z is rewritten
+          if (!mbar_wait(&ctl->zempty[zb], ((nz >> 1) & 1) ^ 1, abort_w)) {
+            give_up(36);
             ok = false;
             break;
           }
-          // Z chunks: (row i, 8-pair chunk c8); 8 consecutive threads share row i
-          for (int ch = tid_b; ch < BM * 8; ch += NBUILD * 32) {
-            const int i = ch >> 3, c8 = ch & 7;
-            const short2 ee = tab[kb * 8 + c8];
+          ++nz;
+          unsigned char* z = sm + zb * NT * Z_BYTES;
+#pragma unroll 4
+          for (int i = tid_b >> 3; i < NT * BM; i += NBUILD * 4) {
             uint4 zv = make_uint4(0, 0, 0, 0);
             if (ee.x >= 0) {
               const __nv_bfloat16 xe = *reinterpret_cast<const __nv_bfloat16*>(
@@ -2062,89 +2098,126 @@ __global__ void __launch_bounds__(256, 1)
 #pragma unroll
               for (int h = 0; h < 4; ++h) z2[h] = __hmul2(x2e, a2[h]);
             }
-            *reinterpret_cast<uint4*>(sm + stage * STAGE_BYTES + i * 128 + ((c8 ^ (i & 7)) << 4)) = zv;
+            *reinterpret_cast<uint4*>(z + i * 128 + ((c8 ^ (i & 7)) << 4)) = zv;
           }
           fence_async_smem();
           __syncwarp();
-          if (lane == 0) mbar_arrive(&ctl->zfull[stage]);
-          if (++stage == STAGES) {
-            stage = 0;
-            phase ^= 1;
-          }
+          if (lane == 0) mbar_arrive(&ctl->zfull[zb]);
         }
-        if (!ok) break;
-        if (warp >= 4) {
-          const int q = warp & 3;
-          if (!mbar_wait(&ctl->tfull, acc_phase, abort_w)) {
-            atomicExch(err, 37);
-            ctl->abort_w = 1;
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const int64_t row = (int64_t)mt * BM + q * 32 + lane;    // pool index
-          const float* hrow = Ha + (m + (row < n ? row : 0)) * c;
-          for (int cc = 0; cc < 128; cc += 32) {
-            float q1[32], q2[32];
-            tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + cc, q1);
-            tmem_ld32(tmem + ((uint32_t)(q * 32) << 16) + 128 + cc, q2);
-            if (row < n) {
-#pragma unroll
-              for (int t = 0; t < 32; ++t) {
-                const int k = kc * 128 + cc + t;
-                if (k < c) {
-                  const double hv = (double)hrow[k];
-                  const double wk = hv * (1.0 - hv);
-                  score += wk * (double)q1[t] / (1.0 + eta * wk * (double)q2[t]);
-                }
-              }
-            }
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0) mbar_arrive(&ctl->tempty);
-          if (kc == n_kc - 1) {   // the chain's score is complete: masked running argmax
-            const int64_t row = (int64_t)mt * BM + q * 32 + lane;
-            if (row < n && !mask[ce * rc.mask_stride + row] && score == score &&
-                (score > best[ce] || (score == best[ce] && row < besti[ce]))) {
-              best[ce] = score;
-              besti[ce] = row;
-            }
-          }
-        }
-        acc_phase ^= 1;
-      }
       __syncwarp();
       if (lane == 0) mbar_arrive(&ctl->xempty);
     }
-    if (warp >= 4) {
-      for (int e = 0; e < rc.n; ++e) {
-        double bv = best[e];
-        long long bix = besti[e];
-        for (int o = 16; o > 0; o >>= 1) {
-          const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
-          const long long oi = __shfl_xor_sync(0xffffffffu, bix, o);
-          if (ov > bv || (ov == bv && oi < bix)) {
-            bv = ov;
-            bix = oi;
+  } else if (warp >= 8) {
+    // ---------------- epilogue
+    const int et = (warp - 8) >> 2, q = warp & 3;
+    const uint32_t lanes = (uint32_t)(q * 32) << 16;
+    uint32_t na = 0;
+    bool ok = true;
+    double best[RC_MAX];
+    long long besti[RC_MAX];
+#pragma unroll
+    for (int e = 0; e < RC_MAX; ++e) {
+      best[e] = -INFINITY;
+      besti[e] = LLONG_MAX;
+    }
+    // relative error of the f32 score: 16 roundings a term, c terms (unit 2^-24)
+    const float feps = (float)(c + 40) * 6.0e-8f;
+    for (int64_t mt = blockIdx.x; mt < n_it && ok && !*abort_w; mt += gridDim.x) {
+      const int64_t row = (mt * NT + et) * BM + q * 32 + lane;    // pool index
+      const float* hrow = Ha + (m + (row < n ? row : 0)) * c;
+      double score = 0.0;   // this point's eq. 14 sum over class chunks
+      for (int ch = 0; ch < n_ch && ok; ++ch) {
+        const int ce = ch / n_kc, kc = ch - ce * n_kc;   // chain, class chunk
+        const double eta = rc.eta[ce];
+        if (kc == 0) score = 0.0;
+        const bool open = row < n && !mask[ce * rc.mask_stride + row];
+        const int ab = na % NACC;
+        const uint32_t col = tmem + lanes + ab * BN + et * BN;
+        if (!mbar_wait(&ctl->tfull[ab], (na / NACC) & 1, abort_w)) {
+          give_up(37);
+          ok = false;
+          break;
+        }
+        ++na;
+        tc_fence_after();
+        const int kn = min(128, c - kc * 128);
+        bool need = open;
+        if (n_kc == 1) {
+          // f32 score and its bound.  Terms with 1 + t far from rounding noise only (t > -1/4, not
+          // huge); anything else, and what is not finite, takes the FP64 sum.
+          const float etaf = (float)eta;
+          float s32 = 0.0f, sa = 0.0f, tlo = 0.0f, thi = 0.0f;
+          for (int cc = 0; cc < kn; cc += 16) {
+            float q1[16], q2[16];
+            tmem_ld16(col + cc, q1);
+            tmem_ld16(col + 128 + cc, q2);
+#pragma unroll
+            for (int t = 0; t < 16; ++t) {
+              if (cc + t < kn) {
+                const float h = hrow[cc + t], w = h * (1.0f - h);
+                const float tt = etaf * w * q2[t];
+                const float v = __fdividef(w * q1[t], 1.0f + tt);
+                tlo = fminf(tlo, tt);
+                thi = fmaxf(thi, tt);
+                s32 += v;
+                sa += fabsf(v);
+              }
+            }
+          }
+          const float ub = __fadd_ru(s32, __fadd_ru(__fmul_ru(feps, sa), 1e-30f));
+          const float thr = key_float(*(volatile int*)&ctl->thr[ce]);
+          need = open && (!(ub < thr) || !(sa < 1e37f) || tlo < -0.25f || thi > 1e30f);
+        }
+        if (__any_sync(0xffffffffu, need)) {
+          for (int cc = 0; cc < kn; cc += 16) {
+            float q1[16], q2[16];
+            tmem_ld16(col + cc, q1);
+            tmem_ld16(col + 128 + cc, q2);
+            if (need) {
+#pragma unroll
+              for (int t = 0; t < 16; ++t)
+                if (cc + t < kn) round_term(score, hrow[kc * 128 + cc + t], q1[t], q2[t], eta);
+            }
           }
         }
-        if (lane == 0) {
-          ctl->bval[e * 4 + warp - 4] = bv;
-          ctl->bidx[e * 4 + warp - 4] = bix;
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&ctl->tempty[ab]);
+        if (kc == n_kc - 1 && need && score == score) {   // the chain's score: running argmax
+          if (score > best[ce] || (score == best[ce] && row < besti[ce])) {
+            best[ce] = score;
+            besti[ce] = row;
+            if (n_kc == 1) atomicMax(&ctl->thr[ce], float_key(__double2float_rd(score)));
+          }
         }
+      }
+    }
+    for (int e = 0; e < rc.n; ++e) {
+      double bv = best[e];
+      long long bix = besti[e];
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const long long oi = __shfl_xor_sync(0xffffffffu, bix, o);
+        if (ov > bv || (ov == bv && oi < bix)) {
+          bv = ov;
+          bix = oi;
+        }
+      }
+      if (lane == 0) {
+        ctl->bval[e * 8 + warp - 8] = bv;
+        ctl->bidx[e * 8 + warp - 8] = bix;
       }
     }
   }
   __syncthreads();
   if (threadIdx.x < rc.n) {
     const int e = threadIdx.x;
-    double b = ctl->bval[e * 4];
-    long long bi = ctl->bidx[e * 4];
-    for (int w = 1; w < 4; ++w)
-      if (ctl->bval[e * 4 + w] > b || (ctl->bval[e * 4 + w] == b && ctl->bidx[e * 4 + w] < bi)) {
-        b = ctl->bval[e * 4 + w];
-        bi = ctl->bidx[e * 4 + w];
+    double b = ctl->bval[e * 8];
+    long long bi = ctl->bidx[e * 8];
+    for (int w = 1; w < 4 * NT; ++w)
+      if (ctl->bval[e * 8 + w] > b || (ctl->bval[e * 8 + w] == b && ctl->bidx[e * 8 + w] < bi)) {
+        b = ctl->bval[e * 8 + w];
+        bi = ctl->bidx[e * 8 + w];
       }
     part_val[e * gridDim.x + blockIdx.x] = b;
     part_idx[e * gridDim.x + blockIdx.x] = bi;
@@ -2152,14 +2225,15 @@ __global__ void __launch_bounds__(256, 1)
   if (warp == 1) {
     __syncwarp();
     tc_fence_after();
-    tmem_dealloc(tmem, 256);
+    tmem_dealloc(tmem, 512);
   }
 }
 
 // M~ rows for one Round iteration: row (kc, which, kk) = M_{which, k} symmetric pair weights
-// at pair p of the 8-aligned table (0 where e' < e or beyond d), bf16 hi and lo
+// at pair p of the 8-aligned table (0 where e' < e or beyond d), bf16: per 32 pairs, their hi
+// values and then their lo values (one 128-byte row of a product's operand)
 template <class T>
-__global__ void k_round_mpairs(bf16* Mh, bf16* Ml, const T* M1, const T* M2, const short2* tab,
+__global__ void k_round_mpairs(bf16* Mp, const T* M1, const T* M2, const short2* tab,
                                int c, int d, int kpad, int n_kc) {
   const int row = blockIdx.x;                 // (chain * n_kc + kc)*256 + which*128 + kk
   const int ce = row / (n_kc * 256), kc = (row / 256) % n_kc, which = (row / 128) & 1,
@@ -2173,8 +2247,9 @@ __global__ void k_round_mpairs(bf16* Mh, bf16* Ml, const T* M1, const T* M2, con
     if (k < c && e >= 0 && e2 < d && e2 >= e)
       v = e == e2 ? (float)M[e * d + e] : (float)(M[e * d + e2] + M[e2 * d + e]);
     const bf16 hi = __float2bfloat16_rn(v);
-    Mh[(int64_t)row * kpad + p] = hi;
-    Ml[(int64_t)row * kpad + p] = __float2bfloat16_rn(v - __bfloat162float(hi));
+    bf16* o = Mp + ((int64_t)row * kpad + (p & ~31)) * 2 + (p & 31);
+    o[0] = hi;
+    o[32] = __float2bfloat16_rn(v - __bfloat162float(hi));
   }
 }
 
@@ -3435,17 +3510,14 @@ static int32_t tc_round_scores_t(firal_problem* P, const float* M1, const float*
   const int rows = n_chain * n_kc * BN;
   const size_t mbytes = (size_t)rows * kpad * 2;
   FIRAL_TRY(P->rM.ensure(2 * mbytes));
-  bf16* Mh = P->rM.as<bf16>();
-  bf16* Ml = Mh + mbytes / 2;
+  bf16* Mp = P->rM.as<bf16>();
   ProfScope ps(st, PF_ROUND);
   count_launch(2);
-  k_round_mpairs<float><<<rows, 256, 0, st>>>(Mh, Ml, M1, M2, P->rtab.as<short2>(), c, d, kpad,
-                                              n_kc);
+  k_round_mpairs<float><<<rows, 256, 0, st>>>(Mp, M1, M2, P->rtab.as<short2>(), c, d, kpad, n_kc);
   FIRAL_CUDA_TRY(cudaGetLastError());
-  CUtensorMap mX, mMh, mMl;
+  CUtensorMap mX, mM;
   FIRAL_TRY(make_map(&mX, P->Xb.p, P->Np, DP, BM, DP, false));
-  FIRAL_TRY(make_map(&mMh, Mh, (uint64_t)rows, kpad, BN, BK, true));
-  FIRAL_TRY(make_map(&mMl, Ml, (uint64_t)rows, kpad, BN, BK, true));
+  FIRAL_TRY(make_map(&mM, Mp, (uint64_t)rows, 2 * kpad, BN, 64, true));
   RoundChains rc{};
   rc.n = n_chain;
   rc.mask_stride = P->n;
@@ -3453,15 +3525,28 @@ static int32_t tc_round_scores_t(firal_problem* P, const float* M1, const float*
   static bool attr[4] = {false, false, false, false};
   const int ai = DP == 16 ? 0 : DP == 32 ? 1 : DP == 64 ? 2 : 3;
   if (!attr[ai]) {
-    FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_tc_round<DP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        L<DP>::SMEM));
+    FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_tc_round<DP, 1>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        L<DP, 1>::SMEM));
+    FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_tc_round<DP, 2>,
+                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                        L<DP, 2>::SMEM));
     attr[ai] = true;
   }
-  const int n_mt = (int)((P->n + BM - 1) / BM);
-  const int grid = std::min(n_mt, sms);
-  k_tc_round<DP><<<grid, 256, L<DP>::SMEM, st>>>(mX, mMh, mMl, P->rtab.as<short2>(),
-                                                  P->Ha.as<float>(), mask, P->m, P->n, c, n_kc,
-                                                  kblocks, rc, pv, pi, tc_error_word(P));
+  // Two tiles an item once one each does not cover the points (a second round of one-tile items
+  // costs more than the wider item), and only with one class chunk: the FP64 sums of several
+  // chunks need the second accumulator to run beside the products.
+  const int64_t n_mt = (P->n + BM - 1) / BM;
+  const bool pair = n_kc == 1 && n_mt > sms;
+  const int grid = (int)std::min<int64_t>(pair ? (n_mt + 1) / 2 : n_mt, sms);
+  if (pair)
+    k_tc_round<DP, 2><<<grid, L<DP, 2>::THREADS, L<DP, 2>::SMEM, st>>>(
+        mX, mM, P->rtab.as<short2>(), P->Ha.as<float>(), mask, P->m, P->n, c, n_kc, kblocks, rc,
+        pv, pi, tc_error_word(P));
+  else
+    k_tc_round<DP, 1><<<grid, L<DP, 1>::THREADS, L<DP, 1>::SMEM, st>>>(
+        mX, mM, P->rtab.as<short2>(), P->Ha.as<float>(), mask, P->m, P->n, c, n_kc, kblocks, rc,
+        pv, pi, tc_error_word(P));
   FIRAL_CUDA_TRY(cudaGetLastError());
   *np_out = grid;
   return FIRAL_OK;

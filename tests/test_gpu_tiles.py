@@ -28,6 +28,59 @@ def dev(a):
     return torch.from_numpy(np.ascontiguousarray(a)).cuda()
 
 
+# one tile per item up to 152 tiles of 128 points, two beyond; a last item of one tile, of one
+# point, and full; several class chunks (c > 128) keep one tile; one chunk exactly full
+@pytest.mark.parametrize("n,d,c", [(19456, 16, 5), (19457, 16, 5), (19585, 12, 7), (38912, 16, 3),
+                                   (38913, 20, 4), (20000, 8, 130), (19500, 8, 128), (1, 16, 4),
+                                   (129, 70, 6)])
+def test_round_scores_over_item_shapes(api, handle, n, d, c):
+    """First picks against the FP64 oracle where its top-1/top-2 gap exceeds 1e-3, as in the mixed
+    Round tests; otherwise a near tie.  The reported point must also be unselected."""
+    p = make_problem(n, d, c, seed=n % 97 + d, x_dtype="bf16", h_dtype="float32")
+    b = min(3, n)
+    prob = api.Problem(handle, dev(p.X).to(torch.bfloat16), dev(p.h),
+                       dev(p.Xo).to(torch.bfloat16), dev(p.ho), p.lam, precision="mixed")
+    z = np.full(n, float(b) / n)
+    ref, info = approx.round_select(p, z, b, record=True)
+    sel = prob.round(dev(z.astype(np.float32)), b)[0].cpu().tolist()
+    assert len(set(sel)) == b and min(sel) >= 0 and max(sel) < n
+    for t in range(b):
+        if sel[t] == ref[t]:
+            continue
+        sc = info["scores"][t]
+        assert info["gap"][t] <= 1e-3, (t, sel, ref)
+        assert sc[sel[t]] >= sc[ref[t]] - 1e-3 * abs(sc[ref[t]]), (t, sc[sel[t]], sc[ref[t]])
+        break
+
+
+def test_round_ties_take_the_lowest_index(api, handle):
+    """Equal points have equal scores, bit for bit: the first of them wins wherever the two lie
+    (other tile of the item, other item, other block), although the f32 bound skips most FP64
+    sums."""
+    p = make_problem(25000, 16, 6, seed=5, x_dtype="bf16", h_dtype="float32")
+    X, h = dev(p.X).to(torch.bfloat16), dev(p.h)
+    z = torch.full((p.n,), 1.0 / p.n, dtype=torch.float32, device="cuda")
+
+    def first():
+        prob = api.Problem(handle, X, h, dev(p.Xo).to(torch.bfloat16), dev(p.ho), p.lam,
+                           precision="mixed")
+        s = prob.round(z, 1)[0].cpu().tolist()[0]
+        prob.close()
+        return s
+
+    best = first()
+    for j in (best + 128, best + 129, best + 256, 24999, 3):
+        j %= p.n
+        if j == best:
+            continue
+        keep = X[j].clone(), h[j].clone()
+        X[j], h[j] = X[best], h[best]
+        # the duplicate moves Sigma by one row in 25,000: the pair stays on top of the others by
+        # its gap, and of the pair the lower index wins
+        assert first() in (min(best, j),), (best, j)
+        X[j], h[j] = keep
+
+
 @pytest.mark.parametrize("x_dtype,h_dtype", [("bf16", "float32"), ("float32", "float64"),
                                              ("float64", "float32")])
 def test_pooled_rows_from_every_storage_type(api, handle, x_dtype, h_dtype):
