@@ -81,6 +81,27 @@ def test_round_ties_take_the_lowest_index(api, handle):
         X[j], h[j] = keep
 
 
+@pytest.mark.parametrize("d", [56, 57, 63, 64, 112, 113, 126, 128])
+@pytest.mark.parametrize("n,c", [(700, 5), (5003, 9)])
+def test_ordered_blocks_padded_tile(api, handle, n, c, d):
+    """B_k alone (the ordered sums) on either side of the padded tiles' range: f32 sums of n terms,
+    each with three roundings, against float64 (bound n 2^-24 on the terms' absolute sum)."""
+    p = make_problem(n, d, c, seed=d, x_dtype="float32", h_dtype="float32")
+    prob = api.Problem(handle, dev(p.X), dev(p.h), dev(p.Xo), dev(p.ho), p.lam, precision="fp32")
+    g = torch.Generator(device="cuda").manual_seed(d)
+    z = torch.rand(n, generator=g, device="cuda", dtype=torch.float32)
+    B = prob.precond_blocks(z)
+    B = (B if torch.is_tensor(B) else B[0]).double().cpu().numpy().reshape(c, d, d)
+    X = np.concatenate([p.Xo, p.X]).astype(np.float32).astype(np.float64)
+    h = np.concatenate([p.ho, p.h]).astype(np.float32).astype(np.float64)
+    w = np.concatenate([np.ones(len(p.Xo)), z.double().cpu().numpy()])
+    for k in range(c):
+        a = w * h[:, k] * (1 - h[:, k])
+        ref = (X * a[:, None]).T @ X + p.lam * np.eye(d)
+        mag = (np.abs(X) * a[:, None]).T @ np.abs(X) + p.lam * np.eye(d)
+        assert np.all(np.abs(B[k] - ref) <= (len(w) + 8) * 2.0 ** -24 * mag), k
+
+
 @pytest.mark.parametrize("x_dtype,h_dtype", [("bf16", "float32"), ("float32", "float64"),
                                              ("float64", "float32")])
 def test_pooled_rows_from_every_storage_type(api, handle, x_dtype, h_dtype):
