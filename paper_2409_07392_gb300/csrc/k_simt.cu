@@ -141,8 +141,8 @@ int32_t copy_rows(bool dbl, void* dst, const void* a, int64_t ma, const void* b,
 // elsewhere).  One pass that writes every element of X and h once: no zero fill, no stacked copy
 // of the inputs in their own type.  Bound by the writes of h (N x C, of which a pool's columns
 // are a few percent).  A warp takes 8 consecutive rows; its entry is found by bisection.
-// Stacking and copying 64 pools of 1.3 M rows, 3 groups of up to 400 classes (3.2 GB of h): 6.3 ms
-// as fills, 2-D copies and a copy; 0.43 ms here (7.6 TB/s).
+// Stacking and copying 64 pools of 1.4 M rows, 3 groups of up to 410 classes (1.7 GB of h, 0.3 of x):
+// 6.3 ms as fills, 2-D copies and a copy; 0.43 ms here (4.5 TB/s written).
 constexpr int STACK_RW = 8;
 template <class T, class Tx, class Th>
 __global__ void __launch_bounds__(256) k_stack_rows(T* __restrict__ X, T* __restrict__ H,

@@ -3572,14 +3572,14 @@ int32_t tc_round_scores(firal_problem* P, const void* M1, const void* M2, const 
 // pool's c_q classes, direction P~ with the pool's class means removed):
 //   a_ikj = x_i . P~_j[:, k]                      MMA1: 128 rows x (probe, class), K = features
 //   alpha_ij = sum_k h_ik a_ikj,   psi_ikj = w_i h_ik (a_ikj - alpha_ij)     f32, CUDA cores
-//   out_j[:, k] += sum_i psi_ikj x_i              MMA2: features x (probe, class), K = rows
+//   out_j[:, k] += sum_i psi_ikj x_i              MMA2: (probe, class) x features, K = rows
 // P~ and psi enter as bf16 hi + lo (x is exact in bf16), so both products carry about 2^-17
 // relative rounding, and nothing cancels: each psi is the row's own contribution.  Column
 // (probe j, class k) is j cpad + k, cpad = the pool's class count rounded up to 8, 16 or 32,
 // so one 32-column TMEM load holds whole probes; a probe group of at most 128 columns is one
-// unit of work, so a pool with cpad s > 128 runs as several groups.  MMA2 takes x^T (the
-// staged x^T tile, K-major, 128 rows of which the first dp are features) and psi as an
-// MN-major operand, so each epilogue thread writes its row's psi values as 16-byte runs.
+// unit of work, so a pool with cpad s > 128 runs as several groups.  MMA2 takes psi as an
+// MN-major operand, so each epilogue thread writes its row's psi values as 16-byte runs, and the
+// staged x^T tile (K-major, dp rows).
 // Work list: segments of at most SEG_TILES 128-row tiles of one pool's rows (its labelled
 // rows and its pool rows are separate segments); an item is one probe group of a segment, and
 // the host deals the items to the CTAs longest first (sched: per-CTA offsets, then items as
@@ -3718,20 +3718,68 @@ struct PwEpi {
   int s, sp, d;
 };
 
+// An item whose D accumulator is still to be written out: where its partial rows go
+struct PwOut {
+  uint32_t item;
+  int sgw, cq, cpad, grp, nc;
+};
+
+// D of a finished item -> its partial rows, [class][probe][feature]; the thread holds column i
+// (its TMEM lane) and a half of the features.  False when the wait gave up.
+template <int DP>
+__device__ __forceinline__ bool pw_write_item(const PwEpi& E, const PwOut& o) {
+  using namespace pw_cfg;
+  const int db = o.item & 1;
+  if (!mbar_wait(&E.ctl->d_full[db], (o.item >> 1) & 1, E.abort_w)) {
+    E.ctl->abort_w = 1;
+    atomicExch(E.err, 48);
+    return false;
+  }
+  tc_fence_after();
+  constexpr int NF = DP == 16 ? 16 : DP / 2;   // features per thread
+  const int e0 = E.half * NF;
+  if (DP > 16 || E.half == 0) {
+    float v[NF];
+    const uint32_t a = E.tmem + E.lanes + TD + db * NU + e0;
+    if (NF == 32) tmem_ld32(a, v);
+    else tmem_ld16(a, v);
+    const int jl = E.i / o.cpad, kl = E.i - jl * o.cpad;
+    const int j = o.grp * (NU / o.cpad) + jl;
+    if (E.i < o.nc && kl < o.cq && j < E.s) {
+      float* p = E.part + ((int64_t)(o.sgw + kl) * E.sp + j) * E.d + e0;
+      const int ne = E.d - e0;
+      if ((E.d & 3) == 0) {
+#pragma unroll
+        for (int t = 0; t < NF; t += 4)
+          if (t < ne)
+            *reinterpret_cast<float4*>(p + t) = make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
+      } else if ((E.d & 1) == 0) {
+#pragma unroll
+        for (int t = 0; t < NF; t += 2)
+          if (t < ne) *reinterpret_cast<float2*>(p + t) = make_float2(v[t], v[t + 1]);
+      } else {
+#pragma unroll
+        for (int t = 0; t < NF; ++t)
+          if (t < ne) p[t] = v[t];
+      }
+    }
+  }
+  tc_fence_before();
+  __syncwarp();
+  if (E.lane == 0) mbar_arrive(&E.ctl->d_empty[db]);
+  return true;
+}
+
 // One work item (segment sg of pool pq, probe group grp of nc columns) of the epilogue, with
-// the pool's classes padded to CPAD: per tile, psi into the MN-major operand; at the end, the
-// item's partial rows from the D accumulator.  u counts the units seen; false when a wait gave
-// up (the abort word and the error word are set).
+// the pool's classes padded to CPAD: per tile, psi into the MN-major operand; after the first
+// tile, the previous item's D (prev), whose last product has passed by then.  u counts the units
+// seen; false when a wait gave up (the abort word and the error word are set).
 template <int CPAD, int DP>
-__device__ __forceinline__ bool pw_epi_item(const PwEpi& E, uint32_t& u, uint32_t item,
-                                            const int4& sg, const int4& pq, int grp, int nc) {
+__device__ __forceinline__ bool pw_epi_item(const PwEpi& E, uint32_t& u, const int4& sg,
+                                            const int4& pq, int nc, const PwOut* prev) {
   using namespace pw_cfg;
   const int i = E.i, lane = E.lane, cq = pq.y;
   const int t0 = sg.y >> 7, t1 = (sg.z - 1) >> 7;
-  auto give_up = [&](int code) {
-    E.ctl->abort_w = 1;
-    atomicExch(E.err, code);
-  };
   float hn[CPAD], wn;
   {
     const int64_t row = (int64_t)t0 * 128 + i;
@@ -3751,18 +3799,33 @@ __device__ __forceinline__ bool pw_epi_item(const PwEpi& E, uint32_t& u, uint32_
     const uint32_t ph = (u >> 1) & 1;
     if (!mbar_wait(&E.ctl->s_full[b], ph, E.abort_w) ||
         !mbar_wait(&E.ctl->psi_empty[b], ph ^ 1, E.abort_w)) {
-      give_up(47);
+      E.ctl->abort_w = 1;
+      atomicExch(E.err, 47);
       return false;
     }
     ++u;
     tc_fence_after();
     unsigned char* psi_row = E.sm + OFF_PSI + b * PSI_BUF + i * 128;
-    for (int ch = E.half; ch < nc / 32; ch += 2) {
-      uint32_t ra[32];
-      tmem_ld32_async(E.tmem + E.lanes + TS + b * NU + ch * 32, ra);
+    const uint32_t ta = E.tmem + E.lanes + TS + b * NU;
+    const int ch = E.half, ch2 = ch + 2;   // the thread's 32-column chunks
+    auto put = [&](const uint32_t (&r)[32], int c0) {
+      unsigned char* hi = psi_row + (c0 >> 1) * PSI_ATOM;   // 64-column atom of the chunk
+      pw_psi_chunk<CPAD>(r, wh2, winv, hi, hi + 2 * PSI_ATOM, (c0 & 1) * 4, i & 7);
+    };
+    if (CPAD <= 16 && ch2 < nc / 32) {   // both loads in flight (CPAD = 32: no registers for it)
+      uint32_t ra[32], rb[32];
+      tmem_ld32_async(ta + ch * 32, ra);
+      tmem_ld32_async(ta + ch2 * 32, rb);
       tmem_wait_ld();
-      unsigned char* hi = psi_row + (ch >> 1) * PSI_ATOM;   // 64-column atom of the chunk
-      pw_psi_chunk<CPAD>(ra, wh2, winv, hi, hi + 2 * PSI_ATOM, (ch & 1) * 4, i & 7);
+      put(ra, ch);
+      put(rb, ch2);
+    } else {
+      for (int c0 = ch; c0 < nc / 32; c0 += 2) {
+        uint32_t ra[32];
+        tmem_ld32_async(ta + c0 * 32, ra);
+        tmem_wait_ld();
+        put(ra, c0);
+      }
     }
     tc_fence_before();
     fence_async_smem();
@@ -3771,37 +3834,8 @@ __device__ __forceinline__ bool pw_epi_item(const PwEpi& E, uint32_t& u, uint32_
       mbar_arrive(&E.ctl->s_empty[b]);
       mbar_arrive(&E.ctl->psi_full[b]);
     }
+    if (t == t0 && prev && !pw_write_item<DP>(E, *prev)) return false;
   }
-  // item end: D -> the item's partial rows, [class][probe][feature]; the thread holds feature
-  // e (its TMEM lane) of the columns of its half
-  const int db = item & 1;
-  if (!mbar_wait(&E.ctl->d_full[db], (item >> 1) & 1, E.abort_w)) {
-    give_up(48);
-    return false;
-  }
-  tc_fence_after();
-  {
-    constexpr int LC = CPAD == 8 ? 3 : CPAD == 16 ? 4 : 5;
-    const int e = i;
-    for (int c0 = E.half * 64; c0 < E.half * 64 + 64; c0 += 32) {
-      if (c0 >= nc) break;
-      uint32_t v[32];
-      tmem_ld32_async(E.tmem + E.lanes + TD + db * NU + c0, v);
-      tmem_wait_ld();
-      if (e < E.d) {
-#pragma unroll
-        for (int t = 0; t < 32; ++t) {
-          const int col = c0 + t, jl = col >> LC, kl = col - (jl << LC);
-          const int j = grp * (NU >> LC) + jl;
-          if (kl < cq && j < E.s)
-            E.part[((int64_t)(sg.w + kl) * E.sp + j) * E.d + e] = __uint_as_float(v[t]);
-        }
-      }
-    }
-  }
-  tc_fence_before();
-  __syncwarp();
-  if (lane == 0) mbar_arrive(&E.ctl->d_empty[db]);
   return true;
 }
 
@@ -3919,9 +3953,8 @@ __global__ void __launch_bounds__(384, 1)
     struct Pend {
       uint32_t u, item;
       bool first, last;
-      int nc;
     };
-    Pend pend{0, 0, false, false, 0};
+    Pend pend{0, 0, false, false};
     bool have = false;
     uint32_t nt = 0, ni = 0;
     bool ok = true;
@@ -3932,21 +3965,22 @@ __global__ void __launch_bounds__(384, 1)
           (p.first && !mbar_wait(&ctl->d_empty[db], ((p.item >> 1) & 1) ^ 1, abort_w)))
         return false;
       tc_fence_after();
-      // D (lanes = features, columns = the unit's (probe, class) columns) += x^T psi:
-      // A = the x^T tile (K-major; rows past dp are not features and their D rows are unused),
-      // B = psi (MN-major: rows = the tile's rows, 64-column atoms 16 KB apart)
+      // D (lanes = the unit's (probe, class) columns, columns = features) += psi^T x:
+      // A = psi (MN-major: rows = the tile's rows, 64-column atoms 16 KB apart; columns past nc
+      // are stale and their D lanes unused), B = the x^T tile (K-major, DP rows): N = DP, where the
+      // features as M would fill 128 lanes with at most 64 of them
       const uint32_t ps = smem_u32(sm + OFF_PSI + b * PSI_BUF),
                      xt = smem_u32(sm + OFF_XT + b * XT_BYTES);
-      const uint32_t idesc2 = idesc_bf16_f32_bmn(128, p.nc);
+      constexpr uint32_t idesc2 = idesc_bf16_f32_amn(128, DP);
 #pragma unroll
       for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const uint64_t ad = sdesc_sw128(xt + kb * DP * 128 + k * 32);
-          const uint32_t b0 = ps + (kb * 64 + k * 16) * 128;
+          const uint64_t xd = sdesc_sw128(xt + kb * DP * 128 + k * 32);
+          const uint32_t a0 = ps + (kb * 64 + k * 16) * 128;
           const uint32_t acc = (p.first && kb == 0 && k == 0) ? 0u : 1u;
-          umma_bf16(tmem + TD + db * NU, ad, sdesc_sw128_mn(b0, PSI_ATOM), idesc2, acc);
-          umma_bf16(tmem + TD + db * NU, ad, sdesc_sw128_mn(b0 + 2 * PSI_ATOM, PSI_ATOM), idesc2,
+          umma_bf16(tmem + TD + db * NU, sdesc_sw128_mn(a0, PSI_ATOM), xd, idesc2, acc);
+          umma_bf16(tmem + TD + db * NU, sdesc_sw128_mn(a0 + 2 * PSI_ATOM, PSI_ATOM), xd, idesc2,
                     1u);
         }
       umma_commit(&ctl->psi_empty[b]);
@@ -3982,7 +4016,7 @@ __global__ void __launch_bounds__(384, 1)
         if (t == t1) umma_commit(&ctl->pt_empty);
         ++nt;
         if (have && !mma2(pend)) { give_up(46); ok = false; break; }
-        pend = Pend{u, item, t == t0, t == t1, nc};
+        pend = Pend{u, item, t == t0, t == t1};
         have = true;
       }
     }
@@ -3996,16 +4030,19 @@ __global__ void __launch_bounds__(384, 1)
                   lane, abort_w, err, HaT, w, part, N, s, sp, d};
     uint32_t u = 0, ni = 0;
     bool ok = true;
+    PwOut out{};
     for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
       const int code = sched[gridDim.x + 1 + it], grp = code & (GRP_MAX - 1);
       const int4 sg = seg_tab[code / GRP_MAX];
       const int4 pq = pool_tab[sg.x];
       const int nc = pw_ncols(pq.z, sp, grp);
-      const uint32_t item = ni++;
-      if (pq.z == 8) ok = pw_epi_item<8, DP>(E, u, item, sg, pq, grp, nc);
-      else if (pq.z == 16) ok = pw_epi_item<16, DP>(E, u, item, sg, pq, grp, nc);
-      else ok = pw_epi_item<32, DP>(E, u, item, sg, pq, grp, nc);
+      const PwOut* prev = ni ? &out : nullptr;
+      if (pq.z == 8) ok = pw_epi_item<8, DP>(E, u, sg, pq, nc, prev);
+      else if (pq.z == 16) ok = pw_epi_item<16, DP>(E, u, sg, pq, nc, prev);
+      else ok = pw_epi_item<32, DP>(E, u, sg, pq, nc, prev);
+      out = PwOut{ni++, sg.w, pq.y, pq.z, grp, nc};
     }
+    if (ok && ni && !*abort_w) pw_write_item<DP>(E, out);
   }
   __syncthreads();
   if (warp == 2) {
@@ -4082,18 +4119,17 @@ __global__ void __launch_bounds__(PWF_THREADS) k_pw_finish(float* out, const flo
     const int64_t o = (int64_t)j * D + (int64_t)(pt.x + kl) * d + e;
     float acc = lam * (V[o] - vm[e]);
     // a pool's segments are consecutive: its partial of segment g lies g cq rows after the first;
-    // eight loads in flight, added in segment order
+    // sixteen loads in flight, added in segment order
     const float* ps = part + ((int64_t)((ns ? seg_tab[sr.x].w : 0) + kl) * sp + j) * d + e;
     const int64_t step = (int64_t)cq * sp * d;
-    int g = 0;
-    for (; g + 8 <= ns; g += 8) {
-      float v[8];
+    for (int g = 0; g < ns; g += 16) {
+      float v[16];
 #pragma unroll
-      for (int x = 0; x < 8; ++x) v[x] = ps[(g + x) * step];
+      for (int x = 0; x < 16; ++x) v[x] = g + x < ns ? ps[(g + x) * step] : 0.0f;
 #pragma unroll
-      for (int x = 0; x < 8; ++x) acc += v[x];
+      for (int x = 0; x < 16; ++x)
+        if (g + x < ns) acc += v[x];
     }
-    for (; g < ns; ++g) acc += ps[g * step];
     t[kl * 64 + e] = acc;
   }
   __syncthreads();
@@ -4302,11 +4338,13 @@ static int32_t tc_apply_pw_t(firal_problem* P, const float* w, const float* V, i
   cudaStream_t st = P->H->stream;
   const int c = P->c, d = P->d;
   const int Qe = pool_count(P->pt);
-  FIRAL_TRY(P->vmean.ensure((size_t)s * Qe * d * sizeof(float)));
+  // means and packed rows sized for the gradient's two operands: growing them there frees memory,
+  // which waits for the device
+  FIRAL_TRY(P->vmean.ensure((size_t)2 * s * Qe * d * sizeof(float)));
   FIRAL_TRY(P->qmean.ensure((size_t)s * Qe * d * sizeof(float)));
   const int sp = (s + 7) / 8 * 8;
   const int64_t prows = 2LL * sp * P->pw_cpad_total;
-  FIRAL_TRY(P->pw_pk.ensure((size_t)prows * 64 * 2));
+  FIRAL_TRY(P->pw_pk.ensure((size_t)2 * prows * 64 * 2));
   FIRAL_TRY(P->pw_part.ensure((size_t)std::max<int64_t>(1, P->pw_segcls_total) * sp * d *
                               sizeof(float)));
   {

@@ -220,9 +220,9 @@ __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) |
          ((uint32_t)(M >> 4) << 24);
 }
-// ... with B MN-major (bit 16)
-__host__ __device__ constexpr uint32_t idesc_bf16_f32_bmn(int M, int N) {
-  return idesc_bf16_f32(M, N) | (1u << 16);
+// ... with A MN-major (bit 15)
+__host__ __device__ constexpr uint32_t idesc_bf16_f32_amn(int M, int N) {
+  return idesc_bf16_f32(M, N) | (1u << 15);
 }
 
 // Byte offset of element (row, k) (k < 64) in a 128-byte-swizzled K-major bf16 tile.
