@@ -1,6 +1,7 @@
 // C-ABI entry points (include/firal.h) and host orchestration of the Relax and Round steps.
 #include <algorithm>
 #include <cmath>
+#include <initializer_list>
 #include <map>
 #include <tuple>
 #include <cstdlib>
@@ -105,9 +106,9 @@ ProfScope::~ProfScope() {
 // Buffers of destroyed problems are parked here and handed to later allocations on the same
 // device instead of going back to the driver: freeing a large problem's buffers costs about
 // 20 ms, and a caller that builds one problem per call (firal_relax, firal_round) pays it
-// every time.  Only firal_problem_destroy parks, after synchronising the problem's stream, so
-// a parked block has no kernel in flight; every other release still calls cudaFree (which
-// synchronises the device).  Bounded by FIRAL_CACHE_BYTES (default 64 GiB, 0 disables);
+// every time.  firal_problem_destroy and drop_temps (a call's own buffers) park, after
+// synchronising the stream that used them, so a parked block has no kernel in flight; every other
+// release still calls cudaFree (which synchronises the device).  Bounded by FIRAL_CACHE_BYTES (default 64 GiB, 0 disables);
 // firal_cache_trim returns every parked block.
 namespace {
 struct ParkedBlock {
@@ -219,6 +220,17 @@ void DBuf::park() {
   if (p && !cache_park(p, bytes)) cudaFree(p);
   p = nullptr;
   bytes = 0;
+}
+
+// The end of a call's temporaries, all last used on st: parked once st has drained (freed if it
+// reports an error).  Three pooled problems' stacked z alone took 4.3 ms of cudaFree of the 33 ms
+// of 64 batched pools.
+void drop_temps(cudaStream_t st, std::initializer_list<DBuf*> bufs) {
+  const bool synced = cudaStreamSynchronize(st) == cudaSuccess;
+  for (DBuf* b : bufs) {
+    if (synced) b->park();
+    else b->release();
+  }
 }
 
 // tensor-core entry points (k_tc.cu); return FIRAL_ERR_UNSUPPORTED when not built
@@ -668,10 +680,9 @@ int32_t relax_step_impl(firal_problem* P, const firal_relax_opts* o, int32_t t, 
 // their Cholesky factors, shared by every eta of a sweep.
 struct RoundSetup {
   DBuf Sig, L;
-  ~RoundSetup() {
-    Sig.release();
-    L.release();
-  }
+  cudaStream_t st;
+  explicit RoundSetup(cudaStream_t st_) : st(st_) {}
+  ~RoundSetup() { drop_temps(st, {&Sig, &L}); }
 };
 
 int32_t round_setup(firal_problem* P, const void* zr, RoundSetup& rs) {
@@ -704,9 +715,8 @@ int32_t round_chains(firal_problem* P, const RoundSetup& rs, int32_t b, const do
   const double* L = rs.L.as<double>();
   DBuf Bm, Binv, Hk, M1, M2, eig, nu, mask, pv, pi, score, Tg, Ht, Hot, Sig3;
   auto rel = [&]() {
-    for (DBuf* bf : {&Bm, &Binv, &Hk, &M1, &M2, &eig, &nu, &mask, &pv, &pi, &score, &Tg, &Ht,
-                     &Hot, &Sig3})
-      bf->release();
+    drop_temps(st, {&Bm, &Binv, &Hk, &M1, &M2, &eig, &nu, &mask, &pv, &pi, &score, &Tg, &Ht,
+                    &Hot, &Sig3});
   };
   const int np = (int)std::max<int64_t>((P->n + 127) / 128, P->sms);
   // per chain: tridiagonal forms (2 c d), Gershgorin bounds (2 c), nu's per-SM partials
@@ -810,7 +820,7 @@ int32_t round_impl(firal_problem* P, const void* zr, int32_t b, const firal_roun
   if (sharded(P)) return fail(FIRAL_ERR_UNSUPPORTED, "Round does not take a row-sharded problem");
   if (b < 1 || b > P->n) return fail(FIRAL_ERR_ARG, "budget must be in [1, n]");
   if (P->dbl && P->d > 90) return fail(FIRAL_ERR_UNSUPPORTED, "FP64 Round supports d <= 90");
-  RoundSetup rs;
+  RoundSetup rs(P->H->stream);
   FIRAL_TRY(round_setup(P, zr, rs));
   const double eta = (o && o->eta > 0) ? o->eta : 8.0 * std::sqrt((double)P->D);
   FIRAL_TRY(round_chains(P, rs, b, &eta, 1, sel, stats));
@@ -1098,7 +1108,7 @@ int32_t batched_pooled(firal_handle* H, int32_t nq, const firal_pool* pools,
   std::vector<DBuf> zcat;
   auto destroy_all = [&]() {
     for (auto* p : probs) firal_problem_destroy(p);
-    for (auto& z : zcat) z.release();
+    for (auto& z : zcat) drop_temps(st, {&z});
   };
   int32_t rc = FIRAL_OK;
   for (auto& kv : groups)
@@ -1159,9 +1169,7 @@ int32_t selected_min_eig(firal_problem* P, const int32_t* sel, int32_t b, double
   const size_t blk = (size_t)c * d * d;
   DBuf Hs, Lid, eig;
   auto rel = [&]() {
-    Hs.release();
-    Lid.release();
-    eig.release();
+    drop_temps(st, {&Hs, &Lid, &eig});
   };
   int32_t rc = FIRAL_OK;
   if ((rc = Hs.ensure(blk * 8)) != FIRAL_OK || (rc = Lid.ensure(blk * 8)) != FIRAL_OK ||
@@ -1198,7 +1206,7 @@ int32_t round_sweep_impl(firal_problem* P, const void* zr, int32_t b, const doub
   if (sharded(P)) return fail(FIRAL_ERR_UNSUPPORTED, "Round does not take a row-sharded problem");
   if (P->dbl && P->d > 90) return fail(FIRAL_ERR_UNSUPPORTED, "FP64 Round supports d <= 90");
   // the eta-independent set-up once, then one chain per eta
-  RoundSetup rs;
+  RoundSetup rs(P->H->stream);
   FIRAL_TRY(round_setup(P, zr, rs));
   // the chains of up to 8 values of eta side by side (one score launch per pick for all)
   for (int e0 = 0; e0 < neta; e0 += 8) {
@@ -1336,7 +1344,7 @@ int32_t firal_problem_destroy(firal_problem* P) {
   // every kernel of the problem ran on the handle's stream (graph replays join it before
   // returning): after this synchronisation its buffers can be parked for reuse
   const bool synced = cudaStreamSynchronize(P->H->stream) == cudaSuccess;
-  exact_release(P);
+  exact_release(P, synced);
   for (DBuf* b : {&P->Xa, &P->Ha, &P->HaT, &P->w_sig, &P->w_p, &P->S_p, &P->S_sig, &P->Pblk,
                   &P->Minv, &P->HoBlk, &P->walpha, &P->Dpart, &P->syrk_part, &P->form_part, &P->form_pk, &P->blk_w, &P->cgX, &P->cgR,
                   &P->cgP, &P->cgQ, &P->cgZ, &P->cgcols, &P->cgpart1, &P->cgpart2, &P->V, &P->U,
@@ -1615,7 +1623,7 @@ int32_t firal_block_eigvals(firal_handle* H, int32_t c, int32_t d, const double*
     rc = chol_inv(true, Sig, c, d, nullptr, nullptr, L.as<double>(), not_spd_flag(H), H->stream);
   if (rc == FIRAL_OK) rc = tilde_eigvals(L.as<double>(), Hm, c, d, eig, H->stream);
   if (rc == FIRAL_OK) rc = read_flags(H);
-  L.release();
+  drop_temps(H->stream, {&L});
   return record(H, rc);
 }
 
@@ -1722,7 +1730,7 @@ int32_t lr_fit_impl(firal_handle* H, const void* Xv, const int32_t* y, int64_t m
   const int64_t D = (int64_t)c * d;
   DBuf h, R, g, dW, Wt, ones, part;
   auto rel = [&] {
-    for (DBuf* b : {&h, &R, &g, &dW, &Wt, &ones, &part}) b->release();
+    drop_temps(st, {&h, &R, &g, &dW, &Wt, &ones, &part});
   };
   int32_t rc = FIRAL_OK;
 #define TRYL(x)          \
@@ -1827,7 +1835,7 @@ int32_t al_impl(firal_handle* H, const void* Xp, const int32_t* yp, int64_t n, c
   FIRAL_TRY(labels_in_range(yl0, m, c, st));
   DBuf Xpv, Xl, yl, Xr, hr, hl, W, z, idx, sl;
   auto rel = [&] {
-    for (DBuf* bf : {&Xpv, &Xl, &yl, &Xr, &hr, &hl, &W, &z, &idx, &sl}) bf->release();
+    drop_temps(st, {&Xpv, &Xl, &yl, &Xr, &hr, &hl, &W, &z, &idx, &sl});
   };
   int32_t rc = FIRAL_OK;
 #define TRYA(x)          \
@@ -1930,7 +1938,7 @@ int32_t firal_lr_probs(firal_handle* H, const void* X, int32_t x_dtype, const vo
   if (rc == FIRAL_OK) rc = lr_probs(dbl, Xv.p, W, rows, d, c, h_out, H->stream);
   if (rc == FIRAL_OK && cudaStreamSynchronize(H->stream) != cudaSuccess)
     rc = fail(FIRAL_ERR_CUDA, "lr_probs failed");
-  Xv.release();
+  drop_temps(H->stream, {&Xv});
   return record(H, rc);
 }
 
@@ -1953,7 +1961,7 @@ int32_t firal_lr_fit(firal_handle* H, const void* X, int32_t x_dtype, const int3
                      &gn);
   if (iters_out) *iters_out = it;
   if (gnorm_out) *gnorm_out = gn;
-  Xv.release();
+  drop_temps(H->stream, {&Xv});
   return record(H, rc);
 }
 

@@ -371,7 +371,7 @@ int32_t exact_relax(firal_problem* P, double budget, int T, double beta0, const 
                     void* z, double* hist);
 int32_t exact_round(firal_problem* P, const void* zd, int b, double eta, int exclude,
                     int32_t* sel, double* r_host, double* nu_host, int* evals);
-void exact_release(firal_problem* P);
+void exact_release(firal_problem* P, bool park);   // park: the problem's stream has drained
 int32_t dense_gemm(bool dbl, cudaStream_t st, bool ta, bool tb, int M, int N, int K,
                    double alpha, const void* A, int64_t lda, const void* B, int64_t ldb,
                    double beta, void* C, int64_t ldc);

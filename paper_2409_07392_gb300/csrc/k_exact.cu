@@ -1423,13 +1423,14 @@ int32_t exact_round(firal_problem* P, const void* zd, int b, double eta, int exc
   return round_t<float>(P, (const float*)zd, b, eta, exclude, sel, r_host, nu_host, evals);
 }
 
-void exact_release(firal_problem* P) {
+void exact_release(firal_problem* P, bool park) {
   if (!P->ex) return;
   ExactWs& ex = *P->ex;
-  for (auto& b : ex.m) b.release();
+  auto drop = [park](DBuf& b) { park ? b.park() : b.release(); };
+  for (auto& b : ex.m) drop(b);
   for (DBuf* b : {&ex.pairs, &ex.part, &ex.gpart, &ex.K, &ex.YZ, &ex.negr, &ex.mask, &ex.argp,
                   &ex.flag, &ex.scal})
-    b->release();
+    drop(*b);
   delete P->ex;
   P->ex = nullptr;
 }
