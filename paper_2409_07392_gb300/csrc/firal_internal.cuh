@@ -197,6 +197,7 @@ struct firal_problem {
   bool S_p_ready = false;
   // scratch of the Hessian apply
   firal::DBuf walpha, Dpart, syrk_part;
+  firal::DBuf terms;             // f32 block sums: both operands of some rows of every range
   firal::DBuf form_pk;           // CUDA-core row forms: packed coefficient tiles
   firal::DBuf form_part;         // CUDA-core quadratic forms and scores: per-block row partials
   firal::DBuf blk_w;             // f32 block sums of Round: w h (1 - h) (N x c)

@@ -50,11 +50,9 @@ __device__ __forceinline__ void cp_wait0() { asm volatile("cp.async.wait_group 0
 
 // ------------------------------------------------------------------------------------------
 // k_row_outer: part[split][m][n] = sum over the split's rows of A[i][m] B[i][n]
-//   OP 0 (low-rank part): m = j c + k, A = h_ik walpha_ij; n = e, B = x_ie
-//   OP 2 (Exact-FIRAL):   m = class pair (k, l), A = wsc w_i (delta_kl h_ik - h_ik h_il); n and B
-//                         as OP 1 (f32 only)
-//   OP 1 (block sums):    m = which c + k, A = w_i h_ik (which 0) or w_i h_ik (1 - h_ik)
-//                         (which 1); n = pair (e, f), e <= f, B = x_ie x_if
+//   OP 0 (low-rank part):   m = j c + k, A = h_ik walpha_ij; n = e, B = x_ie
+//   OP 1 (FP64 block sums): m = which c + k, A = w_i h_ik (which 0) or w_i h_ik (1 - h_ik)
+//                           (which 1); n = pair (e, f), e <= f, B = x_ie x_if
 // The tile is GM TM x GN TN outputs, GM GN threads active; rows in steps of BK, the next
 // step's h, x and factors in flight (cp.async) while this one is multiplied.
 // ------------------------------------------------------------------------------------------
@@ -69,8 +67,6 @@ struct OuterArgs {
   int64_t rps;       // rows per split
   int d, c, s;
   int which0;        // OP 1: first output kind (0: w h, 1: w h (1 - h))
-  const int2* pairs; // OP 2: class pairs; w may be null (weights 1), all scaled by wsc
-  float wsc;
   int M, Nn;         // outputs in all
   int GM, GN;
   T* part;
@@ -197,43 +193,38 @@ __global__ __launch_bounds__(512, 1) void k_row_outer_d(const OuterArgs<double> 
   }
 }
 
-// f32: TM x 8 outputs per thread.  Row q of a thread's TM is tile row
+// f32, OP 0: 8 x 8 outputs per thread.  Row q of a thread's 8 is tile row
 // (q / 4) 4 GM + 4 mg + q % 4, column y is (y / 4) 4 GN + 4 ng + y % 4; a warp covers 8 column
 // groups x 4 row groups where GN allows, which is the fewest shared-memory wavefronts.
 // One barrier per step.  A step's multiply-adds run in four quarters; each quarter first reads
-// its share of the next step's operands (h and its factors from global memory, OP 0's x too;
-// OP 1: two rows of pair factors from x in shared memory, and x of the step after from global
-// memory), multiplies, and then writes that share to the other buffer, so that the loads'
-// latency is covered and only one share is held in registers.
+// its share of the next step's operands (h, its factors and x), multiplies, and then writes that
+// share to the other buffer, so that the loads' latency is covered and only one share is held in
+// registers.
 // Bound by issue slots: the multiply-adds alone run at 53-57 TFLOP/s (78 is the part's peak, 65
-// an 8 x 8 outer product from registers), with the operands' loads and stores 43 (low-rank part,
-// n = 21,000, c = 1000, d = 64, s = 16: 1.01 ms, 2.88 before; Round's blocks at n = 1M, d = 128,
-// c = 100: 75 ms, 177 before) and, forming pairs, 29 (block sums, same n, c, d: 3.0 ms, 8.6
-// before).  Staging by cp.async with a separate pass over the tile ran at 31.
+// an 8 x 8 outer product from registers), with the operands' loads and stores 40-43 (n = 21,000,
+// c = 1000, d = 64, s = 16: 1.08 ms, 2.88 before).  Staging by cp.async with a separate pass over
+// the tile ran at 31.
 // VH 4: rows of h and x 16-byte aligned, 16 rows per step; otherwise VH values of h per load
 // (8-byte aligned rows: 2), x by single values, 8 rows per step.
-template <int OP, int VH>
+template <int VH>
 struct OuterCfg {
   static constexpr int BK = VH == 4 ? 16 : 8;
   static constexpr int NI = VH == 4 ? 4 : VH == 2 ? 8 : 12;   // loads of h per thread and step
   static constexpr int VX = VH == 4 ? 4 : 1;
   static constexpr int NX = VH == 4 ? 4 : 8;                  // loads of x per thread and step
 };
-template <int OP, int TM, int VH>
+template <int VH>
 __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a) {
-  using Cfg = OuterCfg<OP, VH>;
-  constexpr int BK = Cfg::BK, NI = Cfg::NI, NX = Cfg::NX, VX = Cfg::VX, TN = 8;
+  using Cfg = OuterCfg<VH>;
+  constexpr int BK = Cfg::BK, NI = Cfg::NI, NX = Cfg::NX, VX = Cfg::VX, TM = 8, TN = 8;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int BM = a.GM * TM, BN = a.GN * TN;
   const int d = a.d, c = a.c;
-  const int dS = OP == 0 ? BN : (d + 3) & ~3;              // staged x row
   const int bm0 = blockIdx.x * BM, bn0 = blockIdx.y * BN;
-  const int j0 = OP == 0 ? bm0 / c : 0;
+  const int j0 = bm0 / c;
   float* As = (float*)smem_raw;                // [2][BK][BM]
   float* Bs = As + 2 * BK * BM;                // [2][BK][BN]
-  float* Xs = Bs + 2 * BK * BN;                // OP 1: [2][BK][dS]
-  int* mcol = (int*)(OP == 0 ? Xs : Xs + 2 * BK * dS);   // [BM] class | (probe or kind) << 16
-  int* nmap = mcol + BM;                       // OP 1: [BN] e | f << 16
+  int* mcol = (int*)(Bs + 2 * BK * BN);        // [BM] class | probe << 16
   const int tid = threadIdx.x, nt = blockDim.x;
   int mg, ng;
   if ((a.GN & 7) == 0) {
@@ -246,26 +237,16 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
   const bool act = mg < a.GM && ng < a.GN;
   for (int q = tid; q < BM; q += nt) {
     const int m = bm0 + q;
-    if (OP == 2)
-      mcol[q] = m < a.M ? a.pairs[m].x | a.pairs[m].y << 16 : -1;
-    else
-      mcol[q] = m < a.M ? (m % c) | ((OP == 0 ? m / c - j0 : m / c + a.which0) << 16) : -1;
+    mcol[q] = m < a.M ? (m % c) | (m / c - j0) << 16 : -1;
   }
-  if (OP != 0)
-    for (int q = tid; q < BN; q += nt) {
-      int e = 0, f = 0;
-      if (bn0 + q < a.Nn) feature_pair(bn0 + q, d, e, f);
-      nmap[q] = bn0 + q < a.Nn ? e | (f << 16) : -1;
-    }
   __syncthreads();
   const int64_t i0 = a.r0 + (int64_t)blockIdx.z * a.rps;
   const int64_t i1 = min(a.r1, i0 + a.rps);
   const int rows = i0 < i1 ? (int)(i1 - i0) : 0;
   const int steps = (rows + BK - 1) / BK;
   const int hw = BM / VH, hn = BK * hw;        // loads of h per row and step
-  const int xw = dS / VX, xn = BK * xw;        // loads of x
-  const int xo = OP == 0 ? bn0 : 0;
-  // the loads' places, fixed over the steps: class | (probe or kind) << 12 | row of the step << 24
+  const int xw = BN / VX, xn = BK * xw;        // loads of x
+  // the loads' places, fixed over the steps: class | probe << 12 | row of the step << 24
   // (-1: none), and the offset of x
   int hp[NI], xp[NX];
 #pragma unroll
@@ -276,7 +257,7 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
 #pragma unroll
   for (int u = 0; u < NX; ++u) {
     const int idx = tid + u * nt, pr = idx / xw, q = (idx - pr * xw) * VX;
-    xp[u] = idx < xn && xo + q < d ? pr * d + q : -1;
+    xp[u] = idx < xn && bn0 + q < d ? pr * d + q : -1;
   }
   constexpr int QI = NI / 4, QX = NX / 4;   // loads per quarter
   float hr[QI][VH], wr[QI], xr[QX][VX];
@@ -284,7 +265,7 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
     const int64_t ib = i0 + (int64_t)t * BK;
     const int lim = min(BK, rows - t * BK);
     const float* H = a.Ha + ib * c;
-    const float* W = OP == 0 ? a.w + ib * a.s + j0 : a.w + ib;
+    const float* W = a.w + ib * a.s + j0;
 #pragma unroll
     for (int v = 0; v < QI; ++v) {
       const int hu = hp[qt * QI + v], pr = hu >> 24;
@@ -305,14 +286,8 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
           hr[v][VH > 1 ? 1 : 0] = r.y;
         } else {
           hr[v][0] = *h;
-          if (OP == 2) {
-            const int l = hu >> 12 & 0xfff;
-            const float hk = *h;
-            hr[v][0] = (l == (hu & 0xfff) ? hk : 0.0f) - hk * H[pr * c + l];
-          }
         }
-        wr[v] = OP == 0 ? W[pr * a.s + (hu >> 12 & 0xfff)]
-                        : OP == 1 ? W[pr] : a.wsc * (a.w ? W[pr] : 1.0f);
+        wr[v] = W[pr * a.s + (hu >> 12 & 0xfff)];
       }
     }
   };
@@ -324,10 +299,7 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
       if (idx >= hn) break;
       float r[VH];
 #pragma unroll
-      for (int z = 0; z < VH; ++z) {
-        r[z] = wr[v] * hr[v][z];
-        if (OP == 1 && (hp[qt * QI + v] & 0x1000)) r[z] *= 1.0f - hr[v][z];
-      }
+      for (int z = 0; z < VH; ++z) r[z] = wr[v] * hr[v][z];
       if (VH == 4)
         *reinterpret_cast<float4*>(A + idx * VH) =
             make_float4(r[0], r[VH > 1 ? 1 : 0], r[VH > 2 ? 2 : 0], r[VH > 3 ? 3 : 0]);
@@ -338,7 +310,7 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
     }
   };
   auto load_x = [&](int t, int qt) {
-    const float* X = a.Xa + (i0 + (int64_t)t * BK) * d + xo;
+    const float* X = a.Xa + (i0 + (int64_t)t * BK) * d + bn0;
     const int lim = min(BK, rows - t * BK) * d;   // offsets of a step's rows lie below rows d
 #pragma unroll
     for (int v = 0; v < QX; ++v) {
@@ -357,7 +329,7 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
     }
   };
   auto store_x = [&](int t, int qt) {
-    float* X = OP == 0 ? Bs + (t & 1) * BK * BN : Xs + (t & 1) * BK * dS;
+    float* X = Bs + (t & 1) * BK * BN;
 #pragma unroll
     for (int v = 0; v < QX; ++v) {
       const int idx = tid + (qt * QX + v) * nt;
@@ -369,18 +341,6 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
         X[idx] = xr[v][0];
     }
   };
-  // pairs of step t: warp w takes rows w, w + warps, ..; lane l columns l + 32 i, quarter by
-  // quarter of the multiply-adds (i = quarter, quarter + 4, ..)
-  const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-  auto pair_rows = [&](int t, int q, int pr0) {
-    const float* X = Xs + (t & 1) * BK * dS;
-    float* B = Bs + (t & 1) * BK * BN + q;
-    const int ef = nmap[q];
-    const float* xe = X + (ef < 0 ? 0 : ef & 0xffff);
-    const float* xf = X + (ef < 0 ? 0 : ef >> 16);
-    for (int pr = pr0; pr < BK; pr += nw) B[pr * BN] = ef < 0 ? 0.0f : xe[pr * dS] * xf[pr * dS];
-  };
-
   float acc[TM][TN];
 #pragma unroll
   for (int x = 0; x < TM; ++x)
@@ -393,40 +353,19 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
       load_x(0, qt);
       store_a(0, qt);
       store_x(0, qt);
-      if (OP != 0 && steps > 1) {
-        load_x(1, qt);
-        store_x(1, qt);
-      }
-    }
-    if (OP != 0) {
-      __syncthreads();
-      for (int q = lane; q < BN; q += 32) pair_rows(0, q, wid);
     }
     __syncthreads();
   }
   for (int t = 0; t < steps; ++t) {
-    const bool more = t + 1 < steps, morex = OP == 0 ? more : t + 2 < steps;
+    const bool more = t + 1 < steps;
     const float* A = As + (t & 1) * BK * BM + mg * 4;
     const float* B = Bs + (t & 1) * BK * BN + ng * 4;
     const int va = a.GM * 4, vb = a.GN * 4;
 #pragma unroll
     for (int qt = 0; qt < 4; ++qt) {
-      if (more) load_h(t + 1, qt);
-      if (morex) load_x(OP == 0 ? t + 1 : t + 2, qt);
-      float pe[2] = {0.0f, 0.0f}, pf[2] = {0.0f, 0.0f};
-      const int pq = lane + qt * 32;
-      const bool pair = OP != 0 && more && pq < BN;
-      if (pair) {
-        const int ef = nmap[pq];
-        const float* X = Xs + ((t + 1) & 1) * BK * dS + wid * dS;
-        if (ef >= 0) {
-          pe[0] = X[ef & 0xffff];
-          pf[0] = X[ef >> 16];
-          if (wid + nw < BK) {
-            pe[1] = X[nw * dS + (ef & 0xffff)];
-            pf[1] = X[nw * dS + (ef >> 16)];
-          }
-        }
+      if (more) {
+        load_h(t + 1, qt);
+        load_x(t + 1, qt);
       }
       if (act) {
 #pragma unroll
@@ -448,15 +387,10 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
         A += BK / 4 * BM;
         B += BK / 4 * BN;
       }
-      if (pair) {
-        float* P = Bs + ((t + 1) & 1) * BK * BN + wid * BN + pq;
-        P[0] = pe[0] * pf[0];
-        if (wid + nw < BK) P[nw * BN] = pe[1] * pf[1];
-        if (wid + 2 * nw < BK) pair_rows(t + 1, pq, wid + 2 * nw);
-        for (int q = pq + 128; q < BN; q += 128) pair_rows(t + 1, q, wid);
+      if (more) {
+        store_a(t + 1, qt);
+        store_x(t + 1, qt);
       }
-      if (more) store_a(t + 1, qt);
-      if (morex) store_x(OP == 0 ? t + 1 : t + 2, qt);
     }
     __syncthreads();
   }
@@ -492,7 +426,6 @@ int row_vec(const void* q, int cols) {
 }
 // k_row_outer_f's VH: 4 needs both operands' rows aligned
 int outer_vh(const OuterArgs<float>& a) {
-  if (a.pairs) return 1;   // two values of h per element
   const int h = row_vec(a.Ha, a.c);
   return h == 4 && row_vec(a.Xa, a.d) == 4 ? 4 : h >= 2 ? 2 : 1;
 }
@@ -518,7 +451,7 @@ OuterPlan outer_plan(const OuterArgs<T>& a, int sms) {
   const int64_t rows = a.r1 - a.r0;
   const int TN = dbl ? 2 : 8;
   OuterPlan p{};
-  p.TM = dbl ? 2 : (OP == 1 && M <= 32 ? 4 : 8);
+  p.TM = dbl ? 2 : 8;
   const int nt = dbl ? 512 : 256;
   const int max_gn = dbl ? 64 : 16;
   const int ng = (Nn + TN - 1) / TN, mg = (M + p.TM - 1) / p.TM;
@@ -535,7 +468,7 @@ OuterPlan outer_plan(const OuterArgs<T>& a, int sms) {
     int need = p.GM * p.GN;
     if (!dbl) {
       const int hn = bk * p.GM * p.TM / vh;
-      const int xn = bk * (OP == 0 ? p.GN * 8 : (a.d + 3) / 4 * 4) / (vh == 4 ? 4 : 1);
+      const int xn = bk * p.GN * 8 / (vh == 4 ? 4 : 1);
       need = std::max({need, (hn + ni - 1) / ni, (xn + nx - 1) / nx});
     }
     p.threads = std::max(128, (need + 31) / 32 * 32);
@@ -562,15 +495,14 @@ OuterPlan outer_plan(const OuterArgs<T>& a, int sms) {
   return p;
 }
 
-template <int OP, int TM, int VH>
+template <int VH>
 int32_t outer_launch_f(const OuterArgs<float>& a, const OuterPlan& p, cudaStream_t st) {
-  const int BK = OuterCfg<OP, VH>::BK, BM = p.GM * TM, BN = p.GN * 8, dS = (a.d + 3) & ~3;
-  const size_t smem =
-      ((size_t)2 * BK * (BM + BN + (OP != 0 ? dS : 0)) + BM + (OP != 0 ? BN : 0)) * 4;
-  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_outer_f<OP, TM, VH>,
+  const int BK = OuterCfg<VH>::BK, BM = p.GM * 8, BN = p.GN * 8;
+  const size_t smem = ((size_t)2 * BK * (BM + BN) + BM) * 4;
+  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_outer_f<VH>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
   count_launch();
-  k_row_outer_f<OP, TM, VH><<<dim3(p.tm, p.tn, p.splits), p.threads, smem, st>>>(a);
+  k_row_outer_f<VH><<<dim3(p.tm, p.tn, p.splits), p.threads, smem, st>>>(a);
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
 }
@@ -591,19 +523,14 @@ int32_t outer_run(OuterArgs<double> a, const OuterPlan& p, cudaStream_t st) {
 
 template <int OP>
 int32_t outer_run(OuterArgs<float> a, const OuterPlan& p, cudaStream_t st) {
+  static_assert(OP == 0, "the f32 block sums are pair_sums");
   a.GM = p.GM;
   a.GN = p.GN;
   a.rps = p.rps;
   const int vh = outer_vh(a);
-  if constexpr (OP == 2) return outer_launch_f<2, 8, 1>(a, p, st);
-  if constexpr (OP == 1) if (p.TM == 4) {
-    if (vh == 4) return outer_launch_f<OP, 4, 4>(a, p, st);
-    if (vh == 2) return outer_launch_f<OP, 4, 2>(a, p, st);
-    return outer_launch_f<OP, 4, 1>(a, p, st);
-  }
-  if (vh == 4) return outer_launch_f<OP, 8, 4>(a, p, st);
-  if (vh == 2) return outer_launch_f<OP, 8, 2>(a, p, st);
-  return outer_launch_f<OP, 8, 1>(a, p, st);
+  if (vh == 4) return outer_launch_f<4>(a, p, st);
+  if (vh == 2) return outer_launch_f<2>(a, p, st);
+  return outer_launch_f<1>(a, p, st);
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1189,6 +1116,233 @@ void block_ranges(OuterPlan& p, int64_t N, int64_t rows, int d, int c, int sms) 
   p.splits = (int)std::max<int64_t>(1, (rows + p.rps - 1) / p.rps);   // ranges that hold rows
 }
 
+// ------------------------------------------------------------------------------------------
+// Block sums over feature pairs, f32 (eq. 13's S and B_k with M = (kind, class), Exact-FIRAL's dense
+// sums with M = class pair): out[m][p] = sum_i A[i][m] Z[i][p], p a pair e <= f of features,
+//   Z = x_e x_f;   A = w h_k (kind 0), w h_k (1 - h_k) (kind 1), wsc w (delta_kl h_k - h_k h_l)
+// Both operands are written out first (k_outer_terms), a bounded number of rows of every range at a
+// time, so that the product is nothing but copies and multiply-adds: 8 x 16 outputs per thread,
+// six 16-byte shared loads per 128 multiply-adds.  Forming A and Z tile by tile inside the product
+// cost more issue slots than the operands' traffic costs time: 29 TFLOP/s at n = 21,000, c = 1000,
+// d = 64 (3.0 ms), now 44 (1.90 ms and 0.09 for the operands); Exact-FIRAL's sums at n = 5,000,
+// c = d = 50 1.02 -> 0.36 ms.  Three blocks per SM at the square tile (168 registers, a few spills
+// outside the loop): 408 tiles take one wave of 456 slots, not two of 304 (2.43 ms).  Rows of a
+// range are added in order.
+// ------------------------------------------------------------------------------------------
+struct PairSum {
+  const float* Xa;
+  const float* Ha;
+  const float* w;      // row weights; class pairs: may be null (weights 1), all scaled by wsc
+  const int2* pairs;   // class pairs, or null: kinds and classes
+  int64_t r0, r1;      // rows of the sum
+  int64_t rps;         // rows per range
+  int splits;          // ranges
+  int d, c, which0;    // which0: the first kind
+  float wsc;
+  int M, Nn, lda, ldz; // outputs, and row lengths of A and Z (multiples of 4, zero-padded)
+  int64_t t0, L;       // this pass: rows [t0, t0 + L) of every range
+  float* A;
+  float* Z;
+  float* part;         // splits x M x Nn
+};
+
+constexpr int TERM_ROWS = 16;
+__global__ __launch_bounds__(256) void k_outer_terms(const PairSum a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* xs = (float*)smem_raw;   // [TERM_ROWS][d]
+  __shared__ float ws[TERM_ROWS];
+  const int z = blockIdx.y;
+  const int64_t l0 = (int64_t)blockIdx.x * TERM_ROWS;        // row of the pass
+  const int64_t i0 = a.r0 + z * a.rps + a.t0 + l0;
+  const int64_t end = min(a.r1, a.r0 + (z + 1) * a.rps);
+  const int nr = (int)max((int64_t)0, min((int64_t)TERM_ROWS, min(a.L - l0, end - i0)));
+  if (nr == 0) return;
+  for (int q = threadIdx.x; q < nr * a.d; q += blockDim.x) xs[q] = a.Xa[i0 * a.d + q];
+  if (threadIdx.x < nr) ws[threadIdx.x] = a.w ? a.w[i0 + threadIdx.x] : 1.0f;
+  __syncthreads();
+  const int64_t row = z * a.L + l0;
+  const float* H = a.Ha + i0 * a.c;
+  float* A = a.A + row * a.lda;
+  for (int m = threadIdx.x; m < a.lda; m += blockDim.x) {
+    if (a.pairs) {
+      const int2 kl = m < a.M ? a.pairs[m] : make_int2(0, 0);
+      for (int r = 0; r < nr; ++r) {
+        const float hk = H[r * a.c + kl.x];
+        const float v = (kl.x == kl.y ? hk : 0.0f) - hk * H[r * a.c + kl.y];
+        A[(int64_t)r * a.lda + m] = m < a.M ? a.wsc * ws[r] * v : 0.0f;
+      }
+    } else {
+      const int kind = m / a.c + a.which0, k = m % a.c;
+      for (int r = 0; r < nr; ++r) {
+        const float h = H[r * a.c + k];
+        float v = ws[r] * h;
+        if (kind) v *= 1.0f - h;
+        A[(int64_t)r * a.lda + m] = m < a.M ? v : 0.0f;
+      }
+    }
+  }
+  float* Z = a.Z + row * a.ldz;
+  for (int p = threadIdx.x; p < a.ldz; p += blockDim.x) {
+    int e = 0, f = 0;
+    if (p < a.Nn) feature_pair(p, a.d, e, f);
+    for (int r = 0; r < nr; ++r)
+      Z[(int64_t)r * a.ldz + p] = p < a.Nn ? xs[r * a.d + e] * xs[r * a.d + f] : 0.0f;
+  }
+}
+
+// GM thread groups of 8 rows m, 128 / GM of 16 columns: 128 x 128, 64 x 256 or 32 x 512 outputs
+template <int GM>
+struct PairTile {
+  static constexpr int BM = 8 * GM, BN = 16 * (128 / GM), BK = 16, ST = 3;
+  static constexpr int SMEM = ST * BK * (BM + BN) * 4;
+};
+template <int GM>
+__global__ __launch_bounds__(128, GM == 16 ? 3 : 2) void k_outer_gemm(const PairSum a) {
+  using C = PairTile<GM>;
+  constexpr int BM = C::BM, BN = C::BN, BK = C::BK, ST = C::ST, GN = 128 / GM;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* As = (float*)smem_raw;     // [ST][BK][BM]
+  float* Zs = As + ST * BK * BM;    // [ST][BK][BN]
+  const int tid = threadIdx.x, z = blockIdx.z;
+  // a warp covers 32 / GW row groups x GW column groups
+  constexpr int GW = GN < 8 ? GN : GM == 16 ? 8 : GN < 32 ? GN : 32;
+  const int mg = tid / 32 * (32 / GW) % GM + tid % 32 / GW;
+  const int ng = (tid / 32 * (32 / GW) / GM) * GW + tid % GW;
+  const int bm0 = blockIdx.x * BM, bn0 = blockIdx.y * BN;
+  const int64_t left = min(a.r1, a.r0 + (z + 1) * a.rps) - (a.r0 + z * a.rps + a.t0);
+  const int n = (int)max((int64_t)0, min(a.L, left));
+  if (n == 0 && a.t0 > 0) return;   // the range ended in an earlier pass
+  const int steps = (n + BK - 1) / BK;
+  const float* A = a.A + (int64_t)z * a.L * a.lda + bm0;
+  const float* Z = a.Z + (int64_t)z * a.L * a.ldz + bn0;
+  const int am = a.lda - bm0, zn = a.ldz - bn0;   // columns there are
+  auto load = [&](int t) {
+    if (t < steps) {
+      const int lim = n - t * BK;
+      float* As_ = As + t % ST * BK * BM;
+      float* Zs_ = Zs + t % ST * BK * BN;
+      const float* A_ = A + (int64_t)t * BK * a.lda;
+      const float* Z_ = Z + (int64_t)t * BK * a.ldz;
+#pragma unroll
+      for (int u = 0; u < BK * BM / 512; ++u) {
+        const int idx = tid + u * 128, r = idx / (BM / 4), q = idx % (BM / 4) * 4;
+        const bool ok = r < lim && q < am;
+        cp_async<16>(As_ + r * BM + q, ok ? A_ + (int64_t)r * a.lda + q : a.A, ok);
+      }
+#pragma unroll
+      for (int u = 0; u < BK * BN / 512; ++u) {
+        const int idx = tid + u * 128, r = idx / (BN / 4), q = idx % (BN / 4) * 4;
+        const bool ok = r < lim && q < zn;
+        cp_async<16>(Zs_ + r * BN + q, ok ? Z_ + (int64_t)r * a.ldz + q : a.Z, ok);
+      }
+    }
+    cp_commit();
+  };
+  float acc[8][16];
+  float* out = a.part + (int64_t)z * a.M * a.Nn;
+#pragma unroll
+  for (int x = 0; x < 8; ++x) {
+    const int m = bm0 + (x / 4) * (BM / 2) + mg * 4 + x % 4;
+#pragma unroll
+    for (int y = 0; y < 16; ++y) {
+      const int p = bn0 + (y / 4) * (BN / 4) + ng * 4 + y % 4;
+      acc[x][y] = a.t0 > 0 && m < a.M && p < a.Nn ? out[(int64_t)m * a.Nn + p] : 0.0f;
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < ST - 1; ++t) load(t);
+  for (int t = 0; t < steps; ++t) {
+    cp_wait<ST - 2>();
+    __syncthreads();   // step t has landed for all; every thread is done with step t - 1
+    load(t + ST - 1);
+    const float* As_ = As + t % ST * BK * BM + mg * 4;
+    const float* Zs_ = Zs + t % ST * BK * BN + ng * 4;
+#pragma unroll 4
+    for (int r = 0; r < BK; ++r) {   // rows past the end are zero in both
+      float av[8], zv[16];
+#pragma unroll
+      for (int v = 0; v < 2; ++v)
+        *reinterpret_cast<float4*>(av + 4 * v) =
+            *reinterpret_cast<const float4*>(As_ + r * BM + v * (BM / 2));
+#pragma unroll
+      for (int v = 0; v < 4; ++v)
+        *reinterpret_cast<float4*>(zv + 4 * v) =
+            *reinterpret_cast<const float4*>(Zs_ + r * BN + v * (BN / 4));
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+#pragma unroll
+        for (int y = 0; y < 16; ++y) acc[x][y] = fmaf(av[x], zv[y], acc[x][y]);
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < 8; ++x) {
+    const int m = bm0 + (x / 4) * (BM / 2) + mg * 4 + x % 4;
+    if (m >= a.M) continue;
+#pragma unroll
+    for (int y = 0; y < 16; ++y) {
+      const int p = bn0 + (y / 4) * (BN / 4) + ng * 4 + y % 4;
+      if (p < a.Nn) out[(int64_t)m * a.Nn + p] = acc[x][y];
+    }
+  }
+}
+
+// The tile that covers M x Nn with the fewest outputs
+int pair_tile(int M, int Nn, int64_t* tiles) {
+  int best = 16;
+  int64_t ba = INT64_MAX;
+  for (int gm : {16, 8, 4}) {
+    const int bm = 8 * gm, bn = 16 * (128 / gm);
+    const int64_t t = (int64_t)((M + bm - 1) / bm) * ((Nn + bn - 1) / bn);
+    if (t * bm * bn < ba) {
+      ba = t * bm * bn;
+      best = gm;
+      *tiles = t;
+    }
+  }
+  return best;
+}
+
+template <int GM>
+int32_t outer_gemm(const PairSum& a, cudaStream_t st) {
+  using C = PairTile<GM>;
+  FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_outer_gemm<GM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      C::SMEM));
+  count_launch();
+  k_outer_gemm<GM><<<dim3((a.M + C::BM - 1) / C::BM, (a.Nn + C::BN - 1) / C::BN, a.splits), 128,
+                     C::SMEM, st>>>(a);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
+// a: everything but the operands' buffers and the passes.  The operands take at most TERM_BYTES
+// (and at least TERM_ROWS rows of every range).
+constexpr int64_t TERM_BYTES = (int64_t)1 << 29;
+int32_t pair_sums(firal_problem* P, PairSum a) {
+  cudaStream_t st = P->H->stream;
+  a.lda = (a.M + 3) & ~3;
+  a.ldz = (a.Nn + 3) & ~3;
+  const int64_t row = (int64_t)(a.lda + a.ldz) * sizeof(float);
+  const int64_t most = std::max<int64_t>(1, std::min(a.rps, a.r1 - a.r0));   // rows of a range
+  a.L = std::max<int64_t>(TERM_ROWS, TERM_BYTES / (row * a.splits) / TERM_ROWS * TERM_ROWS);
+  a.L = std::min(a.L, (most + TERM_ROWS - 1) / TERM_ROWS * TERM_ROWS);
+  FIRAL_TRY(P->terms.ensure((size_t)(a.L * a.splits * row)));
+  a.A = P->terms.as<float>();
+  a.Z = a.A + a.L * a.splits * a.lda;
+  int64_t tiles = 0;
+  const int gm = pair_tile(a.M, a.Nn, &tiles);
+  const size_t smem = (size_t)TERM_ROWS * a.d * sizeof(float);
+  a.t0 = 0;
+  do {
+    count_launch();
+    k_outer_terms<<<dim3((unsigned)((a.L + TERM_ROWS - 1) / TERM_ROWS), a.splits), 256, smem, st>>>(a);
+    FIRAL_CUDA_TRY(cudaGetLastError());
+    FIRAL_TRY(gm == 16 ? outer_gemm<16>(a, st) : gm == 8 ? outer_gemm<8>(a, st)
+                                                          : outer_gemm<4>(a, st));
+    a.t0 += a.L;
+  } while (a.t0 < most);
+  return FIRAL_OK;
+}
+
 template <class T>
 int32_t syrk_t(firal_problem* P, const T* w, int64_t rows, double lamS, T* outS, double lamP,
                double* outP) {
@@ -1197,34 +1351,60 @@ int32_t syrk_t(firal_problem* P, const T* w, int64_t rows, double lamS, T* outS,
   const int nw = (outS ? 1 : 0) + (outP ? 1 : 0);
   if (nw == 0) return FIRAL_OK;
   const int np = d * (d + 1) / 2;
-  OuterArgs<T> a{};
-  a.Xa = P->Xa.as<T>();
-  a.Ha = P->Ha.as<T>();
-  a.w = w;
-  a.r0 = 0;
-  a.r1 = rows;
-  a.d = d;
-  a.c = c;
-  a.s = 1;
-  a.which0 = outS ? 0 : 1;
-  a.M = nw * c;
-  a.Nn = np;
-  OuterPlan p = outer_plan<1>(a, P->sms);
-  if (sizeof(T) == 4) block_ranges(p, P->N, rows, d, c, P->sms);
-  FIRAL_TRY(P->syrk_part.ensure((size_t)a.M * a.Nn * p.splits * sizeof(T)));
-  a.part = P->syrk_part.as<T>();
+  const int M = nw * c;
+  int splits = 1;
+  T* part = nullptr;
   ProfScope ps(st, PF_SYRK);
-  FIRAL_TRY(outer_run<1>(a, p, st));
-  const int64_t per = (int64_t)a.M * np, half = (int64_t)c * np;
+  if constexpr (sizeof(T) == 8) {
+    OuterArgs<T> a{};
+    a.Xa = P->Xa.as<T>();
+    a.Ha = P->Ha.as<T>();
+    a.w = w;
+    a.r0 = 0;
+    a.r1 = rows;
+    a.d = d;
+    a.c = c;
+    a.s = 1;
+    a.which0 = outS ? 0 : 1;
+    a.M = M;
+    a.Nn = np;
+    const OuterPlan p = outer_plan<1>(a, P->sms);
+    splits = p.splits;
+    FIRAL_TRY(P->syrk_part.ensure((size_t)M * np * splits * sizeof(T)));
+    part = a.part = P->syrk_part.as<T>();
+    FIRAL_TRY(outer_run<1>(a, p, st));
+  } else {
+    OuterPlan p{};
+    block_ranges(p, P->N, rows, d, c, P->sms);
+    splits = p.splits;
+    FIRAL_TRY(P->syrk_part.ensure((size_t)M * np * splits * sizeof(T)));
+    part = P->syrk_part.as<T>();
+    PairSum a{};
+    a.Xa = P->Xa.as<float>();
+    a.Ha = P->Ha.as<float>();
+    a.w = w;
+    a.r0 = 0;
+    a.r1 = rows;
+    a.rps = p.rps;
+    a.splits = splits;
+    a.d = d;
+    a.c = c;
+    a.which0 = outS ? 0 : 1;
+    a.M = M;
+    a.Nn = np;
+    a.part = part;
+    FIRAL_TRY(pair_sums(P, a));
+  }
+  const int64_t per = (int64_t)M * np, half = (int64_t)c * np;
   const dim3 blk(32, 8);
   const unsigned grid = (unsigned)((half + 31) / 32);
   if (outS) {
     count_launch();
-    k_pair_expand<T><<<grid, blk, 0, st>>>(a.part, p.splits, half, per, np, d, lamS, nullptr, outS);
+    k_pair_expand<T><<<grid, blk, 0, st>>>(part, splits, half, per, np, d, lamS, nullptr, outS);
   }
   if (outP) {
     count_launch();
-    k_pair_expand<T><<<grid, blk, 0, st>>>(a.part + (outS ? half : 0), p.splits, half, per, np, d,
+    k_pair_expand<T><<<grid, blk, 0, st>>>(part + (outS ? half : 0), splits, half, per, np, d,
                                            lamP, outP, nullptr);
   }
   FIRAL_CUDA_TRY(cudaGetLastError());
@@ -1540,13 +1720,15 @@ int32_t apply_t(firal_problem* P, const T* w, const T* Sblk, const T* V, int s, 
     ProfScope ps(st, PF_DTERM);
     FIRAL_TRY(outer_run<0>(o, p, st));
   }
-  // one probe per block and the splits over thread groups (a power of two, at most 1024 threads)
-  // while that leaves the blocks few; 4 probes per block once the classes alone fill the chip
+  // the splits over thread groups (a power of two, at most 1024 threads) while the blocks are few,
+  // and one probe per block in place of 4 while blocks of 4 would fill less than half the chip
+  // (c = 101, d = 100, s = 10: 26 us as 1,010 blocks of one probe, each S_k read ten times; 18 as 303)
   const int dpad = (d + 31) / 32 * 32;
-  const bool few = (int64_t)c * ((s + 3) / 4) < 4 * P->sms;
-  const int JB = few ? 1 : 4;
+  const int64_t quads = (int64_t)c * ((s + 3) / 4);
+  const bool few = quads < 4 * P->sms;
+  const int JB = 2 * quads < P->sms ? 1 : 4;
   int SG = 1;
-  while (few && 2 * SG * dpad <= 1024 && 2 * SG <= p.splits) SG *= 2;
+  while (few && 2 * SG * JB * dpad <= 1024 && 2 * SG <= p.splits) SG *= 2;
   const size_t smem = ((size_t)JB * d + (size_t)SG * JB * dpad) * sizeof(T);
   ProfScope ps(st, PF_COMBINE);
   count_launch();
@@ -1662,7 +1844,7 @@ int32_t round_scores_f32(firal_problem* P, const float* M1, const float* M2, con
 // pairs with M_kl staged pair by pair, took 1,830 and 2,760.
 int32_t pair_sums_f32(firal_problem* P, int64_t r0, int64_t rows, const float* w, double wsc,
                       const int2* pairs, int npairs, DBuf& part, int* splits) {
-  OuterArgs<float> a{};
+  PairSum a{};
   a.Xa = P->Xa.as<float>();
   a.Ha = P->Ha.as<float>();
   a.w = w ? w - r0 : nullptr;
@@ -1670,17 +1852,27 @@ int32_t pair_sums_f32(firal_problem* P, int64_t r0, int64_t rows, const float* w
   a.r1 = r0 + rows;
   a.d = P->d;
   a.c = P->c;
-  a.s = 1;
   a.pairs = pairs;
   a.wsc = (float)wsc;
   a.M = npairs;
   a.Nn = P->d * (P->d + 1) / 2;
-  const OuterPlan p = outer_plan<2>(a, P->sms);
-  FIRAL_TRY(part.ensure((size_t)a.M * a.Nn * p.splits * sizeof(float)));
+  // ranges: two blocks per SM, whole waves where the row count allows it, at most 1024 rows in one
+  // f32 sum, partials of at most 512 MiB
+  int64_t tiles = 1;
+  pair_tile(a.M, a.Nn, &tiles);
+  const int64_t slots = 2LL * P->sms;
+  int64_t want = std::max<int64_t>({1, slots / tiles, (rows + 1023) / 1024});
+  if (want * tiles > slots) want = std::max(want, (want * tiles + slots - 1) / slots * slots / tiles);
+  want = std::min(want, (rows + 31) / 32);
+  want = std::min(want, ((int64_t)1 << 29) / ((int64_t)a.M * a.Nn * 4));
+  want = std::max<int64_t>(1, std::min<int64_t>(want, 65535));
+  a.rps = std::max<int64_t>(1, (rows + want - 1) / want);
+  a.splits = (int)std::max<int64_t>(1, (rows + a.rps - 1) / a.rps);
+  FIRAL_TRY(part.ensure((size_t)a.M * a.Nn * a.splits * sizeof(float)));
   a.part = part.as<float>();
-  *splits = p.splits;
+  *splits = a.splits;
   ProfScope ps(P->H->stream, PF_EXACT_BUILD);
-  return outer_run<2>(a, p, P->H->stream);
+  return pair_sums(P, a);
 }
 
 int32_t pair_forms_f32(firal_problem* P, const int2* pairs, int npairs, const float* M, float* g,
