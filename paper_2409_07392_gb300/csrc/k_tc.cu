@@ -3850,7 +3850,7 @@ __global__ void __launch_bounds__(384, 1)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   PwCtl* ctl = (PwCtl*)(sm + OFF_CTL);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ctl->x_full[b], 1);
@@ -3948,8 +3948,13 @@ __global__ void __launch_bounds__(384, 1)
       const uint32_t cnt = (nt + 1 - b) / 2;
       if (cnt) mbar_wait_drain(&ctl->xt_full[b], (cnt - 1) & 1);
     }
-  } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer: MMA1 of unit u, then MMA2 of unit u - 1
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: MMA1 of unit u, then MMA2 of unit u - 1.  The whole warp runs the
+    // loop and one elected lane issues: under a branch on the lane the operands of every MMA pass
+    // through vector registers, about 110 cycles an MMA against the 64 it takes
+    auto wait = [&](uint64_t* bar, uint32_t ph) {   // the same answer in every lane
+      return __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_w)) != 0;
+    };
     struct Pend {
       uint32_t u, item;
       bool first, last;
@@ -3961,67 +3966,76 @@ __global__ void __launch_bounds__(384, 1)
     auto mma2 = [&](const Pend& p) -> bool {
       const int b = p.u & 1, db = p.item & 1;
       const uint32_t ph = (p.u >> 1) & 1;
-      if (!mbar_wait(&ctl->psi_full[b], ph, abort_w) || !mbar_wait(&ctl->xt_full[b], ph, abort_w) ||
-          (p.first && !mbar_wait(&ctl->d_empty[db], ((p.item >> 1) & 1) ^ 1, abort_w)))
+      if (!wait(&ctl->psi_full[b], ph) || !wait(&ctl->xt_full[b], ph) ||
+          (p.first && !wait(&ctl->d_empty[db], ((p.item >> 1) & 1) ^ 1)))
         return false;
       tc_fence_after();
       // D (lanes = the unit's (probe, class) columns, columns = features) += psi^T x:
       // A = psi (MN-major: rows = the tile's rows, 64-column atoms 16 KB apart; columns past nc
       // are stale and their D lanes unused), B = the x^T tile (K-major, DP rows): N = DP, where the
       // features as M would fill 128 lanes with at most 64 of them
-      const uint32_t ps = smem_u32(sm + OFF_PSI + b * PSI_BUF),
-                     xt = smem_u32(sm + OFF_XT + b * XT_BYTES);
+      const uint64_t pd = sdesc_sw128_mn(smem_u32(sm + OFF_PSI + b * PSI_BUF), PSI_ATOM),
+                     xd = sdesc_sw128(smem_u32(sm + OFF_XT + b * XT_BYTES));
+      const uint32_t dt = tmem + TD + db * NU;
       constexpr uint32_t idesc2 = idesc_bf16_f32_amn(128, DP);
+      if (elect_one()) {
 #pragma unroll
-      for (int kb = 0; kb < 2; ++kb)
+        for (int kb = 0; kb < 2; ++kb)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint64_t xd = sdesc_sw128(xt + kb * DP * 128 + k * 32);
-          const uint32_t a0 = ps + (kb * 64 + k * 16) * 128;
-          const uint32_t acc = (p.first && kb == 0 && k == 0) ? 0u : 1u;
-          umma_bf16(tmem + TD + db * NU, sdesc_sw128_mn(a0, PSI_ATOM), xd, idesc2, acc);
-          umma_bf16(tmem + TD + db * NU, sdesc_sw128_mn(a0 + 2 * PSI_ATOM, PSI_ATOM), xd, idesc2,
-                    1u);
-        }
-      umma_commit(&ctl->psi_empty[b]);
-      umma_commit(&ctl->xt_empty[b]);
-      if (p.last) umma_commit(&ctl->d_full[db]);
+          for (int k = 0; k < 4; ++k) {   // descriptors advance by bytes / 16
+            const uint64_t x1 = xd + (kb * DP * 128 + k * 32) / 16;
+            const uint64_t p1 = pd + (kb * 64 + k * 16) * 128 / 16;
+            umma_bf16(dt, p1, x1, idesc2, (kb | k) == 0 ? (p.first ? 0u : 1u) : 1u);
+            umma_bf16(dt, p1 + 2 * PSI_ATOM / 16, x1, idesc2, 1u);
+          }
+        umma_commit(&ctl->psi_empty[b]);
+        umma_commit(&ctl->xt_empty[b]);
+        if (p.last) umma_commit(&ctl->d_full[db]);
+      }
+      __syncwarp();
       return true;
     };
-    for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
+    for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok; ++it) {
       const int code = sched[gridDim.x + 1 + it], grp = code & (GRP_MAX - 1);
       const int4 sg = seg_tab[code / GRP_MAX];
       const int4 pq = pool_tab[sg.x];
       const int t0 = sg.y >> 7, t1 = (sg.z - 1) >> 7;
       const int nc = pw_ncols(pq.z, sp, grp);
       const uint32_t idesc1 = idesc_bf16_f32(128, nc);
-      if (!mbar_wait(&ctl->pt_full, ni & 1, abort_w)) { give_up(44); ok = false; break; }
+      if (!wait(&ctl->pt_full, ni & 1)) { give_up(44); ok = false; break; }
       const uint32_t item = ni++;
       for (int t = t0; t <= t1; ++t) {
         const uint32_t u = nt;
         const int b = u & 1;
         const uint32_t ph = (u >> 1) & 1;
-        if (!mbar_wait(&ctl->x_full[b], ph, abort_w) ||
-            !mbar_wait(&ctl->s_empty[b], ph ^ 1, abort_w)) { give_up(45); ok = false; break; }
-        tc_fence_after();
-        const uint32_t xa = smem_u32(sm + OFF_XA + b * XA_BYTES), pt = smem_u32(sm + OFF_PT);
-#pragma unroll
-        for (int k = 0; k < DP / 16; ++k) {
-          const uint64_t ad = sdesc_sw128(xa + k * 32);
-          umma_bf16(tmem + TS + b * NU, ad, sdesc_sw128(pt + k * 32), idesc1, k > 0 ? 1u : 0u);
-          umma_bf16(tmem + TS + b * NU, ad, sdesc_sw128(pt + PT_HALF + k * 32), idesc1, 1u);
+        if (!wait(&ctl->x_full[b], ph) || !wait(&ctl->s_empty[b], ph ^ 1)) {
+          give_up(45);
+          ok = false;
+          break;
         }
-        umma_commit(&ctl->s_full[b]);
-        umma_commit(&ctl->x_empty[b]);
-        if (t == t1) umma_commit(&ctl->pt_empty);
+        tc_fence_after();
+        const uint64_t xd = sdesc_sw128(smem_u32(sm + OFF_XA + b * XA_BYTES)),
+                       pd = sdesc_sw128(smem_u32(sm + OFF_PT));
+        if (elect_one()) {
+#pragma unroll
+          for (int k = 0; k < DP / 16; ++k) {
+            umma_bf16(tmem + TS + b * NU, xd + 2 * k, pd + 2 * k, idesc1, k > 0 ? 1u : 0u);
+            umma_bf16(tmem + TS + b * NU, xd + 2 * k, pd + PT_HALF / 16 + 2 * k, idesc1, 1u);
+          }
+          umma_commit(&ctl->s_full[b]);
+          umma_commit(&ctl->x_empty[b]);
+          if (t == t1) umma_commit(&ctl->pt_empty);
+        }
+        __syncwarp();
         ++nt;
         if (have && !mma2(pend)) { give_up(46); ok = false; break; }
         pend = Pend{u, item, t == t0, t == t1};
         have = true;
       }
     }
-    if (ok && have && !*abort_w && !mma2(pend)) give_up(46);
-    umma_commit(&ctl->drain);
+    if (ok && have && !mma2(pend)) give_up(46);
+    if (elect_one()) umma_commit(&ctl->drain);
+    __syncwarp();
     mbar_wait_drain(&ctl->drain, 0);
   } else if (warp >= 4) {
     // ---------------- epilogue
