@@ -238,6 +238,7 @@ int32_t tc_prepare(firal_problem* P);
 int32_t tc_prepare_operands(firal_problem* P);
 int32_t tc_hessian_apply(firal_problem* P, const void* w, const void* Sblk, const void* V, int s,
                          void* out, double* pq, double lam_null);
+int32_t tc_pw_cg(firal_problem* P, int s, double tol, int fixed, bool first, int* host_active);
 int32_t tc_quad_forms(firal_problem* P, const void* A, const void* B, int s, double scale,
                       void* g);
 int32_t tc_syrk_blocks(firal_problem* P, const void* w, double lamS, void* outS, double lamP,
@@ -480,9 +481,14 @@ int32_t pcg_run(firal_problem* P, const void* B, int s, const firal_cg_opts& cg,
       for (int j = 0; j < ns; ++j) any |= cols[j].active != 0;
       if (!any) break;
     }
-    FIRAL_TRY(apply(P, P->w_sig.p, P->S_sig.p, P->cgP.p, s, P->cgQ.p, P->cgpart1.as<double>()));
     const int slot = (it + 1) & 1;
-    FIRAL_TRY(cg_iterate_tail(P, s, tol, fixed, lag ? rd.at(slot, ns) : nullptr));
+    int* flags = lag ? rd.at(slot, ns) : nullptr;
+    if (P->pw && !sharded(P)) {
+      FIRAL_TRY(tc_pw_cg(P, s, tol, fixed, it == 0, flags));
+    } else {
+      FIRAL_TRY(apply(P, P->w_sig.p, P->S_sig.p, P->cgP.p, s, P->cgQ.p, P->cgpart1.as<double>()));
+      FIRAL_TRY(cg_iterate_tail(P, s, tol, fixed, flags));
+    }
     if (lag) FIRAL_CUDA_TRY(cudaEventRecord(rd.ev[slot], st));
   }
   FIRAL_CUDA_TRY(cudaMemcpyAsync(X_out, P->cgX.p, (size_t)s * P->D * vsize(P),

@@ -4178,6 +4178,215 @@ __global__ void __launch_bounds__(PWF_THREADS) k_pw_finish(float* out, const flo
   }
 }
 
+// Everything of a CG iteration but the apply's product, for one (pool q, probe j): the columns of
+// the fused apply are independent, so one block takes a column from the apply's partials to the
+// next packed direction.  With u the column's direction p:
+//   Q = Sigma p (k_pw_finish), alpha = rho / <p, Q>, x += alpha p, r -= alpha Q, z_k = M_k^{-1} r_k,
+//   the stop test on <r, r>, beta = <r, z> / rho, p = z + beta p, P~ and its means (k_pw_pack)
+// with the arithmetic and the order of additions of those kernels and of k_cg_alpha, k_cg_update,
+// k_cg_beta and k_cg_pupdate, whose five launches (28 us an iteration at 50,000 x 50 x 10, 40
+// columns; 60 us over 3 groups of 64 pools) it replaces: 22 and 41 us.  Bound by the chains of loads and
+// FP64 additions of one column; a stopped column only reports itself.
+__global__ void __launch_bounds__(PWF_THREADS) k_pw_cg(
+    const float* __restrict__ part, const float* __restrict__ Minv, float* __restrict__ X,
+    float* __restrict__ R, float* __restrict__ Pd, float* __restrict__ vmean, bf16* __restrict__ Pk,
+    CGCol* __restrict__ cols, const int4* __restrict__ pool_tab, const int2* __restrict__ pseg,
+    const int4* __restrict__ seg_tab, double lam, double tol, int fixed, int sp, int d, int64_t D,
+    int Qe, int* host_active) {
+  constexpr int NG = PWF_THREADS / 64;
+  __shared__ float t[32 * 64], ps[32 * 64];   // Q, then r; p
+  __shared__ double red[NG][64];
+  __shared__ float qm[64];
+  __shared__ double dots[2][32];
+  __shared__ double s_scal;
+  __shared__ int s_live;
+  const int q = blockIdx.x, j = blockIdx.y, tid = threadIdx.x;
+  const int warp = tid >> 5, lane = tid & 31;
+  const int slot = j * Qe + q;
+  if (!cols[slot].active) {
+    if (tid == 0 && host_active) host_active[slot] = 0;
+    return;
+  }
+  const int4 pt = pool_tab[q];   // first class, classes, padded classes, padded classes before
+  const int2 sr = pseg[q];
+  const int cq = pt.y, ns = sr.y - sr.x, nel = cq * d;
+  float* vm = vmean + (j * Qe + q) * d;
+  const int64_t base = (int64_t)j * D + (int64_t)pt.x * d;   // element kl d + e of the column
+  const float flam = (float)lam;
+  auto warp_add = [](double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+  };
+  // Q before its projection
+  const float* p0 = part + ((int64_t)(ns ? seg_tab[sr.x].w : 0) * sp + j) * d;
+  const int64_t step = (int64_t)cq * sp * d;
+  for (int idx = tid; idx < nel; idx += PWF_THREADS) {
+    const int kl = idx / d, e = idx - kl * d;
+    const float p = Pd[base + idx];
+    ps[kl * 64 + e] = p;
+    float acc = flam * (p - vm[e]);
+    const float* pp = p0 + (int64_t)kl * sp * d + e;
+    for (int g = 0; g < ns; g += 16) {
+      float v[16];
+#pragma unroll
+      for (int x = 0; x < 16; ++x) v[x] = g + x < ns ? pp[(g + x) * step] : 0.0f;
+#pragma unroll
+      for (int x = 0; x < 16; ++x)
+        if (g + x < ns) acc += v[x];
+    }
+    t[kl * 64 + e] = acc;
+  }
+  __syncthreads();
+  {
+    const int e = tid & 63, gr = tid >> 6;
+    double acc = 0.0;
+    if (e < d)
+      for (int kl = gr; kl < cq; kl += NG) acc += (double)t[kl * 64 + e];
+    red[gr][e] = acc;
+    __syncthreads();
+    if (tid < 64 && e < d) {
+      double tot = 0.0;
+      for (int g = 0; g < NG; ++g) tot += red[g][e];
+      qm[e] = (float)(tot / cq);
+    }
+    __syncthreads();
+  }
+  // the projection and <p, Q>, one warp per class
+  for (int kl = warp; kl < cq; kl += PWF_THREADS / 32) {
+    double dot = 0.0;
+    for (int e = lane; e < d; e += 32) {
+      const float v = t[kl * 64 + e] - qm[e] + (float)(lam * (double)vm[e]);
+      t[kl * 64 + e] = v;
+      dot += (double)ps[kl * 64 + e] * (double)v;
+    }
+    dot = warp_add(dot);
+    if (lane == 0) dots[0][kl] = dot;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const double pq = warp_add(lane < cq ? dots[0][lane] : 0.0);
+    if (lane == 0) {
+      CGCol cc = cols[slot];
+      if (pq > 0.0 && isfinite(pq)) {
+        cc.alpha = cc.rho / pq;
+      } else {
+        cc.active = 0;
+        cc.alpha = 0.0;
+        if (host_active) host_active[slot] = 0;
+      }
+      cols[slot] = cc;
+      s_scal = cc.alpha;
+      s_live = cc.active;
+    }
+  }
+  __syncthreads();
+  if (!s_live) return;
+  const float a = (float)s_scal;
+  for (int idx = tid; idx < nel; idx += PWF_THREADS) {
+    const int kl = idx / d, e = idx - kl * d;
+    X[base + idx] = fmaf(a, ps[kl * 64 + e], X[base + idx]);
+    const float r = fmaf(-a, t[kl * 64 + e], R[base + idx]);
+    R[base + idx] = r;
+    t[kl * 64 + e] = r;
+  }
+  __syncthreads();
+  // z = M^{-1} r (kept in registers: at most 4 elements a thread) and the two dots
+  float z[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int idx = tid + u * PWF_THREADS;
+    z[u] = 0.0f;
+    if (idx < nel) {
+      const int kl = idx / d, e = idx - kl * d;
+      const float* Mk = Minv + (int64_t)(pt.x + kl) * d * d + e;
+      const float* r = t + kl * 64;
+      float acc = 0.0f;
+#pragma unroll 16
+      for (int f = 0; f < d; ++f) acc = fmaf(Mk[f * d], r[f], acc);
+      z[u] = acc;
+    }
+  }
+  __shared__ float zs[32 * 64];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int idx = tid + u * PWF_THREADS;
+    if (idx < nel) zs[idx / d * 64 + idx % d] = z[u];
+  }
+  __syncthreads();
+  for (int kl = warp; kl < cq; kl += PWF_THREADS / 32) {
+    double rr = 0.0, rz = 0.0;
+    for (int e0 = 0; e0 < d; e0 += 32) {
+      const int e = e0 + lane;
+      const double r = e < d ? (double)t[kl * 64 + e] : 0.0;
+      const double zz = e < d ? (double)zs[kl * 64 + e] : 0.0;
+      rr += warp_add(r * r);
+      rz += warp_add(r * zz);
+    }
+    if (lane == 0) {
+      dots[0][kl] = rr;
+      dots[1][kl] = rz;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const double rr = warp_add(lane < cq ? dots[0][lane] : 0.0);
+    const double rz = warp_add(lane < cq ? dots[1][lane] : 0.0);
+    if (lane == 0) {
+      CGCol cc = cols[slot];
+      cc.iters += 1;
+      cc.relres = sqrt(rr / cc.bnorm2);
+      if (!fixed && cc.relres <= tol) {
+        cc.active = 0;
+      } else {
+        cc.beta = rz / cc.rho;
+        cc.rho = rz;
+      }
+      cols[slot] = cc;
+      s_scal = cc.beta;
+      s_live = cc.active;
+      if (host_active) host_active[slot] = cc.active;
+    }
+  }
+  __syncthreads();
+  if (!s_live) return;
+  const float b = (float)s_scal;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int idx = tid + u * PWF_THREADS;
+    if (idx < nel) {
+      const int o = idx / d * 64 + idx % d;
+      const float p = fmaf(b, ps[o], z[u]);
+      Pd[base + idx] = p;
+      ps[o] = p;
+    }
+  }
+  __syncthreads();
+  // the next apply's packed rows (padding rows and features are zero since the first k_pw_pack)
+  {
+    const int e = tid & 63, gr = tid >> 6;
+    double acc = 0.0;
+    if (gr < 4 && e < d)
+      for (int kl = gr; kl < cq; kl += 4) acc += (double)ps[kl * 64 + e];
+    if (gr < 4) red[gr][e] = acc;
+    __syncthreads();
+    if (tid < 64 && e < d) {
+      const double tt = ((red[0][e] + red[1][e]) + red[2][e]) + red[3][e];
+      qm[e] = (float)(tt / cq);
+      vm[e] = qm[e];
+    }
+    __syncthreads();
+  }
+  const int64_t n1 = (int64_t)pt.z * sp, r0 = 2LL * sp * pt.w + (int64_t)j * pt.z;
+  for (int idx = tid; idx < nel; idx += PWF_THREADS) {
+    const int kl = idx / d, e = idx - kl * d;
+    const float v = ps[kl * 64 + e] - qm[e];
+    const bf16 hi = __float2bfloat16_rn(v);
+    Pk[(r0 + kl) * 64 + e] = hi;
+    Pk[(r0 + n1 + kl) * 64 + e] = __float2bfloat16_rn(v - __bfloat162float(hi));
+  }
+}
+
 // out_j[:, k] = lam (V_j[:, k] - pool mean) + the pool's segment partials in segment order
 __global__ void k_pw_combine(float* out, const float* V, const float* vmean, const float* part,
                              const int4* pool_tab, const int2* pseg, const int4* seg_tab,
@@ -4345,12 +4554,13 @@ static int32_t pw_schedule(firal_problem* P, int sp, bool quad, int* grid_out,
   return FIRAL_OK;
 }
 
+// The fused apply's product: the segment partials of every probe of V (packed first if pack; else
+// the packed rows and their means are there).
 template <int DP>
-static int32_t tc_apply_pw_t(firal_problem* P, const float* w, const float* V, int s, float* out,
-                             double* pq, double lam) {
+static int32_t tc_pw_product_t(firal_problem* P, const float* w, const float* V, int s, bool pack) {
   using namespace pw_cfg;
   cudaStream_t st = P->H->stream;
-  const int c = P->c, d = P->d;
+  const int d = P->d;
   const int Qe = pool_count(P->pt);
   // means and packed rows sized for the gradient's two operands: growing them there frees memory,
   // which waits for the device
@@ -4361,7 +4571,7 @@ static int32_t tc_apply_pw_t(firal_problem* P, const float* w, const float* V, i
   FIRAL_TRY(P->pw_pk.ensure((size_t)2 * prows * 64 * 2));
   FIRAL_TRY(P->pw_part.ensure((size_t)std::max<int64_t>(1, P->pw_segcls_total) * sp * d *
                               sizeof(float)));
-  {
+  if (pack) {
     ProfScope ps(st, PF_SPLIT);
     count_launch();
     k_pw_pack<<<dim3((unsigned)Qe, (unsigned)sp), 256, 0, st>>>(
@@ -4393,6 +4603,24 @@ static int32_t tc_apply_pw_t(firal_problem* P, const float* w, const float* V, i
                                          tc_error_word(P));
     FIRAL_CUDA_TRY(cudaGetLastError());
   }
+  return FIRAL_OK;
+}
+
+static int32_t tc_pw_product(firal_problem* P, const float* w, const float* V, int s, bool pack) {
+  switch (P->dp) {
+    case 16: return tc_pw_product_t<16>(P, w, V, s, pack);
+    case 32: return tc_pw_product_t<32>(P, w, V, s, pack);
+    default: return tc_pw_product_t<64>(P, w, V, s, pack);
+  }
+}
+
+static int32_t tc_apply_pw(firal_problem* P, const float* w, const float* V, int s, float* out,
+                           double* pq, double lam) {
+  cudaStream_t st = P->H->stream;
+  const int c = P->c, d = P->d;
+  const int Qe = pool_count(P->pt);
+  const int sp = (s + 7) / 8 * 8;
+  FIRAL_TRY(tc_pw_product(P, w, V, s, true));
   ProfScope ps(st, PF_COMBINE);
   if (!sharded(P)) {
     count_launch();
@@ -4420,13 +4648,20 @@ static int32_t tc_apply_pw_t(firal_problem* P, const float* w, const float* V, i
   return FIRAL_OK;
 }
 
-static int32_t tc_apply_pw(firal_problem* P, const float* w, const float* V, int s, float* out,
-                           double* pq, double lam) {
-  switch (P->dp) {
-    case 16: return tc_apply_pw_t<16>(P, w, V, s, out, pq, lam);
-    case 32: return tc_apply_pw_t<32>(P, w, V, s, out, pq, lam);
-    default: return tc_apply_pw_t<64>(P, w, V, s, out, pq, lam);
-  }
+// One CG iteration of a problem on the fused apply (not sharded; first: its direction is not packed
+// yet): the product and k_pw_cg.
+int32_t tc_pw_cg(firal_problem* P, int s, double tol, int fixed, bool first, int* host_active) {
+  FIRAL_TRY(tc_pw_product(P, P->w_sig.as<float>(), P->cgP.as<float>(), s, first));
+  const int Qe = pool_count(P->pt), sp = (s + 7) / 8 * 8;
+  ProfScope ps(P->H->stream, PF_CG);
+  count_launch();
+  k_pw_cg<<<dim3((unsigned)Qe, (unsigned)s), PWF_THREADS, 0, P->H->stream>>>(
+      P->pw_part.as<float>(), P->Minv.as<float>(), P->cgX.as<float>(), P->cgR.as<float>(),
+      P->cgP.as<float>(), P->vmean.as<float>(), P->pw_pk.as<bf16>(), P->cgcols.as<CGCol>(),
+      P->pw_pool.as<int4>(), P->pw_pseg.as<int2>(), P->pw_seg.as<int4>(), P->lambda, tol, fixed, sp,
+      P->d, P->D, Qe, host_active);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
 }
 
 // ------------------------------------------------------------------------------------------
