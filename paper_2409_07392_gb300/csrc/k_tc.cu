@@ -627,7 +627,7 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   TcCtl* ctl = (TcCtl*)(sm + CTL_OFF);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   constexpr int PPN = BN / (NPART * DP);   // probes per N tile
   // MODE 4 tiles carry only 8 MMAs (K = 64, hi and lo), little next to the serial barrier,
   // fence and commit latency of issuing them; two issuer threads (warps 1 and 3) take
@@ -803,8 +803,11 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
         phase ^= 1;
       }
     }
-  } else if ((warp == 1 || (NMMA == 2 && warp == 3)) && lane == 0) {
-    // ---------------- MMA issuer(s)
+  } else if (warp == 1 || (NMMA == 2 && warp == 3)) {
+    // ---------------- MMA issuer(s): the whole warp runs the loop, one elected lane issues
+    auto wait = [&](uint64_t* bar, uint32_t ph) {   // the same answer in every lane
+      return __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_w)) != 0;
+    };
     const int mi = warp == 3 ? 1 : 0;
     uint64_t* turn = ctl->yfull;   // MODE 4 issuer tokens (the D-GEMM's y barriers, unused here)
     int nturn = 0;                 // token waits done by this issuer
@@ -816,10 +819,10 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
     uint32_t acc_phase = 0;
     int xcount = 0;
     Cur cu = cur_first();
-    for (bool more = Q3 ? cu.mt < n_mt : cur_set(cu); more && !*abort_w; more = cur_next(cu)) {
+    for (bool more = Q3 ? cu.mt < n_mt : cur_set(cu); more; more = cur_next(cu)) {
       const int mt = cu.mt, nt = cu.nt;
       if (Q3 && nt == 0) {
-        if (!mbar_wait(&ctl->xfull[xcount & 1], (xcount >> 1) & 1, abort_w)) {
+        if (!wait(&ctl->xfull[xcount & 1], (xcount >> 1) & 1)) {
           raise_abort(ctl, err, 7);
           break;
         }
@@ -833,20 +836,23 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
             stage = 0;
             phase ^= 1;
           }
-        if (Q3 && nt == n_nt - 1) umma_commit(&ctl->xempty[(xcount - 1) & 1]);
+        if (Q3 && nt == n_nt - 1) {
+          if (elect_one()) umma_commit(&ctl->xempty[(xcount - 1) & 1]);
+          __syncwarp();
+        }
         if (++acc == NACC) {
           acc = 0;
           acc_phase ^= 1;
         }
         continue;
       }
-      if (!mbar_wait(&ctl->tempty[acc], acc_phase ^ 1, abort_w)) {
+      if (!wait(&ctl->tempty[acc], acc_phase ^ 1)) {
         raise_abort(ctl, err, 2);
         break;
       }
       // issuer 0 holds the token for the CTA's first tile; every other tile waits for it
       if (NMMA == 2 && !(mi == 0 && first_tile)) {
-        if (!mbar_wait(&turn[mi], nturn & 1, abort_w)) {
+        if (!wait(&turn[mi], nturn & 1)) {
           raise_abort(ctl, err, 8);
           break;
         }
@@ -857,55 +863,62 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
       const uint32_t d = tmem + acc * ACC_COLS;
       bool ok = true;
       for (int kb = kb_lo; kb < kb_hi; ++kb) {
-        if (!mbar_wait(&ctl->full[stage], phase, abort_w)) {
+        if (!wait(&ctl->full[stage], phase)) {
           raise_abort(ctl, err, 3);
           ok = false;
           break;
         }
-        if (NMMA == 2 && kb == kb_hi - 1) mbar_arrive(&turn[mi ^ 1]);   // pass the token
+        if (NMMA == 2 && kb == kb_hi - 1 && lane == 0) mbar_arrive(&turn[mi ^ 1]);   // pass the token
         tc_fence_after();
         const uint32_t a0 = Q3
                                 ? smem_u32(sm + XBUF + ((xcount - 1) & 1) * XB3(DP) + kb * A_BYTES)
                                 : smem_u32(sm + stage * SB);
         const uint32_t b0 = Q3 ? smem_u32(sm + stage * SB) : a0 + OFF_B;
+        const uint64_t ad = sdesc_sw128(a0), bd = sdesc_sw128(b0);   // advance by bytes / 16
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < BK / 16; ++k) {
-          umma_bf16(d, sdesc_sw128(a0 + k * 32), sdesc_sw128(b0 + k * 32), idesc,
-                    (kb != kb_lo || k != 0) ? 1u : 0u);
-          if (Q3)   // x (A_lo; B_lo) into the same columns: a and b to ~2^-16
-            umma_bf16(d, sdesc_sw128(a0 + k * 32), sdesc_sw128(b0 + C3_BYTES + k * 32), idesc, 1u);
-          if (HLO) {
-            const uint64_t al = sdesc_sw128(a0 + A_BYTES + k * 32);
-            if (MODE == 2) {
-              constexpr uint32_t idesc_h = idesc_bf16_f32(BM, BN / 2);
-              umma_bf16(d, al, sdesc_sw128(b0 + k * 32), idesc_h, 1u);
-            } else {
-              constexpr uint32_t idesc_p = idesc_bf16_f32(BM, DP);
+          for (int k = 0; k < BK / 16; ++k) {
+            umma_bf16(d, ad + 2 * k, bd + 2 * k, idesc, (kb != kb_lo || k != 0) ? 1u : 0u);
+            if (Q3)   // x (A_lo; B_lo) into the same columns: a and b to ~2^-16
+              umma_bf16(d, ad + 2 * k, bd + C3_BYTES / 16 + 2 * k, idesc, 1u);
+            if (HLO) {
+              const uint64_t al = ad + A_BYTES / 16 + 2 * k;
+              if (MODE == 2) {
+                constexpr uint32_t idesc_h = idesc_bf16_f32(BM, BN / 2);
+                umma_bf16(d, al, bd + 2 * k, idesc_h, 1u);
+              } else {
+                constexpr uint32_t idesc_p = idesc_bf16_f32(BM, DP);
 #pragma unroll
-              for (int jj = 0; jj < PPN; ++jj)
-                umma_bf16(d + jj * NPART * DP, al,
-                          sdesc_sw128(b0 + jj * NPART * DP * 128 + k * 32), idesc_p, 1u);
+                for (int jj = 0; jj < PPN; ++jj)
+                  umma_bf16(d + jj * NPART * DP, al, bd + jj * NPART * DP * 128 / 16 + 2 * k,
+                            idesc_p, 1u);
+              }
             }
           }
+          umma_commit(&ctl->empty[stage]);
         }
-        umma_commit(&ctl->empty[stage]);
+        __syncwarp();
         if (++stage == NST) {
           stage = 0;
           phase ^= 1;
         }
       }
       if (!ok) break;
-      umma_commit(&ctl->tfull[acc]);
       // MODE 3/4: the resident x tile is free once the point tile's last MMAs complete (each
       // issuer commits for its own)
-      if (Q3 && nt == n_nt - 1) umma_commit(&ctl->xempty[(xcount - 1) & 1]);
+      if (elect_one()) {
+        umma_commit(&ctl->tfull[acc]);
+        if (Q3 && nt == n_nt - 1) umma_commit(&ctl->xempty[(xcount - 1) & 1]);
+      }
+      __syncwarp();
       if (++acc == NACC) {
         acc = 0;
         acc_phase ^= 1;
       }
     }
     // drain: the barrier completes once every MMA issued above (by each issuer) has completed
-    umma_commit(&ctl->drain);
+    if (elect_one()) umma_commit(&ctl->drain);
+    __syncwarp();
     mbar_wait_drain(&ctl->drain, 0);
   } else if (warp >= 4) {
     // ---------------- epilogue: one pool row per thread
@@ -2985,7 +2998,7 @@ __global__ void __launch_bounds__(384, 1)
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   QfCtl* ctl = (QfCtl*)(sm + OFF_CTL);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ctl->x_full[b], 1);
@@ -3068,42 +3081,51 @@ __global__ void __launch_bounds__(384, 1)
     drain(ctl->x_full, 2, nx);
     drain(ctl->h_full, NHB, nh);
     drain(ctl->c_full, NCS, nc);
-  } else if (warp == 1 && lane == 0) {
-    // ---------------- MMA issuer
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: the whole warp runs the loop, one elected lane issues
+    auto wait = [&](uint64_t* bar, uint32_t ph) {   // the same answer in every lane
+      return __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_w)) != 0;
+    };
     constexpr uint32_t idesc = idesc_bf16_f32(128, 128), idesc256 = idesc_bf16_f32(128, 256);
     uint32_t nx = 0, nc = 0;
     bool ok = true;
-    for (int mt = blockIdx.x; mt < n_mt && ok && !*abort_w; mt += gridDim.x) {
+    for (int mt = blockIdx.x; mt < n_mt && ok; mt += gridDim.x) {
       const int bx = nx & 1;
-      if (!mbar_wait(&ctl->x_full[bx], (nx >> 1) & 1, abort_w)) { give_up(64); break; }
+      if (!wait(&ctl->x_full[bx], (nx >> 1) & 1)) { give_up(64); break; }
       const uint32_t xa = smem_u32(sm + OFF_X + bx * XT);
       const int units = nkc * np2;
       for (int un = 0; un < units && ok; ++un) {
         const int cs = (int)(nc % NCS), b = nc & 1;
-        if (!mbar_wait(&ctl->c_full[cs], (nc / NCS) & 1, abort_w) ||
-            !mbar_wait(&ctl->s_empty[b], ((nc >> 1) & 1) ^ 1, abort_w)) { give_up(65); ok = false; break; }
+        if (!wait(&ctl->c_full[cs], (nc / NCS) & 1) ||
+            !wait(&ctl->s_empty[b], ((nc >> 1) & 1) ^ 1)) { give_up(65); ok = false; break; }
         tc_fence_after();
         const uint32_t cb = smem_u32(sm + OFF_C + cs * CST);
         const uint32_t ta = tmem + 256 * b, tb = ta + 128;
+        const uint64_t xd = sdesc_sw128(xa), cd = sdesc_sw128(cb);   // advance by bytes / 16
+        if (elect_one()) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const uint64_t ad = sdesc_sw128(xa + k * 32);
-          // rows [A hi | B hi] are contiguous: one N = 256 product fills both accumulators;
-          // then B lo alone (exact A) or [A lo | B lo] (general A)
-          umma_bf16(ta, ad, sdesc_sw128(cb + k * 32), idesc256, k > 0 ? 1u : 0u);
-          if (AEXACT)
-            umma_bf16(tb, ad, sdesc_sw128(cb + 2 * 16384 + k * 32), idesc, 1u);
-          else
-            umma_bf16(ta, ad, sdesc_sw128(cb + 2 * 16384 + k * 32), idesc256, 1u);
+          for (int k = 0; k < 4; ++k) {
+            const uint64_t ad = xd + 2 * k, c1 = cd + 2 * k, c2 = c1 + 2 * 16384 / 16;
+            // rows [A hi | B hi] are contiguous: one N = 256 product fills both accumulators;
+            // then B lo alone (exact A) or [A lo | B lo] (general A)
+            umma_bf16(ta, ad, c1, idesc256, k > 0 ? 1u : 0u);
+            if (AEXACT)
+              umma_bf16(tb, ad, c2, idesc, 1u);
+            else
+              umma_bf16(ta, ad, c2, idesc256, 1u);
+          }
+          umma_commit(&ctl->c_empty[cs]);
+          umma_commit(&ctl->s_full[b]);
         }
-        umma_commit(&ctl->c_empty[cs]);
-        umma_commit(&ctl->s_full[b]);
+        __syncwarp();
         ++nc;
       }
-      umma_commit(&ctl->x_empty[bx]);
+      if (elect_one()) umma_commit(&ctl->x_empty[bx]);
+      __syncwarp();
       ++nx;
     }
-    umma_commit(&ctl->drain);
+    if (elect_one()) umma_commit(&ctl->drain);
+    __syncwarp();
     mbar_wait_drain(&ctl->drain, 0);
   } else if (warp >= 4 && AEXACT) {
     // ---------------- epilogue, exact first operand: row r = TMEM lane, class box `box` (32
@@ -4715,7 +4737,7 @@ __global__ void __launch_bounds__(384, 1)
   unsigned char* sm = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   PwCtl* ctl = (PwCtl*)(sm + OFF_CTL);
   float* red = (float*)(sm + OFF_RED);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int b = 0; b < 2; ++b) {
       mbar_init(&ctl->x_full[b], 1);
@@ -4788,10 +4810,14 @@ __global__ void __launch_bounds__(384, 1)
       if (cnt) mbar_wait_drain(&ctl->x_full[b], (cnt - 1) & 1);
     }
     if (ni) mbar_wait_drain(&ctl->pt_full, (ni - 1) & 1);
-  } else if (warp == 1 && lane == 0) {
+  } else if (warp == 1) {
+    // ---------------- MMA issuer: the whole warp runs the loop, one elected lane issues
+    auto wait = [&](uint64_t* bar, uint32_t ph) {   // the same answer in every lane
+      return __all_sync(0xffffffffu, mbar_wait(bar, ph, abort_w)) != 0;
+    };
     uint32_t nt = 0, ni = 0;
     bool ok = true;
-    for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
+    for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok; ++it) {
       const int4 sg = seg_tab[sched[gridDim.x + 1 + it]];
       if (skip(sg)) continue;
       const int4 pq = pool_tab[sg.x];
@@ -4799,33 +4825,41 @@ __global__ void __launch_bounds__(384, 1)
       const int t0 = sg.y >> 7, t1 = (sg.z - 1) >> 7;
       for (int grp = 0; grp < ng && ok; ++grp) {
         const uint32_t idesc1 = idesc_bf16_f32(128, pw_ncols(pq.z, sp, grp));
-        if (!mbar_wait(&ctl->pt_full, ni & 1, abort_w)) { give_up(53); ok = false; break; }
+        if (!wait(&ctl->pt_full, ni & 1)) { give_up(53); ok = false; break; }
         ++ni;
         for (int t = t0; t <= t1; ++t) {
           const int b = nt & 1;
           const uint32_t ph = (nt >> 1) & 1;
-          if (!mbar_wait(&ctl->x_full[b], ph, abort_w) ||
-              !mbar_wait(&ctl->s_empty[b], ph ^ 1, abort_w)) { give_up(54); ok = false; break; }
-          tc_fence_after();
-          const uint32_t xa = smem_u32(sm + OFF_XA + b * pw_cfg::XA_BYTES),
-                         pa = smem_u32(sm + OFF_PA), pb = smem_u32(sm + OFF_PB);
-          const uint32_t ta = tmem + 256 * b, tb = ta + 128;
-#pragma unroll
-          for (int k = 0; k < DP / 16; ++k) {
-            const uint64_t ad = sdesc_sw128(xa + k * 32);
-            umma_bf16(ta, ad, sdesc_sw128(pa + k * 32), idesc1, k > 0 ? 1u : 0u);
-            umma_bf16(ta, ad, sdesc_sw128(pa + PT_HALF + k * 32), idesc1, 1u);
-            umma_bf16(tb, ad, sdesc_sw128(pb + k * 32), idesc1, k > 0 ? 1u : 0u);
-            umma_bf16(tb, ad, sdesc_sw128(pb + PT_HALF + k * 32), idesc1, 1u);
+          if (!wait(&ctl->x_full[b], ph) || !wait(&ctl->s_empty[b], ph ^ 1)) {
+            give_up(54);
+            ok = false;
+            break;
           }
-          umma_commit(&ctl->s_full[b]);
-          umma_commit(&ctl->x_empty[b]);
-          if (t == t1) umma_commit(&ctl->pt_empty);
+          tc_fence_after();
+          const uint64_t xd = sdesc_sw128(smem_u32(sm + OFF_XA + b * pw_cfg::XA_BYTES)),
+                         pa = sdesc_sw128(smem_u32(sm + OFF_PA)),
+                         pb = sdesc_sw128(smem_u32(sm + OFF_PB));   // advance by bytes / 16
+          const uint32_t ta = tmem + 256 * b, tb = ta + 128;
+          if (elect_one()) {
+#pragma unroll
+            for (int k = 0; k < DP / 16; ++k) {
+              const uint64_t ad = xd + 2 * k;
+              umma_bf16(ta, ad, pa + 2 * k, idesc1, k > 0 ? 1u : 0u);
+              umma_bf16(ta, ad, pa + PT_HALF / 16 + 2 * k, idesc1, 1u);
+              umma_bf16(tb, ad, pb + 2 * k, idesc1, k > 0 ? 1u : 0u);
+              umma_bf16(tb, ad, pb + PT_HALF / 16 + 2 * k, idesc1, 1u);
+            }
+            umma_commit(&ctl->s_full[b]);
+            umma_commit(&ctl->x_empty[b]);
+            if (t == t1) umma_commit(&ctl->pt_empty);
+          }
+          __syncwarp();
           ++nt;
         }
       }
     }
-    umma_commit(&ctl->drain);
+    if (elect_one()) umma_commit(&ctl->drain);
+    __syncwarp();
     mbar_wait_drain(&ctl->drain, 0);
   } else if (warp >= 4) {
     const int quad = warp & 3, half = (warp - 4) >> 2;
