@@ -318,10 +318,10 @@ int32_t set_step(int64_t* t_dev, int64_t v, cudaStream_t st) {
 // out[k][e][f] = sum_split part[split][k][e][f] (+ lam on the diagonal), as double and/or T
 template <class T>
 __global__ void k_syrk_reduce(const T* part, int splits, int64_t per, int d, double lam,
-                              double* out_d, T* out_t, const T* add = nullptr) {
+                              double* out_d, T* out_t) {
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < per;
        idx += (int64_t)gridDim.x * blockDim.x) {
-    double acc = add ? (double)add[idx] : 0.0;
+    double acc = 0.0;
 #pragma unroll 8
     for (int sp = 0; sp < splits; ++sp) acc += (double)part[(int64_t)sp * per + idx];
     const int64_t ef = idx % ((int64_t)d * d);
@@ -332,15 +332,55 @@ __global__ void k_syrk_reduce(const T* part, int splits, int64_t per, int d, dou
   }
 }
 
+// The same from partials by feature pair (rows of npq values, e <= f), for the tensor-core sums:
+// each pair is added once and written to both places.  Bound by the FP64 additions.
+__global__ void k_pair_blocks(const float* __restrict__ part, int splits, int64_t c, int np,
+                              int npq, int d, double lam, double* out_d, float* out_t,
+                              const float* __restrict__ add) {
+  const int64_t per = c * npq;
+  for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < per;
+       idx += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t k = idx / npq;
+    const int p = (int)(idx - k * npq);
+    if (p >= np) continue;
+    int e, f;
+    feature_pair(p, d, e, f);
+    const int64_t o1 = (k * d + e) * d + f, o2 = (k * d + f) * d + e;
+    double acc = add ? (double)add[o1] : 0.0;
+#pragma unroll 8
+    for (int sp = 0; sp < splits; ++sp) acc += (double)part[(int64_t)sp * per + idx];
+    if (e == f) acc += lam;
+    if (out_d) out_d[o1] = out_d[o2] = acc;
+    if (out_t) out_t[o1] = out_t[o2] = (float)acc;
+  }
+}
+
+int32_t pair_blocks_f32(firal_problem* P, const float* partS, const float* partP, int npq,
+                        int splits, double lamS, float* outS, double lamP, double* outP,
+                        const float* addS) {
+  cudaStream_t st = P->H->stream;
+  const int np = P->d * (P->d + 1) / 2;
+  const int g = grid_for((int64_t)P->c * npq, 256, 65535);
+  ProfScope ps(st, PF_SYRK);
+  count_launch((outS ? 1 : 0) + (outP ? 1 : 0));
+  if (outS)
+    k_pair_blocks<<<g, 256, 0, st>>>(partS, splits, P->c, np, npq, P->d, lamS, nullptr, outS, addS);
+  if (outP)
+    k_pair_blocks<<<g, 256, 0, st>>>(partP, splits, P->c, np, npq, P->d, lamP, outP, nullptr,
+                                     nullptr);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
 int32_t syrk_reduce_f32(firal_problem* P, const float* partS, const float* partP, int splits,
-                        double lamS, float* outS, double lamP, double* outP, const float* addS) {
+                        double lamS, float* outS, double lamP, double* outP) {
   cudaStream_t st = P->H->stream;
   const int64_t per = (int64_t)P->c * P->d * P->d;
   const int g = grid_for(per, 256, 4096);
   ProfScope ps(st, PF_SYRK);
   count_launch((outS ? 1 : 0) + (outP ? 1 : 0));
   if (outS)
-    k_syrk_reduce<float><<<g, 256, 0, st>>>(partS, splits, per, P->d, lamS, nullptr, outS, addS);
+    k_syrk_reduce<float><<<g, 256, 0, st>>>(partS, splits, per, P->d, lamS, nullptr, outS);
   if (outP) k_syrk_reduce<float><<<g, 256, 0, st>>>(partP, splits, per, P->d, lamP, outP, nullptr);
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;

@@ -1504,7 +1504,7 @@ template <int MODE>
 __global__ void __launch_bounds__(256, 1)
     k_tc_bsum(const __grid_constant__ CUtensorMap mapA0, const __grid_constant__ CUtensorMap mapA1,
               const __grid_constant__ CUtensorMap mapZ0, const __grid_constant__ CUtensorMap mapZ1,
-              float* __restrict__ part, int c, int d, int npairs, int n_mt, int n_nt,
+              float* __restrict__ part, int c, int npq, int n_mt, int n_nt,
               int splits, int64_t kb_per_split, int64_t kb_total, int32_t* err,
               const int4* __restrict__ klist, int kbL) {
   using namespace b_cfg;
@@ -1675,15 +1675,9 @@ __global__ void __launch_bounds__(256, 1)
       if (kb0 >= kb1) {
         // empty unit (pooled problems): zero partial block
         if (k < c) {
-          float* out = part + ((int64_t)sp * c + k) * d * d;
-          for (int t = 0; t < BN; ++t) {
-            const int p = nt * BN + t;
-            if (p >= npairs) break;
-            int e, e2;
-            pair_of(p, d, e, e2);
-            out[e * d + e2] = 0.0f;
-            out[e2 * d + e] = 0.0f;
-          }
+          float* out = part + ((int64_t)sp * c + k) * npq;
+          for (int p = nt * BN; p < npq && p < nt * BN + BN; p += 4)
+            *reinterpret_cast<float4*>(out + p) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
         continue;
       }
@@ -1697,7 +1691,10 @@ __global__ void __launch_bounds__(256, 1)
         }
         tc_fence_after();
         const uint32_t tS = tmem + lanes, tL = tmem + lanes + COL_LONG;
-        float* out = part + ((int64_t)sp * c + k) * d * d;
+        // partials by pair, rows of npq (whole 16-byte runs): a thread's 32 pairs are one line.  As
+        // full blocks they were two scattered 4-byte stores each, 0.9 GB of sectors a launch at
+        // 410 classes, d = 64 and 17 splits
+        float* out = part + ((int64_t)sp * c + k) * npq;
         for (int cc = 0; cc < BN; cc += 32) {
           float v[32];
           tmem_ld32(tS + cc, v);
@@ -1710,20 +1707,12 @@ __global__ void __launch_bounds__(256, 1)
           if (!last) {
             tmem_st32(tL + cc, v);
           } else if (k < c) {
-            int e = 0, e2 = 0;
             const int p0 = nt * BN + cc;
-            if (p0 < npairs) pair_of(p0, d, e, e2);
 #pragma unroll
-            for (int t = 0; t < 32; ++t) {
-              if (p0 + t < npairs) {
-                out[e * d + e2] = v[t];
-                out[e2 * d + e] = v[t];
-                if (++e2 == d) {
-                  ++e;
-                  e2 = e;
-                }
-              }
-            }
+            for (int t = 0; t < 32; t += 4)
+              if (p0 + t < npq)
+                *reinterpret_cast<float4*>(out + p0 + t) =
+                    make_float4(v[t], v[t + 1], v[t + 2], v[t + 3]);
           }
         }
         tc_fence_before();
@@ -1814,15 +1803,18 @@ __global__ void k_weighted_hT(bf16* Ahi, bf16* Alo, bf16* AP, const float* Ha, c
   __shared__ float tile[64][33];
   __shared__ float ws[64], wS[64];
   __shared__ int cs[64];
-  const int64_t rb = (int64_t)blockIdx.x * 64;
+  int64_t kb = blockIdx.x;
   const int cb = blockIdx.y * 32;
   // pooled: the block sums read, for each 128-class tile, the labelled rows' K-steps and its
-  // pools' K-steps only (K list {first, end, ...}); the other blocks stay unwritten
+  // pools' K-steps only (K list {first, end, steps in all, ..}); the others stay unwritten.  The
+  // grid holds the longest list, not every K-step: 200,000 mostly empty blocks took 160 us a
+  // launch at 0.8 M rows and 410 classes
   if (klist) {
-    const int64_t kb = blockIdx.x;
     const int4 kl = klist[cb / 128];
-    if (kb >= kbL && (kb < kl.x || kb >= kl.y)) return;
+    if (kb >= kl.z) return;
+    if (kb >= kbL) kb = kl.x + (kb - kbL);
   }
+  const int64_t rb = kb * 64;
   for (int i = threadIdx.y; i < 64; i += blockDim.y) {
     const int64_t r = rb + i;
     const int col = cb + threadIdx.x;
@@ -1845,7 +1837,7 @@ __global__ void k_weighted_hT(bf16* Ahi, bf16* Alo, bf16* AP, const float* Ha, c
     // the diagonal-part operator takes u = h - e_m on centred rows
     const float v0 = ws0 * (cs[t2] == col ? h0 - 1.0f : h0);
     const float v1 = ws1 * (cs[t2 + 1] == col ? h1 - 1.0f : h1);
-    const int64_t o = ((int64_t)blockIdx.x * cpb + col) * 64 + t2;
+    const int64_t o = (kb * cpb + col) * 64 + t2;
     if (Ahi) {
       const __nv_bfloat162 hi = __floats2bfloat162_rn(v0, v1);
       *reinterpret_cast<__nv_bfloat162*>(Ahi + o) = hi;
@@ -2665,7 +2657,8 @@ static int32_t tc_labelled_blocks(firal_problem* P) {
   FIRAL_TRY(P->S_lab.ensure((size_t)per * sizeof(float)));
   FIRAL_TRY(P->w_lab.ensure((size_t)P->N * sizeof(float)));
   FIRAL_TRY(fill_weights(false, P->w_lab.p, m, 1.0, nullptr, 0.0, P->n, st));
-  FIRAL_TRY(P->syrk_part.ensure((size_t)per * sizeof(float)));
+  const int npq = (npairs + 3) / 4 * 4;
+  FIRAL_TRY(P->syrk_part.ensure((size_t)c * npq * sizeof(float)));
   FIRAL_TRY(P->Aw.ensure((size_t)3 * asz * 2));
   bf16* Ahi = P->Aw.as<bf16>();
   bf16* Alo = Ahi + asz;
@@ -2683,11 +2676,11 @@ static int32_t tc_labelled_blocks(firal_problem* P) {
   FIRAL_TRY(make_map(&mZ1, P->Zp.as<bf16>() + npp * Np, zrows, BK, BN, BK, true));
   const int tiles = n_mt * n_nt;
   k_tc_bsum<0><<<std::min(tiles, P->sms), 256, Cfg<0>::SMEM, st>>>(
-      mA0, mA1, mZ0, mZ1, P->syrk_part.as<float>(), c, d, npairs, n_mt, n_nt, 1, kbm, kbm,
+      mA0, mA1, mZ0, mZ1, P->syrk_part.as<float>(), c, npq, n_mt, n_nt, 1, kbm, kbm,
       tc_error_word(P), nullptr, 0);
   FIRAL_CUDA_TRY(cudaGetLastError());
-  FIRAL_TRY(syrk_reduce_f32(P, P->syrk_part.as<float>(), nullptr, 1, 0.0, P->S_lab.as<float>(),
-                            0.0, nullptr));
+  FIRAL_TRY(pair_blocks_f32(P, P->syrk_part.as<float>(), nullptr, npq, 1, 0.0,
+                            P->S_lab.as<float>(), 0.0, nullptr, nullptr));
   P->slab_ready = true;
   return FIRAL_OK;
 }
@@ -2730,7 +2723,8 @@ int32_t tc_syrk_blocks(firal_problem* P, const void* wv, double lamS, void* outS
   const int64_t kbps = (kL + splits - 1) / splits;
   splits = (int)((kL + kbps - 1) / kbps);
   P->tune_used.bsum_splits = splits;
-  const int64_t per = (int64_t)c * d * d;
+  const int npq = (npairs + 3) / 4 * 4;
+  const int64_t per = (int64_t)c * npq;
   FIRAL_TRY(P->syrk_part.ensure((size_t)per * splits * 2 * sizeof(float)));
   float* pS = P->syrk_part.as<float>();
   float* pP = pS + per * splits;
@@ -2756,7 +2750,7 @@ int32_t tc_syrk_blocks(firal_problem* P, const void* wv, double lamS, void* outS
     const bool lab_sep = s1 && outS && sig && P->m > 0 && lab_rows(P) == 0;
     if (lab_sep && !P->slab_ready) FIRAL_TRY(tc_labelled_blocks(P));
     count_launch(1 + (outS ? 1 : 0) + (outP ? 1 : 0));
-    k_weighted_hT<<<dim3((unsigned)(Np / 64), (unsigned)(cpb / 32)), dim3(32, 8), 0, st>>>(
+    k_weighted_hT<<<dim3((unsigned)kL, (unsigned)(cpb / 32)), dim3(32, 8), 0, st>>>(
         outS ? Ahi : nullptr, s1 ? nullptr : Alo, outP ? AP : nullptr, P->Ha.as<float>(), w,
         P->N, c, Np, cpb,
         P->n_cen > 0 ? P->cen.as<int>() : nullptr, lab_sep ? P->m : lab_rows(P),
@@ -2773,26 +2767,26 @@ int32_t tc_syrk_blocks(firal_problem* P, const void* wv, double lamS, void* outS
     const int grid = std::min(units, sms);
     if (outS && s1) {
       // one product: A_hi against the pair operand's bf16 part
-      k_tc_bsum<1><<<grid, 256, Cfg<1>::SMEM, st>>>(mA0, mA0, mZ0, mZ0, pS, c, d, npairs, n_mt,
+      k_tc_bsum<1><<<grid, 256, Cfg<1>::SMEM, st>>>(mA0, mA0, mZ0, mZ0, pS, c, npq, n_mt,
                                                     n_nt, splits, kbps, kb_total,
                                                     tc_error_word(P), P->kr_bsum.as<int4>(),
                                                     P->kbL);
       FIRAL_CUDA_TRY(cudaGetLastError());
     } else if (outS) {
-      k_tc_bsum<0><<<grid, 256, Cfg<0>::SMEM, st>>>(mA0, mA1, mZ0, mZ1, pS, c, d, npairs, n_mt,
+      k_tc_bsum<0><<<grid, 256, Cfg<0>::SMEM, st>>>(mA0, mA1, mZ0, mZ1, pS, c, npq, n_mt,
                                                     n_nt, splits, kbps, kb_total,
                                                     tc_error_word(P), P->kr_bsum.as<int4>(),
                                                     P->kbL);
       FIRAL_CUDA_TRY(cudaGetLastError());
     }
     if (outP) {
-      k_tc_bsum<1><<<grid, 256, Cfg<1>::SMEM, st>>>(mA2, mA2, mZ0, mZ0, pP, c, d, npairs, n_mt,
+      k_tc_bsum<1><<<grid, 256, Cfg<1>::SMEM, st>>>(mA2, mA2, mZ0, mZ0, pP, c, npq, n_mt,
                                                     n_nt, splits, kbps, kb_total,
                                                     tc_error_word(P), P->kr_bsum.as<int4>(),
                                                     P->kbL);
       FIRAL_CUDA_TRY(cudaGetLastError());
     }
-    return syrk_reduce_f32(P, outS ? pS : nullptr, outP ? pP : nullptr, splits, lamS,
+    return pair_blocks_f32(P, outS ? pS : nullptr, outP ? pP : nullptr, npq, splits, lamS,
                            (float*)outS, lamP, outP, lab_sep ? P->S_lab.as<float>() : nullptr);
   }
 }
