@@ -608,7 +608,7 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
                const float* __restrict__ hrow = nullptr, int c = 0, int64_t m = 0,
                float gscale = 0.0f, const int* __restrict__ cen = nullptr,
                const float* __restrict__ cen_am = nullptr, float* __restrict__ cen_rho = nullptr,
-               int64_t wskip = 0) {
+               int64_t wskip = 0, int nkl = 64, const __grid_constant__ CUtensorMap mapPL = {}) {
   using namespace alpha_cfg;
   // MODE 3 stages hold the x tile and two 128-row coefficient tiles (hi and lo), followed by
   // a double buffer of f32 h tiles
@@ -778,12 +778,14 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
           break;
         }
         unsigned char* st = sm + stage * SB;
-        mbar_expect_tx(&ctl->full[stage], SB);
+        const bool lastc = Q3 && cu.chunk == nkcq - 1;   // the narrower last chunk
+        mbar_expect_tx(&ctl->full[stage], lastc ? 4 * nkl * 128 : SB);
         if (Q3) {
           // coefficient tiles of (probe j, chunk kc) sit at row block (j nkc + kc) 2 + hl
           const int ntc = KCM ? cu.probe * nkcq + cu.chunk : nt;
-          tma_load_2d(st, &mapP, &ctl->full[stage], kb * BK, (2 * ntc) * 128);
-          tma_load_2d(st + C3_BYTES, &mapP, &ctl->full[stage], kb * BK, (2 * ntc + 1) * 128);
+          const CUtensorMap* mc = lastc ? &mapPL : &mapP;
+          tma_load_2d(st, mc, &ctl->full[stage], kb * BK, (2 * ntc) * 128);
+          tma_load_2d(st + C3_BYTES, mc, &ctl->full[stage], kb * BK, (2 * ntc + 1) * 128);
         } else {
           tma_load_2d(st, &mapH, &ctl->full[stage], kb * BK, mt * BM);
           if (HLO) tma_load_2d(st + A_BYTES, &mapHL, &ctl->full[stage], kb * BK, mt * BM);
@@ -812,7 +814,8 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
     uint64_t* turn = ctl->yfull;   // MODE 4 issuer tokens (the D-GEMM's y barriers, unused here)
     int nturn = 0;                 // token waits done by this issuer
     bool first_tile = true;
-    constexpr uint32_t idesc = idesc_bf16_f32(BM, Q3 ? 128 : BN);
+    constexpr uint32_t idesc_all = idesc_bf16_f32(BM, Q3 ? 128 : BN);
+    const uint32_t idesc_last = idesc_bf16_f32(BM, 2 * nkl);
     int stage = 0;
     uint32_t phase = 0;
     int acc = 0;
@@ -861,6 +864,7 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
       first_tile = false;
       tc_fence_after();
       const uint32_t d = tmem + acc * ACC_COLS;
+      const uint32_t idesc = Q3 && cu.chunk == nkcq - 1 ? idesc_last : idesc_all;
       bool ok = true;
       for (int kb = kb_lo; kb < kb_hi; ++kb) {
         if (!wait(&ctl->full[stage], phase)) {
@@ -940,8 +944,10 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
       const int64_t row = (int64_t)mt * BM + q * 32 + lane;
       if (Q3) {
         // per-point quadratic forms (eq. 11) from a = x.A_j[:,k], b = x.B_j[:,k] (K = d), the
-        // hi and lo coefficient products summed in TMEM; 64 classes per tile, columns
-        // [a (64) | b (64)]; term 1 = sum_k h a b, term 2 = (sum_k h a)(sum_k h b) with the
+        // hi and lo coefficient products summed in TMEM; nk = 64 classes per tile (nkl, a multiple
+        // of 8, in the last chunk: at 100 classes 208 columns instead of 256, 316 -> 300 us at
+        // n = 200,000, d = 128, s = 16), columns
+        // [a (nk) | b (nk)]; term 1 = sum_k h a b, term 2 = (sum_k h a)(sum_k h b) with the
         // exact f32 h, staged by TMA in 128-byte-swizzled boxes of 32 classes
         const int kc = cu.kr;   // position of the tile's chunk in this point tile's order
         const int hi = cu.hi;
@@ -958,11 +964,12 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
         const uint32_t tb = tmem + ((uint32_t)(q * 32) << 16) + acc * ACC_COLS;
         const unsigned char* hbuf = sm + HBUF + hb * H3_BYTES;
         const int r = q * 32 + lane;
+        const int nk = cu.chunk == nkc - 1 ? nkl : 64;
 #pragma unroll 1
-        for (int box = 0; box < (own ? 2 : 0); ++box) {
+        for (int box = 0; box < (own ? (nk + 31) / 32 : 0); ++box) {
           uint32_t ra[32], rb[32];
           tmem_ld32_async(tb + box * 32, ra);
-          tmem_ld32_async(tb + 64 + box * 32, rb);
+          tmem_ld32_async(tb + nk + box * 32, rb);
           // h of classes (2u, 2u + 1) as one packed pair
           uint64_t hv[16];
           const unsigned char* hrow_s = hbuf + box * (H3_BYTES / 2) + r * 128;
@@ -974,6 +981,11 @@ __global__ void __launch_bounds__(MODE == 4 ? 384 : 256, 1)
             hv[2 * ch + 1] = h4.y;
           }
           tmem_wait_ld();
+          if (nk - box * 32 < 32) {   // columns past nk hold other values: their classes add zero
+#pragma unroll
+            for (int t = 0; t < 32; ++t)
+              if (t >= nk - box * 32) ra[t] = rb[t] = 0;
+          }
           // four partial sums per quantity (classes t mod 4), two per packed pair: short
           // dependency chains, half the f32 instructions of the scalar form
           uint64_t pab[2] = {0, 0}, pa[2] = {0, 0}, pb[2] = {0, 0};
@@ -2801,22 +2813,23 @@ int32_t tc_syrk_blocks(firal_problem* P, const void* wv, double lamS, void* outS
 // term2 from the alpha-GEMM on [A; B] with f32 output (MODE 1).
 // ------------------------------------------------------------------------------------------
 // Coefficient rows of the feature-contracted quadratic forms: row ((j nkc + kc) 2 + hl) 128 + r
-// holds, over the features e < dp, the class-mean-projected A_j (r < 64, class 64 kc + r) or
-// B_j (r >= 64, class 64 kc + r - 64), as bf16 hi (hl = 0) or lo (hl = 1); zero for classes
-// >= c or e >= d.  means: [A; B] class means, (2 s) x pools x d.
+// holds, over the features e < dp, the class-mean-projected A_j (r < nk, class 64 kc + r) or
+// B_j (nk <= r < 2 nk, class 64 kc + r - nk), as bf16 hi (hl = 0) or lo (hl = 1); zero for classes
+// >= c or e >= d.  nk = 64, in the last chunk nkl.  means: [A; B] class means, (2 s) x pools x d.
 __global__ void k_build_coef(bf16* Cf, const float* A, const float* B, const float* mean, int s,
-                             int c, int d, int dp, int64_t D, int nkc, PoolTab pt) {
+                             int c, int d, int dp, int64_t D, int nkc, int nkl, PoolTab pt) {
   const int rb = blockIdx.x;                 // ((j nkc + kc) 2 + hl)
   const int hl = rb & 1, kc = (rb >> 1) % nkc, j = (rb >> 1) / nkc;
   const int Qe = pool_count(pt);
   for (int idx = threadIdx.x; idx < 128 * dp; idx += blockDim.x) {
     const int r = idx / dp, e = idx - r * dp;
-    const bool isb = r >= 64;
-    const int k = kc * 64 + (isb ? r - 64 : r);
+    const int nk = kc == nkc - 1 ? nkl : 64;
+    const bool isb = r >= nk;
+    const int k = kc * 64 + (isb ? r - nk : r);
     const float* src = isb ? B : A;
     const int jm = isb ? s + j : j;
     float v = 0.0f;
-    if (k < c && e < d)
+    if (r < 2 * nk && k < c && e < d)
       v = src[(int64_t)j * D + (int64_t)k * d + e] - mean[(jm * Qe + pool_of(pt, k)) * d + e];
     const bf16 hi = __float2bfloat16_rn(v);
     Cf[((int64_t)rb * 128 + r) * dp + e] = hl ? __float2bfloat16_rn(v - __bfloat162float(hi)) : hi;
@@ -3386,12 +3399,13 @@ static int32_t tc_quad_t(firal_problem* P, const float* A, const float* B, int s
     // bf16, A and B as hi + lo); the epilogue forms sum_k h a b - (sum_k h a)(sum_k h b)
     // with the exact f32 h row and accumulates over the probes (MODE 3)
     const int nkc = cp / 64;
+    const int nkl = (c - (nkc - 1) * 64 + 7) / 8 * 8;   // classes of the last chunk
     const int64_t crow = (int64_t)s * nkc * 2 * 128;
     FIRAL_TRY(P->gq_m.ensure((size_t)crow * DP * 2));
     count_launch(2);
     k_build_coef<<<(unsigned)(s * nkc * 2), 256, 0, st>>>(P->gq_m.as<bf16>(), AB, AB + (size_t)s * D,
                                                          P->vmean.as<float>(), s, c, d, DP, D,
-                                                         nkc, P->pt);
+                                                         nkc, nkl, P->pt);
     FIRAL_CUDA_TRY(cudaGetLastError());
     // s <= 16: class-chunk-major order (MODE 4), each h tile loaded once per chunk
     const bool kcm = s <= S4MAX;
@@ -3408,9 +3422,10 @@ static int32_t tc_quad_t(firal_problem* P, const float* A, const float* B, int s
                                             SMEM3(DP)));
       attr3[a3] = true;
     }
-    CUtensorMap mX, mC, mHf;
+    CUtensorMap mX, mC, mCL, mHf;
     FIRAL_TRY(make_map(&mX, P->Xb.p, Np, DP, BM, BK, true));
     FIRAL_TRY(make_map(&mC, P->gq_m.p, crow, DP, 128, BK, true));
+    FIRAL_TRY(make_map(&mCL, P->gq_m.p, crow, DP, 2 * nkl, BK, true));
     FIRAL_TRY(make_map_f32(&mHf, P->Ha.p, P->N, c, BM));
     const int n_mt = (int)(Np / BM), n_nt = s * nkc;
     if (kcm) {
@@ -3418,11 +3433,13 @@ static int32_t tc_quad_t(firal_problem* P, const float* A, const float* B, int s
       FIRAL_CUDA_TRY(cudaMemsetAsync(g, 0, (size_t)P->n * sizeof(float), st));
       k_tc_alpha<DP, 4, 2, 0><<<std::min(n_mt, sms), 384, SMEM4(DP), st>>>(
           mX, mC, mHf, P->Xb.as<bf16>(), nullptr, nullptr, g, P->N, Np, s, DP / BK, n_mt, n_nt,
-          0, d, tc_error_word(P), nullptr, P->Ha.as<float>(), c, P->m, (float)(scale / s));
+          0, d, tc_error_word(P), nullptr, P->Ha.as<float>(), c, P->m, (float)(scale / s), nullptr,
+          nullptr, nullptr, 0, nkl, mCL);
     } else {
       k_tc_alpha<DP, 3, 2, 0><<<std::min(n_mt, sms), 256, SMEM3(DP), st>>>(
           mX, mC, mHf, P->Xb.as<bf16>(), nullptr, nullptr, g, P->N, Np, s, DP / BK, n_mt, n_nt,
-          0, d, tc_error_word(P), nullptr, P->Ha.as<float>(), c, P->m, (float)(scale / s));
+          0, d, tc_error_word(P), nullptr, P->Ha.as<float>(), c, P->m, (float)(scale / s), nullptr,
+          nullptr, nullptr, 0, nkl, mCL);
     }
     FIRAL_CUDA_TRY(cudaGetLastError());
     return FIRAL_OK;
