@@ -125,3 +125,28 @@ def test_pooled_rows_from_every_storage_type(api, handle, x_dtype, h_dtype):
         e_pooled = float((z.double() - z32).norm() / z32.norm())
         e_single = float((single("mixed") - z32).norm() / z32.norm())
         assert e_pooled < 1.25 * e_single + 1e-5, (e_pooled, e_single)
+
+
+@pytest.mark.parametrize("n,d,c", [(17000, 128, 4), (8500, 128, 9)])
+def test_block_sums_in_several_passes(api, handle, n, d, c):
+    """FP32 block sums whose operands exceed one pass (512 MiB; the second shape stays within it):
+    the diagonal part S through one Hessian apply, against float64 with the sum bound (n + m + d +
+    c + 8 roundings of f32 on the magnitudes)."""
+    p = make_problem(n, d, c, seed=c, x_dtype="float32", h_dtype="float32")
+    prob = api.Problem(handle, dev(p.X), dev(p.h), dev(p.Xo), dev(p.ho), p.lam, precision="fp32")
+    g = torch.Generator(device="cuda").manual_seed(c)
+    z = torch.rand(n, generator=g, device="cuda", dtype=torch.float32) / n
+    V = torch.randn((2, c * d), generator=g, device="cuda", dtype=torch.float32)
+    out = prob.hessian_apply(V, z).double().reshape(2, c, d)
+    X = torch.cat([dev(p.Xo), dev(p.X)]).double()
+    h = torch.cat([dev(p.ho), dev(p.h)]).double()
+    w = torch.cat([torch.ones(len(p.Xo), device="cuda", dtype=torch.float64), z.double()])
+    Vd = V.double().reshape(2, c, d)
+
+    def form(X, V, sign):
+        t = torch.einsum("ie,ske->isk", X, V)
+        al = torch.einsum("isk,ik->is", t, h)
+        return torch.einsum("isk,ie->ske", (t + sign * al[:, :, None]) * (w[:, None] * h)[:, None],
+                            X) + p.lam * V
+    ref, mag = form(X, Vd, -1.0), form(X.abs(), Vd.abs(), 1.0)
+    assert bool(((out - ref).abs() <= (len(w) + d + c + 8) * 2.0 ** -23 * mag).all())
