@@ -574,6 +574,7 @@ int32_t problem_create_impl(firal_handle* H, const firal_pool* pool, const firal
   if (stacked) {
     const size_t tb = stacked->size() * sizeof(StackRows);
     TRYC(P->stack_tab.ensure(tb));
+    P->stack_n = (int)stacked->size();
     if (cudaMemcpyAsync(P->stack_tab.p, stacked->data(), tb, cudaMemcpyHostToDevice, st) !=
         cudaSuccess)
       return cleanup(fail(FIRAL_ERR_CUDA, "copy of the pools' row table"));

@@ -214,6 +214,7 @@ struct firal_problem {
   firal::DBuf vmean, qmean;      // class means of the probe block / of the raw apply (s x d)
   firal::DBuf Aw;                // block sums: (w h)^T hi, lo and (w h (1 - h))^T (3 x cp x Np)
   firal::DBuf stack_tab;         // pooled problems: the StackRows the rows came from
+  int stack_n = 0;
   firal::DBuf Zp;                // block sums: x (x) x on the pair triangle, bf16 hi and lo
   firal::DBuf gq_ab, gq_m, gq_part;  // tensor-core quadratic forms: [A;B], M~ pairs, partials
   firal::DBuf rtab, rM;          // Round on tensor cores: 8-pair chunk table, M~ hi/lo rows
@@ -280,6 +281,7 @@ int32_t stack_rows(bool dbl, void* X, void* H, const StackRows* tab, int nent, i
                    int C, int32_t x_dtype, int32_t h_dtype, cudaStream_t st);
 int32_t transpose(bool dbl, void* dst, const void* src, int64_t rows, int cols, cudaStream_t st);
 int32_t class_major_h(firal_problem* P);
+int32_t class_major_own(firal_problem* P);   // pooled, f32: the rows' own pools' classes only
 int32_t fill_weights(bool dbl, void* w, int64_t m, double lab_val, const void* z, double zconst,
                      int64_t n, cudaStream_t st);
 int32_t probes(bool dbl, void* V, uint64_t seed, int64_t t, int s, int64_t D, cudaStream_t st,

@@ -5,16 +5,18 @@
 //                forms (eq. 11) and the eq. 14 scores of Round
 //   k_row_form_d the first two in FP64
 //   k_row_outer  sums over the rows of A[i][m] B[i][n]: the low-rank part of the Hessian apply
-//                (m = (probe, class), n = feature) and the weighted block sums of eq. 13
-//                (m = class, n = pair of features)
+//                (m = (probe, class), n = feature), in FP64 also the weighted block sums of
+//                eq. 13 (m = class, n = pair of features)
+//   k_outer_gemm the f32 block sums and Exact-FIRAL's dense sums, operands written out first
+//   k_block_ord  the f32 block sums with every addition in a fixed order
 //
-// Both are dense products with one operand made on the fly.  f32: 8 x 8 outputs per thread from
-// shared memory, plain fmaf: the packed form (fma.rn.f32x2) has the same peak on this part and
-// needs one operand duplicated, which cost more in shared-memory reads than it saved in issue
-// slots (43 against 53 TFLOP/s with operands resident).  FP64: the part issues two FP64
-// multiply-adds per SM and cycle, so operand traffic is free and what counts is that no lane
-// multiplies padding and every SM has work; tiles are 2 x 2 outputs per thread with the tile's
-// width taken from the problem instead of a power of two.
+// All are dense products.  f32: 8 x 8 or 8 x 16 outputs per thread from shared memory, plain
+// fmaf: the packed form (fma.rn.f32x2) has the same peak on this part and needs one operand
+// duplicated, which cost more in shared-memory reads than it saved in issue slots (43 against 53
+// TFLOP/s with operands resident).  FP64: the part issues two FP64 multiply-adds per SM and
+// cycle, so operand traffic is free and what counts is that no lane multiplies padding and every
+// SM has work; tiles are 2 x 2 outputs per thread with the tile's width taken from the problem
+// instead of a power of two.
 #include <cuda_bf16.h>
 
 #include <algorithm>

@@ -224,6 +224,50 @@ int32_t class_major_h(firal_problem* P) {
   return transpose(P->dbl, P->HaT.p, P->Ha.p, P->N, P->c, P->H->stream);
 }
 
+// The class-major h of a pooled problem where its own kernels read it: each row's own pool's
+// classes (at most 32), 32 rows a block; the rest of the array stays unwritten.  64 pools of 1.4 M
+// rows: 0.91 ms as a transposition of all 1.7 GB, below 0.2 here.
+__global__ void __launch_bounds__(256) k_class_major_own(float* __restrict__ dst,
+                                                         const float* __restrict__ src,
+                                                         const StackRows* __restrict__ tab,
+                                                         int nent, int64_t N, int C) {
+  __shared__ float tile[32][33];
+  __shared__ int c0s[32], cs[32];
+  const int64_t rb = (int64_t)blockIdx.x * 32;
+  if (threadIdx.x < 32 && rb + threadIdx.x < N) {
+    const int64_t r = rb + threadIdx.x;
+    int lo = 0, hi = nent - 1;
+    while (lo < hi) {
+      const int mid = (lo + hi + 1) >> 1;
+      if (tab[mid].row0 <= r) lo = mid;
+      else hi = mid - 1;
+    }
+    c0s[threadIdx.x] = tab[lo].c0;
+    cs[threadIdx.x] = tab[lo].c;
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int i = warp + 8 * u;
+    if (rb + i < N && lane < cs[i]) tile[i][lane] = src[(rb + i) * C + c0s[i] + lane];
+  }
+  __syncthreads();
+  if (rb + lane < N)
+    for (int k = warp; k < cs[lane]; k += 8) dst[(int64_t)(c0s[lane] + k) * N + rb + lane] = tile[lane][k];
+}
+
+int32_t class_major_own(firal_problem* P) {
+  if (P->HaT.p) return FIRAL_OK;
+  FIRAL_TRY(P->HaT.ensure((size_t)P->N * P->c * sizeof(float)));
+  ProfScope ps(P->H->stream, PF_PREP);
+  count_launch();
+  k_class_major_own<<<(unsigned)((P->N + 31) / 32), 256, 0, P->H->stream>>>(
+      P->HaT.as<float>(), P->Ha.as<float>(), P->stack_tab.as<StackRows>(), P->stack_n, P->N, P->c);
+  FIRAL_CUDA_TRY(cudaGetLastError());
+  return FIRAL_OK;
+}
+
 // weights over all rows: [lab_val] * m, then z (or zconst) on the pool rows
 template <class T>
 __global__ void k_fill_w(T* w, int64_t m, T lab_val, const T* z, T zconst, int64_t n) {

@@ -1744,61 +1744,44 @@ __global__ void __launch_bounds__(256, 1)
 // Z[p][i] = x_ie x_ie' for pair p = (e, e') of the row-major triangle, as bf16 hi and lo (exact);
 // rows p >= npairs and columns of padding points are zero.  K-block-major layout
 // [i / 64][p][i % 64] (npp rows per block): every 128 x 64 TMA tile is one contiguous 16 KB
-// run.  Block = 64 points (staged point-major in shared memory) x every pair; a thread takes
-// pairs p, p + 256, ... (consecutive threads read consecutive e' of the staged rows) and
-// writes each pair's 64 points as four 32-byte pieces.  Zlo may be NULL: the lo part is left out.
+// run.  Block = 64 points (staged feature-major in shared memory) x every pair; a thread makes
+// 8 points of a pair (one 16-byte load per factor), and the 8 threads of a pair write its 128-byte
+// row together.  Bound by the writes: 5.0 GB for 64 pools (Z_hi alone) took 1.39 ms when a thread
+// wrote a pair's whole row in four pieces, 0.94 here.  Zlo may be NULL: the lo part is left out.
 __global__ void __launch_bounds__(256) k_build_z(bf16* Zhi, bf16* Zlo, const bf16* Xb, int d,
                                                  int dp, int npairs, int64_t npp) {
-  __shared__ __align__(16) bf16 xs[64 * 128];
+  constexpr int LD = 72;   // points of a feature: 144-byte rows, 16-byte aligned
+  __shared__ __align__(16) bf16 xs[128 * LD];
   const int64_t i0 = (int64_t)blockIdx.x * 64;
-  {
-    const uint4* src = reinterpret_cast<const uint4*>(Xb + i0 * dp);
-    uint4* dst = reinterpret_cast<uint4*>(xs);
-    for (int t = threadIdx.x; t < 64 * dp / 8; t += blockDim.x) dst[t] = src[t];
+  for (int t = threadIdx.x; t < 64 * dp / 2; t += blockDim.x) {
+    const int i = t / (dp / 2), e = t % (dp / 2) * 2;
+    const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162*>(Xb + (i0 + i) * dp + e);
+    xs[e * LD + i] = v.x;
+    xs[(e + 1) * LD + i] = v.y;
   }
   __syncthreads();
-  const int d2 = 2 * d + 1;
-  for (int p = threadIdx.x; p < npp; p += blockDim.x) {
-    // row e of the triangle: the largest e with e d - e (e - 1) / 2 <= p
-    int e = 0, e2 = 0;
-    const bool real = p < npairs;
-    if (real) {
-      e = (int)((d2 - sqrtf((float)(d2 * d2 - 8 * p))) * 0.5f);
-      e = e < 0 ? 0 : (e >= d ? d - 1 : e);
-      while (e > 0 && e * d - e * (e - 1) / 2 > p) --e;
-      while (e + 1 < d && (e + 1) * d - (e + 1) * e / 2 <= p) ++e;
-      e2 = e + (p - (e * d - e * (e - 1) / 2));
-    }
-    bf16* zh = Zhi + ((int64_t)blockIdx.x * npp + p) * 64;
-    bf16* zl = Zlo ? Zlo + ((int64_t)blockIdx.x * npp + p) * 64 : nullptr;
-#pragma unroll 1
-    for (int c16 = 0; c16 < 4; ++c16) {
-      uint4 hv[2], lv[2];
+  const int g = threadIdx.x & 7;   // points 8 g .. 8 g + 7
+  for (int p = threadIdx.x >> 3; p < npp; p += 32) {
+    uint4 hv = make_uint4(0, 0, 0, 0), lv = make_uint4(0, 0, 0, 0);
+    if (p < npairs) {
+      int e, e2;
+      feature_pair(p, d, e, e2);
+      const uint4 a = *reinterpret_cast<const uint4*>(xs + e * LD + 8 * g);
+      const uint4 b = *reinterpret_cast<const uint4*>(xs + e2 * LD + 8 * g);
+      const bf16* x = reinterpret_cast<const bf16*>(&a);
+      const bf16* y = reinterpret_cast<const bf16*>(&b);
+      bf16* h = reinterpret_cast<bf16*>(&hv);
+      bf16* l = reinterpret_cast<bf16*>(&lv);
 #pragma unroll
-      for (int hh = 0; hh < 2; ++hh) {
-        hv[hh] = make_uint4(0, 0, 0, 0);
-        lv[hh] = make_uint4(0, 0, 0, 0);
-        if (real) {
-          bf16* h = reinterpret_cast<bf16*>(&hv[hh]);
-          bf16* l = reinterpret_cast<bf16*>(&lv[hh]);
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int i = c16 * 16 + hh * 8 + q;
-            const float z = __bfloat162float(xs[i * dp + e]) * __bfloat162float(xs[i * dp + e2]);
-            h[q] = __float2bfloat16_rn(z);
-            l[q] = __float2bfloat16_rn(z - __bfloat162float(h[q]));
-          }
-        }
-      }
-      uint4* oh = reinterpret_cast<uint4*>(zh + c16 * 16);
-      oh[0] = hv[0];
-      oh[1] = hv[1];
-      if (Zlo) {
-        uint4* ol = reinterpret_cast<uint4*>(zl + c16 * 16);
-        ol[0] = lv[0];
-        ol[1] = lv[1];
+      for (int q = 0; q < 8; ++q) {
+        const float z = __bfloat162float(x[q]) * __bfloat162float(y[q]);
+        h[q] = __float2bfloat16_rn(z);
+        l[q] = __float2bfloat16_rn(z - __bfloat162float(h[q]));
       }
     }
+    const int64_t o = ((int64_t)blockIdx.x * npp + p) * 64 + 8 * g;
+    *reinterpret_cast<uint4*>(Zhi + o) = hv;
+    if (Zlo) *reinterpret_cast<uint4*>(Zlo + o) = lv;
   }
 }
 
@@ -1808,15 +1791,17 @@ __global__ void __launch_bounds__(256) k_build_z(bf16* Zhi, bf16* Zlo, const bf1
 // (A_hi only if Ahi, A_lo only if Ahi and Alo, A_P only if AP)
 // with u = h, or u = h - e_m on centred rows (cen, may be NULL); rows below wskip take weight
 // 0 in A_hi and A_lo (their part of the Hessian apply runs on CUDA cores).
-// Block = one 64-point block x 32 classes; each warp store writes one 128-byte row run.
+// Block = one 64-point block x 64 classes, h read as 256-byte runs of 16-byte loads (single values
+// where the rows are not aligned); each warp store writes one 128-byte row run.  Bound by HBM:
+// 8 GB at n = 1M, c = 1000 (h once, A_hi and A_P) 2.33 ms with 32 classes of single loads, 1.42 here.
 __global__ void k_weighted_hT(bf16* Ahi, bf16* Alo, bf16* AP, const float* Ha, const float* w,
                               int64_t N, int c, int64_t Np, int cpb, const int* cen,
                               int64_t wskip, const int4* klist = nullptr, int kbL = 0) {
-  __shared__ float tile[64][33];
+  __shared__ float tile[64][65];
   __shared__ float ws[64], wS[64];
   __shared__ int cs[64];
   int64_t kb = blockIdx.x;
-  const int cb = blockIdx.y * 32;
+  const int cb = blockIdx.y * 64;
   // pooled: the block sums read, for each 128-class tile, the labelled rows' K-steps and its
   // pools' K-steps only (K list {first, end, steps in all, ..}); the others stay unwritten.  The
   // grid holds the longest list, not every K-step: 200,000 mostly empty blocks took 160 us a
@@ -1827,12 +1812,35 @@ __global__ void k_weighted_hT(bf16* Ahi, bf16* Alo, bf16* AP, const float* Ha, c
     if (kb >= kbL) kb = kl.x + (kb - kbL);
   }
   const int64_t rb = kb * 64;
-  for (int i = threadIdx.y; i < 64; i += blockDim.y) {
-    const int64_t r = rb + i;
-    const int col = cb + threadIdx.x;
-    tile[i][threadIdx.x] = (r < N && col < c) ? Ha[r * c + col] : 0.0f;
+  const int tid = threadIdx.y * 32 + threadIdx.x;
+  if ((c & 3) == 0) {   // (Ha starts on a 16-byte boundary)
+    float4 v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t r = rb + (tid >> 4) + 16 * u;
+      const int col = cb + (tid & 15) * 4;
+      v[u] = (r < N && col < c) ? *reinterpret_cast<const float4*>(Ha + r * c + col)
+                                : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      float* t = &tile[(tid >> 4) + 16 * u][(tid & 15) * 4];
+      t[0] = v[u].x;
+      t[1] = v[u].y;
+      t[2] = v[u].z;
+      t[3] = v[u].w;
+    }
+  } else {
+    float v[16];
+    const int col = cb + (tid & 63);
+#pragma unroll
+    for (int u = 0; u < 16; ++u) {
+      const int64_t r = rb + (tid >> 6) + 4 * u;
+      v[u] = (r < N && col < c) ? Ha[r * c + col] : 0.0f;
+    }
+#pragma unroll
+    for (int u = 0; u < 16; ++u) tile[(tid >> 6) + 4 * u][tid & 63] = v[u];
   }
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x;
   if (tid < 64) {
     ws[tid] = rb + tid < N ? w[rb + tid] : 0.0f;
     wS[tid] = rb + tid >= wskip ? ws[tid] : 0.0f;
@@ -1842,7 +1850,8 @@ __global__ void k_weighted_hT(bf16* Ahi, bf16* Alo, bf16* AP, const float* Ha, c
   const int t2 = 2 * threadIdx.x;   // points rb + t2, rb + t2 + 1
   const float w0 = ws[t2], w1 = ws[t2 + 1];
   const float ws0 = wS[t2], ws1 = wS[t2 + 1];
-  for (int i = threadIdx.y; i < 32; i += blockDim.y) {
+#pragma unroll 2
+  for (int i = threadIdx.y; i < 64; i += 8) {
     const int col = cb + i;
     if (col >= cpb) continue;
     const float h0 = tile[t2][i], h1 = tile[t2 + 1][i];
@@ -2677,7 +2686,7 @@ static int32_t tc_labelled_blocks(firal_problem* P) {
   FIRAL_TRY(tc_bsum_launch_attrs());
   ProfScope ps(st, PF_SYRK);
   count_launch(2);
-  k_weighted_hT<<<dim3((unsigned)kbm, (unsigned)(cpb / 32)), dim3(32, 8), 0, st>>>(
+  k_weighted_hT<<<dim3((unsigned)kbm, (unsigned)(cpb / 64)), dim3(32, 8), 0, st>>>(
       Ahi, Alo, nullptr, P->Ha.as<float>(), P->w_lab.as<float>(), P->N, c, Np, cpb, nullptr, 0);
   FIRAL_CUDA_TRY(cudaGetLastError());
   CUtensorMap mA0, mA1, mZ0, mZ1;
@@ -2762,7 +2771,7 @@ int32_t tc_syrk_blocks(firal_problem* P, const void* wv, double lamS, void* outS
     const bool lab_sep = s1 && outS && sig && P->m > 0 && lab_rows(P) == 0;
     if (lab_sep && !P->slab_ready) FIRAL_TRY(tc_labelled_blocks(P));
     count_launch(1 + (outS ? 1 : 0) + (outP ? 1 : 0));
-    k_weighted_hT<<<dim3((unsigned)kL, (unsigned)(cpb / 32)), dim3(32, 8), 0, st>>>(
+    k_weighted_hT<<<dim3((unsigned)kL, (unsigned)(cpb / 64)), dim3(32, 8), 0, st>>>(
         outS ? Ahi : nullptr, s1 ? nullptr : Alo, outP ? AP : nullptr, P->Ha.as<float>(), w,
         P->N, c, Np, cpb,
         P->n_cen > 0 ? P->cen.as<int>() : nullptr, lab_sep ? P->m : lab_rows(P),
@@ -4505,8 +4514,12 @@ int32_t tc_setup_pw(firal_problem* P, const std::vector<int>& coff,
         P->X64.as<bf16>(), P->Xb.as<bf16>(), P->Np, P->dp);
     FIRAL_CUDA_TRY(cudaGetLastError());
   }
-  // h read class-major by the fused kernels (one coalesced run of a tile's rows per class)
-  FIRAL_TRY(class_major_h(P));
+  // h read class-major by the fused kernels (one coalesced run of a tile's rows per class); in a
+  // pooled problem only a row's own pool's classes, so only those are written
+  if (P->pt.Q)
+    FIRAL_TRY(class_major_own(P));
+  else
+    FIRAL_TRY(class_major_h(P));
   // the host vectors are read by the copies
   FIRAL_CUDA_TRY(cudaStreamSynchronize(st));
   P->pw_pool_h = ptab;
