@@ -3624,8 +3624,9 @@ int32_t tc_round_scores(firal_problem* P, const void* M1, const void* M2, const 
 // staged x^T tile (K-major, dp rows).
 // Work list: segments of at most SEG_TILES 128-row tiles of one pool's rows (its labelled
 // rows and its pool rows are separate segments); an item is one probe group of a segment, and
-// the host deals the items to the CTAs longest first (sched: per-CTA offsets, then items as
-// segment GRP_MAX + group), so a single pool of 50,000 rows (49 segments) still fills the chip.
+// the host deals the items to the CTAs longest first (sched: per-CTA offsets, then a pair
+// (segment, group) per item: any number of probes), so a single pool of 50,000 rows (49 segments)
+// still fills the chip.
 // A tile that also holds rows of another pool runs once per pool with the other rows masked.  An item accumulates out in TMEM and writes one partial; a
 // per-class combine adds a pool's partials in segment order.
 // Pipeline: the x and x^T tiles, the S accumulator (TMEM), the psi operand (shared memory) and
@@ -3649,7 +3650,6 @@ constexpr int OFF_PT = 0, OFF_XA = 2 * PT_HALF, OFF_XT = OFF_XA + 2 * XA_BYTES;
 constexpr int OFF_PSI = OFF_XT + 2 * XT_BYTES, OFF_CTL = OFF_PSI + 2 * PSI_BUF;
 constexpr int SMEM = OFF_CTL + 256 + 1024;
 constexpr uint32_t TS = 0, TD = 256;              // TMEM columns: S (2 x 128) | D (2 x 128)
-constexpr int GRP_MAX = 64;   // probe groups of a segment: 32 classes x 256 probes / NU
 }  // namespace pw_cfg
 
 struct PwCtl {   // < 256 bytes
@@ -3659,6 +3659,12 @@ struct PwCtl {   // < 256 bytes
   int abort_w;
 };
 static_assert(sizeof(PwCtl) <= 256, "control block must fit in 256 bytes");
+
+// Item it of the apply's work list: (segment, probe group), from an 8-byte boundary after the CTAs'
+// offsets.
+__device__ __forceinline__ int2 pw_item(const int* sched, int it) {
+  return reinterpret_cast<const int2*>(sched + ((gridDim.x + 2) & ~1u))[it];
+}
 
 // Probe groups of a pool (cpad, sp): ceil(cpad sp / 128); columns of group grp.
 __device__ __forceinline__ int pw_ngrp(int cpad, int sp) {
@@ -3933,8 +3939,9 @@ __global__ void __launch_bounds__(384, 1)
     uint32_t nt = 0, ni = 0;   // tiles and items loaded
     bool ok = true;
     for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
-      const int code = sched[gridDim.x + 1 + it], grp = code & (GRP_MAX - 1);
-      const int4 sg = seg_tab[code / GRP_MAX];
+      const int2 item_sg = pw_item(sched, it);
+      const int grp = item_sg.y;
+      const int4 sg = seg_tab[item_sg.x];
       const int4 pq = pool_tab[sg.x];
       const int n1 = pq.z * sp, pbase = 2 * sp * pq.w;
       const int nc = pw_ncols(pq.z, sp, grp);
@@ -3971,7 +3978,7 @@ __global__ void __launch_bounds__(384, 1)
     uint32_t nt = 0;
     bool ok = true;
     for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
-      const int4 sg = seg_tab[sched[gridDim.x + 1 + it] / GRP_MAX];
+      const int4 sg = seg_tab[pw_item(sched, it).x];
       for (int t = sg.y >> 7; t <= (sg.z - 1) >> 7; ++t) {
         const int b = nt & 1;
         if (!mbar_wait(&ctl->xt_empty[b], ((nt >> 1) & 1) ^ 1, abort_w)) {
@@ -4038,8 +4045,9 @@ __global__ void __launch_bounds__(384, 1)
       return true;
     };
     for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok; ++it) {
-      const int code = sched[gridDim.x + 1 + it], grp = code & (GRP_MAX - 1);
-      const int4 sg = seg_tab[code / GRP_MAX];
+      const int2 item_sg = pw_item(sched, it);
+      const int grp = item_sg.y;
+      const int4 sg = seg_tab[item_sg.x];
       const int4 pq = pool_tab[sg.x];
       const int t0 = sg.y >> 7, t1 = (sg.z - 1) >> 7;
       const int nc = pw_ncols(pq.z, sp, grp);
@@ -4088,8 +4096,9 @@ __global__ void __launch_bounds__(384, 1)
     bool ok = true;
     PwOut out{};
     for (int it = sched[blockIdx.x]; it < sched[blockIdx.x + 1] && ok && !*abort_w; ++it) {
-      const int code = sched[gridDim.x + 1 + it], grp = code & (GRP_MAX - 1);
-      const int4 sg = seg_tab[code / GRP_MAX];
+      const int2 item_sg = pw_item(sched, it);
+      const int grp = item_sg.y;
+      const int4 sg = seg_tab[item_sg.x];
       const int4 pq = pool_tab[sg.x];
       const int nc = pw_ncols(pq.z, sp, grp);
       const PwOut* prev = ni ? &out : nullptr;
@@ -4534,9 +4543,9 @@ int32_t tc_setup_pw(firal_problem* P, const std::vector<int>& coff,
   return FIRAL_OK;
 }
 
-// The CTAs' segment lists for sp padded probes (quad: the gradient, which skips the labelled
-// rows' segments): each segment costs (tiles + 1) x probe groups, and the segments go longest
-// first to the least-loaded CTA (ties to the lowest index), which keeps the slowest CTA within
+// The CTAs' work lists for sp padded probes.  Apply: (segment, probe group) items of cost tiles + 1;
+// gradient (quad): segments, the labelled rows' left out, of cost (tiles + 1) x probe groups.  They
+// go longest first to the least-loaded CTA (ties to the lowest index), which keeps the slowest CTA within
 // a few percent of the mean where striding left it up to 2x.  Made once per (sp, quad), before
 // any graph capture (the first MD step runs eagerly); each CTA walks its list in pool order.
 static int32_t pw_schedule(firal_problem* P, int sp, bool quad, int* grid_out,
@@ -4547,7 +4556,11 @@ static int32_t pw_schedule(firal_problem* P, int sp, bool quad, int* grid_out,
       *sched_out = sc.buf.as<int>();
       return FIRAL_OK;
     }
-  std::vector<std::pair<int64_t, int>> items;
+  struct Item {
+    int64_t cost;
+    int seg, grp;
+  };
+  std::vector<Item> items;
   for (int g = 0; g < (int)P->pw_seg_h.size(); ++g) {
     const int4 sg = P->pw_seg_h[g];
     if (quad && (int64_t)sg.z <= P->m) continue;
@@ -4557,30 +4570,33 @@ static int32_t pw_schedule(firal_problem* P, int sp, bool quad, int* grid_out,
     // apply: an item is one probe group of a segment (each group writes its own partial);
     // gradient: a segment (its groups add to the same entries of g in group order)
     if (quad)
-      items.push_back({(tiles + 1) * ng, g});
+      items.push_back({(tiles + 1) * ng, g, 0});
     else
-      for (int grp = 0; grp < ng; ++grp) items.push_back({tiles + 1, g * pw_cfg::GRP_MAX + grp});
+      for (int grp = 0; grp < ng; ++grp) items.push_back({tiles + 1, g, grp});
   }
   const int grid = std::max(1, std::min<int>(P->sms, (int)items.size()));
   std::stable_sort(items.begin(), items.end(),
-                   [](const std::pair<int64_t, int>& a, const std::pair<int64_t, int>& b) {
-                     return a.first > b.first;
-                   });
-  std::vector<std::vector<int>> lists(grid);
+                   [](const Item& a, const Item& b) { return a.cost > b.cost; });
+  std::vector<std::vector<std::pair<int, int>>> lists(grid);   // (segment, group)
   std::vector<int64_t> load(grid, 0);
   for (const auto& it : items) {
     int best = 0;
     for (int b = 1; b < grid; ++b)
       if (load[b] < load[best]) best = b;
-    lists[best].push_back(it.second);
-    load[best] += it.first;
+    lists[best].push_back({it.seg, it.grp});
+    load[best] += it.cost;
   }
   std::vector<int> tab(grid + 1, 0);
   for (int b = 0; b < grid; ++b) {
     std::sort(lists[b].begin(), lists[b].end());
     tab[b + 1] = tab[b] + (int)lists[b].size();
   }
-  for (int b = 0; b < grid; ++b) tab.insert(tab.end(), lists[b].begin(), lists[b].end());
+  if (!quad && (grid & 1) == 0) tab.push_back(0);   // pw_item's pairs: 8-byte aligned
+  for (int b = 0; b < grid; ++b)
+    for (const auto& it : lists[b]) {
+      tab.push_back(it.first);
+      if (!quad) tab.push_back(it.second);
+    }
   firal_problem::PwSched sc;
   sc.sp = sp;
   sc.quad = quad;
