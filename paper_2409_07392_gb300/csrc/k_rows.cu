@@ -410,6 +410,7 @@ __global__ __launch_bounds__(256, 2) void k_row_outer_f(const OuterArgs<float> a
   }
 }
 
+constexpr size_t OUTER_SMEM = 220 * 1024;   // the most a block of k_row_outer may ask for
 template <int OP>
 size_t outer_smem_d(int GM, int GN, int d, int c) {
   constexpr int BK = OUTER_BK;
@@ -440,7 +441,8 @@ struct OuterPlan {
 };
 
 // The tile takes its width from the outputs (groups of TN columns up to 128 of them), then as
-// many row groups as the block has threads for, both cut to equal tiles, so that little of a
+// many row groups as the block has threads for (FP64: and shared memory, which one column group
+// of up to 512 row groups, d <= 2, exceeds), both cut to equal tiles, so that little of a
 // tile is padding at any class count or feature width (the fixed 64 x 64 tile multiplied 54
 // empty class columns at c = 10: 413 us a launch at n = 50,000, d = 50, s = 20; now 56).
 // Splits: enough blocks for two per SM (one at FP64: 512 threads), whole waves where the row
@@ -462,7 +464,7 @@ OuterPlan outer_plan(const OuterArgs<T>& a, int sms) {
   p.tn = (ng + gn - 1) / gn;
   p.GN = (ng + p.tn - 1) / p.tn;
   int gm = std::min(mg, nt / p.GN);
-  // f32: the block's threads must also cover a step's loads
+  // f32: the block's threads must also cover a step's loads; FP64: the tile must fit
   const int bk = vh == 4 ? 16 : 8, ni = vh == 4 ? 4 : vh == 2 ? 8 : 12, nx = vh == 4 ? 4 : 8;
   for (;; --gm) {
     p.tm = (mg + gm - 1) / gm;
@@ -474,7 +476,8 @@ OuterPlan outer_plan(const OuterArgs<T>& a, int sms) {
       need = std::max({need, (hn + ni - 1) / ni, (xn + nx - 1) / nx});
     }
     p.threads = std::max(128, (need + 31) / 32 * 32);
-    if (p.threads <= nt || gm == 1) break;
+    const bool fits = !dbl || outer_smem_d<OP>(p.GM, p.GN, a.d, a.c) <= OUTER_SMEM;
+    if ((p.threads <= nt && fits) || gm == 1) break;
   }
   const int64_t tiles = (int64_t)p.tm * p.tn;
   const int64_t slots = (int64_t)sms * (dbl ? 1 : 2);
@@ -502,7 +505,7 @@ int32_t outer_launch_f(const OuterArgs<float>& a, const OuterPlan& p, cudaStream
   const int BK = OuterCfg<VH>::BK, BM = p.GM * 8, BN = p.GN * 8;
   const size_t smem = ((size_t)2 * BK * (BM + BN) + BM) * 4;
   FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_outer_f<VH>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, OUTER_SMEM));
   count_launch();
   k_row_outer_f<VH><<<dim3(p.tm, p.tn, p.splits), p.threads, smem, st>>>(a);
   FIRAL_CUDA_TRY(cudaGetLastError());
@@ -516,7 +519,7 @@ int32_t outer_run(OuterArgs<double> a, const OuterPlan& p, cudaStream_t st) {
   a.rps = p.rps;
   const size_t smem = outer_smem_d<OP>(p.GM, p.GN, a.d, a.c);
   FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_outer_d<OP>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, OUTER_SMEM));
   count_launch();
   k_row_outer_d<OP><<<dim3(p.tm, p.tn, p.splits), p.threads, smem, st>>>(a);
   FIRAL_CUDA_TRY(cudaGetLastError());
