@@ -640,10 +640,15 @@ __global__ void k_row_combine(const T* __restrict__ S, const T* __restrict__ V,
 // groups of 4 inner indices of one unit, so its share of a row's sum stays in registers; the
 // groups meet in shared memory once per tile.  Blocks: 128 rows x a range of units
 // (blockIdx.y).
+// MODE 2 adds x_e (x.M_k[e]) over the features as sums of two floats (two_prod, two_sum), which
+// hold what an FP64 sum does: eq. 14 compares points whose scores differ by little, and f32 sums
+// moved them by 1e-8 to 9e-8.  Some 10 f32 instructions a term: a pick takes 620 us at n = 5,000,
+// d = c = 50 (605 with f32 sums), 640 at n = 100,000, d = 16, c = 64 (551).  An FP64 multiply-add and
+// the conversions of its factors would take the FP64 pipe three times as long as the row's products.
 // Bound by issue slots and, per tile, the latency of the row coefficients: 40 TFLOP/s for alpha
 // at n = 21,000, c = 1000, d = 64, s = 16 (1.08 ms; one thread per row took 4.67), the quadratic
 // forms at n = 50,000, d = 50, c = 10, s = 20 100 us (175 before), the eq. 14 scores at
-// n = 5,000, d = c = 50 110 us (2,840 before: 40 blocks, one after another over the classes).
+// n = 5,000, d = c = 50 about 125 us (2,840 before: 40 blocks, one after another over the classes).
 // The coefficient tiles are packed first (k_form_pack), feature-major, so that a step of the
 // main loop is staged by whole 16-byte copies at any alignment.
 // ------------------------------------------------------------------------------------------
@@ -672,6 +677,20 @@ struct FormArgs {
 // features padded to whole steps of 16
 __host__ __device__ inline int form_dk(int d) { return (d + 15) / 16 * 16; }
 
+// hi + lo += b, exactly but for the rounding of lo (two-sum: Knuth, The Art of Computer Programming
+// 2, 4.2.2)
+__device__ __forceinline__ void two_sum(float& hi, float& lo, float b) {
+  const float s = __fadd_rn(hi, b), t = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, t)), __fsub_rn(b, t)));
+  hi = s;
+}
+// hi + lo += x y: the product's rounding error by one fused multiply-add
+__device__ __forceinline__ void two_prod(float& hi, float& lo, float x, float y) {
+  const float p = __fmul_rn(x, y);
+  lo = __fadd_rn(lo, __fmaf_rn(x, y, -p));
+  two_sum(hi, lo, p);
+}
+
 // One thread: one tile column, 8 features.
 template <int MODE>
 __global__ __launch_bounds__(256) void k_form_pack(const FormArgs a, int64_t total) {
@@ -693,19 +712,29 @@ __global__ __launch_bounds__(256) void k_form_pack(const FormArgs a, int64_t tot
       src += ok ? (int64_t)(kl.x * a.d + v) * a.ldm + (int64_t)kl.y * a.d : 0;
     } else {
       if (MODE != 0 && col >= 64) src = a.B;
-      src += ok ? u * a.ustride + (int64_t)v * a.d : 0;
+      src += ok ? u * a.ustride + (MODE == 2 ? v : (int64_t)v * a.d) : 0;
     }
+    // MODE 2 takes column v of M_k (symmetric but for the rounding of its f32 products), in runs of
+    // consecutive threads
+    const int es = MODE == 2 ? a.d : 1;
     float* dst = a.pk + ((int64_t)T * dK + e0) * 128 + col;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) dst[e * 128] = ok && e0 + e < a.d ? src[e0 + e] : 0.0f;
+    for (int e = 0; e < 8; ++e) dst[e * 128] = ok && e0 + e < a.d ? src[(e0 + e) * es] : 0.0f;
   }
 }
+
+__host__ __device__ constexpr int form_nv(int mode) {
+  return mode == 0 || mode == 3 ? 1 : mode == 1 ? 3 : 2;
+}
+__host__ __device__ constexpr int form_ns(int mode) { return mode == 2 ? 4 : form_nv(mode); }
 
 // KC features per step: 16, or 8 where that lets two blocks share an SM
 template <int MODE, int KC>
 __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
   constexpr bool ONE = MODE == 0 || MODE == 3;            // one coefficient block
-  constexpr int NV = ONE ? 1 : MODE == 1 ? 3 : 2;         // values per (row, unit)
+  // values per (row, unit): in red, and in sum as floats (MODE 2: one form at a time as two floats,
+  // two forms as doubles)
+  constexpr int NV = form_nv(MODE), NS = form_ns(MODE);
   constexpr int GC = ONE ? 32 : 16;                       // column groups per tile
   constexpr int LD = FORM_LD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -713,7 +742,8 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
   float* xs = (float*)smem_raw;              // [dK][LD]
   float* vs = xs + (size_t)dK * LD;          // [2][KC][128]
   float* red = vs + 2 * KC * 128;            // [NV][128][GC + 1]
-  float* sum = red + NV * 128 * (GC + 1);    // [NV][UB][128]
+  float* sum = red + NV * 128 * (GC + 1);    // [NV][UB][128] (MODE 2: doubles, [2][UB][128])
+  double* dsum = reinterpret_cast<double*>(sum);
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   // a warp covers 8 column groups x 4 row groups
   const int tx = (wid & 1) * 8 + (lane & 7), ty = (wid >> 1) * 4 + (lane >> 3);
@@ -733,7 +763,7 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
       cp_async<4>(xs + e * LD + r, a.Xa + (ok ? (i0 + r) * d + e : 0), ok);
     }
   }
-  for (int q = tid; q < NV * a.UB * 128; q += 256) sum[q] = 0.0f;
+  for (int q = tid; q < NS * a.UB * 128; q += 256) sum[q] = 0.0f;
   // step kk of tile (cc, p): KC rows of 512 bytes
   auto stage = [&](int cc, int p, int kk, int b) {
     const float* src = a.pk + ((((int64_t)blockIdx.y * a.CC + cc) * tpb + p) * dK + kk * KC) * 128;
@@ -783,6 +813,51 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
         for (int q = 0; q < qn; ++q) multiply(q);
       }
     }
+    if (MODE == 2) {
+      // the two forms one after the other through the same shared sums
+      const int ul = tx / gpu, v = cc * a.kc + (tx - ul * gpu) * 4;
+      const bool uv = ul < a.PJ && u0 + p * a.PJ + ul < u1;
+      float fh[2][8], fl[2][8];
+#pragma unroll
+      for (int x = 0; x < 8; ++x) {
+        const int r = (x / 4) * 64 + ty * 4 + (x & 3);
+        fh[0][x] = fl[0][x] = fh[1][x] = fl[1][x] = 0.0f;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float xe = uv && v + q < a.inner ? xs[(v + q) * LD + r] : 0.0f;
+          two_prod(fh[0][x], fl[0][x], xe, acc[x][q]);
+          two_prod(fh[1][x], fl[1][x], xe, acc[x][4 + q]);
+        }
+      }
+#pragma unroll
+      for (int which = 0; which < 2; ++which) {
+        if (which) __syncthreads();   // the first form's groups have been added
+#pragma unroll
+        for (int x = 0; x < 8; ++x) {
+          const int r = (x / 4) * 64 + ty * 4 + (x & 3);
+          red[r * (GC + 1) + tx] = fh[which][x];
+          red[(128 + r) * (GC + 1) + tx] = fl[which][x];
+        }
+        __syncthreads();
+        for (int q = tid; q < a.PJ * 128; q += 256) {
+          const int r = q & 127, slot = p * a.PJ + (q >> 7);
+          if (u0 + slot < u1) {
+            const float* rp = red + r * (GC + 1) + (q >> 7) * gpu;
+            float hi = 0.0f, lo = 0.0f;
+            for (int x = 0; x < gpu; ++x) {
+              two_sum(hi, lo, rp[x]);
+              lo = __fadd_rn(lo, rp[128 * (GC + 1) + x]);
+            }
+            // (an infinite sum's lo is NaN)
+            dsum[(which * a.UB + slot) * 128 + r] +=
+                isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+          }
+        }
+      }
+      cc = cn;
+      p = pn;
+      continue;
+    }
     // per row: this thread's 4 (MODE 0: 2 x 4) inner indices
 #pragma unroll
     for (int g = 0; g < (ONE ? 2 : 1); ++g) {
@@ -794,7 +869,7 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
         const int r = (x / 4) * 64 + ty * 4 + (x & 3);
         const int64_t i = i0 + r;
         float cf[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        if (MODE >= 2) {
+        if (MODE == 3) {
 #pragma unroll
           for (int q = 0; q < 4; ++q)
             if (uv && v + q < a.inner) cf[q] = xs[(v + q) * LD + r];
@@ -820,14 +895,11 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
           const float va = acc[x][g * 4 + q], vb = acc[x][4 + q];
           if (ONE) {
             s0 = fmaf(cf[q], va, s0);
-          } else if (MODE == 1) {
+          } else {
             const float ha = cf[q] * va;
             s0 = fmaf(ha, vb, s0);
             s1 += ha;
             s2 = fmaf(cf[q], vb, s2);
-          } else {
-            s0 = fmaf(cf[q], va, s0);
-            s1 = fmaf(cf[q], vb, s1);
           }
         }
         red[r * (GC + 1) + grp] = s0;
@@ -860,7 +932,9 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
     const int64_t i = i0 + tid;
     double q = 0.0;
     for (int ul = 0; ul < u1 - u0; ++ul) {
-      const double v0 = sum[ul * 128 + tid], v1 = ONE ? 0.0 : sum[(a.UB + ul) * 128 + tid];
+      const double v0 = MODE == 2 ? dsum[ul * 128 + tid] : (double)sum[ul * 128 + tid];
+      const double v1 = ONE ? 0.0 : MODE == 2 ? dsum[(a.UB + ul) * 128 + tid]
+                                              : (double)sum[(a.UB + ul) * 128 + tid];
       if (MODE == 3) {
         const int2 kl = a.pairs[u0 + ul];
         const double hk = (double)a.Ha[i * a.c + kl.x], hl = (double)a.Ha[i * a.c + kl.y];
@@ -880,14 +954,14 @@ __global__ __launch_bounds__(256, 2) void k_row_form(const FormArgs a) {
 
 // Units per tile and block for `rows` rows: kc spreads the inner range over equal chunks of at
 // most the tile; units per block: as many as keep the grid's last wave full (two blocks per
-// SM), at most 16 (shared-memory sums).
-void form_plan(FormArgs& a, int tile, int64_t rows, int sms) {
+// SM), at most `most` (shared-memory sums: 16, or 8 where they are doubles).
+void form_plan(FormArgs& a, int tile, int64_t rows, int sms, int most = 16) {
   a.CC = (a.inner + tile - 1) / tile;
   a.kc = ((a.inner + a.CC - 1) / a.CC + 3) / 4 * 4;
-  a.PJ = std::min(std::max(1, tile / a.kc), std::min(a.units, 16));
+  a.PJ = std::min(std::max(1, tile / a.kc), std::min(a.units, most));
   const int64_t rt = (rows + 127) / 128;
   double best = 1e300;
-  for (int nb = 1; nb <= 16 / a.PJ; ++nb) {
+  for (int nb = 1; nb <= most / a.PJ; ++nb) {
     const int ub = nb * a.PJ;
     const int64_t y = (a.units + ub - 1) / ub;
     if (nb > 1 && (nb - 1) * a.PJ >= a.units) break;
@@ -902,10 +976,10 @@ void form_plan(FormArgs& a, int tile, int64_t rows, int sms) {
 
 template <int MODE, int KC>
 int32_t form_launch_k(const FormArgs& a, int64_t rows, int ny, cudaStream_t st) {
-  constexpr int NV = MODE == 0 || MODE == 3 ? 1 : MODE == 1 ? 3 : 2;
+  constexpr int NV = form_nv(MODE), NS = form_ns(MODE);
   constexpr int GC = MODE == 0 || MODE == 3 ? 32 : 16;
   const size_t smem = ((size_t)form_dk(a.d) * FORM_LD + 2 * KC * 128 +
-                       (size_t)NV * 128 * (GC + 1) + (size_t)NV * a.UB * 128) *
+                       (size_t)NV * 128 * (GC + 1) + (size_t)NS * a.UB * 128) *
                       4;
   FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_form<MODE, KC>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
@@ -1831,7 +1905,8 @@ int32_t round_scores_f32(firal_problem* P, const float* M1, const float* M2, con
   a.inner = P->d;
   a.ustride = (int64_t)P->d * P->d;
   a.eta = eta;
-  form_plan(a, 64, P->n, P->sms);
+  // sums of 16 classes where two blocks still share an SM
+  form_plan(a, 64, P->n, P->sms, P->d <= 80 ? 16 : 8);
   FIRAL_TRY(P->form_part.ensure((size_t)((a.units + a.UB - 1) / a.UB) * P->n * sizeof(double)));
   a.part = P->form_part.as<double>();
   ProfScope ps(st, PF_ROUND);
