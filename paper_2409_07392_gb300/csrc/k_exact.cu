@@ -353,8 +353,10 @@ int32_t gemm(cudaStream_t st, bool ta, bool tb, int M, int N, int K, double alph
 // past j the trailing matrix, and a step is one update a_ik -= l_i v_k with v_k = Y_jk, 1 / L_jj
 // or l_k left, at and right of column j, published through shared memory.  Latency-bound (two
 // barriers, a square root and a reciprocal per step, the next pivot's overlapped with the
-// update): 68 us for a 128 x 128 f32 tile; in shared memory, with the inverse as a second
-// pass of row-by-row substitutions, a 64 x 64 tile took 59.
+// update): 78 us for a 128 x 128 f32 tile; in shared memory, with the inverse as a second
+// pass of row-by-row substitutions, a 64 x 64 tile took 59.  Root and quotients are rounded once:
+// rsqrt(v) and its products, up to 2 units in the last place off over a whole column and the
+// inverse, took 68 us and put f up to 1.3 times as far from 64 bits.
 // A pivot that is not positive and finite sets *flag; the tiles are then not to be used.
 template <class T, int R>
 __global__ __launch_bounds__(256) void k_potrf_diag(T* A, T* Winv, int64_t ld, int j0, int jb,
@@ -380,9 +382,15 @@ __global__ __launch_bounds__(256) void k_potrf_diag(T* A, T* Winv, int64_t ld, i
       if (k > i) At[(int64_t)i * ld + k] = Wt[(int64_t)i * ld + k] = T(0);
   auto pivot = [&](T v) {
     if (!(v > T(0)) || !(v < T(INFINITY))) bad = 1;
-    const T r = rsqrt(v);
-    piv[0] = v * r;
-    piv[1] = r;
+    const T p = sqrt(v);
+    piv[0] = p;
+    piv[1] = T(1) / p;
+  };
+  // v / p from the rounded reciprocal r of p: the product's residual, exact by a fused multiply-add,
+  // gives the rounded quotient (P. Markstein, IBM J. Res. Dev. 34, 1990)
+  auto divide = [](T v, T p, T r) {
+    const T q = v * r;
+    return fma(fma(-q, p, v), r, q);
   };
   if (tid == 0) pivot(a[0]);
 #pragma unroll
@@ -395,20 +403,20 @@ __global__ __launch_bounds__(256) void k_potrf_diag(T* A, T* Winv, int64_t ld, i
         if (tid == 0) atomicExch(flag, 1);
         return;
       }
-      const T r = piv[1];
+      const T p = piv[0], r = piv[1];
       if (tk == tj) {                // column j
 #pragma unroll
         for (int x = bj; x < R; ++x) {
           const int i = ti + 16 * x;
           T& v = a[x * (x + 1) / 2 + bj];
           if (i > j) {
-            const T l = v * r;
+            const T l = divide(v, p, r);
             vec[i] = l;
             if (i < jb) At[(int64_t)i * ld + j] = l;
             v = T(0);
           } else if (i == j) {
             vec[j] = r;
-            At[(int64_t)j * ld + j] = piv[0];
+            At[(int64_t)j * ld + j] = p;
             v = r;
           }
         }
@@ -419,7 +427,7 @@ __global__ __launch_bounds__(256) void k_potrf_diag(T* A, T* Winv, int64_t ld, i
           const int k = tk + 16 * y;
           T& v = a[bj * (bj + 1) / 2 + y];
           if (k < j) {
-            v *= r;
+            v = divide(v, p, r);
             vec[k] = v;
           }
         }
