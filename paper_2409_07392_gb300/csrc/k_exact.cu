@@ -85,14 +85,18 @@ constexpr int K_TO_M1 = 4;     // op(A) lower triangular: k < m0 + BM
 
 // C (M x N) = alpha op(A) op(B) + beta C for every batch z (operands offset by z sA, z sB,
 // z sC elements).  op(A) is M x K (A row-major M x K, or K x M when
-// TA); op(B) is K x N (B row-major K x N, or N x K when TB).  lower: tiles wholly above the
-// diagonal are skipped (the caller uses only the lower triangle).  beta == 0 never reads C.
+// TA); op(B) is K x N (B row-major K x N, or N x K when TB).  tri: 1, tiles wholly above the
+// diagonal are skipped (the caller uses only the lower triangle); -b, tiles wholly below the
+// diagonal's b x b blocks are (it uses the upper triangle of blocks).  beta == 0 never reads C.
 // A may alias C only when one CTA covers every column of C (N <= BM) and reads only its own
 // rows of A: all of a CTA's reads finish before its epilogue writes.
+__device__ __forceinline__ bool skip_tile(int tri, int m0, int n0, int BM) {
+  return tri > 0 ? n0 >= m0 + BM : tri < 0 && n0 + BM <= m0 / -tri * -tri;
+}
 template <class T, bool TA, bool TB>
 __global__ __launch_bounds__(256) void k_gemm(int M, int N, int K, T alpha, const T* A,
                                               int64_t lda, const T* B, int64_t ldb, T beta,
-                                              T* C, int64_t ldc, int lower, int kflags,
+                                              T* C, int64_t ldc, int tri, int kflags,
                                               int64_t sA, int64_t sB, int64_t sC) {
   A += blockIdx.z * sA;
   B += blockIdx.z * sB;
@@ -104,7 +108,7 @@ __global__ __launch_bounds__(256) void k_gemm(int M, int N, int K, T alpha, cons
   __shared__ __align__(16) T Bs[2][GBK][BN + PAD];
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  if (lower && n0 >= m0 + BM) return;
+  if (skip_tile(tri, m0, n0, BM)) return;
   int kb = 0, ke = K;
   if (kflags & K_FROM_N0) kb = max(kb, n0);
   if (kflags & K_FROM_M0) kb = max(kb, m0);
@@ -203,7 +207,7 @@ __global__ __launch_bounds__(256) void k_gemm(int M, int N, int K, T alpha, cons
 template <bool TA, bool TB, bool VEC>
 __global__ __launch_bounds__(256, 2) void k_gemm_f(int M, int N, int K, float alpha, const float* A,
                                                    int64_t lda, const float* B, int64_t ldb,
-                                                   float beta, float* C, int64_t ldc, int lower,
+                                                   float beta, float* C, int64_t ldc, int tri,
                                                    int kflags, int64_t sA, int64_t sB,
                                                    int64_t sC) {
   A += blockIdx.z * sA;
@@ -215,7 +219,7 @@ __global__ __launch_bounds__(256, 2) void k_gemm_f(int M, int N, int K, float al
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const int tx = (wid & 1) * 8 + (lane & 7), ty = (wid >> 1) * 4 + (lane >> 3);
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BM;
-  if (lower && n0 >= m0 + BM) return;
+  if (skip_tile(tri, m0, n0, BM)) return;
   int kb = 0, ke = K;
   if (kflags & K_FROM_N0) kb = max(kb, n0);
   if (kflags & K_FROM_M0) kb = max(kb, m0);
@@ -311,7 +315,7 @@ __global__ __launch_bounds__(256, 2) void k_gemm_f(int M, int N, int K, float al
 template <class T>
 int32_t gemm(cudaStream_t st, bool ta, bool tb, int M, int N, int K, double alpha, const T* A,
              int64_t lda, const T* B, int64_t ldb, double beta, T* C, int64_t ldc,
-             bool lower = false, int kflags = 0, int batch = 1, int64_t sA = 0, int64_t sB = 0,
+             int tri = 0, int kflags = 0, int batch = 1, int64_t sA = 0, int64_t sB = 0,
              int64_t sC = 0) {
   if (M <= 0 || N <= 0 || batch <= 0) return FIRAL_OK;
   constexpr int BM = GemmCfg<T>::BM;
@@ -319,8 +323,7 @@ int32_t gemm(cudaStream_t st, bool ta, bool tb, int M, int N, int K, double alph
   ProfScope ps(st, PF_EXACT_GEMM);
   count_launch();
   const T a = (T)alpha, b = (T)beta;
-  const int lw = lower ? 1 : 0;
-#define FIRAL_GEMM_ARGS M, N, K, a, A, lda, B, ldb, b, C, ldc, lw, kflags, sA, sB, sC
+#define FIRAL_GEMM_ARGS M, N, K, a, A, lda, B, ldb, b, C, ldc, tri, kflags, sA, sB, sC
   if constexpr (sizeof(T) == 4) {
     const auto al = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
     const bool vec = al(A) && al(B) && lda % 4 == 0 && ldb % 4 == 0 && sA % 4 == 0 && sB % 4 == 0;
@@ -492,7 +495,7 @@ int32_t potrf_trtri(cudaStream_t st, T* A, T* W, T* Tmp, int64_t D, int* flag) {
                         A21, D));
       // A22 -= L21 L21^T (lower tiles)
       FIRAL_TRY(gemm<T>(st, false, true, rest, rest, jb, -1.0, A21, D, A21, D, 1.0, A21 + jb, D,
-                        true));
+                        1));
     }
   }
   // W = L^{-1} by doubling: [[P, 0], [Q, R]]^{-1} = [[P^-1, 0], [-R^-1 Q P^-1, R^-1]].  At
@@ -504,18 +507,18 @@ int32_t potrf_trtri(cudaStream_t st, T* A, T* W, T* Tmp, int64_t D, int* flag) {
     if (nfull > 0) {
       // Tmp_q (s x s) = Q_q P_q^{-1}; P^{-1} is lower triangular
       FIRAL_TRY(gemm<T>(st, false, false, (int)s, (int)s, (int)s, 1.0, A + s * D, D, W, D, 0.0,
-                        Tmp, s, false, K_FROM_N0, nfull, step, step, s * s));
+                        Tmp, s, 0, K_FROM_N0, nfull, step, step, s * s));
       // W_q[c0.., o..] = -R_q^{-1} Tmp_q; R^{-1} is lower triangular
       FIRAL_TRY(gemm<T>(st, false, false, (int)s, (int)s, (int)s, -1.0, W + s * (D + 1), D, Tmp,
-                        s, 0.0, W + s * D, D, false, K_TO_M1, nfull, step, s * s, step));
+                        s, 0.0, W + s * D, D, 0, K_TO_M1, nfull, step, s * s, step));
     }
     const int64_t o = 2 * s * nfull, c0 = o + s;
     if (c0 < D) {
       const int cs = (int)(D - c0);
       FIRAL_TRY(gemm<T>(st, false, false, cs, (int)s, (int)s, 1.0, A + c0 * D + o, D,
-                        W + o * D + o, D, 0.0, Tmp, s, false, K_FROM_N0));
+                        W + o * D + o, D, 0.0, Tmp, s, 0, K_FROM_N0));
       FIRAL_TRY(gemm<T>(st, false, false, cs, (int)s, cs, -1.0, W + c0 * D + c0, D, Tmp, s, 0.0,
-                        W + c0 * D + o, D, false, K_TO_M1));
+                        W + c0 * D + o, D, 0, K_TO_M1));
     }
   }
   return FIRAL_OK;
@@ -1154,18 +1157,20 @@ int32_t objective_t(firal_problem* P, const T* z, double* f_host, T* g) {
   FIRAL_TRY(clear_flag(P));
   FIRAL_TRY(potrf_trtri<T>(st, A, W, T1, D, P->ex->flag.as<int>()));
   // Sigma^{-1} = W^T W
-  FIRAL_TRY(gemm<T>(st, true, false, (int)D, (int)D, (int)D, 1.0, W, D, W, D, 0.0, S, D, true,
+  FIRAL_TRY(gemm<T>(st, true, false, (int)D, (int)D, (int)D, 1.0, W, D, W, D, 0.0, S, D, 1,
                     K_FROM_N0 | K_FROM_M0));
   FIRAL_TRY(sym_from_lower<T>(st, S, D));
   double* f_dev = ex.scal.as<double>();
   FIRAL_TRY(dot_scaled(P->dbl, S, mat<T>(ex, EX_HP), D * D, 1.0, f_dev + 64, f_dev, st));
   if (g) {
-    // M = Sigma^{-1} H_p Sigma^{-1}, then g_i = -Tr(H_i M) (eq. 6)
+    // M = Sigma^{-1} H_p Sigma^{-1}, then g_i = -Tr(H_i M) (eq. 6), which reads the blocks M_kl,
+    // k <= l.  The diagonal blocks are needed whole: M is symmetric, but x^T M_kk x with the two
+    // roundings of each pair of elements is closer to 64 bits than with one of them mirrored (g over
+    // twelve shapes: 1.2e-6 against 1.4e-6)
     FIRAL_TRY(gemm<T>(st, false, false, (int)D, (int)D, (int)D, 1.0, S, D, mat<T>(ex, EX_HP), D,
                       0.0, T1, D));
     FIRAL_TRY(gemm<T>(st, false, false, (int)D, (int)D, (int)D, 1.0, T1, D, S, D, 0.0, M, D,
-                      true));      // symmetric: the lower tiles, then mirrored
-    FIRAL_TRY(sym_from_lower<T>(st, M, D));
+                      -P->d));
     bool done = false;
     if constexpr (sizeof(T) == 4)
       FIRAL_TRY(pair_forms_f32(P, ex.pairs.as<int2>(), ex.npairs, M, g, &done));
@@ -1209,7 +1214,7 @@ int32_t trace_inv_pows(firal_problem* P, double nu, double* v2, double* v3, int*
   FIRAL_TRY(combine<T>(st, X, 1.0, mat<T>(ex, EX_MHAT), 0.0, nullptr, 0.0, nullptr, nu, D));
   FIRAL_TRY(clear_flag(P));
   FIRAL_TRY(potrf_trtri<T>(st, X, W, mat<T>(ex, EX_T), D, ex.flag.as<int>()));
-  FIRAL_TRY(gemm<T>(st, true, false, (int)D, (int)D, (int)D, 1.0, W, D, W, D, 0.0, S, D, true,
+  FIRAL_TRY(gemm<T>(st, true, false, (int)D, (int)D, (int)D, 1.0, W, D, W, D, 0.0, S, D, 1,
                     K_FROM_N0 | K_FROM_M0));
   FIRAL_TRY(sym_from_lower<T>(st, S, D));
   FIRAL_TRY(gemm<T>(st, false, false, (int)D, (int)D, (int)D, 1.0, S, D, S, D, 0.0, S2, D));
@@ -1309,9 +1314,9 @@ int32_t round_t(firal_problem* P, const T* zd, int b, double eta, int exclude, i
     if (bad) return fail(FIRAL_ERR_NOT_SPD, "Sigma_diamond is not positive definite");
   }
   FIRAL_TRY(gemm<T>(st, false, false, (int)D, (int)D, (int)D, 1.0, Linv, D, Ho, D, 0.0, T1, D,
-                    false, K_TO_M1));
+                    0, K_TO_M1));
   FIRAL_TRY(gemm<T>(st, false, true, (int)D, (int)D, (int)D, 1.0, T1, D, Linv, D, 0.0, Hho, D,
-                    true));
+                    1));
   FIRAL_TRY(sym_from_lower<T>(st, Hho, D));
   FIRAL_CUDA_TRY(cudaMemsetAsync(Hsum, 0, DD, st));
   FIRAL_CUDA_TRY(cudaMemsetAsync(Mhat, 0, DD, st));
@@ -1331,7 +1336,7 @@ int32_t round_t(firal_problem* P, const T* zd, int b, double eta, int exclude, i
     FIRAL_TRY(combine<T>(st, A, nu, Sig, eta, Hsum, eta / b, Ho, 0.0, D));
     FIRAL_TRY(clear_flag(P));
     FIRAL_TRY(potrf_trtri<T>(st, A, W, T1, D, ex.flag.as<int>()));
-    FIRAL_TRY(gemm<T>(st, true, false, (int)D, (int)D, (int)D, 1.0, W, D, W, D, 0.0, S, D, true,
+    FIRAL_TRY(gemm<T>(st, true, false, (int)D, (int)D, (int)D, 1.0, W, D, W, D, 0.0, S, D, 1,
                       K_FROM_N0 | K_FROM_M0));
     FIRAL_TRY(sym_from_lower<T>(st, S, D));                              // S = G^{-1}
     FIRAL_TRY(dot_scaled(P->dbl, Sig, S, D * D, 1.0, sc + 64, sc + 2, st));   // Tr(Sigma G^-1)
@@ -1378,7 +1383,7 @@ int32_t round_t(firal_problem* P, const T* zd, int b, double eta, int exclude, i
       FIRAL_CUDA_TRY(cudaGetLastError());
     }
     FIRAL_TRY(combine<T>(st, Mhat, 1.0, Mhat, eta / b, Hho, 0.0, nullptr, 0.0, D));
-    FIRAL_TRY(gemm<T>(st, false, true, (int)D, (int)D, c, eta, Z, c, Y, c, 1.0, Mhat, D, true));
+    FIRAL_TRY(gemm<T>(st, false, true, (int)D, (int)D, c, eta, Z, c, Y, c, 1.0, Mhat, D, 1));
     // nu_{t+1}: root of sum_j (nu + lambda_j(eta H~))^{-2} = 1 (eq. 10), bracketed by nu_t
     int ev = 0;
     FIRAL_TRY(nu_root<T>(P, nu, &nu, &ev));
