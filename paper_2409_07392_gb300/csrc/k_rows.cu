@@ -989,16 +989,29 @@ int32_t form_launch_k(const FormArgs& a, int64_t rows, int ny, cudaStream_t st) 
   return FIRAL_OK;
 }
 
+// Per-block row partials (blocks of units x rows x 8 bytes) of at most FORM_PART_BYTES: the rows run
+// in chunks of whole tiles beyond that.  Unbounded, Exact-FIRAL's forms would take 10 GB at n = 1 M,
+// c = 200, d = 50.  Rows of a chunk:
+constexpr int64_t FORM_PART_BYTES = (int64_t)1 << 28;
+int64_t form_chunk(int64_t rows, int64_t ny, int tile) {
+  const int64_t most = std::max<int64_t>(tile, FORM_PART_BYTES / (8 * ny) / tile * tile);
+  return std::min(rows, most);
+}
+
+// pack: the coefficients' tiles are not there yet
 template <int MODE>
-int32_t form_launch(firal_problem* P, FormArgs a, int64_t rows, int* ny, cudaStream_t st) {
+int32_t form_launch(firal_problem* P, FormArgs a, int64_t rows, int* ny, cudaStream_t st,
+                    bool pack = true) {
   *ny = (a.units + a.UB - 1) / a.UB;
   const int dK = form_dk(a.d);
   const int64_t tiles = (int64_t)*ny * a.CC * (a.UB / a.PJ);
   FIRAL_TRY(P->form_pk.ensure((size_t)tiles * dK * 128 * sizeof(float)));
   a.pk = P->form_pk.as<float>();
-  const int64_t total = tiles * (dK / 8) * 128;
-  count_launch();
-  k_form_pack<MODE><<<(unsigned)std::min<int64_t>((total + 255) / 256, 65536), 256, 0, st>>>(a, total);
+  if (pack) {
+    const int64_t total = tiles * (dK / 8) * 128;
+    count_launch();
+    k_form_pack<MODE><<<(unsigned)std::min<int64_t>((total + 255) / 256, 65536), 256, 0, st>>>(a, total);
+  }
   if (a.d <= 96) return form_launch_k<MODE, 16>(a, rows, *ny, st);
   return form_launch_k<MODE, 8>(a, rows, *ny, st);
 }
@@ -1013,8 +1026,8 @@ constexpr int FORM_D_STAGE = 512;   // doubles of a probe's coefficients staged 
 template <int MODE>
 __global__ __launch_bounds__(256) void k_row_form_d(
     const double* __restrict__ Xa, const double* __restrict__ HaT, const double* __restrict__ w,
-    const double* __restrict__ A, const double* __restrict__ B, int64_t row0, int64_t N, int d,
-    int c, int s, int64_t D, double* __restrict__ walpha, double* __restrict__ part) {
+    const double* __restrict__ A, const double* __restrict__ B, int64_t row0, int64_t row1, int64_t N,
+    int d, int c, int s, int64_t D, double* __restrict__ walpha, double* __restrict__ part) {
   constexpr int KC = 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nw = blockDim.x >> 5, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -1025,11 +1038,11 @@ __global__ __launch_bounds__(256) void k_row_form_d(
   __shared__ double red[8][33];
   const int64_t i0 = row0 + (int64_t)blockIdx.x * 32;
   const int64_t i = i0 + lane;
-  const bool rv = i < N;
+  const bool rv = i < row1;
   const int j = blockIdx.y * nw + wid;
 #pragma unroll 8
   for (int r = wid; r < 32; r += nw)
-    for (int e = lane; e < d; e += 32) xs[r * ldx + e] = i0 + r < N ? Xa[(i0 + r) * d + e] : 0.0;
+    for (int e = lane; e < d; e += 32) xs[r * ldx + e] = i0 + r < row1 ? Xa[(i0 + r) * d + e] : 0.0;
   __syncthreads();
   double s0 = 0.0, s1 = 0.0, s2 = 0.0;
   const double* x = xs + lane * ldx;
@@ -1100,7 +1113,7 @@ __global__ __launch_bounds__(256) void k_row_form_d(
   if (wid == 0 && rv) {
     double q = 0.0;
     for (int x2 = 0; x2 < nw; ++x2) q += red[x2][lane];
-    part[blockIdx.y * (N - row0) + (i - row0)] = q;
+    part[blockIdx.y * (row1 - row0) + (i - row0)] = q;
   }
 }
 
@@ -1115,14 +1128,14 @@ int form_d_warps(int64_t rows, int s, int sms) {
 
 template <int MODE>
 int32_t form_d_launch(const double* Xa, const double* HaT, const double* w, const double* A,
-                      const double* B, int64_t row0, int64_t N, int d, int c, int s, int64_t D,
-                      double* walpha, double* part, int nw, cudaStream_t st) {
+                      const double* B, int64_t row0, int64_t row1, int64_t N, int d, int c, int s,
+                      int64_t D, double* walpha, double* part, int nw, cudaStream_t st) {
   const size_t smem = ((size_t)32 * (d | 1) + (size_t)(MODE == 1 ? 2 : 1) * nw * FORM_D_STAGE) * 8;
   FIRAL_CUDA_TRY(cudaFuncSetAttribute(k_row_form_d<MODE>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
   count_launch();
-  k_row_form_d<MODE><<<dim3((unsigned)((N - row0 + 31) / 32), (s + nw - 1) / nw), nw * 32, smem,
-                       st>>>(Xa, HaT, w, A, B, row0, N, d, c, s, D, walpha, part);
+  k_row_form_d<MODE><<<dim3((unsigned)((row1 - row0 + 31) / 32), (s + nw - 1) / nw), nw * 32, smem,
+                       st>>>(Xa, HaT, w, A, B, row0, row1, N, d, c, s, D, walpha, part);
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
 }
@@ -1140,21 +1153,22 @@ __global__ void k_form_sum(const double* __restrict__ part, int ny, int64_t n, d
 }
 
 // eq. 14: the blocks' partial scores added per row, then the masked argmax of each 128 rows
-// (lowest index on ties)
+// (lowest index on ties); r0: the pool's index of the first of the n rows
 __global__ __launch_bounds__(128) void k_score_argmax(const double* __restrict__ part, int ny,
-                                                      int64_t n, const uint8_t* __restrict__ mask,
+                                                      int64_t n, int64_t r0,
+                                                      const uint8_t* __restrict__ mask,
                                                       double* part_val, int64_t* part_idx) {
   __shared__ double bv[4];
   __shared__ int64_t bi[4];
   const int64_t i = (int64_t)blockIdx.x * 128 + threadIdx.x;
   double val = -INFINITY;
   int64_t idx = INT64_MAX;
-  if (i < n && !mask[i]) {
+  if (i < n && !mask[r0 + i]) {
     double q = 0.0;
     for (int y = 0; y < ny; ++y) q += part[y * n + i];
     if (q == q) {
       val = q;
-      idx = i;
+      idx = r0 + i;
     }
   }
   for (int o = 16; o > 0; o >>= 1) {
@@ -1754,7 +1768,7 @@ int32_t apply_t(firal_problem* P, const T* w, const T* Sblk, const T* V, int s, 
   {
     ProfScope ps(st, PF_ALPHA);
     if constexpr (sizeof(T) == 8) {
-      FIRAL_TRY(form_d_launch<0>(P->Xa.as<double>(), P->HaT.as<double>(), w, V, nullptr, 0, N, d,
+      FIRAL_TRY(form_d_launch<0>(P->Xa.as<double>(), P->HaT.as<double>(), w, V, nullptr, 0, N, N, d,
                                  c, s, D, P->walpha.as<double>(), nullptr, form_d_warps(N, s, P->sms),
                                  st));
     } else {
@@ -1848,23 +1862,17 @@ int32_t quad_forms_simt(firal_problem* P, const void* A, const void* B, int s, d
   cudaStream_t st = P->H->stream;
   const int d = P->d, c = P->c;
   ProfScope ps(st, PF_QUAD);
-  int ny = 0;
+  FormArgs a{};
+  int nw = 0, ny = 0;
   if (P->dbl) {
     FIRAL_TRY(class_major_h(P));
-    const int nw = form_d_warps(P->n, s, P->sms);
+    nw = form_d_warps(P->n, s, P->sms);
     ny = (s + nw - 1) / nw;
-    FIRAL_TRY(P->form_part.ensure((size_t)ny * P->n * sizeof(double)));
-    FIRAL_TRY(form_d_launch<1>(P->Xa.as<double>(), P->HaT.as<double>(), nullptr,
-                               (const double*)A, (const double*)B, P->m, P->N, d, c, s, P->D,
-                               nullptr, P->form_part.as<double>(), nw, st));
   } else {
-    FormArgs a{};
     a.Xa = P->Xa.as<float>();
     a.Ha = P->Ha.as<float>();
     a.A = (const float*)A;
     a.B = (const float*)B;
-    a.row0 = P->m;
-    a.N = P->N;
     a.d = d;
     a.c = c;
     a.units = s;
@@ -1872,19 +1880,29 @@ int32_t quad_forms_simt(firal_problem* P, const void* A, const void* B, int s, d
     a.ustride = P->D;
     a.vec = row_vec(a.Ha, c) == 4;
     form_plan(a, 64, P->n, P->sms);
-    FIRAL_TRY(P->form_part.ensure((size_t)((s + a.UB - 1) / a.UB) * P->n * sizeof(double)));
-    a.part = P->form_part.as<double>();
-    FIRAL_TRY(form_launch<1>(P, a, P->n, &ny, st));
+    ny = (s + a.UB - 1) / a.UB;
   }
-  count_launch();
-  const unsigned grid = (unsigned)std::min<int64_t>((P->n + 255) / 256, 4096);
-  if (P->dbl)
-    k_form_sum<double><<<grid, 256, 0, st>>>(P->form_part.as<double>(), ny, P->n, -scale / s,
-                                             (double*)g);
-  else
-    k_form_sum<float><<<grid, 256, 0, st>>>(P->form_part.as<double>(), ny, P->n, -scale / s,
-                                            (float*)g);
-  FIRAL_CUDA_TRY(cudaGetLastError());
+  const int64_t chunk = form_chunk(P->n, ny, P->dbl ? 32 : 128);
+  FIRAL_TRY(P->form_part.ensure((size_t)ny * chunk * sizeof(double)));
+  double* part = a.part = P->form_part.as<double>();
+  for (int64_t r = 0; r < P->n; r += chunk) {
+    const int64_t rows = std::min(chunk, P->n - r);
+    const unsigned grid = (unsigned)std::min<int64_t>((rows + 255) / 256, 4096);
+    if (P->dbl) {
+      FIRAL_TRY(form_d_launch<1>(P->Xa.as<double>(), P->HaT.as<double>(), nullptr,
+                                 (const double*)A, (const double*)B, P->m + r, P->m + r + rows,
+                                 P->N, d, c, s, P->D, nullptr, part, nw, st));
+      count_launch();
+      k_form_sum<double><<<grid, 256, 0, st>>>(part, ny, rows, -scale / s, (double*)g + r);
+    } else {
+      a.row0 = P->m + r;
+      a.N = a.row0 + rows;
+      FIRAL_TRY(form_launch<1>(P, a, rows, &ny, st, r == 0));
+      count_launch();
+      k_form_sum<float><<<grid, 256, 0, st>>>(part, ny, rows, -scale / s, (float*)g + r);
+    }
+    FIRAL_CUDA_TRY(cudaGetLastError());
+  }
   return FIRAL_OK;
 }
 
@@ -1897,8 +1915,6 @@ int32_t round_scores_f32(firal_problem* P, const float* M1, const float* M2, con
   a.Ha = P->Ha.as<float>();
   a.A = M1;
   a.B = M2;
-  a.row0 = P->m;
-  a.N = P->N;
   a.d = P->d;
   a.c = P->c;
   a.units = P->c;
@@ -1907,14 +1923,23 @@ int32_t round_scores_f32(firal_problem* P, const float* M1, const float* M2, con
   a.eta = eta;
   // sums of 16 classes where two blocks still share an SM
   form_plan(a, 64, P->n, P->sms, P->d <= 80 ? 16 : 8);
-  FIRAL_TRY(P->form_part.ensure((size_t)((a.units + a.UB - 1) / a.UB) * P->n * sizeof(double)));
+  int ny = (a.units + a.UB - 1) / a.UB;
+  const int64_t chunk = form_chunk(P->n, ny, 128);
+  FIRAL_TRY(P->form_part.ensure((size_t)ny * chunk * sizeof(double)));
   a.part = P->form_part.as<double>();
   ProfScope ps(st, PF_ROUND);
-  int ny = 0;
-  FIRAL_TRY(form_launch<2>(P, a, P->n, &ny, st));
-  count_launch();
-  k_score_argmax<<<np, 128, 0, st>>>(a.part, ny, P->n, mask, pv, pi);
-  FIRAL_CUDA_TRY(cudaGetLastError());
+  for (int64_t r = 0; r < P->n; r += chunk) {
+    const int64_t rows = std::min(chunk, P->n - r);
+    a.row0 = P->m + r;
+    a.N = a.row0 + rows;
+    FIRAL_TRY(form_launch<2>(P, a, rows, &ny, st, r == 0));
+    // (the last chunk's launch also fills the partials past the last row)
+    const int64_t blocks = r + rows < P->n ? rows / 128 : np - r / 128;
+    count_launch();
+    k_score_argmax<<<(unsigned)blocks, 128, 0, st>>>(a.part, ny, rows, r, mask, pv + r / 128,
+                                                     pi + r / 128);
+    FIRAL_CUDA_TRY(cudaGetLastError());
+  }
   return FIRAL_OK;
 }
 
@@ -1962,8 +1987,6 @@ int32_t pair_forms_f32(firal_problem* P, const int2* pairs, int npairs, const fl
   a.Xa = P->Xa.as<float>();
   a.Ha = P->Ha.as<float>();
   a.A = M;
-  a.row0 = P->m;
-  a.N = P->N;
   a.d = P->d;
   a.c = P->c;
   a.units = npairs;
@@ -1973,16 +1996,23 @@ int32_t pair_forms_f32(firal_problem* P, const int2* pairs, int npairs, const fl
   form_plan(a, 128, P->n, P->sms);
   const int64_t ny = (npairs + a.UB - 1) / a.UB;
   *done = false;
-  if (ny > 4096) return FIRAL_OK;   // very many classes of few features: partials too large
-  FIRAL_TRY(P->form_part.ensure((size_t)ny * P->n * sizeof(double)));
+  // very many classes of few features: the packed tiles would take several times M's memory
+  if (ny > 4096) return FIRAL_OK;
+  const int64_t chunk = form_chunk(P->n, ny, 128);
+  FIRAL_TRY(P->form_part.ensure((size_t)ny * chunk * sizeof(double)));
   a.part = P->form_part.as<double>();
   ProfScope ps(st, PF_EXACT_QUAD);
-  int y = 0;
-  FIRAL_TRY(form_launch<3>(P, a, P->n, &y, st));
-  count_launch();
-  k_form_sum<float><<<(unsigned)std::min<int64_t>((P->n + 255) / 256, 4096), 256, 0, st>>>(
-      P->form_part.as<double>(), y, P->n, 1.0, g);
-  FIRAL_CUDA_TRY(cudaGetLastError());
+  for (int64_t r = 0; r < P->n; r += chunk) {
+    const int64_t rows = std::min(chunk, P->n - r);
+    a.row0 = P->m + r;
+    a.N = a.row0 + rows;
+    int y = 0;
+    FIRAL_TRY(form_launch<3>(P, a, rows, &y, st, r == 0));
+    count_launch();
+    k_form_sum<float><<<(unsigned)std::min<int64_t>((rows + 255) / 256, 4096), 256, 0, st>>>(
+        a.part, y, rows, 1.0, g + r);
+    FIRAL_CUDA_TRY(cudaGetLastError());
+  }
   *done = true;
   return FIRAL_OK;
 }
