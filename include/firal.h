@@ -398,8 +398,9 @@ int32_t firal_exact_round(firal_problem* problem, const void* z_relaxed, int32_t
 /* Destroyed problems park their device buffers in a process-wide cache (bounded by the
  * FIRAL_CACHE_BYTES environment variable, default 64 GiB; 0 disables it), from which later
  * problems on the same device take buffers of a similar size instead of calling cudaMalloc.
- * firal_cache_trim returns every parked buffer to the driver; firal_cache_bytes reports how
- * many bytes are parked. */
+ * firal_cache_trim returns every parked buffer to the driver (an allocation that finds the
+ * device full does so too, once, before it fails); firal_cache_bytes reports how many bytes
+ * are parked. */
 int32_t firal_cache_trim(void);
 int64_t firal_cache_bytes(void);
 

@@ -108,8 +108,9 @@ ProfScope::~ProfScope() {
 // 20 ms, and a caller that builds one problem per call (firal_relax, firal_round) pays it
 // every time.  firal_problem_destroy and drop_temps (a call's own buffers) park, after
 // synchronising the stream that used them, so a parked block has no kernel in flight; every other
-// release still calls cudaFree (which synchronises the device).  Bounded by FIRAL_CACHE_BYTES (default 64 GiB, 0 disables);
-// firal_cache_trim returns every parked block.
+// release still calls cudaFree (which synchronises the device).  Bounded by FIRAL_CACHE_BYTES (default
+// 64 GiB, 0 disables); firal_cache_trim returns every parked block, and so does an allocation that
+// finds the device full, before it tries once more.
 namespace {
 struct ParkedBlock {
   void* p;
@@ -160,6 +161,30 @@ bool cache_park(void* p, size_t bytes) {
   c.held += bytes;
   return true;
 }
+// Give every parked block back to the driver; whether there was one.
+bool cache_clear() {
+  BlockCache& c = block_cache();
+  std::vector<ParkedBlock> blocks;
+  {
+    std::lock_guard<std::mutex> g(c.mu);
+    blocks.swap(c.blocks);
+    c.held = 0;
+  }
+  int cur = 0;
+  cudaGetDevice(&cur);
+  for (const ParkedBlock& b : blocks) {
+    cudaSetDevice(b.dev);
+    cudaFree(b.p);
+  }
+  cudaSetDevice(cur);
+  return !blocks.empty();
+}
+// This thread records a graph (replay_steps): nothing is freed meanwhile.
+thread_local bool g_capturing = false;
+struct CaptureScope {
+  CaptureScope() { g_capturing = true; }
+  ~CaptureScope() { g_capturing = false; }
+};
 }  // namespace
 
 int32_t DBuf::ensure(size_t nbytes) {
@@ -177,7 +202,12 @@ int32_t DBuf::ensure(size_t nbytes) {
     return FIRAL_OK;
   }
   cudaError_t e = cudaMalloc(&p, nbytes);
+  if (e == cudaErrorMemoryAllocation && !g_capturing && cache_clear()) {
+    cudaGetLastError();   // the failed attempt's, or the next launch check would report it
+    e = cudaMalloc(&p, nbytes);
+  }
   if (e != cudaSuccess) {
+    cudaGetLastError();
     p = nullptr;
     return fail(FIRAL_ERR_NOMEM, std::string("cudaMalloc(") + std::to_string(nbytes) +
                                      "): " + cudaGetErrorString(e));
@@ -885,9 +915,12 @@ int32_t replay_steps(firal_handle* H, std::vector<firal_problem*>& probs,
   FIRAL_CUDA_TRY(cudaStreamBeginCapture(cap, cudaStreamCaptureModeRelaxed));
   cudaEventRecord(fork, cap);
   for (int i = 0; i < nstreams; ++i) cudaStreamWaitEvent(ss.st[i], fork, 0);
-  for (int p = 0; p < np && rc == FIRAL_OK; ++p) {
-    H->stream = ss.st[p % nstreams];
-    rc = relax_step_impl(probs[p], &opts[p], 0, budgets[p], zs[p], nullptr, true);
+  {
+    CaptureScope recording;
+    for (int p = 0; p < np && rc == FIRAL_OK; ++p) {
+      H->stream = ss.st[p % nstreams];
+      rc = relax_step_impl(probs[p], &opts[p], 0, budgets[p], zs[p], nullptr, true);
+    }
   }
   H->stream = user;
   for (int i = 0; i < nstreams; ++i) {
@@ -2036,20 +2069,7 @@ int32_t firal_set_default_tuning(firal_handle* H, const firal_tuning* t) {
 }
 
 int32_t firal_cache_trim(void) {
-  BlockCache& c = block_cache();
-  std::vector<ParkedBlock> blocks;
-  {
-    std::lock_guard<std::mutex> g(c.mu);
-    blocks.swap(c.blocks);
-    c.held = 0;
-  }
-  int cur = 0;
-  cudaGetDevice(&cur);
-  for (const ParkedBlock& b : blocks) {
-    cudaSetDevice(b.dev);
-    cudaFree(b.p);
-  }
-  cudaSetDevice(cur);
+  cache_clear();
   return FIRAL_OK;
 }
 
