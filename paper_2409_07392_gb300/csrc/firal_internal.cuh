@@ -299,7 +299,7 @@ int32_t precond_apply(firal_problem* P, const void* R, int s, void* Z);
 int32_t tick(int64_t* t_dev, cudaStream_t st);
 int32_t set_step(int64_t* t_dev, int64_t v, cudaStream_t st);
 int32_t syrk_reduce_f32(firal_problem* P, const float* partS, const float* partP, int splits,
-                        double lamS, float* outS, double lamP, double* outP);
+                        int64_t stride, double lamS, float* outS, double lamP, double* outP);
 int32_t pair_blocks_f32(firal_problem* P, const float* partS, const float* partP, int npq,
                         int splits, double lamS, float* outS, double lamP, double* outP,
                         const float* addS);

@@ -1504,16 +1504,18 @@ int32_t syrk_t(firal_problem* P, const T* w, int64_t rows, double lamS, T* outS,
   return FIRAL_OK;
 }
 
-// pw[i][k] = w_i h_ik, then (both) w_i h_ik (1 - h_ik); only the second when !both
+// pw[i] = w_i h_ik over the classes (if hasS), then w_i h_ik (1 - h_ik) (if hasP); blockDim.y rows
+// a block
 __global__ void k_block_weights(const float* __restrict__ Ha, const float* __restrict__ w,
-                                int64_t rows, int c, bool both, float* __restrict__ pw) {
-  const int cc = both ? 2 * c : c;
-  for (int64_t i = blockIdx.x; i < rows; i += gridDim.x) {
+                                int64_t rows, int c, bool hasS, bool hasP, float* __restrict__ pw) {
+  const int cc = (hasS ? c : 0) + (hasP ? c : 0);
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.y + threadIdx.y; i < rows;
+       i += (int64_t)gridDim.x * blockDim.y) {
     const float wi = w[i];
     for (int k = threadIdx.x; k < c; k += blockDim.x) {
       const float h = Ha[i * c + k], wh = wi * h;
-      if (both) pw[i * cc + k] = wh;
-      pw[i * cc + cc - c + k] = wh * (1.0f - h);
+      if (hasS) pw[i * cc + k] = wh;
+      if (hasP) pw[i * cc + cc - c + k] = wh * (1.0f - h);
     }
   }
 }
@@ -1522,9 +1524,19 @@ __global__ void k_block_weights(const float* __restrict__ Ha, const float* __res
 // (and w h for S), rows in order within their range, over the full square, as both (e, f) and
 // (f, e) are used.  For results that amplify the sums' rounding: Round's nu and scores (B_k
 // alone: its Sigma blocks and B(H_o), firal_precond_blocks), and the classifier refit, whose line
-// search compares losses at their f32 noise (S and B_k over few rows).  It is OP 0's product with
-// m = (kind and class k, feature e): A = x_e p_k, B = x_f.
+// search compares losses at their f32 noise (S and B_k over few rows).  Also for few (kind, class)
+// rows (few_outputs), of which pair_sums multiplies at least 32, after writing every pair of features
+// out.  It is OP 0's product with m = (kind and class k, feature e): A = x_e p_k, B = x_f.
 constexpr int64_t FEW_ROWS = 256;   // one range at any class count
+
+// Up to 8 (kind, class) rows, a quarter of pair_sums' smallest tile, where either the features are wide
+// or the rows many: one apply with s = 1, pair_sums and here, at c = 2: d = 128 2,011 and 400 us at
+// n = 100,000, 196 and 112 at 5,000; d = 50 455 and 293 at 100,000 but 106 and 116 at 5,000, where the
+// ranges of 256 rows are a chain of latencies (c = 5: 107 and 135).  At d = 50 the lines cross near
+// 13,000 rows.
+bool few_outputs(int outputs, int d, int64_t rows) {
+  return outputs <= 8 && (d > 56 || rows >= 16384);
+}
 
 // The same sums, class blocks of d <= DP features padded to DP (64 or 128), one class to DP DP / 128
 // threads of 8 x 16 outputs each.  One staged row of x serves both operands: the left one,
@@ -1632,7 +1644,7 @@ int32_t block_ord(const float* Xa, const float* pw, int64_t rows, int64_t rps, i
 int32_t blocks_ordered_f32(firal_problem* P, const float* w, int64_t rows, double lamS,
                            float* outS, double lamP, double* outP) {
   cudaStream_t st = P->H->stream;
-  const int d = P->d, c = P->c, cc = (outS ? 1 : 0) * c + c;
+  const int d = P->d, c = P->c, cc = (outS ? c : 0) + (outP ? c : 0);
   const int64_t per = (int64_t)c * d * d;
   OuterArgs<float> a{};
   a.Xa = a.Ha = P->Xa.as<float>();
@@ -1652,9 +1664,10 @@ int32_t blocks_ordered_f32(firal_problem* P, const float* w, int64_t rows, doubl
     ProfScope ps(st, PF_SYRK);
     if (rows > 0) {
       count_launch();
-      k_block_weights<<<(unsigned)std::min<int64_t>(rows, 65536), std::min(256, (c + 31) / 32 * 32),
-                        0, st>>>(P->Ha.as<float>(), w, rows, c, outS != nullptr,
-                                 P->blk_w.as<float>());
+      const int tx = std::min(256, (c + 31) / 32 * 32), ty = 256 / tx;
+      k_block_weights<<<(unsigned)std::min<int64_t>((rows + ty - 1) / ty, 65536), dim3(tx, ty), 0,
+                        st>>>(P->Ha.as<float>(), w, rows, c, outS != nullptr,
+                                 outP != nullptr, P->blk_w.as<float>());
       FIRAL_CUDA_TRY(cudaGetLastError());
     }
     // the padded tile where it wastes less than a quarter of its outputs
@@ -1665,8 +1678,9 @@ int32_t blocks_ordered_f32(firal_problem* P, const float* w, int64_t rows, doubl
     else
       FIRAL_TRY(outer_run<0>(a, p, st));
   }
-  // S and B_k together: one range (few rows), S's blocks before B_k's
-  return syrk_reduce_f32(P, a.part, a.part + (outS ? per : 0), p.splits, lamS, outS, lamP, outP);
+  // a range's blocks: S's, then B_k's
+  return syrk_reduce_f32(P, a.part, a.part + (outS ? per : 0), p.splits, (int64_t)cc * d * d, lamS,
+                         outS, lamP, outP);
 }
 
 // The apply of one vector over few rows (the classifier refit's solves), f32, in two launches and
@@ -1836,7 +1850,10 @@ int32_t apply_t(firal_problem* P, const T* w, const T* Sblk, const T* V, int s, 
 int32_t syrk_blocks(firal_problem* P, const void* w, double lamS, void* outS, double lamP,
                     double* outP, int64_t rows) {
   if (rows < 0) rows = P->N;
-  if (!P->dbl && (!outS || (outP && rows == P->N && rows <= FEW_ROWS)))
+  const int kinds = (outS ? 1 : 0) + (outP ? 1 : 0);
+  if (kinds == 0) return FIRAL_OK;
+  if (!P->dbl && (!outS || few_outputs(kinds * P->c, P->d, rows) ||
+                  (outP && rows == P->N && rows <= FEW_ROWS)))
     return blocks_ordered_f32(P, (const float*)w, rows, lamS, (float*)outS, lamP, outP);
   if (P->dbl) return syrk_t<double>(P, (const double*)w, rows, lamS, (double*)outS, lamP, outP);
   return syrk_t<float>(P, (const float*)w, rows, lamS, (float*)outS, lamP, outP);

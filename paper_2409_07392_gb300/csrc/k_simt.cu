@@ -359,15 +359,16 @@ int32_t set_step(int64_t* t_dev, int64_t v, cudaStream_t st) {
 // ------------------------------------------------------------------------------------------
 // Reductions of the tensor-core path's split sums (the CUDA-core paths' are in k_rows.cu)
 // ------------------------------------------------------------------------------------------
-// out[k][e][f] = sum_split part[split][k][e][f] (+ lam on the diagonal), as double and/or T
+// out[k][e][f] = sum_split part[split][k][e][f] (+ lam on the diagonal), as double and/or T; a
+// split's blocks lie `stride` values after the one's before it
 template <class T>
-__global__ void k_syrk_reduce(const T* part, int splits, int64_t per, int d, double lam,
-                              double* out_d, T* out_t) {
+__global__ void k_syrk_reduce(const T* part, int splits, int64_t per, int64_t stride, int d,
+                              double lam, double* out_d, T* out_t) {
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < per;
        idx += (int64_t)gridDim.x * blockDim.x) {
     double acc = 0.0;
 #pragma unroll 8
-    for (int sp = 0; sp < splits; ++sp) acc += (double)part[(int64_t)sp * per + idx];
+    for (int sp = 0; sp < splits; ++sp) acc += (double)part[sp * stride + idx];
     const int64_t ef = idx % ((int64_t)d * d);
     const int e = (int)(ef / d), f = (int)(ef % d);
     if (e == f) acc += lam;
@@ -417,15 +418,16 @@ int32_t pair_blocks_f32(firal_problem* P, const float* partS, const float* partP
 }
 
 int32_t syrk_reduce_f32(firal_problem* P, const float* partS, const float* partP, int splits,
-                        double lamS, float* outS, double lamP, double* outP) {
+                        int64_t stride, double lamS, float* outS, double lamP, double* outP) {
   cudaStream_t st = P->H->stream;
   const int64_t per = (int64_t)P->c * P->d * P->d;
   const int g = grid_for(per, 256, 4096);
   ProfScope ps(st, PF_SYRK);
   count_launch((outS ? 1 : 0) + (outP ? 1 : 0));
   if (outS)
-    k_syrk_reduce<float><<<g, 256, 0, st>>>(partS, splits, per, P->d, lamS, nullptr, outS);
-  if (outP) k_syrk_reduce<float><<<g, 256, 0, st>>>(partP, splits, per, P->d, lamP, outP, nullptr);
+    k_syrk_reduce<float><<<g, 256, 0, st>>>(partS, splits, per, stride, P->d, lamS, nullptr, outS);
+  if (outP)
+    k_syrk_reduce<float><<<g, 256, 0, st>>>(partP, splits, per, stride, P->d, lamP, outP, nullptr);
   FIRAL_CUDA_TRY(cudaGetLastError());
   return FIRAL_OK;
 }
