@@ -5,20 +5,22 @@
 //
 // Layout: every d~ x d~ matrix is row-major with leading dimension d~; row and column index
 // k d + e stand for class k and feature e (the Kronecker order of eq. 2).  Everything runs in
-// the problem's vec type (float, or double for FIRAL_FP64); the factorisation and inverse of
-// each diagonal tile, the Round's c x c systems and all scalar reductions use double.
+// the problem's vec type (float, or double for FIRAL_FP64); the Round's c x c systems and all
+// scalar reductions use double.
 //
 // Building blocks:
-//   * k_pair_syrk + k_pair_reduce: sum_i w_i H_i (+ base matrices) built per class pair
-//     (k, l), k <= l, as sum_i w_i q_i^{kl} x_i x_i^T with q^{kl} = delta_kl h_k - h_k h_l
-//     (eq. 2 written block by block), mirrored into the lower blocks;
-//   * k_gemm: C = alpha op(A) op(B) + beta C, SIMT, 128 x 128 (float) / 64 x 64 (double)
-//     tiles, with optional skipping of tiles above the diagonal and of K ranges that a
-//     triangular operand makes zero;
-//   * k_potrf_diag: Cholesky and inverse of one 64 x 64 diagonal tile; with k_gemm it makes
-//     the blocked right-looking Cholesky and the blocked (doubling) triangular inverse;
-//   * k_pair_quad: x_i^T M_kl x_i for every class pair -- the exact gradient and the c x c
-//     matrices of the Round scores;
+//   * sum_i w_i H_i (+ base matrices) built per class pair (k, l), k <= l, as
+//     sum_i w_i q_i^{kl} x_i x_i^T with q^{kl} = delta_kl h_k - h_k h_l (eq. 2 written block by
+//     block), mirrored into the lower blocks: float, pair_sums_f32 (k_rows.cu) +
+//     k_pair_reduce_tri; double, k_pair_syrk + k_pair_reduce;
+//   * k_gemm_f (float, 128 x 128 tiles) and k_gemm (double, 64 x 64): C = alpha op(A) op(B) +
+//     beta C, SIMT, with optional skipping of tiles on one side of the diagonal and of K ranges
+//     that a triangular operand makes zero;
+//   * k_potrf_diag: Cholesky and inverse of one diagonal tile (float 128 x 128, double 64 x 64);
+//     with the products it makes the blocked right-looking Cholesky and the blocked (doubling)
+//     triangular inverse;
+//   * x_i^T M_kl x_i for every class pair: float gradient, pair_forms_f32 (k_rows.cu); double
+//     gradient and the c x c matrices of the Round scores, k_pair_quad;
 //   * k_exact_score: eq. 9's trace for one candidate from its c x c matrices (Woodbury).
 #include <cuda_runtime.h>
 
@@ -202,6 +204,7 @@ __global__ __launch_bounds__(256) void k_gemm(int M, int N, int K, T alpha, cons
 // those of k_gemm<float>.  128 x 128 x 16 tiles, 8 x 8 outputs per thread, a warp 8 x 4 thread
 // groups; 16-byte loads where the operands allow (VEC), each quarter of a step reading one item
 // of the next tile before its multiply-adds and storing it after them, one barrier per step.
+// Loads pass through registers.
 // D = 2500: about 38 TFLOP/s on full products (400 tiles, 1.3 waves of two blocks per SM); scalar
 // loads of 8-deep stages with the whole next tile held in registers ran at 33.
 template <bool TA, bool TB, bool VEC>

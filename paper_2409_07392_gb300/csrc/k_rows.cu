@@ -1198,9 +1198,10 @@ __global__ __launch_bounds__(128) void k_score_argmax(const double* __restrict__
 // Row ranges of the f32 block sums.  The rows' weights span the labelled rows' 1 and the pool's
 // b / n, so a long f32 chain drops part of the small terms: at n = 1M, d = 128, c = 100 Round's
 // blocks come out 2e-4 low and its nu 6e-4, and an apply over 400,000 rows and 360 classes
-// carries 3e-5.  That error is part of the results, so the ranges depend on the shape alone and
-// stay as they are (finer ones move those results by more than f32 calls may differ between
-// versions); rows run in order within each.
+// carries 3e-5.  That error is part of the results and finer ranges would move them by as much, so
+// the ranges are those the sums have always had: enough for four blocks per SM at one class a block
+// (four classes at d <= 64), rows in order within each.  They follow the SM count, so another device
+// or a smaller SM budget adds in other ranges.
 void block_ranges(OuterPlan& p, int64_t N, int64_t rows, int d, int c, int sms) {
   const int64_t groups = d > 64 ? c : (c + 3) / 4;
   int64_t n = std::max<int64_t>((4 * (int64_t)sms + groups - 1) / groups, (N + 65535) / 65536);

@@ -213,10 +213,9 @@ int32_t transpose(bool dbl, void* dst, const void* src, int64_t rows, int cols, 
   return FIRAL_OK;
 }
 
-// Class-major copy h^T (c x N) read by the CUDA-core kernels.  FP32 / FP64 problems make it
-// when they are created; a mixed-precision problem needs it only for the FP64-accumulated
-// block sums of Round and makes it on first use (never inside a stream capture: Round and the
-// block-sum entry points are not captured).
+// Class-major copy h^T (c x N), read by the FP64 kernels and by the fused per-point kernels.  FP64
+// problems and mixed problems on the fused kernels make it when they are created (pooled ones only
+// their own pools' classes: class_major_own); FP32 kernels read rows and make none.
 int32_t class_major_h(firal_problem* P) {
   if (P->HaT.p) return FIRAL_OK;
   const size_t vs = P->dbl ? sizeof(double) : sizeof(float);
